@@ -243,6 +243,51 @@ def run(state):
                 seq_lens=s["seq_lens"])
 
 
+# ------------------------------------------------------------------------- 64-bit answer
+def _exact_attn(s):
+    """The attention of `s` in 64 bits: visible keys are the committed prefix and, among the draft
+    nodes, the node itself and all its ancestors."""
+    q, B, N = s["q"], s["q"].shape[0], s["q"].shape[1]
+    Hq, D, Hkv = q.shape[2], q.shape[3], s["draft_k"].shape[2]
+    G = Hq // Hkv
+    ptr, idx, lens = s["parent_ptr"].cpu().numpy(), s["parent_idx"].cpu().numpy(), s["seq_lens"].cpu().numpy()
+    out = torch.empty(q.shape, dtype=torch.float64, device=_DEV)
+    for b in range(B):
+        L = int(lens[b])
+        see = np.eye(N, dtype=bool)
+        for v in range(N):              # (parents come before their children)
+            for p in idx[b, ptr[b, v]:ptr[b, v + 1]]:
+                see[v] |= see[p]
+        hide = ~torch.from_numpy(see).to(_DEV).repeat_interleave(G, 0)
+        for c in range(Hkv):
+            k = torch.cat((s["k_cache"][b, :L, c], s["draft_k"][b, :, c])).double()
+            v = torch.cat((s["v_cache"][b, :L, c], s["draft_v"][b, :, c])).double()
+            x = q[b, :, c * G:(c + 1) * G].reshape(N * G, D).double() @ k.T
+            x *= D ** -0.5
+            x[:, L:].masked_fill_(hide, -math.inf)
+            out[b, :, c * G:(c + 1) * G] = (torch.softmax(x, 1) @ v).view(N, G, D)
+    return out
+
+
+def exact(case, seed):
+    kind = case["kind"]
+    if kind in ("accept", "sampled"):
+        return None                     # whole numbers only
+    s = prepare(case, seed)
+    if kind == "attn":
+        return _exact_attn(s)
+    if kind == "step":
+        return dict(mask=None, out=_exact_attn(s), tokens=None, lens=None, nodes=None, k_cache=None, v_cache=None,
+                    seq_lens=None)
+    B, F, V, k = (case[n] for n in ("B", "F", "V", "k"))
+    n0, Ncap = int(s["n0"][0]), case["Ncap"]
+    prob = torch.zeros((B, Ncap), dtype=torch.float64, device=_DEV)
+    new = torch.softmax(s["logits"].double(), 2).topk(k, 2).values.reshape(B, F * k)
+    prob[:, n0:n0 + F * k] = new[:, :Ncap - n0]
+    return dict(tokens=None, tree_parent=None, merge_to=None, leaf=None, prob=prob, num_nodes=None, new_frontier=None,
+                new_frontier_len=None)
+
+
 def work(case):
     c, kind = case, case["kind"]
     if kind == "draft":
