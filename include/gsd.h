@@ -68,16 +68,16 @@ typedef enum gsd_status {
 
 /* kernel selection for gsd_verify_attn */
 /* GSD_ATTN_AUTO takes the tcgen05 kernel when it supports the shape and the stacked rows of one
- * (sequence, kv head), N * Hq/Hkv, number at least 64; everything else runs on the mma.sync
- * kernel, which reaches roughly a sixth of the tensor throughput (group sizes 3, 6, 12, ... and
- * D == 64 therefore stay correct but slow).  Asking for GSD_ATTN_TCGEN05 on a shape it does
- * not support returns GSD_ERR_UNSUPPORTED. */
+ * (sequence, kv head), N * Hq/Hkv, number at least 64 (head dimension 64 or 128, groups of up to
+ * 128 heads); everything else runs on the mma.sync kernel, which reaches roughly a sixth of the
+ * tensor throughput.  Asking for GSD_ATTN_TCGEN05 by name is answered for D == 128 and group
+ * sizes that divide 128 only; other shapes return GSD_ERR_UNSUPPORTED. */
 #define GSD_ATTN_SPLIT_BALANCED (-1)      /* values of gsd_attn_params.num_splits */
 #define GSD_ATTN_SPLIT_PER_SEQUENCE (-2)
 
 #define GSD_ATTN_AUTO 0
 #define GSD_ATTN_MMA  1            /* warp-level mma.sync kernel: D in {64,128}, any N, any group size */
-#define GSD_ATTN_TCGEN05 2         /* tcgen05/TMEM/TMA kernel: D == 128 and Hq/Hkv a divisor of 128 */
+#define GSD_ATTN_TCGEN05 2         /* tcgen05/TMEM/TMA kernel, by name: D == 128 and Hq/Hkv a divisor of 128 */
 
 typedef struct gsd_attn_params {
     int32_t B;            /* sequences */
@@ -91,7 +91,8 @@ typedef struct gsd_attn_params {
                              GSD_ATTN_SPLIT_BALANCED = equal shares of key tiles per CTA, dealt out on the
                              device from seq_lens; GSD_ATTN_SPLIT_PER_SEQUENCE = a split count per sequence,
                              chosen on the device from seq_lens so that all units are about equally long
-                             (both: tcgen05 kernel; the mma.sync kernel reads them as 0) */
+                             (both: tcgen05 kernel with D == 128 and a group size that divides 128; read
+                             as 0 otherwise) */
     int32_t kernel;       /* GSD_ATTN_AUTO / _MMA / _TCGEN05 */
 } gsd_attn_params;
 

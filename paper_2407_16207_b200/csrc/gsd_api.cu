@@ -47,7 +47,10 @@ static int attn_params_ok(const gsd_attn_params* p) {
 
 int attn_pick_kernel(const gsd_attn_params* p) {
     if (p->kernel != GSD_ATTN_AUTO) return p->kernel;
-    // the TMEM kernel pays off once the stacked rows fill its 128-row tiles
+    // The TMEM kernel pays off once the stacked rows fill its 128-row tiles.  D = 64 and groups
+    // that do not divide 128 ran on the mma.sync kernel before, measured at 5 x 8 groups of 3,
+    // D 128, N 77, L 300-1999: 45.4 us there, 28.5 us here; 4 x 8 groups of 4, D 64, N 128,
+    // L 1000-4000: 81 us there, 42 us here (device time of the whole call).
     const int G = p->Hq / p->Hkv;
     if (attn_tcgen05_supports(p->D, G) && p->N * G >= 64) return GSD_ATTN_TCGEN05;
     return GSD_ATTN_MMA;
@@ -60,7 +63,7 @@ AttnPlan attn_make_plan(const gsd_attn_params* p, int sm_count) {
     const int G = p->Hq / p->Hkv;
     const int R = p->N * G;
     const int bn = tc ? 128 : 64;
-    pl.rows_per_item = tc ? 256 : 64;
+    pl.rows_per_item = tc ? 2 * attn_tcgen05_rows(G) : 64;
     pl.dev.tiles_per_unit = (R + pl.rows_per_item - 1) / pl.rows_per_item;
     pl.items = pl.dev.tiles_per_unit * p->B * p->Hkv;
     const int tiles = (p->Lmax + bn - 1) / bn + (p->N + bn - 1) / bn;
@@ -77,7 +80,8 @@ AttnPlan attn_make_plan(const gsd_attn_params* p, int sm_count) {
     // as much traffic as a key tile), so it pays when the lengths of a batch differ by far
     // more than a share - one long context among short ones - and loses otherwise.
     const int tpu = pl.dev.tiles_per_unit;
-    if (tc && p->num_splits == GSD_ATTN_SPLIT_BALANCED && resident <= 1024 && tpu <= resident &&
+    const bool dev_plans = tc && p->D == 128 && 128 % G == 0;
+    if (dev_plans && p->num_splits == GSD_ATTN_SPLIT_BALANCED && resident <= 1024 && tpu <= resident &&
         (long long)pl.items * tiles < (1ll << 30)) {
         pl.dev.balanced = 1;
         // one group of tpu CTAs (a CTA per row-tile item) per share of the line
@@ -88,7 +92,7 @@ AttnPlan attn_make_plan(const gsd_attn_params* p, int sm_count) {
         pl.ws_bytes = plan_part_o_bytes(pl, p->D) + plan_part_ml_bytes(pl) + plan_bal_bytes(pl, p->B);
         return pl;
     }
-    if (tc && p->num_splits == GSD_ATTN_SPLIT_PER_SEQUENCE && resident <= 1024) {
+    if (dev_plans && p->num_splits == GSD_ATTN_SPLIT_PER_SEQUENCE && resident <= 1024) {
         // split counts per sequence, chosen on the device; persistent CTAs walk the units
         pl.dev.balanced = 2;
         pl.ctas = resident;
@@ -188,6 +192,10 @@ extern "C" int gsd_verify_attn(const void* q, const void* k_cache, const void* v
     if (need > 0) {
         if (!workspace || workspace_bytes < need) return GSD_ERR_WORKSPACE;
         if (((uintptr_t)workspace & 255u) != 0) return GSD_ERR_MISALIGNED;
+    }
+    if (p->kernel == GSD_ATTN_TCGEN05 && 128 % (p->Hq / p->Hkv) != 0) {
+        set_error_text("GSD_ATTN_TCGEN05 needs D == 128 and a group size that divides 128");
+        return GSD_ERR_UNSUPPORTED;
     }
     AttnArgs a;
     a.q = q; a.k_cache = k_cache; a.v_cache = v_cache; a.draft_k = draft_k; a.draft_v = draft_v;

@@ -1,11 +1,13 @@
-// gsd_verify_attn, tcgen05 back end for D = 128 (sm_100a): TMA-fed, TMEM-resident
-// flash-attention over the stacked (draft node x GQA head) rows.
+// gsd_verify_attn, tcgen05 back end (sm_100a): TMA-fed, TMEM-resident flash-attention over the
+// stacked (draft node x GQA head) rows, for head dimensions 64 and 128 and groups of up to 128 heads.
 //
 // Tree attention over the flattened token graph (Sec. 4.1) with the committed prefix in the
 // KV cache (Sec. 4.2): row r = (node r / G, head r % G) of kv head c attends to cache rows
 // j < seq_lens[b] and to the draft rows whose bit is set in the node's ancestor mask.
 //
-// A unit of work is up to two row tiles of 128 stacked rows of one (sequence, kv head) and a
+// A unit of work is up to two row tiles of 128 stacked rows (a group size G that does not divide
+// 128: the 128 / G whole nodes that fit; three heads a group use 126 of the 128 rows) of one
+// (sequence, kv head) and a
 // contiguous range of 128-key tiles (prefix tiles, then the draft tiles that hold a visible
 // key for any of its rows).  Warp roles:
 //   warps 0-3   softmax of stream 0 (thread = row = TMEM lane)
@@ -16,7 +18,8 @@
 // A stream is a row tile (two row tiles: both streams see every key tile) or, for a unit with
 // one row tile, the even / odd key tiles of that row tile (merged in the epilogue).  A job is
 // one key tile of one stream; jobs alternate between the streams.
-// TMEM (512 columns): S (128) | P0 (64) | P1 (64) | O0 (128) | O1 (128).  There is one score
+// TMEM (512 columns) at D = 128: S (128) | P0 (64) | P1 (64) | O0 (128) | O1 (128); the layout at
+// D = 64 is in Geo.  There is one score
 // buffer: QK^T of job k+1 is issued as soon as the softmax of job k has pulled its score row
 // into registers, i.e. it runs under that softmax; P (bf16) has a buffer per stream and
 // O_i += P_i V follows when the softmax hands P over (in two halves of 64 keys).  So neither
@@ -38,13 +41,28 @@ namespace {
 
 constexpr int BM = 128;            // rows per row tile
 constexpr int BN = 128;            // keys per tile
-constexpr int HD = 128;            // head dimension
-constexpr int KST = 2;             // K ring stages
-constexpr int VST = 2;             // V ring stages
+constexpr int kMaxStages = 4;      // ring stages at most (barriers are laid out for this many)
 constexpr uint32_t HALF_BYTES = 128 * 64 * 2;     // one [128 rows][64 bf16] swizzled block
-constexpr uint32_t TILE_BYTES = 2 * HALF_BYTES;   // a 128 x 128 bf16 tile (two column halves)
 constexpr int kThreads = 384;
-constexpr uint32_t kSmemBytes = (2 + KST + VST) * TILE_BYTES + 2 * HALF_BYTES + 1024;  // tiles, output staging, alignment slack
+
+// What depends on the head dimension.  A tile is HD / 64 swizzled blocks of 64 columns.  The
+// rings hold 64 KB of K and as much of V either way: two stages of 32 KB or four of 16 KB.  TMEM
+// columns (32-bit words): a bf16 P tile and an accumulator per stream, and the scores.  With
+// HD = 128 that leaves room for ONE score tile, which the streams share; with HD = 64 the
+// accumulators are half as wide and each stream has its own, so a stream's QK^T only waits for
+// that stream's own softmax (at HD = 64 the exponentials cost twice the tensor time: the softmax
+// warps must never wait).
+template <int HD>
+struct Geo {
+    static constexpr int BLOCKS = HD / 64;
+    static constexpr uint32_t TILE_BYTES = BLOCKS * HALF_BYTES;   // a 128 x HD bf16 tile
+    static constexpr int ST = HD == 128 ? 2 : 4;                  // stages of the K ring and of the V ring
+    static constexpr uint32_t SMEM_BYTES = (2 + 2 * ST) * TILE_BYTES + 2 * HALF_BYTES + 1024;  // tiles, output staging, alignment slack
+    static constexpr bool TWO_S = HD == 64;
+    static constexpr uint32_t COL_S0 = 0, COL_P0 = 128, COL_P1 = 192, COL_O0 = 256, COL_O1 = 256 + HD;
+    static constexpr uint32_t COL_S1 = TWO_S ? 384 : COL_S0;
+    static_assert(COL_O1 + HD <= (TWO_S ? 384 : 512), "512 TMEM columns");
+};
 constexpr float kRescaleThreshold = 8.0f;         // log2 units
 constexpr int kUnitTable = 12;                    // units of work per CTA decoded in the prologue (one per warp)
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // default limit of every in-kernel wait
@@ -62,17 +80,14 @@ struct WaitCtl {
     unsigned long long limit_ns;
 };
 
-// TMEM columns (32-bit words): one score tile, a bf16 P tile per stream, an accumulator per stream
-constexpr uint32_t COL_S = 0, COL_P0 = 128, COL_P1 = 192, COL_O0 = 256, COL_O1 = 384;
-
 enum Bar {
     BAR_Q_FULL = 0,
-    BAR_K_FULL = 1,                   // KST
-    BAR_K_EMPTY = BAR_K_FULL + KST,   // KST
-    BAR_V_FULL = BAR_K_EMPTY + KST,   // VST
-    BAR_V_EMPTY = BAR_V_FULL + VST,   // VST
-    BAR_S_FULL = BAR_V_EMPTY + VST,   // 2: the scores of a job of stream i are in S
-    BAR_S_FREE = BAR_S_FULL + 2,      // 2: the softmax of stream i has read them out of S
+    BAR_K_FULL = 1,                          // one per stage
+    BAR_K_EMPTY = BAR_K_FULL + kMaxStages,   // one per stage
+    BAR_V_FULL = BAR_K_EMPTY + kMaxStages,   // one per stage
+    BAR_V_EMPTY = BAR_V_FULL + kMaxStages,   // one per stage
+    BAR_S_FULL = BAR_V_EMPTY + kMaxStages,   // 2: the scores of a job of stream i are in its S
+    BAR_S_FREE = BAR_S_FULL + 2,      // 2: the softmax of stream i has read them out
     BAR_P_READY = BAR_S_FREE + 2,     // 2: keys 0..63 of P_i are in TMEM
     BAR_P_READY2 = BAR_P_READY + 2,   // 2: keys 64..127 of P_i are in TMEM
     BAR_P_FREE = BAR_P_READY2 + 2,    // 2: the PV of a job of stream i (and all before it) has completed
@@ -92,6 +107,7 @@ struct TcParams {
     float* part_ml;
     int32_t* status;
     int B, N, Hq, Hkv, Lmax, G, W, R;
+    int RT;           // stacked rows a row tile holds: the whole nodes that fit 128 rows, 128 / G * G
     float scale_log2;
     PlanDev plan;
     int total_work;   // CTAs of the plan = units of work
@@ -286,30 +302,38 @@ constexpr uint64_t kDescBase = (1ull << 46) | (2ull << 61);   // descriptor vers
 constexpr uint32_t kDescHi = (uint32_t)((kDescBase | ((uint64_t)(1024 >> 4) << 32)) >> 32);
 __device__ __forceinline__ uint32_t desc_lo_kmajor(uint32_t addr) { return ((addr & 0x3FFFFu) >> 4) | (1u << 16); }
 __device__ __forceinline__ uint32_t desc_lo_mnmajor(uint32_t addr) { return ((addr & 0x3FFFFu) >> 4) | ((HALF_BYTES >> 4) << 16); }
-// instruction descriptors: bf16 x bf16 -> fp32, M = 128, N = 128
+// instruction descriptors: bf16 x bf16 -> fp32, M = 128; N = 128 keys
 constexpr uint32_t kIdescQK = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-constexpr uint32_t kIdescPV = kIdescQK | (1u << 16);   // B (= V) is MN-major
+// O += P V: N = head dimension, B (= V) is MN-major
+template <int HD>
+constexpr uint32_t kIdescPV = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | (((uint32_t)HD >> 3) << 17) | ((128u >> 4) << 24);
 
-// S = A B^T over the head dimension (eight k-steps of 16) as one block issued by one elected
+// S = A B^T over the head dimension (HD / 16 k-steps of 16) as one block issued by one elected
 // lane: per k-step one add per operand and the MMA, nothing else.  alo / blo are the low
-// descriptor words of two K-major [128][128] bf16 tiles (two swizzled 64-column blocks each).
-__device__ __forceinline__ void tc_qk8(uint32_t d_tmem, uint32_t alo, uint32_t blo) {
+// descriptor words of two K-major [128][HD] bf16 tiles (HD / 64 swizzled 64-column blocks each).
+template <int HD>
+__device__ __forceinline__ void tc_qk(uint32_t d_tmem, uint32_t alo, uint32_t blo) {
 #define GSD_QK_STEP(OFF, P)                                                         \
     " add.u32 al, %1, " #OFF ";\n add.u32 bl, %2, " #OFF ";\n"                       \
     " mov.b64 a, {al, %3};\n mov.b64 b, {bl, %3};\n"                                \
     " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, " #P ";\n"
-    asm volatile(
-        "{\n .reg .pred q, pt, pf;\n .reg .b64 a, b;\n .reg .b32 al, bl;\n"
-        " elect.sync _|q, 0xffffffff;\n"
-        " setp.eq.u32 pt, %4, %4;\n setp.ne.u32 pf, %4, %4;\n"
-        GSD_QK_STEP(0, pf) GSD_QK_STEP(2, pt) GSD_QK_STEP(4, pt) GSD_QK_STEP(6, pt)
-        GSD_QK_STEP(1024, pt) GSD_QK_STEP(1026, pt) GSD_QK_STEP(1028, pt) GSD_QK_STEP(1030, pt)
-        "}\n"
-        ::"r"(d_tmem), "r"(alo), "r"(blo), "r"(kDescHi), "r"(kIdescQK) : "memory");
+#define GSD_QK_HEAD                                                                 \
+    "{\n .reg .pred q, pt, pf;\n .reg .b64 a, b;\n .reg .b32 al, bl;\n"             \
+    " elect.sync _|q, 0xffffffff;\n"                                                \
+    " setp.eq.u32 pt, %4, %4;\n setp.ne.u32 pf, %4, %4;\n"                          \
+    GSD_QK_STEP(0, pf) GSD_QK_STEP(2, pt) GSD_QK_STEP(4, pt) GSD_QK_STEP(6, pt)
+    if constexpr (HD == 128)
+        asm volatile(
+            GSD_QK_HEAD GSD_QK_STEP(1024, pt) GSD_QK_STEP(1026, pt) GSD_QK_STEP(1028, pt) GSD_QK_STEP(1030, pt) "}\n"
+            ::"r"(d_tmem), "r"(alo), "r"(blo), "r"(kDescHi), "r"(kIdescQK) : "memory");
+    else
+        asm volatile(GSD_QK_HEAD "}\n" ::"r"(d_tmem), "r"(alo), "r"(blo), "r"(kDescHi), "r"(kIdescQK) : "memory");
+#undef GSD_QK_HEAD
 #undef GSD_QK_STEP
 }
 // O (+)= P V for four k-steps of 16 keys: A = 8 TMEM columns of bf16 pairs per step, B = the
 // MN-major V tile (2048 bytes per 16 keys).  `accum_first` = 0 makes the first step overwrite O.
+template <int HD>
 __device__ __forceinline__ void tc_pv4(uint32_t d_tmem, uint32_t a_tmem, uint32_t blo, uint32_t accum_first) {
 #define GSD_PV_STEP(ACOL, BOFF, P)                                                  \
     " add.u32 at, %1, " #ACOL ";\n add.u32 bl, %2, " #BOFF ";\n mov.b64 b, {bl, %3};\n" \
@@ -320,7 +344,7 @@ __device__ __forceinline__ void tc_pv4(uint32_t d_tmem, uint32_t a_tmem, uint32_
         " setp.eq.u32 pt, %4, %4;\n setp.ne.u32 p0, %5, 0;\n"
         GSD_PV_STEP(0, 0, p0) GSD_PV_STEP(8, 128, pt) GSD_PV_STEP(16, 256, pt) GSD_PV_STEP(24, 384, pt)
         "}\n"
-        ::"r"(d_tmem), "r"(a_tmem), "r"(blo), "r"(kDescHi), "r"(kIdescPV), "r"(accum_first) : "memory");
+        ::"r"(d_tmem), "r"(a_tmem), "r"(blo), "r"(kDescHi), "r"(kIdescPV<HD>), "r"(accum_first) : "memory");
 #undef GSD_PV_STEP
 }
 
@@ -399,10 +423,10 @@ __device__ __forceinline__ UnitInfo unit_info(const TcParams& p, int w, int lane
         plan_decode(p.plan, w, item, u.split, u.nsplit, u.slot);
     }
     const int unit = item / p.plan.tiles_per_unit;
-    u.row0 = (item % p.plan.tiles_per_unit) * (2 * BM);
+    u.row0 = (item % p.plan.tiles_per_unit) * (2 * p.RT);
     u.b = unit / p.Hkv;
     u.c = unit % p.Hkv;
-    u.two = u.row0 + BM < p.R;
+    u.two = u.row0 + p.RT < p.R;
     if (!GSD_IN_BOUNDS(u.b >= 0 && u.b < p.B && u.c < p.Hkv && u.row0 < p.R, p.status)) {
         u.b = 0; u.c = 0; u.row0 = 0; u.two = false;      // checking build only: a unit outside the problem
     }
@@ -411,7 +435,7 @@ __device__ __forceinline__ UnitInfo unit_info(const TcParams& p, int w, int lane
     u.L = L;
     // OR the mask rows of the unit's nodes, one node per lane
     const int n_lo = u.row0 / p.G;
-    const int n_hi = (min(u.row0 + 2 * BM, p.R) - 1) / p.G + 1;
+    const int n_hi = (min(u.row0 + 2 * p.RT, p.R) - 1) / p.G + 1;
     unsigned live = 0;
     const uint32_t tail = (p.N & 31) ? (1u << (p.N & 31)) - 1u : 0xFFFFFFFFu;   // valid bits of the last word
     if ((p.W & 3) == 0 && (reinterpret_cast<uintptr_t>(p.mask) & 15u) == 0) {
@@ -457,11 +481,15 @@ __device__ __forceinline__ UnitInfo unit_info(const TcParams& p, int w, int lane
 // counted across units, so the producer and the QK^T issuer run ahead into the next unit
 // (Q, the first K/V tiles and the first QK^T) while the softmax warps still read out the
 // accumulators of the previous one.
+template <int HD>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_dk,
                const __grid_constant__ CUtensorMap tm_dv, const __grid_constant__ CUtensorMap tm_out,
                const TcParams p) {
+    using T = Geo<HD>;
+    constexpr uint32_t TILE_BYTES = T::TILE_BYTES;
+    constexpr int ST = T::ST;
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long s_bars[BAR_COUNT];
     __shared__ uint32_t s_tmem_base;
@@ -470,13 +498,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     __shared__ UnitInfo s_units[kUnitTable];   // the CTA's first units of work, decoded once up front
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int N = p.N, G = p.G, R = p.R;
+    const int N = p.N, G = p.G, R = p.R, RT = p.RT;
 
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sQ = smem_base;                                   // 2 tiles
-    const uint32_t sK = smem_base + 2 * TILE_BYTES;                  // KST tiles
-    const uint32_t sV = sK + KST * TILE_BYTES;                       // VST tiles
-    const uint32_t sStage = sV + VST * TILE_BYTES;                   // one [128][64] bf16 block per softmax warpgroup
+    const uint32_t sK = smem_base + 2 * TILE_BYTES;                  // ST tiles
+    const uint32_t sV = sK + ST * TILE_BYTES;                        // ST tiles
+    const uint32_t sStage = sV + ST * TILE_BYTES;                   // one [128][64] bf16 block per softmax warpgroup
     const uint32_t bar0 = smem_u32(s_bars);
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
     volatile int* abort_flag = &s_wait.abort;
@@ -489,8 +517,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         mbar_init(bar(BAR_Q_FULL), 1);
         mbar_init(bar(BAR_Q_EMPTY), 1);
         mbar_init(bar(BAR_ML_READY), 4);
-        for (int s = 0; s < KST; ++s) { mbar_init(bar(BAR_K_FULL + s), 1); mbar_init(bar(BAR_K_EMPTY + s), 1); }
-        for (int s = 0; s < VST; ++s) { mbar_init(bar(BAR_V_FULL + s), 1); mbar_init(bar(BAR_V_EMPTY + s), 1); }
+        for (int s = 0; s < ST; ++s) {
+            mbar_init(bar(BAR_K_FULL + s), 1); mbar_init(bar(BAR_K_EMPTY + s), 1);
+            mbar_init(bar(BAR_V_FULL + s), 1); mbar_init(bar(BAR_V_EMPTY + s), 1);
+        }
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar(BAR_S_FULL + i), 1);
             mbar_init(bar(BAR_S_FREE + i), 4);     // one arrival per softmax warp
@@ -506,6 +536,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     if (warp == 10) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&s_tmem_base)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (RT < BM) {
+        // a group size that does not divide 128: the copies of Q never write the last rows of a
+        // tile, whose scores and output rows nobody uses; zeros there keep them finite
+        const int words = (BM - RT) * 32;                  // 128-byte rows of one block
+        for (int t = tid; t < 2 * T::BLOCKS * words; t += kThreads) {
+            const int blk = t / words, w = t - blk * words;
+            *reinterpret_cast<uint32_t*>(smem_raw + (sQ - smem_u32(smem_raw)) + blk * HALF_BYTES + RT * 128 + w * 4) = 0u;
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     // The CTA's units: work indices blockIdx.x, blockIdx.x + gridDim.x, ... of a fixed plan, or
     // a run of the table that the planning kernel (this kernel is its programmatic dependent)
@@ -557,42 +597,42 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 ok = mbar_wait(bar(BAR_Q_EMPTY), (au & 1) ^ 1, abort_flag, p.status);
                 if (ok) {
                     const int ntile_rows = u.two ? 2 : 1;
-                    mbar_expect_tx(bar(BAR_Q_FULL), (uint32_t)ntile_rows * TILE_BYTES);
+                    mbar_expect_tx(bar(BAR_Q_FULL), (uint32_t)(ntile_rows * T::BLOCKS * RT) * 128u);
                     for (int i = 0; i < ntile_rows; ++i)
-                        for (int h = 0; h < 2; ++h)
+                        for (int h = 0; h < T::BLOCKS; ++h)
                             tma_load_4d(sQ + i * TILE_BYTES + h * HALF_BYTES, &tm_q, bar(BAR_Q_FULL), h * 64, u.c * G,
-                                        (u.row0 + i * BM) / G, u.b);
+                                        (u.row0 + i * RT) / G, u.b);
                     q_pending = true;
                 }
                 for (int idx = 0; idx < u.ntiles && ok; ++idx) {
                     const TileInfo ti = tile_info(u.t_begin + idx, u.nPT, u.L, u.live);
                     const CUtensorMap* mk = ti.kind == 2 ? &tm_dk : &tm_k;
                     const CUtensorMap* mv = ti.kind == 2 ? &tm_dv : &tm_v;
-                    const int s = kvc % KST;
-                    const uint32_t par = (uint32_t)((kvc / KST) & 1) ^ 1u;
+                    const int s = kvc % ST;
+                    const uint32_t par = (uint32_t)((kvc / ST) & 1) ^ 1u;
                     ok = mbar_wait(bar(BAR_K_EMPTY + s), par, abort_flag, p.status);
                     if (!ok) break;
                     mbar_expect_tx(bar(BAR_K_FULL + s), TILE_BYTES);
                     if (!(p.withhold_first_k && kvc == 0))   // (test hook: the bytes announced above never arrive)
-                        for (int h = 0; h < 2; ++h)
+                        for (int h = 0; h < T::BLOCKS; ++h)
                             tma_load_4d(sK + s * TILE_BYTES + h * HALF_BYTES, mk, bar(BAR_K_FULL + s), h * 64, u.c, ti.key0, u.b);
                     ok = mbar_wait(bar(BAR_V_EMPTY + s), par, abort_flag, p.status);
                     if (!ok) {
                         // the K copy just issued is still in flight: let it land
-                        mbar_wait_slow(bar(BAR_K_FULL + s), (kvc / KST) & 1, abort_flag, nullptr, true);
+                        mbar_wait_slow(bar(BAR_K_FULL + s), (kvc / ST) & 1, abort_flag, nullptr, true);
                         break;
                     }
                     mbar_expect_tx(bar(BAR_V_FULL + s), TILE_BYTES);
-                    for (int h = 0; h < 2; ++h)
+                    for (int h = 0; h < T::BLOCKS; ++h)
                         tma_load_4d(sV + s * TILE_BYTES + h * HALF_BYTES, mv, bar(BAR_V_FULL + s), h * 64, u.c, ti.key0, u.b);
                     ++kvc;
                 }
                 if (!ok) {
                     // gave up: let the copies already in flight land before the CTA retires
                     if (q_pending) mbar_wait_slow(bar(BAR_Q_FULL), au & 1, abort_flag, nullptr, true);
-                    for (int t = max(0, kvc - KST); t < kvc; ++t) {
-                        mbar_wait_slow(bar(BAR_K_FULL + t % KST), (t / KST) & 1, abort_flag, nullptr, true);
-                        mbar_wait_slow(bar(BAR_V_FULL + t % VST), (t / VST) & 1, abort_flag, nullptr, true);
+                    for (int t = max(0, kvc - ST); t < kvc; ++t) {
+                        mbar_wait_slow(bar(BAR_K_FULL + t % ST), (t / ST) & 1, abort_flag, nullptr, true);
+                        mbar_wait_slow(bar(BAR_V_FULL + t % ST), (t / ST) & 1, abort_flag, nullptr, true);
                     }
                 }
             }
@@ -611,9 +651,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         int s_owner = -1;         // stream whose scores were last written to S
         bool ok = true;
         auto wait = [&](int b, uint32_t par) -> bool { return mbar_wait_warp(bar(b), par, abort_flag, p.status); };
-        static_assert(KST == 2, "two K stages are selected by a flag");
         const uint32_t qlo0 = desc_lo_kmajor(sQ), qlo1 = desc_lo_kmajor(sQ + TILE_BYTES);
-        const uint32_t klo0 = desc_lo_kmajor(sK), klo1 = desc_lo_kmajor(sK + TILE_BYTES);
+        const uint32_t klo0 = desc_lo_kmajor(sK);       // (stage st: + st * TILE_BYTES / 16)
         for (int it = 0; it < n_my && ok; ++it) {
             const UnitInfo u = unit_of(it);
             if (u.ntiles == 0) continue;
@@ -622,16 +661,19 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             ok = wait(BAR_Q_FULL, au & 1);
             for (int k = 0; k < njobs && ok; ++k) {
                 const int i = k & 1;
-                const int r = kvc + (two ? (k >> 1) : k), st = r % KST;
+                const int r = kvc + (two ? (k >> 1) : k), st = r % ST;
                 if (!two || i == 0) {
-                    if (!(ok = wait(BAR_K_FULL + st, (r / KST) & 1))) break;
+                    if (!(ok = wait(BAR_K_FULL + st, (r / ST) & 1))) break;
                 }
-                if (s_owner >= 0) {
+                if (T::TWO_S) {
+                    // the scores of the stream's previous job must have left its S
+                    if ((i ? jq1 : jq0) > 0 && !(ok = wait(BAR_S_FREE + i, (uint32_t)((i ? jq1 : jq0) - 1) & 1u))) break;
+                } else if (s_owner >= 0) {
                     // the previous job's scores must have left S
                     if (!(ok = wait(BAR_S_FREE + s_owner, (uint32_t)((s_owner ? jq1 : jq0) - 1) & 1u))) break;
                 }
                 tc_fence_after();
-                tc_qk8(tmem + COL_S, (two && i) ? qlo1 : qlo0, st ? klo1 : klo0);
+                tc_qk<HD>(tmem + (i ? T::COL_S1 : T::COL_S0), (two && i) ? qlo1 : qlo0, klo0 + (uint32_t)st * (TILE_BYTES >> 4));
                 tc_commit(bar(BAR_S_FULL + i));
                 if (!two || i == 1) tc_commit(bar(BAR_K_EMPTY + st));
                 if (k == njobs - 1) tc_commit(bar(BAR_Q_EMPTY));   // every QK^T of the unit is issued
@@ -657,8 +699,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         int jp0 = 0, jp1 = 0;     // jobs issued per stream so far (phase of P_READY / P_FREE)
         bool ok = true;
         auto wait = [&](int b, uint32_t par) -> bool { return mbar_wait_warp(bar(b), par, abort_flag, p.status); };
-        static_assert(VST == 2, "two V stages are selected by a flag");
-        const uint32_t vlo0 = desc_lo_mnmajor(sV), vlo1 = desc_lo_mnmajor(sV + TILE_BYTES);
+        const uint32_t vlo0 = desc_lo_mnmajor(sV);      // (stage st: + st * TILE_BYTES / 16)
         for (int it = 0; it < n_my && ok; ++it) {
             const UnitInfo u = unit_of(it);
             if (u.ntiles == 0) continue;
@@ -667,13 +708,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             const int n1 = two ? u.ntiles : u.ntiles / 2;      // jobs of stream 1
             for (int k = 0; k < njobs && ok; ++k) {
                 const int i = k & 1;
-                const int r = kvc + (two ? (k >> 1) : k), st = r % VST;
+                const int r = kvc + (two ? (k >> 1) : k), st = r % ST;
                 const bool first = k < 2;                      // first job of its stream in this unit
                 const uint32_t par = (uint32_t)(i ? jp1 : jp0) & 1u;
-                const uint32_t vlo = st ? vlo1 : vlo0;
-                const uint32_t tP = tmem + (i ? COL_P1 : COL_P0), tO = tmem + (i ? COL_O1 : COL_O0);
+                const uint32_t vlo = vlo0 + (uint32_t)st * (TILE_BYTES >> 4);
+                const uint32_t tP = tmem + (i ? T::COL_P1 : T::COL_P0), tO = tmem + (i ? T::COL_O1 : T::COL_O0);
                 if (!two || i == 0) {
-                    if (!(ok = wait(BAR_V_FULL + st, (r / VST) & 1))) break;
+                    if (!(ok = wait(BAR_V_FULL + st, (r / ST) & 1))) break;
                 }
                 if (!(ok = wait(BAR_P_READY + i, par))) break;
                 if (first && (i ? au1 : au) > 0) {
@@ -681,10 +722,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     if (!(ok = wait(BAR_O_FREE + i, (uint32_t)((i ? au1 : au) - 1) & 1u))) break;
                 }
                 tc_fence_after();
-                tc_pv4(tO, tP, vlo, first ? 0u : 1u);
+                tc_pv4<HD>(tO, tP, vlo, first ? 0u : 1u);
                 if (!(ok = wait(BAR_P_READY2 + i, par))) break;
                 tc_fence_after();
-                tc_pv4(tO, tP + 32, vlo + 4 * 128, 1u);
+                tc_pv4<HD>(tO, tP + 32, vlo + 4 * 128, 1u);
                 tc_commit(bar(BAR_P_FREE + i));
                 if (!two || i == 1) tc_commit(bar(BAR_V_EMPTY + st));
                 if (k + 2 >= njobs) tc_commit(bar(BAR_O_DONE + i));   // the stream's last job of the unit
@@ -705,9 +746,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         const int i = warp >> 2;                         // stream of this warpgroup
         const int rloc = (warp & 3) * 32 + lane;         // row inside the tile = TMEM lane
         const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t tS = tmem + lane_addr + COL_S;
-        const uint32_t tP = tmem + lane_addr + (i ? COL_P1 : COL_P0);
-        const uint32_t tO = tmem + lane_addr + (i ? COL_O1 : COL_O0);
+        const uint32_t tS = tmem + lane_addr + (i ? T::COL_S1 : T::COL_S0);
+        const uint32_t tP = tmem + lane_addr + (i ? T::COL_P1 : T::COL_P0);
+        const uint32_t tO = tmem + lane_addr + (i ? T::COL_O1 : T::COL_O0);
         int kvc = 0;      // key tiles of all non-empty units so far (ring position of the V tiles)
         int tcnt = 0;     // jobs this stream has processed so far (barrier phase)
         int auc = 0;      // non-empty units this stream has finished so far (barrier phase)
@@ -723,8 +764,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             const int my_n = alt ? (i == 0 ? (ntiles + 1) / 2 : ntiles / 2) : ntiles;
             const int n1 = alt ? ntiles / 2 : ntiles;           // tiles of stream 1 in this unit
             const int b = u.b, c = u.c;
-            const int row = u.row0 + (alt ? 0 : i * BM) + rloc;
-            const bool rvalid = row < R;
+            const int row = u.row0 + (alt ? 0 : i * RT) + rloc;
+            const bool rvalid = rloc < RT && row < R;
             if (warp == 0 && lane == 0) {
                 const int Lraw = p.seq_lens[b];
                 if ((Lraw < 0 || Lraw > p.Lmax) && p.status) atomicOr((unsigned*)p.status, GSD_DEV_BAD_SEQ_LEN);
@@ -796,7 +837,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     if (!ok) break;
                     tc_fence_after();
 #pragma unroll 1
-                    for (int ch = 0; ch < 4; ++ch) {
+                    for (int ch = 0; ch < HD / 32; ++ch) {
                         float v[32];
                         tc_ld32(tO + ch * 32, v);
                         tc_wait_ld();
@@ -890,7 +931,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (ntiles > 0) {
                 tc_fence_after();
 #pragma unroll
-                for (int ch = 0; ch < 4; ++ch) tc_ld32p(tO + ch * 32, acc + ch * 32);
+                for (int ch = 0; ch < HD / 32; ++ch) tc_ld32p(tO + ch * 32, acc + ch * 32);
                 tc_wait_ld();
                 if (alt && n1 > 0) {
                     // merge the odd-tile stream: O = w0 O0 + w1 O1, l = w0 l0 + w1 l1 at the common maximum
@@ -898,9 +939,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     const float m = fmaxf(m_ref, ml1.x);
                     const float m_use = m == -CUDART_INF_F ? 0.f : m;
                     const float w0 = fast_exp2(m_ref - m_use), w1 = fast_exp2(ml1.x - m_use);
-                    const uint32_t tO1 = tmem + lane_addr + COL_O1;
+                    const uint32_t tO1 = tmem + lane_addr + T::COL_O1;
 #pragma unroll
-                    for (int ch = 0; ch < 4; ++ch) {
+                    for (int ch = 0; ch < HD / 32; ++ch) {
                         float v[32];
                         tc_ld32(tO1 + ch * 32, v);
                         tc_wait_ld();
@@ -929,7 +970,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 unsigned char* srow = smem_raw + (stage - smem_u32(smem_raw)) + rloc * 128;
                 const bool issuer = (warp & 3) == 0 && lane == 0;
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
+                for (int h = 0; h < T::BLOCKS; ++h) {
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
                         const int e = h * 64 + k * 8;
@@ -943,7 +984,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     wg_barrier(1 + i);
                     if (issuer) {
-                        tma_store_4d(&tm_out, stage, h * 64, c * G, (u.row0 + (alt ? 0 : i * BM)) / G, b);
+                        tma_store_4d(&tm_out, stage, h * 64, c * G, (u.row0 + (alt ? 0 : i * RT)) / G, b);
                         bulk_commit();
                         bulk_wait_read();          // the staging block may be overwritten again
                     }
@@ -951,7 +992,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 }
             } else if (rvalid) {
                 {
-                    const size_t prow = (size_t)u.slot * (2 * BM) + (alt ? 0 : i * BM) + rloc;
+                    const size_t prow = (size_t)u.slot * (2 * RT) + (alt ? 0 : i * RT) + rloc;
                     if (GSD_IN_BOUNDS(u.slot >= 0 && u.slot < p.slots, p.status)) {
                     float* dst = p.part_o + prow * HD;
 #pragma unroll
@@ -1001,7 +1042,7 @@ EncodeTiledFn encode_fn() {
 }
 
 // [d3][d2][d1][D] bf16 tensor; box = 64 columns x box1 x box2 x 1, 128-byte swizzle, zero fill
-int make_map(CUtensorMap* m, const void* base, uint64_t d1, uint64_t d2, uint64_t d3, uint32_t box1, uint32_t box2) {
+int make_map(CUtensorMap* m, const void* base, uint64_t HD, uint64_t d1, uint64_t d2, uint64_t d3, uint32_t box1, uint32_t box2) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return GSD_ERR_CUDA;
     const cuuint64_t dims[4] = {(cuuint64_t)HD, d1, d2, d3};
@@ -1022,34 +1063,30 @@ int make_map(CUtensorMap* m, const void* base, uint64_t d1, uint64_t d2, uint64_
 
 }  // namespace
 
-bool attn_tcgen05_supports(int D, int G) { return D == HD && G >= 1 && G <= BM && BM % G == 0; }
-
-int launch_attn_tcgen05(const AttnArgs& a) {
-    if (!attn_tcgen05_supports(a.D, a.G)) {
-        set_error_text("tcgen05 back end needs D == 128 and a group size that divides 128");
-        return GSD_ERR_UNSUPPORTED;
-    }
+template <int HD>
+static int launch_tc(const AttnArgs& a) {
+    const int nodes = BM / a.G;           // whole nodes of a row tile
     CUtensorMap tq, tk, tv, tdk, tdv, tout;
     int rc;
-    if ((rc = make_map(&tq, a.q, a.Hq, a.N, a.B, a.G, BM / a.G)) != GSD_OK) return rc;
-    if ((rc = make_map(&tk, a.k_cache, a.Hkv, a.Lmax, a.B, 1, BN)) != GSD_OK) return rc;
-    if ((rc = make_map(&tv, a.v_cache, a.Hkv, a.Lmax, a.B, 1, BN)) != GSD_OK) return rc;
-    if ((rc = make_map(&tdk, a.draft_k, a.Hkv, a.N, a.B, 1, BN)) != GSD_OK) return rc;
-    if ((rc = make_map(&tdv, a.draft_v, a.Hkv, a.N, a.B, 1, BN)) != GSD_OK) return rc;
-    if ((rc = make_map(&tout, a.out, a.Hq, a.N, a.B, a.G, BM / a.G)) != GSD_OK) return rc;
+    if ((rc = make_map(&tq, a.q, HD, a.Hq, a.N, a.B, a.G, nodes)) != GSD_OK) return rc;
+    if ((rc = make_map(&tk, a.k_cache, HD, a.Hkv, a.Lmax, a.B, 1, BN)) != GSD_OK) return rc;
+    if ((rc = make_map(&tv, a.v_cache, HD, a.Hkv, a.Lmax, a.B, 1, BN)) != GSD_OK) return rc;
+    if ((rc = make_map(&tdk, a.draft_k, HD, a.Hkv, a.N, a.B, 1, BN)) != GSD_OK) return rc;
+    if ((rc = make_map(&tdv, a.draft_v, HD, a.Hkv, a.N, a.B, 1, BN)) != GSD_OK) return rc;
+    if ((rc = make_map(&tout, a.out, HD, a.Hq, a.N, a.B, a.G, nodes)) != GSD_OK) return rc;
     TcParams p;
     p.mask = a.mask; p.seq_lens = a.seq_lens; p.out = (__nv_bfloat16*)a.out; p.status = a.status;
     p.B = a.B; p.N = a.N; p.Hq = a.Hq; p.Hkv = a.Hkv; p.Lmax = a.Lmax; p.G = a.G; p.W = a.W;
-    p.R = a.N * a.G; p.scale_log2 = a.scale_log2; p.plan = a.plan.dev;
+    p.R = a.N * a.G; p.RT = nodes * a.G; p.scale_log2 = a.scale_log2; p.plan = a.plan.dev;
     p.part_o = (float*)a.workspace;
     p.part_ml = (float*)((char*)a.workspace + plan_part_o_bytes(a.plan, a.D));
     {
-        // the opt-in for large dynamic shared memory is per device and sticks: do it once
+        // the opt-in for large dynamic shared memory is per kernel and device and sticks: do it once
         static bool done[64] = {};
         int dev = 0;
         GSD_CUDA_TRY(cudaGetDevice(&dev));
         if (dev < 0 || dev >= 64 || !done[dev]) {
-            GSD_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
+            GSD_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<HD>::SMEM_BYTES));
             if (dev >= 0 && dev < 64) done[dev] = true;
         }
     }
@@ -1075,20 +1112,32 @@ int launch_attn_tcgen05(const AttnArgs& a) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)a.plan.ctas);
         cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = kSmemBytes;
+        cfg.dynamicSmemBytes = Geo<HD>::SMEM_BYTES;
         cfg.stream = a.stream;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel, tq, tk, tv, tdk, tdv, tout, p));
+        GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD>, tq, tk, tv, tdk, tdv, tout, p));
         return GSD_OK;
     }
     dim3 grid(a.plan.ctas < di.sm_count ? a.plan.ctas : di.sm_count);
-    attn_tc_kernel<<<grid, kThreads, kSmemBytes, a.stream>>>(tq, tk, tv, tdk, tdv, tout, p);
+    attn_tc_kernel<HD><<<grid, kThreads, Geo<HD>::SMEM_BYTES, a.stream>>>(tq, tk, tv, tdk, tdv, tout, p);
     GSD_CUDA_TRY(cudaGetLastError());
     return GSD_OK;
+}
+
+int attn_tcgen05_rows(int G) { return G <= BM ? BM / G * G : BM; }
+
+bool attn_tcgen05_supports(int D, int G) { return (D == 128 || D == 64) && G >= 1 && G <= BM; }
+
+int launch_attn_tcgen05(const AttnArgs& a) {
+    if (!attn_tcgen05_supports(a.D, a.G)) {
+        set_error_text("tcgen05 back end needs a head dimension of 64 or 128 and a group size of at most 128");
+        return GSD_ERR_UNSUPPORTED;
+    }
+    return a.D == 128 ? launch_tc<128>(a) : launch_tc<64>(a);
 }
 
 void debug_attn_wait(unsigned long long limit_ns, int withhold_first_k) {

@@ -73,7 +73,7 @@ struct PlanDev {
 };
 struct AttnPlan {
     int kernel;         // GSD_ATTN_MMA or GSD_ATTN_TCGEN05
-    int rows_per_item;  // 64 (mma.sync back end) or 256 (tcgen05 back end)
+    int rows_per_item;  // 64 (mma.sync back end) or two row tiles of attn_tcgen05_rows(G) (tcgen05 back end)
     int items;
     int ctas;
     int slots;          // partial-result slots; 0 when nothing is split
@@ -167,6 +167,7 @@ int launch_attn_plan(const AttnArgs& a);      // plans made on the device only: 
 int launch_attn_mma(const AttnArgs& a);
 int launch_attn_tcgen05(const AttnArgs& a);
 bool attn_tcgen05_supports(int D, int G);
+int attn_tcgen05_rows(int G);                 // stacked rows of one row tile
 int launch_attn_merge(const AttnArgs& a);
 // test hook behind gsd_debug_attn_wait (process-wide; 0 restores the default limit)
 void debug_attn_wait(unsigned long long limit_ns, int withhold_first_k);

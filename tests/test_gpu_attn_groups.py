@@ -1,0 +1,61 @@
+"""The tcgen05 attention kernel at head dimension 64 and at group sizes that do not divide 128, as
+the automatic choice takes it, against the fp64 oracle.  Same tolerance as tests/test_gpu_attn.py
+(bf16 output against fp64); sizes sit at the edges of row tiles (128 // G whole nodes of G heads
+each) and of key tiles, with NaN behind every sequence end."""
+import numpy as np
+import pytest
+
+import gsd_inputs as gi
+from gpu_util import out_to_f64
+from test_gpu_attn import assert_close_scaled, cpu_attn, gpu_attn
+
+pytestmark = pytest.mark.gpu
+
+CASES = []
+for _D in (64, 128):
+    for _G in (1, 3, 5, 7, 8, 12, 48, 96, 128):
+        if _D == 128 and 128 % _G == 0:
+            continue
+        _nodes = 128 // _G                       # nodes of a row tile
+        for _N in sorted({max(1, -(-64 // _G)), _nodes, _nodes + 1, 2 * _nodes, 2 * _nodes + 1, 5 * _nodes - 1}):
+            if _N * _G >= 64 and _N <= 300:
+                CASES.append((_D, _G, _N))
+
+
+@pytest.mark.parametrize("D,G,N", CASES, ids=[f"D{d}_G{g}_N{n}" for d, g, n in CASES])
+def test_row_tile_edges(D, G, N):
+    lens = np.array([0, 1, 127, 128, 129, 300], dtype=np.int32)
+    depth = 0 if N == 1 else int(np.ceil(np.log(2 * N + 1) / np.log(3))) + 1
+    cfg = gi.VerifyConfig("t", 7, len(lens), 2 * G, 2, D, 300, N, min(depth, N - 1), 3, 2, 8, 8, 0.5)
+    inp = gi.make_inputs(cfg, 100 * G + N, accept=False)
+    inp["seq_lens"][:] = lens
+    for b, n in enumerate(lens):
+        inp["k_cache"][b, int(n):] = 0x7FC0
+        inp["v_cache"][b, int(n):] = 0x7FC0
+    want = cpu_attn(inp)
+    for splits in (0, 1, 3):
+        assert_close_scaled(out_to_f64(gpu_attn(inp, num_splits=splits)), want)
+
+
+@pytest.mark.parametrize("D,G,Hkv,L,N", [(64, 4, 8, (1000, 4000), 128), (64, 1, 12, 1537, 77), (128, 3, 8, (300, 1999), 77),
+                                         (128, 7, 4, 4097, 200)])
+def test_many_tiles_per_unit(D, G, Hkv, L, N):
+    # rings and barrier phases wrap many times, several units per CTA, split items and their merge
+    cfg = gi.VerifyConfig("t", 7, 4, G * Hkv, Hkv, D, L, N, 10, 4, 3, 8, 8, 0.5)
+    inp = gi.make_inputs(cfg, 11, accept=False, pad_fill="nan")
+    assert_close_scaled(out_to_f64(gpu_attn(inp)), cpu_attn(inp))
+
+
+def test_score_jumps_at_head_dimension_64():
+    # one cache key far above the rest from some tile on: the accumulators are rescaled in place
+    cfg = gi.VerifyConfig("t", 7, 1, 8, 1, 64, 700, 130, 10, 4, 3, 8, 8, 0.5)
+    inp = gi.make_inputs(cfg, 3, accept=False)
+    k, q = gi.bf16_bits_to_f32(inp["k_cache"]), gi.bf16_bits_to_f32(inp["q"])
+    q[0, :, :, 5] = 24.0
+    k[0, :, 0, 5] = 0.0
+    k[0, 300, 0, 5] = 5.0
+    k[0, 650, 0, 5] = 17.0
+    inp["q"], inp["k_cache"] = gi.f32_to_bf16_bits(q), gi.f32_to_bf16_bits(k)
+    dk = gi.bf16_bits_to_f32(inp["draft_k"]); dk[0, :, 0, 5] = 0.0
+    inp["draft_k"] = gi.f32_to_bf16_bits(dk)
+    assert_close_scaled(out_to_f64(gpu_attn(inp)), cpu_attn(inp))
