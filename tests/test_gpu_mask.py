@@ -40,3 +40,26 @@ def test_bad_edges_are_ignored_and_flagged():
     got = gpu_mask(ptr, idx, status)
     assert np.array_equal(got, oracle.build_mask(ptr, idx))
     assert int(status.item()) == 0x1
+
+
+@pytest.mark.parametrize("N,deg", [(33, 6), (100, 3), (512, 9), (512, 1)])
+def test_mask_with_many_parents(N, deg):
+    # more parents per node than sit in registers, more edges than the on-chip copy holds, repeated
+    # and invalid parents
+    rng = np.random.default_rng(N + deg)
+    ptr = np.zeros((2, N + 1), np.int32)
+    idx = np.zeros((2, N * deg), np.int32)
+    for b in range(2):
+        n = 0
+        for v in range(N):
+            d = int(rng.integers(0, deg + 1)) if v else 0
+            idx[b, n:n + d] = rng.integers(max(0, v - 40), v, size=d) if d else 0
+            n += d
+            ptr[b, v + 1] = n
+    for flagged in (False, True):
+        if flagged:
+            idx[1, ptr[1, N] - 1] = N + 3
+            idx[1, ptr[1, N // 2]] = -2
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        assert np.array_equal(gpu_mask(ptr, idx, status), oracle.build_mask(ptr, idx))
+        assert int(status.item()) == (1 if flagged else 0)
