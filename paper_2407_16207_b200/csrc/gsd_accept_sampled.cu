@@ -11,12 +11,13 @@
 //
 // Two launches.  Grid (slices, B*N): each CTA streams one slice of one logits row with 16-byte
 // loads; each of its warps owns a contiguous eighth of the slice and keeps a running
-// (maximum, sum of exponentials) pair, which it leaves in scratch.  The second launch (one CTA
-// per sequence, a programmatic dependent of the first, so it is resident when the stream ends)
-// combines the pairs per node, tests the steps, runs the level-synchronous longest-path
-// relaxation, walks back, and finds the regenerated token: range sums (for P those in scratch;
-// for the residual eight range sums formed on the spot from the two rows of the end node) give
-// the range of the crossing, a block-wide scan over that range gives the index.
+// (maximum, sum of exponentials) pair, which it leaves in scratch.  The second launch (a cluster
+// of up to eight CTAs per sequence, a programmatic dependent of the first, so it is resident when
+// the stream ends): the leading CTA combines the pairs per node, tests the steps, runs the
+// level-synchronous longest-path relaxation and walks back; then the regenerated token: range sums
+// (for P those in scratch; for the residual one per warp of the cluster, formed on the spot from
+// the two rows of the end node and exchanged through distributed shared memory) give the range of
+// the crossing, a block-wide scan over that range gives the index.
 #include "gsd_internal.cuh"
 #include "gsd_path.cuh"
 #include <math_constants.h>
@@ -69,16 +70,23 @@ __device__ __forceinline__ void take1(Ms& r, float x) {
 }
 
 // The row is cut into slices (one CTA each) and every slice into kWarps contiguous ranges (one
-// warp each); in units of float4 when the row is read that way.  Range r = slice * kWarps + warp.
-__device__ __forceinline__ void range_of(int V, int slices, int vec, int r, int& lo, int& hi) {
-    const int unit = vec ? 4 : 1, n = vec ? (V >> 2) : V;
-    const int per = (n + slices - 1) / slices;
+// warp each), in units of the row's 16-byte groups; the first range has the entries before the
+// first 16-byte boundary too, the last one those behind the last group.  Range r = slice * kWarps + warp.
+struct Range {
+    int a0, a1;    // groups
+    int lo, hi;    // entries
+};
+__device__ __forceinline__ Range range_of(RowSpan sp, int V, int slices, int r) {
+    const int per = (sp.nvec + slices - 1) / slices;
     const int slice = r / kWarps, warp = r % kWarps;
-    const int v0 = min(slice * per, n), v1 = min(v0 + per, n);
+    const int v0 = min(slice * per, sp.nvec), v1 = min(v0 + per, sp.nvec);
     const int wlen = (v1 - v0 + kWarps - 1) / kWarps;
-    const int a0 = min(v0 + warp * wlen, v1), a1 = min(a0 + wlen, v1);
-    lo = a0 * unit;
-    hi = a1 * unit;
+    Range g;
+    g.a0 = min(v0 + warp * wlen, v1);
+    g.a1 = min(g.a0 + wlen, v1);
+    g.lo = r == 0 ? 0 : sp.head + g.a0 * 4;
+    g.hi = r == slices * kWarps - 1 ? V : sp.head + g.a1 * 4;
+    return g;
 }
 
 struct SampledArgs {
@@ -96,8 +104,35 @@ struct SampledArgs {
     float2* part;     // [B*N][slices][kWarps] (maximum, sum) of contiguous ranges of the row, in order
     int32_t* status;
     int B, N, V, Ecap, Tcap, slices;
-    int vec;          // rows are read as float4 (decides where the slices of a row begin)
-    int dvec;         // the rows of the draft logits can be read as float4 too
+    int cluster;      // CTAs of the second launch per sequence
+};
+
+// ---- thread-block cluster of the second launch
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ int cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return (int)r;
+}
+// writes `v` to the place of *dst in CTA `rank` of the cluster
+__device__ __forceinline__ void put_remote(void* dst, int rank, uint32_t v) {
+    uint32_t at;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(dst)), "r"(rank));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+}
+
+// four consecutive entries of a row; `vec`: they start on a 16-byte boundary
+__device__ __forceinline__ float4 load4(const float* p, bool vec) {
+    return vec ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+}
+
+constexpr int kMaxCluster = 8;
+
+// What the leading CTA finds out and the others of the cluster need.
+struct Outcome {
+    int edges, end, end_has_child;
+    float mx, sum;
 };
 
 __device__ void finish_sequence(const SampledArgs& a, int b) {
@@ -107,9 +142,14 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
     __shared__ int s_red[kThreads / 32];
     __shared__ float s_scan[kThreads / 32];
     __shared__ float s_rm[kThreads / 32];
+    __shared__ float s_cm[kMaxCluster], s_cs[kMaxCluster];
     __shared__ float s_rsum[kMaxSlices * kWarps];
+    __shared__ Outcome s_outcome;
     __shared__ int s_pick;
-    const int N = a.N, V = a.V, tid = threadIdx.x;
+    const int C = a.cluster, rank = C > 1 ? cluster_rank() : 0;
+    static_assert(kMaxCluster <= kMaxSlices, "one range sum per warp of the cluster");
+    cluster_arrive();                    // (every CTA has started before any writes to another)
+    const int N = a.N, V = a.V, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int32_t* tok = a.tok + (size_t)b * N;
     const float* lg = a.logits + (size_t)b * N * V;
     const float* q = a.q + (size_t)b * N;
@@ -121,20 +161,36 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
     auto combine_pairs = [&]() -> unsigned {
         unsigned flags = 0;
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        for (int v = tid; v < N; v += kThreads) {
+        // a node's pairs are shared by up to four neighbouring threads when there are fewer nodes than
+        // threads: with few rows the rows are cut into many slices, and one thread per node had 128
+        // pairs to go through (2 sequences of N 40, V 128256: 3.7 us of the call)
+        const int tpn = 4 * N <= kThreads ? 4 : 2 * N <= kThreads ? 2 : 1;
+        const int quads = a.slices * (kWarps / 2) / tpn;               // float4s (two pairs each) of one thread
+        for (int t = tid; t < (N * tpn + 31) / 32 * 32; t += kThreads) {
+            const int v = min(t / tpn, N - 1);
             // the pairs were written by other CTAs: read them past L1
             Ms r{-CUDART_INF_F, 0.f};
-            const float4* pp = reinterpret_cast<const float4*>(a.part + ((size_t)b * N + v) * a.slices * kWarps);
-            for (int k = 0; k < a.slices * (kWarps / 2); k += 4) {     // eight pairs (64 bytes) per round, loaded at once
-                float4 t[4];
+            const float4* pp = reinterpret_cast<const float4*>(a.part + ((size_t)b * N + v) * a.slices * kWarps) + (t % tpn) * quads;
+            for (int k = 0; k < quads; k += 4) {                       // eight pairs (64 bytes) per round, loaded at once
+                float4 p[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) t[i] = __ldcg(pp + k + i);
+                for (int i = 0; i < 4; ++i) p[i] = k + i < quads ? __ldcg(pp + k + i) : make_float4(-CUDART_INF_F, 0.f, -CUDART_INF_F, 0.f);
+                float m = r.m;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    r = combine(r, Ms{t[i].x, t[i].y});
-                    r = combine(r, Ms{t[i].z, t[i].w});
-                }
+                for (int i = 0; i < 4; ++i) m = fmaxf(m, fmaxf(p[i].x, p[i].z));
+                if (m == -CUDART_INF_F) continue;
+                float s = r.s * ex2((r.m - m) * kLog2e);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) s += p[i].y * ex2((p[i].x - m) * kLog2e) + p[i].w * ex2((p[i].z - m) * kLog2e);
+                r = Ms{m, s};
             }
+            for (int o = 1; o < tpn; o *= 2) {
+                Ms other;
+                other.m = __shfl_xor_sync(0xFFFFFFFFu, r.m, o);
+                other.s = __shfl_xor_sync(0xFFFFFFFFu, r.s, o);
+                r = combine(r, other);
+            }
+            if (t >= N * tpn || t % tpn != 0) continue;
             s_mx[v] = r.m;
             s_sum[v] = r.s;
             s_uq[v] = u[v] * q[v];       // the left side of the step test, fetched beside the pairs
@@ -142,66 +198,84 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
         }
         return flags;
     };
-    PathIo io;
-    io.tok = tok;
-    io.pptr = a.pptr + (size_t)b * (N + 1);
-    io.pidx = a.pidx + (size_t)b * a.Ecap;
-    io.out_tok = a.out_tok + (size_t)b * a.Tcap;
-    io.out_nodes = a.out_nodes ? a.out_nodes + (size_t)b * a.Tcap : nullptr;
-    io.out_len = a.out_len + b;
-    io.status = a.status;
-    io.N = N; io.V = V; io.Ecap = a.Ecap; io.Tcap = a.Tcap;
-    // the test of one step: the target's probability of v's token under its parent p (one
-    // logit gathered from global memory) against u q
-    const PathResult res = longest_accepted_path_ex<true>(
-        io, 0u,
-        [&](float logit, int p, int v) { return s_uq[v] < ex2((logit - s_mx[p]) * kLog2e) / s_sum[p]; },
-        [&](int p, int v) -> float {
-            if (!GSD_IN_BOUNDS(p >= 0 && p < N && tok[v] >= 0 && tok[v] < V, a.status)) return -CUDART_INF_F;
-            return lg[(size_t)p * V + tok[v]];
-        },
-        combine_pairs);
-    const int s_m = res.edges, s_end = res.end;
-    int32_t* out_tok = io.out_tok;
+    int32_t* out_tok = a.out_tok + (size_t)b * a.Tcap;
+    if (rank == 0) {
+        PathIo io;
+        io.tok = tok;
+        io.pptr = a.pptr + (size_t)b * (N + 1);
+        io.pidx = a.pidx + (size_t)b * a.Ecap;
+        io.out_tok = out_tok;
+        io.out_nodes = a.out_nodes ? a.out_nodes + (size_t)b * a.Tcap : nullptr;
+        io.out_len = a.out_len + b;
+        io.status = a.status;
+        io.N = N; io.V = V; io.Ecap = a.Ecap; io.Tcap = a.Tcap;
+        // the test of one step: the target's probability of v's token under its parent p (one
+        // logit gathered from global memory) against u q
+        const PathResult res = longest_accepted_path_ex<true>(
+            io, 0u,
+            [&](float logit, int p, int v) { return s_uq[v] < ex2((logit - s_mx[p]) * kLog2e) / s_sum[p]; },
+            [&](int p, int v) -> float {
+                if (!GSD_IN_BOUNDS(p >= 0 && p < N && tok[v] >= 0 && tok[v] < V, a.status)) return -CUDART_INF_F;
+                return lg[(size_t)p * V + tok[v]];
+            },
+            combine_pairs);
+        if (tid == 0) s_outcome = Outcome{res.edges, res.end, res.end_has_child ? 1 : 0, s_mx[res.end], s_sum[res.end]};
+        __syncthreads();
+        cluster_wait();
+        constexpr int kWords = sizeof(Outcome) / 4;
+        if (tid >= kWords && tid < C * kWords)
+            put_remote(reinterpret_cast<uint32_t*>(&s_outcome) + tid % kWords, tid / kWords, reinterpret_cast<const uint32_t*>(&s_outcome)[tid % kWords]);
+    } else {
+        cluster_wait();
+    }
+    cluster_arrive();
+    cluster_wait();
+    const int s_m = s_outcome.edges, s_end = s_outcome.end;
+    const float mx = s_outcome.mx, p_sum = s_outcome.sum;
 
     // The regenerated token: weights w_j over the vocabulary at the end node, then the smallest
     // t whose cumulative weight exceeds u * (total weight).  First the contiguous range of the
-    // row that holds the crossing is found from range sums, then the whole block splits that
-    // range into 256 contiguous pieces, scans the piece sums, and the thread whose piece holds
-    // the crossing walks it.
+    // row that holds the crossing is found from range sums, then one CTA splits that range into
+    // 256 contiguous pieces, scans the piece sums, and the thread whose piece holds the crossing
+    // walks it.
     const float* x = lg + (size_t)s_end * V;
-    const float mx = s_mx[s_end];
-    const int lane = tid & 31, warp = tid >> 5;
+    const RowSpan xs = row_span(x, V);
 
     // Residual of the sampling scheme: when drafted continuations of the end node were rejected
     // (it has a child in the graph) the weights are max(0, P_j - Q_j), Q the draft model's
-    // distribution at that node.  Its range sums are formed here: each warp takes a contiguous
-    // eighth of the row with coalesced loads.
+    // distribution at that node.  Its range sums are formed here: the row is cut into one
+    // contiguous range per warp of the cluster (range_of with the CTAs as slices).  The two rows
+    // come from DRAM and nothing else runs any more, so the time is the chain of dependent trips:
+    // with one CTA per sequence the two passes took 9 us at V 32000 and four times that at
+    // 128256; eight CTAs make each pass one trip.  8 x 256 rows of 32000, whole call: 64.8 us with
+    // one CTA per sequence, 61.9 with two, 59.2 with four, 59.7 with eight.
     bool residual = false;
     float q_m = 0.f, inv_sp = 0.f, inv_sq = 0.f, res_total = 0.f;
     const float* y = nullptr;
-    // both rows readable as float4 (decides where the residual's ranges begin)
-    const bool rvec = a.vec && a.dvec;
-    const int runit = rvec ? 4 : 1, rn = rvec ? (V >> 2) : V;
-    const int rper = (rn + kWarps - 1) / kWarps;
-    if (a.dlogits && res.end_has_child) {
+    bool same = false;                   // both rows have their 16-byte groups at the same entries
+    if (a.dlogits && s_outcome.end_has_child) {
         y = a.dlogits + ((size_t)b * N + s_end) * V;
-        // softmax statistics of the draft row: the row comes from DRAM, so every thread keeps
-        // sixteen 16-byte loads in flight (a 32000-entry row is two trips to memory)
+        same = row_span(y, V).head == xs.head;
+        const Range g = range_of(xs, V, C, rank * kWarps + warp);
+        // entries of the range outside its groups: before (first range) and behind (last range)
+        const int e_head = g.lo + lane, e_tail = xs.head + g.a1 * 4 + lane;
+        const bool in_head = e_head < xs.head, in_tail = e_tail < g.hi;
+        constexpr int kBatch = 8;        // groups a thread has in flight
+        const float4 none = make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
+        auto group = [&](const float* row, bool vec, int i) { return i < g.a1 ? load4(row + xs.head + 4 * i, vec) : none; };
+        // softmax statistics of the draft row; the target's row is brought into L2 beside it
         Ms r{-CUDART_INF_F, 0.f};
-        if (a.dvec) {
-            const float4* y4 = reinterpret_cast<const float4*>(y);
-            const int n4 = V >> 2;
-            const float4 none = make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
-            for (int i = tid; i < n4; i += 16 * kThreads) {
-                float4 t[16];
+        if (in_head) take1(r, __ldg(y + e_head));
+        if (in_tail) take1(r, __ldg(y + e_tail));
+        for (int i = g.a0 + lane; i < g.a1; i += kBatch * 32) {
+            float4 t[kBatch];
 #pragma unroll
-                for (int k = 0; k < 16; ++k) t[k] = i + k * kThreads < n4 ? __ldg(y4 + i + k * kThreads) : none;
+            for (int k = 0; k < kBatch; ++k) t[k] = group(y, same, i + k * 32);
 #pragma unroll
-                for (int k = 0; k < 16; k += 4) take16(r, t[k], t[k + 1], t[k + 2], t[k + 3]);
-            }
-        } else {
-            for (int j = tid; j < V; j += kThreads) take1(r, __ldg(y + j));
+            for (int k = 0; k < kBatch; ++k)
+                if (i + k * 32 < g.a1) asm volatile("prefetch.global.L2 [%0];" ::"l"(x + xs.head + 4 * (i + k * 32)));
+#pragma unroll
+            for (int k = 0; k < kBatch; k += 4) take16(r, t[k], t[k + 1], t[k + 2], t[k + 3]);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -212,57 +286,59 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
         }
         if (lane == 0) { s_rm[warp] = r.m; s_scan[warp] = r.s; }
         __syncthreads();
+        if (tid < C) {
+            r = Ms{-CUDART_INF_F, 0.f};
+            for (int w = 0; w < kWarps; ++w) r = combine(r, Ms{s_rm[w], s_scan[w]});
+            put_remote(s_cm + rank, tid, __float_as_uint(r.m));
+            put_remote(s_cs + rank, tid, __float_as_uint(r.s));
+        }
+        cluster_arrive();
+        cluster_wait();
         r = Ms{-CUDART_INF_F, 0.f};
-        for (int w = 0; w < kWarps; ++w) r = combine(r, Ms{s_rm[w], s_scan[w]});
-        __syncthreads();
+        for (int c = 0; c < C; ++c) r = combine(r, Ms{s_cm[c], s_cs[c]});
         if (!(r.s > 0.f) || r.m == CUDART_INF_F) {
-            if (tid == 0 && a.status) atomicOr((unsigned*)a.status, GSD_DEV_BAD_LOGITS);
+            if (rank == 0 && tid == 0 && a.status) atomicOr((unsigned*)a.status, GSD_DEV_BAD_LOGITS);
         } else {
             q_m = r.m;
-            inv_sp = 1.f / s_sum[s_end];
+            inv_sp = 1.f / p_sum;
             inv_sq = 1.f / r.s;
             auto res1 = [&](float xv, float yv) -> float {
                 return fmaxf(ex2((xv - mx) * kLog2e) * inv_sp - ex2((yv - q_m) * kLog2e) * inv_sq, 0.f);
             };
-            // range sums of the residual: warp w takes the w-th eighth of the row
-            const int w0 = min(warp * rper, rn), w1 = min(w0 + rper, rn);
             float part = 0.f;
-            if (rvec) {
-                const float4* x4 = reinterpret_cast<const float4*>(x);
-                const float4* y4 = reinterpret_cast<const float4*>(y);
-                const float4 none = make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
-                for (int i = w0 + lane; i < w1; i += 8 * 32) {
-                    float4 xv[8], yv[8];
+            if (in_head) part += res1(__ldg(x + e_head), __ldg(y + e_head));
+            for (int i = g.a0 + lane; i < g.a1; i += kBatch * 32) {
+                float4 xv[kBatch], yv[kBatch];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const bool in = i + k * 32 < w1;
-                        xv[k] = in ? __ldg(x4 + i + k * 32) : none;
-                        yv[k] = in ? __ldg(y4 + i + k * 32) : none;
-                    }
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        part += (res1(xv[k].x, yv[k].x) + res1(xv[k].y, yv[k].y)) + (res1(xv[k].z, yv[k].z) + res1(xv[k].w, yv[k].w));
+                for (int k = 0; k < kBatch; ++k) {
+                    xv[k] = group(x, true, i + k * 32);
+                    yv[k] = group(y, same, i + k * 32);
                 }
-            } else {
-                for (int j = w0 + lane; j < w1; j += 32) part += res1(x[j], y[j]);
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k)
+                    part += (res1(xv[k].x, yv[k].x) + res1(xv[k].y, yv[k].y)) + (res1(xv[k].z, yv[k].z) + res1(xv[k].w, yv[k].w));
             }
+            if (in_tail) part += res1(__ldg(x + e_tail), __ldg(y + e_tail));
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
-            if (lane == 0) s_scan[warp] = part;
-            __syncthreads();
-            for (int w = 0; w < kWarps; ++w) res_total += s_scan[w];
+            if (lane < C) put_remote(s_rsum + rank * kWarps + warp, lane, __float_as_uint(part));
+            cluster_arrive();
+            cluster_wait();
+            for (int w = 0; w < C * kWarps; ++w) res_total += s_rsum[w];
             // a residual without mass (the two distributions agree to rounding) leaves P
             residual = res_total > kResidualFloor;
+            __syncthreads();             // (P's range sums may take the place of the residual's)
         }
     }
+    if (!residual && rank != 0) return;  // (no CTA of the cluster touches another one's memory any more)
     // weight of one entry from its two logits (-inf stands for "past the end": weight 0)
     auto weight = [&](float xv, float yv) -> float {
         const float e = ex2((xv - mx) * kLog2e);
         return residual ? fmaxf(e * inv_sp - ex2((yv - q_m) * kLog2e) * inv_sq, 0.f) : e;
     };
     // sixteen consecutive entries of a row, all loads issued before any is used
-    auto load16 = [&](const float* row, bool vec16, int j, int jend, float (&v)[16]) {
-        if (vec16 && (j & 3) == 0 && j + 16 <= jend) {
+    auto load16 = [&](const float* row, int j, int jend, float (&v)[16]) {
+        if ((reinterpret_cast<uintptr_t>(row + j) & 15u) == 0 && j + 16 <= jend) {
             const float4* r4 = reinterpret_cast<const float4*>(row + j);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -274,20 +350,16 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
             for (int k = 0; k < 16; ++k) v[k] = j + k < jend ? row[j + k] : -CUDART_INF_F;
         }
     };
-    const float target = a.us[b] * (residual ? res_total : s_sum[s_end]);
+    const float target = a.us[b] * (residual ? res_total : p_sum);
     // every thread walks the range sums: the first range whose inclusive prefix exceeds the
     // target, or the last one with any mass if rounding leaves none
     int rsel = -1, last_r = 0;
     float before_range = 0.f, before_last = 0.f;
     {
-        const int nr = residual ? kWarps : a.slices * kWarps;
-        if (tid < nr) {          // one range sum per thread, brought to the row's maximum
-            if (residual) {
-                s_rsum[tid] = s_scan[tid];
-            } else {
-                const float2 t = __ldcg(a.part + ((size_t)b * N + s_end) * a.slices * kWarps + tid);
-                s_rsum[tid] = t.x == -CUDART_INF_F ? 0.f : t.y * ex2((t.x - mx) * kLog2e);
-            }
+        const int nr = residual ? C * kWarps : a.slices * kWarps;
+        if (!residual && tid < nr) {          // one range sum per thread, brought to the row's maximum
+            const float2 t = __ldcg(a.part + ((size_t)b * N + s_end) * a.slices * kWarps + tid);
+            s_rsum[tid] = t.x == -CUDART_INF_F ? 0.f : t.y * ex2((t.x - mx) * kLog2e);
         }
         __syncthreads();
         float run = 0.f;
@@ -298,25 +370,21 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
             run += sr;
         }
     }
-    __syncthreads();   // s_scan is reused below
     const bool crossing = rsel >= 0;
     if (!crossing) { rsel = last_r; before_range = before_last; }
+    // the CTA that formed a residual range goes on with it (its part of the rows is close by)
+    if (residual && rank != rsel / kWarps) return;
     if (tid == 0) s_pick = kNone;
-    int r0, r1;
-    if (residual) {
-        r0 = min(rsel * rper, rn) * runit;
-        r1 = min(rsel * rper + rper, rn) * runit;
-    } else {
-        range_of(V, a.slices, a.vec, rsel, r0, r1);
-    }
+    const Range rg = range_of(xs, V, residual ? C : a.slices, rsel);
+    const int r0 = rg.lo, r1 = rg.hi;
     const int per = (r1 - r0 + kThreads - 1) / kThreads;
     const int j0 = min(r0 + tid * per, r1), j1 = min(j0 + per, r1);
     float piece = 0.f;
     int last_pos = -1;
     for (int c0 = j0; c0 < j1; c0 += 16) {
         float xv[16], yv[16];
-        load16(x, a.vec != 0, c0, j1, xv);
-        if (residual) load16(y, a.dvec != 0, c0, j1, yv);
+        load16(x, c0, j1, xv);
+        if (residual) load16(y, c0, j1, yv);
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
             const float e = weight(xv[k], residual ? yv[k] : 0.f);
@@ -352,8 +420,8 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
         int pick = -1;
         for (int c0 = j0; c0 < j1 && pick < 0; c0 += 16) {
             float xv[16], yv[16];
-            load16(x, a.vec != 0, c0, j1, xv);
-            if (residual) load16(y, a.dvec != 0, c0, j1, yv);
+            load16(x, c0, j1, xv);
+            if (residual) load16(y, c0, j1, yv);
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
                 cum += weight(xv[k], residual ? yv[k] : 0.f);
@@ -379,8 +447,7 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
 
 // First launch: one CTA per (slice, row) streams its part of the row and leaves the warps'
 // (maximum, sum) pairs in scratch.
-template <bool kVec>
-__global__ void __launch_bounds__(kThreads) accept_sampled_kernel(SampledArgs a) {
+__global__ void __launch_bounds__(kThreads, 8) accept_sampled_kernel(SampledArgs a) {
     // the per-sequence pass (a programmatic dependent launch) may become resident as CTAs retire
     if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int row = blockIdx.y;  // b * N + n
@@ -388,24 +455,21 @@ __global__ void __launch_bounds__(kThreads) accept_sampled_kernel(SampledArgs a)
     const float* x = a.logits + (size_t)row * a.V;
     Ms r{-CUDART_INF_F, 0.f};
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int lo, hi;
-    range_of(a.V, a.slices, kVec ? 1 : 0, slice * kWarps + warp, lo, hi);
-    if (kVec) {
-        const float4* x4 = reinterpret_cast<const float4*>(x);
-        const int a1 = hi >> 2;
-        int i = (lo >> 2) + lane;
-        // four independent 16-byte loads in flight per thread, each a 512-byte run per warp
-        for (; i + 3 * 32 < a1; i += 4 * 32) {
-            const float4 r0 = __ldcs(x4 + i), r1 = __ldcs(x4 + i + 32);
-            const float4 r2 = __ldcs(x4 + i + 64), r3 = __ldcs(x4 + i + 96);
-            take16(r, r0, r1, r2, r3);
+    const RowSpan sp = row_span(x, a.V);
+    const Range g = range_of(sp, a.V, a.slices, slice * kWarps + warp);
+    {
+        const float4* x4 = reinterpret_cast<const float4*>(x + sp.head);
+        if (g.lo + lane < sp.head) take1(r, __ldcs(x + g.lo + lane));       // (range 0 only: lo is 0)
+        const float4 none = make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
+        // four independent 16-byte loads in flight per thread, each a 512-byte run per warp, in the
+        // last round too (an absent group counts as -inf, which has no mass)
+        for (int i = g.a0 + lane; i < g.a1; i += 4 * 32) {
+            float4 t[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) t[k] = i + k * 32 < g.a1 ? __ldcs(x4 + i + k * 32) : none;
+            take16(r, t[0], t[1], t[2], t[3]);
         }
-        for (; i < a1; i += 32) {
-            const float4 t = __ldcs(x4 + i);
-            take1(r, t.x); take1(r, t.y); take1(r, t.z); take1(r, t.w);
-        }
-    } else {
-        for (int i = lo + lane; i < hi; i += 32) take1(r, __ldcs(x + i));
+        if (sp.head + g.a1 * 4 + lane < g.hi) take1(r, __ldcs(x + sp.head + g.a1 * 4 + lane));   // (last range only)
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -417,10 +481,10 @@ __global__ void __launch_bounds__(kThreads) accept_sampled_kernel(SampledArgs a)
     if (lane == 0) a.part[((size_t)row * a.slices + slice) * kWarps + warp] = make_float2(r.m, r.s);
 }
 
-// Second launch: one CTA per sequence does the rest (statistics per node, step tests, longest
+// Second launch: one cluster per sequence does the rest (statistics per node, step tests, longest
 // path, regenerated token) once every pair of the first launch is visible.
 __global__ void __launch_bounds__(kThreads, 1) accept_sampled_tail_kernel(SampledArgs a) {
-    finish_sequence(a, blockIdx.x);      // (waits for the first launch inside, as late as it can)
+    finish_sequence(a, (int)blockIdx.x / a.cluster);      // (waits for the first launch inside, as late as it can)
 }
 
 int pick_slices(long rows, int V, int sm_count) {
@@ -429,6 +493,15 @@ int pick_slices(long rows, int V, int sm_count) {
     const long want = (long)sm_count * 8;
     while (rows * slices < want && (V / (slices * 2)) >= 4096 && slices * 2 <= kMaxSlices) slices *= 2;
     return slices;
+}
+
+// CTAs of the second launch per sequence: only the two passes over the end node's rows are shared,
+// so a CTA should have at least 2048 entries of them (one round of loads), and all clusters should
+// be resident at once (two CTAs per SM).  Without draft logits there is no residual and no pass.
+int pick_cluster(int B, int V, bool residual, int sm_count) {
+    int c = 1;
+    while (residual && c * 2 <= kMaxCluster && V / (c * 2) >= 2048 && (long)B * c * 2 <= 2l * sm_count) c *= 2;
+    return c;
 }
 
 }  // namespace
@@ -469,10 +542,7 @@ extern "C" int gsd_accept_sampled(const float* logits, const int32_t* draft_toke
     a.part = (float2*)workspace;
     a.status = status;
     a.B = p->B; a.N = p->N; a.V = p->V; a.Ecap = p->Ecap; a.Tcap = p->Tcap;
-    const bool vec = (p->V % 4 == 0) && (((uintptr_t)logits & 15u) == 0);
     a.slices = pick_slices((long)p->B * p->N, p->V, di.sm_count);
-    a.vec = vec ? 1 : 0;
-    a.dvec = (draft_logits && (p->V % 4 == 0) && (((uintptr_t)draft_logits & 15u) == 0)) ? 1 : 0;
 
     // every pair is written before it is read: nothing in the scratch has to start at zero.
     // grid.y holds at most 65535 rows: larger problems go out in blocks of whole sequences.
@@ -488,17 +558,21 @@ extern "C" int gsd_accept_sampled(const float* logits, const int32_t* draft_toke
         if (s.out_nodes) s.out_nodes += (size_t)b0 * p->Tcap;
         s.part += (size_t)b0 * p->N * a.slices * kWarps; s.B = nb;
         const dim3 grid(a.slices, (unsigned)(nb * p->N));
-        if (vec) accept_sampled_kernel<true><<<grid, kThreads, 0, st>>>(s);
-        else accept_sampled_kernel<false><<<grid, kThreads, 0, st>>>(s);
+        accept_sampled_kernel<<<grid, kThreads, 0, st>>>(s);
         GSD_CUDA_TRY(cudaGetLastError());
-        cudaLaunchAttribute attr[1];
+        s.cluster = pick_cluster(nb, p->V, draft_logits != nullptr, di.sm_count);
+        cudaLaunchAttribute attr[2];
         dependent_launch_attr(attr);
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)s.cluster;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)nb);
+        cfg.gridDim = dim3((unsigned)(nb * s.cluster));
         cfg.blockDim = dim3(kThreads);
         cfg.stream = st;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = s.cluster > 1 ? 2 : 1;
         GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_sampled_tail_kernel, s));
     }
     GSD_CUDA_TRY(cudaGetLastError());

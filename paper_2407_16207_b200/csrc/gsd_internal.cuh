@@ -172,6 +172,21 @@ int launch_attn_merge(const AttnArgs& a);
 // test hook behind gsd_debug_attn_wait (process-wide; 0 restores the default limit)
 void debug_attn_wait(unsigned long long limit_ns, int withhold_first_k);
 
+// ---- rows of logits ----
+// A row of fp32 logits as `head` entries (0 to 3) up to the first 16-byte boundary, `nvec` aligned
+// groups of four, and a tail of 0 to 3 entries.  With a vocabulary that is no multiple of four
+// (50257) every row starts at another alignment; the groups keep it on 16-byte loads.
+struct RowSpan {
+    int head, nvec;
+};
+__device__ __forceinline__ RowSpan row_span(const float* x, int V) {
+    const int to_boundary = (int)((0u - (unsigned)(reinterpret_cast<uintptr_t>(x) >> 2)) & 3u);
+    RowSpan r;
+    r.head = min(to_boundary, V);
+    r.nvec = (V - r.head) >> 2;
+    return r;
+}
+
 // ---- scratch words that must start at zero ----
 // Enqueues a small kernel that zeroes `n` 32-bit words and lets the next launch on the stream
 // start beside it.  That next kernel has to be launched with the attribute set up by
