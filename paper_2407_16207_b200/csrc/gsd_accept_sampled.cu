@@ -55,14 +55,14 @@ __device__ __forceinline__ void take16(Ms& r, const float4& a, const float4& b, 
     const float m8 = fmaxf(fmaxf(fmaxf(c.x, c.y), fmaxf(c.z, c.w)), fmaxf(fmaxf(d.x, d.y), fmaxf(d.z, d.w)));
     const float m = fmaxf(r.m, fmaxf(m4, m8));
     if (m == -CUDART_INF_F) return;
-    const float k = -m * kLog2e;
-    float s = r.s * ex2(fmaf(r.m, kLog2e, k));
-    s += ex2(fmaf(a.x, kLog2e, k)) + ex2(fmaf(a.y, kLog2e, k)) + ex2(fmaf(a.z, kLog2e, k)) + ex2(fmaf(a.w, kLog2e, k));
+    // (the rounding of m * log2 e is a factor on every term; the sum is brought back by it)
+    const float k = -m * kLog2e, off = fmaf(-m, kLog2e, -k);
+    float s = ex2(fmaf(a.x, kLog2e, k)) + ex2(fmaf(a.y, kLog2e, k)) + ex2(fmaf(a.z, kLog2e, k)) + ex2(fmaf(a.w, kLog2e, k));
     s += ex2(fmaf(b.x, kLog2e, k)) + ex2(fmaf(b.y, kLog2e, k)) + ex2(fmaf(b.z, kLog2e, k)) + ex2(fmaf(b.w, kLog2e, k));
     s += ex2(fmaf(c.x, kLog2e, k)) + ex2(fmaf(c.y, kLog2e, k)) + ex2(fmaf(c.z, kLog2e, k)) + ex2(fmaf(c.w, kLog2e, k));
     s += ex2(fmaf(d.x, kLog2e, k)) + ex2(fmaf(d.y, kLog2e, k)) + ex2(fmaf(d.z, kLog2e, k)) + ex2(fmaf(d.w, kLog2e, k));
+    r.s = fmaf(r.s, ex2((r.m - m) * kLog2e), s * ex2(off));
     r.m = m;
-    r.s = s;
 }
 
 __device__ __forceinline__ void take1(Ms& r, float x) {
