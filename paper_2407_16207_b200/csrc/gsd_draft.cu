@@ -2,10 +2,9 @@
 // k; Sec. 4.2: probability pruning and sibling pruning; Sec. 5.2: tau-redundant nodes; Sec. 5.3:
 // merge edges to the first occurrence).
 //
-// Two launches.  Grid (F, B): the CTA of frontier row (b, fi) streams that row of draft logits
-// once with 16-byte loads - softmax statistics and every thread's two best (logit, token)
-// pairs - lets one warp pick the row's k best among the 512 pairs, and leaves tokens and
-// probabilities in scratch (a row where a thread's second pair is picked is redone exactly).
+// Two launches.  Grid (F, B): the CTA of frontier row (b, fi) - a cluster of them when there are
+// few rows - streams that row of draft logits once with 16-byte loads (softmax statistics and
+// every thread's best), picks the row's k best, and leaves tokens and probabilities in scratch.
 // The second launch (one CTA per sequence, a programmatic dependent of the first) appends the
 // children (k per frontier node, in frontier order), applies the two pruning rules, looks for
 // an earlier node with the same tau-gram for every new node (first occurrence = lowest id),
@@ -20,6 +19,8 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int K = GSD_DRAFT_MAX_K;
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr int kNone = 0x7FFFFFFF;      // "no token": ranks behind every token
+constexpr int kMaxCluster = 8;
 
 __device__ __forceinline__ float ex2(float x) {
     float y;
@@ -30,6 +31,12 @@ __device__ __forceinline__ float ex2(float x) {
 // a candidate ranks before another if its logit is larger, or equal with the lower token id
 __device__ __forceinline__ bool before(float va, int ia, float vb, int ib) {
     return va > vb || (va == vb && ia < ib);
+}
+
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
 }
 
 struct TopK {
@@ -71,6 +78,7 @@ struct DraftArgs {
     float* wk_q;         // [B,F,K]
     int32_t* status;
     int B, F, V, Ncap, k, tau;
+    int cluster;         // CTAs per row of logits
     float theta_prob, theta_sib;
 };
 
@@ -269,113 +277,138 @@ __device__ __forceinline__ void block_best(float& v, int& i, int& owner, float* 
 }
 
 // The k best tokens of one row of logits and their probabilities, in one pass over the row.
-// Every thread streams its strided share (16-byte loads, kBatch in flight) and keeps the running
-// (maximum, sum of exponentials) pair, the best (logit, token) pair it has met and the VALUE of
-// its second best entry - all without a branch, so that no lane of a warp waits for another's
-// rare update.  The 256 best pairs are picked over in two stages, both with shuffles only (ranked
+// Every thread streams its strided share (16-byte loads, a batch in flight while one is worked
+// through) and keeps the running (maximum, sum of exponentials) pair, the best (logit, token) pair
+// it has met and the VALUE of its second best entry - all without a branch, so that no lane of a
+// warp waits for another's rare update.  The 256 best pairs are picked over in two stages (ranked
 // by logit, ties to the lower token id): every warp picks the k best of its 32 pairs, then one
 // warp picks the k best of those 8 k.  That is the exact answer unless some thread's second best
 // entry ranks at or before the k-th pick - then an entry that no thread offered could belong
-// to the k best (for a random row: about one row in fifty).  Such a row is read once more (from
-// L2): the k-th pick bounds the k-th best entry from below, the entries at or before it form a
-// short list, and the pick is repeated over the list.  Only a list longer than 512 (long runs
-// of equal logits) takes the slow exact way: every thread keeps the K best pairs it meets and
-// the block merges the 256 lists.
-constexpr int kBatch = 8;     // 16-byte loads a thread keeps in flight while it streams a row
+// to the k best; the shares of such threads are looked at once more.  Only a list of more than
+// 512 such entries (long runs of equal logits) takes the slow exact way: every thread keeps the K
+// best pairs it meets and the block merges the 256 lists.
+// What bounds it (8 x 64 rows of 32000, k 4, 66 MB): DRAM for the first 8 to 10 us, then the pick
+// of the row that finishes last.
+constexpr int kBatch = 4;     // 16-byte loads of a batch; the next batch is on the way while one is worked through
 struct Best {
     float v1, v2;   // best and second best logit of the thread's share (v2: value only)
     int i1;         // token of the best
 };
-__device__ __forceinline__ void offer_best(Best& t, float x, int idx) {
-    // a thread meets its entries in ascending token order: an equal logit never displaces an earlier one
+// While a row is streamed the best is kept per 16-byte group - its maximum and which group - and
+// the token inside the group is looked up once at the end: 2 instructions per entry instead of 6.
+// `v2` then bounds the entries outside the best group.  `where`: group number, or ~index of a
+// lone entry.
+__device__ __forceinline__ void offer_group(Best& t, float x, int where) {
+    // a thread meets its groups in ascending order: an equal logit never displaces an earlier one
     const bool up = x > t.v1;
     t.v2 = fmaxf(t.v2, up ? t.v1 : x);
-    t.i1 = up ? idx : t.i1;
-    t.v1 = up ? x : t.v1;
+    t.i1 = up ? where : t.i1;
+    t.v1 = fmaxf(t.v1, x);
 }
-// The best of the pairs the 32 lanes hold (ranked by `before`), and the lane that held it.
-__device__ __forceinline__ void warp_best(float& v, int& i, int& src) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float v2 = __shfl_xor_sync(0xFFFFFFFFu, v, o);
-        const int i2 = __shfl_xor_sync(0xFFFFFFFFu, i, o), s2 = __shfl_xor_sync(0xFFFFFFFFu, src, o);
-        if (before(v2, i2, v, i)) { v = v2; i = i2; src = s2; }
-    }
+// Monotone map of the logits (no NaN here; -0 folded onto +0) to unsigned words, in which the warp
+// can take a maximum with one instruction; 0 stands for "no pair".
+__device__ __forceinline__ unsigned ordered(float v) {
+    const unsigned u = __float_as_uint(v == 0.f ? 0.f : v);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float from_ordered(unsigned o) {
+    return __uint_as_float((o & 0x80000000u) ? (o & 0x7FFFFFFFu) : ~o);
 }
 
-// One warp picks the k best of `count` <= 512 (logit, token) pairs in shared memory with
-// shuffles only and writes tokens and probabilities to the row's scratch entries.  Returns (to
-// every lane) bit 0: a pair in an odd slot was picked; bit 1: fewer than k pairs above -inf;
-// the k-th pick is left in (*last_v, *last_i).
-__device__ __forceinline__ int warp_pick_k(const float* s_cv, const int* s_ci, int count, int k, float rm, float rs,
-                                           int32_t* wk_tok, float* wk_q, float* last_v, int* last_i) {
-    const int lane = threadIdx.x & 31;
-    float cv[16];
-    int ci[16];
+// One warp picks the k best of the pairs its lanes hold, kSlots each, ranked by `before`.  A round is
+// two warp-wide reductions (largest logit, then lowest token among those); with shuffle trees
+// the two stages of picks took most of the 4 us between the last load of a row and its result.
+// done(r, v, i) is called by all lanes with the r-th pick; i == kNone: no pair above -inf is left.
+template <int kSlots, class Done>
+__device__ __forceinline__ void warp_pick_k(float (&cv)[kSlots], int (&ci)[kSlots], int k, Done done) {
+    unsigned key[kSlots];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
+    for (int j = 0; j < kSlots; ++j) key[j] = ci[j] == kNone || cv[j] == -CUDART_INF_F ? 0u : ordered(cv[j]);
+    for (int r = 0; r < k; ++r) {
+        unsigned mine = key[0];
+#pragma unroll
+        for (int j = 1; j < kSlots; ++j) mine = max(mine, key[j]);
+        const unsigned top = __reduce_max_sync(0xFFFFFFFFu, mine);
+        int low = kNone;
+#pragma unroll
+        for (int j = 0; j < kSlots; ++j) low = key[j] == top ? min(low, ci[j]) : low;
+        low = top == 0u ? kNone : __reduce_min_sync(0xFFFFFFFFu, low);
+#pragma unroll
+        for (int j = 0; j < kSlots; ++j)
+            if (key[j] == top && ci[j] == low) key[j] = 0u;
+        done(r, top == 0u ? -CUDART_INF_F : from_ordered(top), low);
+    }
+}
+// The same for `count` <= 32 * kSlots pairs in shared memory; the picks go to out_v / out_i (token
+// -1: none was left).
+template <int kSlots>
+__device__ __forceinline__ void warp_pick_k(const float* s_cv, const int* s_ci, int count, int k, float* out_v, int* out_i) {
+    const int lane = threadIdx.x & 31;
+    float cv[kSlots];
+    int ci[kSlots];
+#pragma unroll
+    for (int j = 0; j < kSlots; ++j) {
         const bool in = lane + 32 * j < count;
         cv[j] = in ? s_cv[lane + 32 * j] : -CUDART_INF_F;
-        ci[j] = in ? s_ci[lane + 32 * j] : 0x7FFFFFFF;
+        ci[j] = in ? s_ci[lane + 32 * j] : kNone;
     }
-    int result = 0;
-    float v = -CUDART_INF_F;
-    int i = 0x7FFFFFFF;
-    for (int r = 0; r < k; ++r) {
-        v = -CUDART_INF_F;
-        i = 0x7FFFFFFF;
-        int slot = -1;
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-            if (before(cv[j], ci[j], v, i)) { v = cv[j]; i = ci[j]; slot = lane + 32 * j; }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float v2 = __shfl_xor_sync(0xFFFFFFFFu, v, o);
-            const int i2 = __shfl_xor_sync(0xFFFFFFFFu, i, o), t2 = __shfl_xor_sync(0xFFFFFFFFu, slot, o);
-            if (before(v2, i2, v, i)) { v = v2; i = i2; slot = t2; }
-        }
-        // pairs at -inf are never taken (slot stays -1 when nothing above -inf is left)
-        if (slot >= 0) {
-            if (slot & 1) result |= 1;
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                if (slot == lane + 32 * j) { cv[j] = -CUDART_INF_F; ci[j] = 0x7FFFFFFF; }
-        } else {
-            result |= 2;
-        }
+    warp_pick_k<kSlots>(cv, ci, k, [&](int r, float v, int i) {
         if (lane == 0) {
-            wk_tok[r] = slot < 0 ? -1 : i;
-            wk_q[r] = slot < 0 ? 0.f : ex2((v - rm) * kLog2e) / rs;
+            out_v[r] = v;
+            out_i[r] = i == kNone ? -1 : i;
         }
-    }
-    *last_v = v;
-    *last_i = i;
-    return result;
+    });
 }
 
-template <bool kVec>
+// ---- thread-block cluster: the CTAs that share a row
+__device__ __forceinline__ int cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return (int)r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// writes `v` to the place of *dst in the leading CTA of the cluster
+__device__ __forceinline__ void put_leader(void* dst, uint32_t v) {
+    uint32_t at;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(dst)));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+}
+
+// The row's CTAs (a cluster; usually one) share it in contiguous slices; each finds the k best of
+// its slice and the leading one picks the row's among those.
 __global__ void __launch_bounds__(kThreads, 4) draft_expand_kernel(DraftArgs a) {
     __shared__ float s_cv[2 * kThreads];
     __shared__ int s_ci[2 * kThreads];
     __shared__ float s_rv[kWarps];
     __shared__ int s_ri[kWarps], s_rt[kWarps];
-    __shared__ float s_m[kWarps], s_s[kWarps], s_v2[kWarps];
-    __shared__ int s_redo, s_count, s_ti;
-    __shared__ float s_tv;
+    __shared__ float s_m[kWarps], s_s[kWarps];
+    __shared__ int s_flagged, s_count;
+    __shared__ short s_flag[kThreads];     // threads whose share has to be looked at again
+    __shared__ float s_bv[K];              // the k best of the slice
+    __shared__ int s_bi[K];
+    __shared__ float s_pv[kMaxCluster * K], s_pm[kMaxCluster], s_ps[kMaxCluster];   // what the cluster's CTAs hand in
+    __shared__ int s_pi[kMaxCluster * K];
     // the per-sequence pass (a programmatic dependent launch) may become resident as CTAs retire
     if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int fi = blockIdx.x, b = blockIdx.y;
+    const int C = a.cluster, slice = C > 1 ? cluster_rank() : 0;
+    const int fi = (int)blockIdx.x / C, b = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int V = a.V;
-    const int fl = a.frontier_len[b];
-    if (fi >= fl || fl > a.F) return;
+    if (C > 1) cluster_arrive();           // every CTA has started before any writes to another
     const float* x = a.logits + ((size_t)b * a.F + fi) * V;
-    const float4* x4 = reinterpret_cast<const float4*>(x);
-    const int nvec = V >> 2;
+    // The CTA's slice: 16-byte groups v0 .. v1, the entries before the first 16-byte boundary (first
+    // slice) and those behind the last group (last slice).  Threads meet theirs in ascending order.
+    const RowSpan sp = row_span(x, V);
+    const float4* x4 = reinterpret_cast<const float4*>(x + sp.head);
+    const int per = (sp.nvec + C - 1) / C;
+    const int v0 = min(slice * per, sp.nvec), v1 = min(v0 + per, sp.nvec);
+    const int e_head = slice == 0 && tid < sp.head ? tid : -1;
+    const int e_tail = slice == C - 1 && sp.head + 4 * sp.nvec + tid < V ? sp.head + 4 * sp.nvec + tid : -1;
     float m = -CUDART_INF_F, s = 0.f;        // running maximum and sum
-    Best best{-CUDART_INF_F, -CUDART_INF_F, 0x7FFFFFFF};
+    Best best{-CUDART_INF_F, -CUDART_INF_F, kNone};
     auto take = [&](float val, int idx) {
-        offer_best(best, val, idx);
+        offer_group(best, val, ~idx);
         if (val > m) {
             s = s * ex2((m - val) * kLog2e) + 1.f;
             m = val;
@@ -385,25 +418,22 @@ __global__ void __launch_bounds__(kThreads, 4) draft_expand_kernel(DraftArgs a) 
             s = val;    // NaN poisons the sum and is reported below
         }
     };
-    if (kVec) {
+    {
         const float4 none = make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
-        for (int i = tid; i < nvec; i += kBatch * kThreads) {
-            float4 r[kBatch];
+        auto fetch = [&](float4 (&r)[kBatch], int i) {
 #pragma unroll
-            for (int k = 0; k < kBatch; ++k) r[k] = i + k * kThreads < nvec ? __ldcs(x4 + i + k * kThreads) : none;
+            for (int k = 0; k < kBatch; ++k) r[k] = i + k * kThreads < v1 ? __ldcs(x4 + i + k * kThreads) : none;
+        };
+        auto work = [&](const float4 (&r)[kBatch], int i) {
             float g = m;
-            float nan_probe = 0.f;
 #pragma unroll
             for (int k = 0; k < kBatch; ++k) {
-                const float g4 = fmaxf(fmaxf(r[k].x, r[k].y), fmaxf(r[k].z, r[k].w));
+                const float g4 = max3(fmaxf(r[k].x, r[k].y), r[k].z, r[k].w);
                 g = fmaxf(g, g4);
-                nan_probe += (r[k].x + r[k].y) + (r[k].z + r[k].w);     // NaN if any entry is NaN (or +inf and -inf meet)
-                const int e = (i + k * kThreads) * 4;
-                offer_best(best, r[k].x, e); offer_best(best, r[k].y, e + 1);
-                offer_best(best, r[k].z, e + 2); offer_best(best, r[k].w, e + 3);
+                offer_group(best, g4, i + k * kThreads);
             }
-            if (nan_probe != nan_probe) {
-                // rare: find out entry by entry (a NaN poisons the sum; -inf next to +inf does not)
+            if (g == -CUDART_INF_F) {
+                // nothing finite yet: a NaN would otherwise go unnoticed (below it poisons the sum)
 #pragma unroll
                 for (int k = 0; k < kBatch; ++k) {
                     const float q[4] = {r[k].x, r[k].y, r[k].z, r[k].w};
@@ -411,175 +441,178 @@ __global__ void __launch_bounds__(kThreads, 4) draft_expand_kernel(DraftArgs a) 
                     for (int j = 0; j < 4; ++j)
                         if (q[j] != q[j]) s = q[j];
                 }
+                return;
             }
-            if (g == -CUDART_INF_F) continue;      // nothing finite yet
-            // one rescale per batch
-            const float kk = -g * kLog2e;
-            float acc = s * ex2(fmaf(m, kLog2e, kk));
+            // One rescale per batch.  The rounding of g * log2 e (2^-21 at a logit of 12) would be a
+            // factor on every term, while the probabilities at the end use v - maximum: the
+            // batch's sum is brought back by what was rounded off.
+            const float kk = -g * kLog2e, off = fmaf(-g, kLog2e, -kk);
+            float acc = 0.f;
 #pragma unroll
             for (int k = 0; k < kBatch; ++k)
                 acc += (ex2(fmaf(r[k].x, kLog2e, kk)) + ex2(fmaf(r[k].y, kLog2e, kk))) + (ex2(fmaf(r[k].z, kLog2e, kk)) + ex2(fmaf(r[k].w, kLog2e, kk)));
-            s = acc;
+            s = fmaf(s, ex2((m - g) * kLog2e), acc * ex2(off));
             m = g;
+        };
+        constexpr int kStep = kBatch * kThreads;
+        float4 ra[kBatch], rb[kBatch];
+        fetch(ra, v0 + tid);
+        // (the row is there whether it is on the frontier or not: the first loads need not wait)
+        const int fl = a.frontier_len[b];
+        if (fi >= fl || fl > a.F) {              // (all CTAs of a cluster alike)
+            if (C > 1) cluster_wait();
+            return;
         }
-    } else {
-        for (int i = tid; i < V; i += kThreads) take(__ldcs(x + i), i);
+        if (e_head >= 0) take(__ldcs(x + e_head), e_head);
+        for (int i = v0 + tid; i < v1; i += 2 * kStep) {
+            fetch(rb, i + kStep);                // on the way while the other batch is worked through
+            work(ra, i);
+            fetch(ra, i + 2 * kStep);
+            if (i + kStep < v1) work(rb, i + kStep);
+        }
+        if (e_tail >= 0) take(__ldcs(x + e_tail), e_tail);
     }
-    // stage 1: every warp picks the k best of its 32 pairs; lane r keeps the r-th pick
+    // the token of the best, and the best of the other entries of its group
+    if (best.i1 != kNone) {
+        if (best.i1 < 0) {
+            best.i1 = ~best.i1;
+        } else {
+            const float4 r = x4[best.i1];
+            const float q[4] = {r.x, r.y, r.z, r.w};
+            int at = 3;
+#pragma unroll
+            for (int j = 2; j >= 0; --j)
+                if (q[j] == best.v1) at = j;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (j != at) best.v2 = fmaxf(best.v2, q[j]);
+            best.i1 = sp.head + 4 * best.i1 + at;
+        }
+    }
+    // stage 1: every warp picks the k best of its 32 pairs
     {
-        float cv = best.v1, pv = -CUDART_INF_F;
-        int ci = best.i1, pi = 0x7FFFFFFF;
-        for (int r = 0; r < a.k; ++r) {
-            float v = cv;
-            int i = ci, src = lane;
-            warp_best(v, i, src);
-            if (lane == r) { pv = v; pi = i; }
-            if (src == lane) { cv = -CUDART_INF_F; ci = 0x7FFFFFFF; }      // (a pair at -inf is never taken: its token is none)
-        }
-        if (lane < a.k) { s_cv[warp * K + lane] = pv; s_ci[warp * K + lane] = pi; }
-        float v2 = best.v2;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v2 = fmaxf(v2, __shfl_xor_sync(0xFFFFFFFFu, v2, o));
-        if (lane == 0) s_v2[warp] = v2;
+        float cv[1] = {best.v1};
+        int ci[1] = {best.i1};
+        warp_pick_k<1>(cv, ci, a.k, [&](int r, float v, int i) {
+            if (lane == 0) { s_cv[warp * a.k + r] = v; s_ci[warp * a.k + r] = i; }
+        });
     }
-    // (maximum, sum) of the row
+    // (maximum, sum) of the warp's entries; a NaN sum stays
+    {
+        float wm = m;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float m2 = __shfl_xor_sync(0xFFFFFFFFu, m, o), s2 = __shfl_xor_sync(0xFFFFFFFFu, s, o);
-        const float mm = fmaxf(m, m2);
-        s = (mm == -CUDART_INF_F) ? ((s != s || s2 != s2) ? CUDART_NAN_F : 0.f)
-                                  : s * ex2((m - mm) * kLog2e) + s2 * ex2((m2 - mm) * kLog2e);
-        m = mm;
+        for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xFFFFFFFFu, wm, o));
+        float ws = wm == -CUDART_INF_F ? s : s * ex2((m - wm) * kLog2e);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ws += __shfl_xor_sync(0xFFFFFFFFu, ws, o);
+        if (lane == 0) { s_m[warp] = wm; s_s[warp] = ws; }
     }
-    if (lane == 0) { s_m[warp] = m; s_s[warp] = s; }
-    if (tid == 0) s_redo = 0;
+    if (tid == 0) { s_flagged = 0; s_count = a.k; }
     __syncthreads();
-    float rm = -CUDART_INF_F, rs = 0.f;
-    const size_t w = ((size_t)b * a.F + fi) * K;
-    if (warp == 0) {
-        for (int q = 0; q < kWarps; ++q) {
-            const float mm = fmaxf(rm, s_m[q]);
-            rs = (mm == -CUDART_INF_F) ? ((rs != rs || s_s[q] != s_s[q]) ? CUDART_NAN_F : 0.f)
-                                       : rs * ex2((rm - mm) * kLog2e) + s_s[q] * ex2((s_m[q] - mm) * kLog2e);
-            rm = mm;
-        }
-        if (lane == 0 && (!(rs > 0.f) || rm == CUDART_INF_F) && a.status) atomicOr((unsigned*)a.status, GSD_DEV_BAD_LOGITS);
-        // stage 2: the k best of the 8 k picks (two per lane at most)
-        const int n = kWarps * a.k;
-        float c0 = -CUDART_INF_F, c1 = -CUDART_INF_F;
-        int j0 = 0x7FFFFFFF, j1 = 0x7FFFFFFF;
-        if (lane < n) { c0 = s_cv[(lane / a.k) * K + lane % a.k]; j0 = s_ci[(lane / a.k) * K + lane % a.k]; }
-        if (lane + 32 < n) { c1 = s_cv[((lane + 32) / a.k) * K + (lane + 32) % a.k]; j1 = s_ci[((lane + 32) / a.k) * K + (lane + 32) % a.k]; }
-        float tv = -CUDART_INF_F;
-        int ti = 0x7FFFFFFF;
-        bool short_row = false;
-        for (int r = 0; r < a.k; ++r) {
-            const bool second = before(c1, j1, c0, j0);
-            float v = second ? c1 : c0;
-            int i = second ? j1 : j0, src = lane;
-            warp_best(v, i, src);
-            if (src == lane) {
-                if (second) { c1 = -CUDART_INF_F; j1 = 0x7FFFFFFF; } else { c0 = -CUDART_INF_F; j0 = 0x7FFFFFFF; }
-            }
-            const bool none = i == 0x7FFFFFFF;
-            short_row |= none;
-            if (lane == 0) {
-                a.wk_tok[w + r] = none ? -1 : i;
-                a.wk_q[w + r] = none ? 0.f : ex2((v - rm) * kLog2e) / rs;
-            }
-            tv = v;
-            ti = i;
-        }
-        // an entry that no thread offered can rank at or before the k-th pick only if some
-        // thread's second best does
-        float v2 = lane < kWarps ? s_v2[lane] : -CUDART_INF_F;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v2 = fmaxf(v2, __shfl_xor_sync(0xFFFFFFFFu, v2, o));
-        const bool redo = v2 > -CUDART_INF_F && v2 >= tv;
-        if (lane == 0) {
-            s_redo = redo ? 1 : 0;
-            s_tv = tv;
-            s_ti = ti;
-            s_count = 0;
-            // (a row that goes through the second pass finds out there whether it is short of k entries)
-            if (short_row && !redo && a.status) atomicOr((unsigned*)a.status, GSD_DEV_BAD_LOGITS);
-        }
-    }
+    // stage 2: the k best of the 8 k picks
+    if (warp == 0) warp_pick_k<kWarps * K / 32>(s_cv, s_ci, kWarps * a.k, a.k, s_bv, s_bi);
     __syncthreads();
-    if (!s_redo) return;
-    // Second pass (about one random row in fifty): the k-th pick is a lower bound on the row's
-    // k-th best entry, so everything that ranks at or before it is collected from the row (now
-    // in L2) and the pick is repeated over that list.
-    const float tv = s_tv;
-    const int ti = s_ti;
-    __syncthreads();                        // the pairs have been read: the list takes their place
-    auto consider = [&](float val, int idx) {
-        if (val > tv || (val == tv && idx <= ti)) {
+    // An entry that no thread offered can rank at or before the k-th pick only if it is in the share
+    // of a thread whose second best does (about one random row in fifty has such a thread).
+    const float tv = s_bv[a.k - 1];
+    const int ti = s_bi[a.k - 1] < 0 ? kNone : s_bi[a.k - 1];
+    const bool again = best.v2 > -CUDART_INF_F && best.v2 >= tv;
+    if (again) s_flag[atomicAdd(&s_flagged, 1)] = (short)tid;
+    if (__syncthreads_or(again)) {
+        // Those shares are read once more (from L2; a warp takes a share, so a row of 32000 is one
+        // trip), and the k picks together with what ranks at or before the last of them and
+        // had not been offered make a short list that holds the k best.  (Reading the whole row again
+        // took 8 us instead of 2.5, for 15 of 512 rows, and the call waits for the last row.)
+        if (tid < a.k) { s_cv[tid] = s_bv[tid]; s_ci[tid] = s_bi[tid] < 0 ? kNone : s_bi[tid]; }
+        __syncthreads();
+        auto consider = [&](float val, int idx) {
+            if (val == -CUDART_INF_F || !(val > tv || (val == tv && idx <= ti))) return;
+            for (int r = 0; r < a.k; ++r)
+                if (s_bi[r] == idx) return;
             const int slot = atomicAdd(&s_count, 1);
             if (slot < 2 * kThreads) { s_cv[slot] = val; s_ci[slot] = idx; }
+        };
+        for (int f = warp; f < s_flagged; f += kWarps) {
+            const int t = s_flag[f];
+            if (lane == 0 && slice == 0 && t < sp.head) consider(x[t], t);
+            if (lane == 0 && slice == C - 1 && sp.head + 4 * sp.nvec + t < V) consider(x[sp.head + 4 * sp.nvec + t], sp.head + 4 * sp.nvec + t);
+            for (int i = v0 + t + lane * kThreads; i < v1; i += 32 * kThreads) {
+                const float4 r = x4[i];
+                const int e = sp.head + i * 4;
+                consider(r.x, e); consider(r.y, e + 1); consider(r.z, e + 2); consider(r.w, e + 3);
+            }
         }
-    };
-    if (kVec) {
-        const float4 none = make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
-        for (int i = tid; i < nvec; i += 8 * kThreads) {
-            float4 r[8];
+        __syncthreads();
+        const int count = s_count;
+        if (count <= 2 * kThreads) {
+            if (warp == 0) warp_pick_k<2 * kThreads / 32>(s_cv, s_ci, count, a.k, s_bv, s_bi);
+        } else {
+            // more than 512 entries rank before the bound (long runs of equal logits in one thread's
+            // share): per-thread lists of the K best pairs, merged by the block
+            TopK t;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) r[k] = i + k * kThreads < nvec ? x4[i + k * kThreads] : none;
+            for (int j = 0; j < K; ++j) {
+                t.v[j] = -CUDART_INF_F;
+                t.i[j] = kNone;
+            }
+            if (e_head >= 0) offer(t, x[e_head], e_head);
+            for (int i = v0 + tid; i < v1; i += kThreads) {
+                const float4 r = x4[i];
+                const int e = sp.head + 4 * i;
+                offer(t, r.x, e); offer(t, r.y, e + 1); offer(t, r.z, e + 2); offer(t, r.w, e + 3);
+            }
+            if (e_tail >= 0) offer(t, x[e_tail], e_tail);
+            int head = 0;
+            for (int r = 0; r < a.k; ++r) {
+                float v = -CUDART_INF_F;
+                int i = kNone;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int e = (i + k * kThreads) * 4;
-                if (fmaxf(fmaxf(r[k].x, r[k].y), fmaxf(r[k].z, r[k].w)) >= tv) {
-                    consider(r[k].x, e); consider(r[k].y, e + 1); consider(r[k].z, e + 2); consider(r[k].w, e + 3);
+                for (int j = 0; j < K; ++j)
+                    if (j == head) { v = t.v[j]; i = t.i[j]; }
+                int owner = tid;
+                block_best(v, i, owner, s_rv, s_ri, s_rt);
+                if (owner == tid && i != kNone) ++head;
+                if (tid == 0) {
+                    s_bv[r] = v;
+                    s_bi[r] = i == kNone ? -1 : i;       // fewer than k entries above -inf
                 }
             }
         }
-    } else {
-        for (int i = tid; i < V; i += kThreads) consider(x[i], i);
+        __syncthreads();
     }
-    __syncthreads();
-    const int count = s_count;
-    if (count <= 2 * kThreads) {
-        if (warp == 0) {
-            float lv;
-            int li;
-            const int res = warp_pick_k(s_cv, s_ci, count, a.k, rm, rs, a.wk_tok + w, a.wk_q + w, &lv, &li);
-            if (lane == 0 && (res & 2) && a.status) atomicOr((unsigned*)a.status, GSD_DEV_BAD_LOGITS);
+    // (maximum, sum) of `n` parts of the row
+    auto sum_up = [](const float* pm, const float* ps, int n, float& rm, float& rs) {
+        rm = -CUDART_INF_F;
+        for (int q = 0; q < n; ++q) rm = fmaxf(rm, pm[q]);
+        rs = 0.f;
+        for (int q = 0; q < n; ++q) rs += rm == -CUDART_INF_F ? ps[q] : ps[q] * ex2((pm[q] - rm) * kLog2e);
+    };
+    float rm, rs;
+    sum_up(s_m, s_s, kWarps, rm, rs);
+    if (C > 1) {
+        // hand the slice's result to the leading CTA, which picks the row's k best
+        cluster_wait();
+        if (tid < a.k) {
+            put_leader(s_pv + slice * a.k + tid, __float_as_uint(s_bi[tid] < 0 ? -CUDART_INF_F : s_bv[tid]));
+            put_leader(s_pi + slice * a.k + tid, (uint32_t)(s_bi[tid] < 0 ? kNone : s_bi[tid]));
         }
-        return;
+        if (tid == 0) {
+            put_leader(s_pm + slice, __float_as_uint(rm));
+            put_leader(s_ps + slice, __float_as_uint(rs));
+        }
+        cluster_arrive();
+        cluster_wait();
+        if (slice != 0) return;
+        if (warp == 0) warp_pick_k<kMaxCluster * K / 32>(s_pv, s_pi, C * a.k, a.k, s_bv, s_bi);
+        __syncthreads();
+        sum_up(s_pm, s_ps, C, rm, rs);
     }
-    {
-        // more than 512 entries rank before the bound (long runs of equal logits in one thread's
-        // share): per-thread lists of the K best pairs, merged by the block
-        TopK t;
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            t.v[j] = -CUDART_INF_F;
-            t.i[j] = 0x7FFFFFFF;
-        }
-        if (kVec) {
-            for (int i = tid; i < nvec; i += kThreads) {
-                const float4 r = x4[i];
-                offer(t, r.x, 4 * i); offer(t, r.y, 4 * i + 1); offer(t, r.z, 4 * i + 2); offer(t, r.w, 4 * i + 3);
-            }
-        } else {
-            for (int i = tid; i < V; i += kThreads) offer(t, x[i], i);
-        }
-        int head = 0;
-        for (int r = 0; r < a.k; ++r) {
-            float v = -CUDART_INF_F;
-            int i = 0x7FFFFFFF;
-#pragma unroll
-            for (int j = 0; j < K; ++j)
-                if (j == head) { v = t.v[j]; i = t.i[j]; }
-            int owner = tid;
-            block_best(v, i, owner, s_rv, s_ri, s_rt);
-            if (owner == tid && i != 0x7FFFFFFF) ++head;
-            if (tid == 0) {
-                if (i == 0x7FFFFFFF && a.status) atomicOr((unsigned*)a.status, GSD_DEV_BAD_LOGITS);   // fewer than k entries above -inf
-                a.wk_tok[w + r] = i == 0x7FFFFFFF ? -1 : i;
-                a.wk_q[w + r] = v == -CUDART_INF_F ? 0.f : ex2((v - rm) * kLog2e) / rs;
-            }
-        }
+    if (tid < a.k) {
+        const size_t w = ((size_t)b * a.F + fi) * K;
+        const bool none = s_bi[tid] < 0;
+        a.wk_tok[w + tid] = s_bi[tid];
+        a.wk_q[w + tid] = none ? 0.f : ex2((s_bv[tid] - rm) * kLog2e) / rs;
+        if ((none || !(rs > 0.f) || rm == CUDART_INF_F) && a.status) atomicOr((unsigned*)a.status, GSD_DEV_BAD_LOGITS);
     }
 }
 
@@ -587,6 +620,17 @@ __global__ void __launch_bounds__(kThreads, 4) draft_expand_kernel(DraftArgs a) 
 // row's result of the first launch is visible.
 __global__ void __launch_bounds__(kThreads) draft_grow_kernel(DraftArgs a) {
     grow_sequence(a, blockIdx.x);        // (waits for the first launch inside, as late as it can)
+}
+
+// CTAs per row of logits: with fewer rows than half the SMs the rows are shared, down to 4096
+// entries (four rounds of a CTA's loads) per CTA.  8 rows of 128256: 25.3 us in one CTA each, 16.9
+// in eight.  With more rows sharing does not pay, since every slice has to find its own k best and
+// the slices without an outstanding entry need the second look more often: 120 rows of 32000, k 8:
+// 24.3 us in one CTA each, 26.1 in two, 27.9 in four (before the second look became cheap).
+int pick_cluster(long rows, int V, int sm_count) {
+    int c = 1;
+    while (c < kMaxCluster && rows * c * 2 <= sm_count && V / (c * 2) >= 4096) c *= 2;
+    return c;
 }
 
 }  // namespace
@@ -613,6 +657,8 @@ extern "C" int gsd_draft_expand(const float* logits, const int32_t* frontier, co
     const size_t need = gsd_draft_expand_workspace_bytes(p);
     if (!workspace || workspace_bytes < need) return GSD_ERR_WORKSPACE;
     if (((uintptr_t)workspace & 7u) != 0) return GSD_ERR_MISALIGNED;
+    DeviceInfo di;
+    if (device_info(&di) != 0) return GSD_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
     DraftArgs a;
     a.logits = logits; a.frontier = frontier; a.frontier_len = frontier_len;
@@ -625,14 +671,20 @@ extern "C" int gsd_draft_expand(const float* logits, const int32_t* frontier, co
     a.B = p->B; a.F = p->F; a.V = p->V; a.Ncap = p->Ncap; a.k = p->k; a.tau = p->tau;
     a.theta_prob = p->theta_prob; a.theta_sib = p->theta_sib;
     // every scratch entry is written before it is read: nothing has to start at zero
-    const bool vec = (p->V % 4 == 0) && (((uintptr_t)logits & 15u) == 0);
-    dim3 grid((unsigned)p->F, (unsigned)p->B);
-    if (vec) draft_expand_kernel<true><<<grid, kThreads, 0, st>>>(a);
-    else draft_expand_kernel<false><<<grid, kThreads, 0, st>>>(a);
-    GSD_CUDA_TRY(cudaGetLastError());
-    cudaLaunchAttribute attr[1];
-    dependent_launch_attr(attr);
+    a.cluster = pick_cluster((long)p->B * p->F, p->V, di.sm_count);
     cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)a.cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)p->F * (unsigned)a.cluster, (unsigned)p->B);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.cluster > 1 ? 1 : 0;
+    GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, draft_expand_kernel, a));
+    dependent_launch_attr(attr);
     cfg.gridDim = dim3((unsigned)p->B);
     cfg.blockDim = dim3(kThreads);
     cfg.stream = st;
