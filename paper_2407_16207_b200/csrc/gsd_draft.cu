@@ -395,6 +395,8 @@ __global__ void __launch_bounds__(kThreads, 4) draft_expand_kernel(DraftArgs a) 
     const int fi = (int)blockIdx.x / C, b = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int V = a.V;
+    const int fl = a.frontier_len[b];
+    if (fi >= fl || fl > a.F) return;      // (all CTAs of a cluster alike; such rows are not read)
     if (C > 1) cluster_arrive();           // every CTA has started before any writes to another
     const float* x = a.logits + ((size_t)b * a.F + fi) * V;
     // The CTA's slice: 16-byte groups v0 .. v1, the entries before the first 16-byte boundary (first
@@ -457,12 +459,6 @@ __global__ void __launch_bounds__(kThreads, 4) draft_expand_kernel(DraftArgs a) 
         constexpr int kStep = kBatch * kThreads;
         float4 ra[kBatch], rb[kBatch];
         fetch(ra, v0 + tid);
-        // (the row is there whether it is on the frontier or not: the first loads need not wait)
-        const int fl = a.frontier_len[b];
-        if (fi >= fl || fl > a.F) {              // (all CTAs of a cluster alike)
-            if (C > 1) cluster_wait();
-            return;
-        }
         if (e_head >= 0) take(__ldcs(x + e_head), e_head);
         for (int i = v0 + tid; i < v1; i += 2 * kStep) {
             fetch(rb, i + kStep);                // on the way while the other batch is worked through
