@@ -1,4 +1,6 @@
-"""ctypes binding of libgsd.so with the same names as the C ABI (include/gsd.h).
+"""Binding of libgsd.so with the same names as the C ABI (include/gsd.h).  The calls of a serving
+iteration go through a CPython extension (csrc/gsd_native.cpp) when their arguments are the plain
+case, and through ctypes otherwise; both load the same library.
 
 The functions take torch tensors (CUDA tensors for the device calls, CPU tensors for the
 host-buffer step), check dtype / shape / contiguity, and pass raw pointers, sizes and the
@@ -115,6 +117,31 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+# The library's functions the extension calls, in the order of its table.
+_NATIVE_CALLS = ("gsd_verify_attn", "gsd_verify_attn_workspace_bytes", "gsd_accept", "gsd_accept_workspace_bytes",
+                 "gsd_accept_sampled", "gsd_accept_sampled_workspace_bytes", "gsd_draft_expand",
+                 "gsd_draft_expand_workspace_bytes", "gsd_build_mask", "gsd_commit_kv")
+_native = None
+_native_lib: Optional[ctypes.CDLL] = None      # the library the extension is bound to
+
+
+def native():
+    """The CPython extension (built in-tree beside the library), bound to the loaded library."""
+    global _native, _native_lib
+    L = lib()
+    if _native is None:
+        try:
+            from . import _native as module
+        except ImportError as e:
+            raise GsdError(-100, f"the extension _native.so is missing or does not load ({e}): run "
+                                 "`python -m paper_2407_16207_b200.build`") from e
+        _native = module
+    if _native_lib is not L:
+        _native.bind(*(ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in _NATIVE_CALLS))
+        _native_lib = L
+    return _native
+
+
 def _check(rc: int) -> None:
     if rc != 0:
         L = lib()
@@ -192,6 +219,13 @@ def gsd_verify_attn(q, k_cache, v_cache, draft_k, draft_v, ancestor_mask, seq_le
                     status: Optional[torch.Tensor] = None) -> torch.Tensor:
     """DAG-masked attention of the draft nodes; see gsd_verify_attn in include/gsd.h.
     Enqueued on the current stream; returns `out` [B,N,Hq,D] bf16."""
+    fast = _native if _lib is not None and _lib is _native_lib else native()
+    r = fast.verify_attn(q, k_cache, v_cache, draft_k, draft_v, ancestor_mask, seq_lens, out, softmax_scale, num_splits, kernel,
+                         workspace, status)
+    if r is not None:
+        if r.__class__ is int:
+            _check(r)
+        return r
     _check_attn_tensors(q, k_cache, v_cache, draft_k, draft_v, ancestor_mask, seq_lens, True)
     if out is None:
         out = torch.empty_like(q)
@@ -222,6 +256,13 @@ def gsd_accept(logits, draft_tokens, parent_ptr, parent_idx, *, Tcap: int = 0,
                ) -> Tuple[torch.Tensor, torch.Tensor, Optional[torch.Tensor]]:
     """Greedy verification + longest accepted path; see gsd_accept in include/gsd.h.
     Returns (accepted_tokens [B,Tcap], accepted_len [B], accepted_nodes [B,Tcap] or None)."""
+    if out is None:
+        fast = _native if _lib is not None and _lib is _native_lib else native()
+        r = fast.accept(logits, draft_tokens, parent_ptr, parent_idx, Tcap, want_nodes, workspace, status)
+        if r is not None:
+            if r.__class__ is int:
+                _check(r)
+            return r
     if logits.dim() != 3:
         raise ValueError("logits must be [B,N,V]")
     B, N, V = logits.shape
@@ -268,6 +309,14 @@ def gsd_accept_sampled(logits, draft_tokens, parent_ptr, parent_idx, draft_q, u_
     include/gsd.h.  `draft_logits` [B,N,V] (optional) makes the regenerated token come from the
     residual max(0, P - Q).  Returns (accepted_tokens [B,Tcap], accepted_len [B], accepted_nodes
     or None)."""
+    if out is None:
+        fast = _native if _lib is not None and _lib is _native_lib else native()
+        r = fast.accept_sampled(logits, draft_tokens, parent_ptr, parent_idx, draft_q, u_accept, u_sample, draft_logits, Tcap,
+                                want_nodes, workspace, status)
+        if r is not None:
+            if r.__class__ is int:
+                _check(r)
+            return r
     if logits.dim() != 3:
         raise ValueError("logits must be [B,N,V]")
     B, N, V = logits.shape
@@ -315,6 +364,14 @@ def gsd_draft_expand(logits, frontier, frontier_len, tokens, tree_parent, merge_
                      ) -> Tuple[torch.Tensor, torch.Tensor]:
     """One growth step of the draft token graph, in place; see gsd_draft_expand in include/gsd.h.
     Returns (new_frontier [B,F*k], new_frontier_len [B])."""
+    if out is None:
+        fast = _native if _lib is not None and _lib is _native_lib else native()
+        r = fast.draft_expand(logits, frontier, frontier_len, tokens, tree_parent, merge_to, leaf, prob, num_nodes, k, tau,
+                              theta_prob, theta_sib, workspace, status)
+        if r is not None:
+            if r.__class__ is int:
+                _check(r)
+            return r
     if logits.dim() != 3:
         raise ValueError("logits must be [B,F,V]")
     B, F, V = logits.shape
@@ -351,6 +408,12 @@ def gsd_build_mask(parent_ptr, parent_idx, out: Optional[torch.Tensor] = None, *
                    status: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Ancestor bitmask [B,N,ceil(N/32)] (int32 words) from the parent CSR; see gsd_build_mask in
     include/gsd.h.  Enqueued on the current stream."""
+    fast = _native if _lib is not None and _lib is _native_lib else native()
+    r = fast.build_mask(parent_ptr, parent_idx, out, status)
+    if r is not None:
+        if r.__class__ is int:
+            _check(r)
+        return r
     B, N1 = parent_ptr.shape
     N = N1 - 1
     Ecap = parent_idx.shape[1]
@@ -398,6 +461,10 @@ def gsd_commit_kv(k_cache, v_cache, draft_k, draft_v, accepted_nodes, accepted_l
                   status: Optional[torch.Tensor] = None) -> None:
     """Append the draft K/V rows of the accepted path to the cache in place and advance
     seq_lens; see gsd_commit_kv in include/gsd.h.  Enqueued on the current stream."""
+    fast = _native if _lib is not None and _lib is _native_lib else native()
+    r = fast.commit_kv(k_cache, v_cache, draft_k, draft_v, accepted_nodes, accepted_len, seq_lens, status)
+    if r is not None:
+        return _check(r)
     B, Lmax, Hkv, D = k_cache.shape
     N = draft_k.shape[1]
     Tcap = accepted_nodes.shape[1]

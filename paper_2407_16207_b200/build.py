@@ -1,9 +1,11 @@
-"""Builds libgsd.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libgsd.so (the C-ABI CUDA library, nvcc for sm_100a) and the CPython extension that
+marshals the calls, both in-tree."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -11,6 +13,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libgsd.so")
 LIB_CHECK = os.path.join(PKG, "libgsd_check.so")
+NATIVE = os.path.join(PKG, "_native.so")
 OBJ_DIR = os.path.join(PKG, "_build")
 SOURCES = ["gsd_api.cu", "gsd_accept.cu", "gsd_accept_sampled.cu", "gsd_draft.cu", "gsd_attn_mma.cu", "gsd_attn_tc.cu", "gsd_attn_plan.cu", "gsd_commit.cu", "gsd_mask.cu", "gsd_unmerge.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
@@ -29,6 +32,30 @@ def _stale(target: str, deps) -> bool:
         return True
     t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def build_native(force: bool = False) -> str:
+    """Compile csrc/gsd_native.cpp (host code only) against the installed torch and CPython."""
+    import torch
+    src = os.path.join(CSRC, "gsd_native.cpp")
+    if not force and not _stale(NATIVE, [src, os.path.join(ROOT, "include", "gsd.h"), torch.__file__]):
+        return NATIVE
+    base = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.sep in _nvcc() else "/usr/local/cuda"
+    tmp = NATIVE + f".tmp{os.getpid()}"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-isystem", os.path.join(base, "include"),
+           "-isystem", os.path.join(base, "include", "torch", "csrc", "api", "include"),
+           "-isystem", os.path.join(cuda, "include"), "-isystem", sysconfig.get_paths()["include"],
+           src, "-o", tmp, "-L", os.path.join(base, "lib"), "-Wl,-rpath," + os.path.join(base, "lib"),
+           "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+        raise RuntimeError("c++ failed: " + " ".join(cmd))
+    os.replace(tmp, NATIVE)
+    return NATIVE
 
 
 def build(force: bool = False, verbose: bool = False, checked: bool = False) -> str:
@@ -69,4 +96,5 @@ def build(force: bool = False, verbose: bool = False, checked: bool = False) -> 
 
 
 if __name__ == "__main__":
+    print(build_native(force="--force" in sys.argv))
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv, checked="--checked" in sys.argv))
