@@ -64,6 +64,7 @@ AttnPlan attn_make_plan(const gsd_attn_params* p, int sm_count) {
     const int R = p->N * G;
     const int bn = tc ? 128 : 64;
     pl.rows_per_item = tc ? 2 * attn_tcgen05_rows(G) : 64;
+    pl.part_rows = tc ? 256 : 64;
     pl.dev.tiles_per_unit = (R + pl.rows_per_item - 1) / pl.rows_per_item;
     pl.items = pl.dev.tiles_per_unit * p->B * p->Hkv;
     const int tiles = (p->Lmax + bn - 1) / bn + (p->N + bn - 1) / bn;

@@ -1,5 +1,4 @@
-// gsd_verify_attn, warp-level tensor-core back end (mma.sync m16n8k16 bf16, fp32
-// accumulate) and the split-KV merge pass.
+// gsd_verify_attn, warp-level tensor-core back end (mma.sync m16n8k16 bf16, fp32 accumulate).
 //
 // Tree attention over the flattened token graph (Sec. 4.1): every draft node attends to
 // the committed prefix held in the KV cache (Sec. 4.2) and to the draft nodes named by its
@@ -69,7 +68,7 @@ struct MmaParams {
     const uint32_t* mask;
     const int32_t* seq_lens;
     __nv_bfloat16* out;
-    float* part_o;   // [slot][64][D]
+    float* part_o;   // [slot][D / 4][64] float4
     float* part_ml;  // [slot][64][2]
     PlanDev plan;
     int32_t* status;
@@ -329,125 +328,15 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if (!rvalid[h]) continue;
-            const size_t prow = (size_t)slot * BM + rloc[h];
             if (!GSD_IN_BOUNDS(slot >= 0 && slot < p.slots, p.status)) continue;
-            float* dst = p.part_o + prow * D;
 #pragma unroll
             for (int dt = 0; dt < DT; ++dt) {
                 const int col = dt * 8 + (lane & 3) * 2;
-                *reinterpret_cast<float2*>(dst + col) = make_float2(o[dt][h * 2], o[dt][h * 2 + 1]);
+                float* dst = p.part_o + (((size_t)slot * (D / 4) + col / 4) * BM + rloc[h]) * 4 + col % 4;
+                *reinterpret_cast<float2*>(dst) = make_float2(o[dt][h * 2], o[dt][h * 2 + 1]);
             }
-            if ((lane & 3) == 0) *reinterpret_cast<float2*>(p.part_ml + prow * 2) = make_float2(m_run[h], l_run[h]);
+            if ((lane & 3) == 0) *reinterpret_cast<float2*>(p.part_ml + ((size_t)slot * BM + rloc[h]) * 2) = make_float2(m_run[h], l_run[h]);
         }
-    }
-}
-
-// Merge of split-KV partial results: one warp per (split item, row of the item).
-//   m = max_s m_s;  out = sum_s 2^(m_s - m) O_s / sum_s 2^(m_s - m) l_s
-struct MergeParams {
-    const float* part_o;
-    const float* part_ml;
-    __nv_bfloat16* out;
-    PlanDev plan;
-    int N, Hq, Hkv, G, R, D, rows_per_item, items;
-    int rows_used;     // min(rows_per_item, R): rows of an item that can exist
-    long warps_total;  // split items * rows_used
-    const int* bal_hdr;      // balanced plan: [0] = items to merge (known on the device only)
-    const int4* bal_merge;   // balanced plan: (pair, first slot, slots) per pair to merge, else nullptr
-    int bal_groups;          // balanced plan: groups of CTAs
-    SeqTable seq;            // per-sequence plan (hdr == nullptr otherwise); the grid then covers every item
-};
-
-__global__ void __launch_bounds__(256, 4) attn_merge_kernel(MergeParams p) {
-    const long w = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (w >= p.warps_total) return;
-    const int lane = threadIdx.x & 31;
-    const int k = (int)(w / p.rows_used), rloc = (int)(w % p.rows_used);
-    // the k-th item that owns slots: group a comes first when it is split at all
-    int item, nsplit, slot0;
-    const int split_a = p.plan.splits_a > 1 ? p.plan.items_a : 0;
-    if (p.bal_merge) {
-        // the list of cut items was made on the device; the grid covers the most there can be
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        const int tpu = p.plan.tiles_per_unit, rt = k % tpu;
-        const int listed = p.bal_hdr[0];
-        const int4 rec = p.bal_merge[k / tpu];       // a (sequence, kv head) pair that was cut (read beside the count)
-        if (k / tpu >= listed) return;
-        item = rec.x * tpu + rt; slot0 = rt * 2 * p.bal_groups + rec.y; nsplit = rec.z;
-    } else if (p.seq.hdr) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        const int per_seq = p.Hkv * p.plan.tiles_per_unit;
-        const int b = k / per_seq;
-        nsplit = p.seq.nsplit[b];
-        if (nsplit == 1) return;                       // the item was stored by its only unit
-        item = k;
-        slot0 = p.seq.slot_off[b] + (k - b * per_seq) * nsplit;
-    } else if (k < split_a) {
-        item = k; nsplit = p.plan.splits_a; slot0 = k * p.plan.splits_a;
-    } else {
-        item = p.plan.items_a + (k - split_a); nsplit = p.plan.splits_b;
-        slot0 = split_a * p.plan.splits_a + (k - split_a) * p.plan.splits_b;
-    }
-    const int unit = item / p.plan.tiles_per_unit;
-    const int row = (item % p.plan.tiles_per_unit) * p.rows_per_item + rloc;
-    if (row >= p.R) return;
-    const int b = unit / p.Hkv, c = unit % p.Hkv;
-    // Launched as a programmatic dependent of the attention kernel: the blocks may become
-    // resident while that kernel drains; its partial results are only visible after this wait.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // A row costs one trip to memory when it has up to four parts (maxima, sums and accumulators
-    // of all of them are fetched together), and two more per further group of four.
-    const float* ml_base = p.part_ml + ((size_t)slot0 * p.rows_per_item + rloc) * 2;
-    const size_t ml_stride = (size_t)p.rows_per_item * 2;
-    const int per_lane = p.D / 32;  // 2 or 4 consecutive floats per lane
-    const float* o_base = p.part_o + ((size_t)slot0 * p.rows_per_item + rloc) * p.D + lane * per_lane;
-    const size_t o_stride = (size_t)p.rows_per_item * p.D;
-    auto fetch = [&](int s0, float2 (&ml)[4], float4 (&v)[4]) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const bool in = s0 + j < nsplit;
-            ml[j] = in ? *reinterpret_cast<const float2*>(ml_base + (size_t)(s0 + j) * ml_stride)
-                       : make_float2(-CUDART_INF_F, 0.f);
-            const float* src = o_base + (size_t)(s0 + j) * o_stride;
-            if (!in) v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-            else if (per_lane == 4) v[j] = *reinterpret_cast<const float4*>(src);
-            else { const float2 t = *reinterpret_cast<const float2*>(src); v[j] = make_float4(t.x, t.y, 0.f, 0.f); }
-        }
-    };
-    float2 ml[4];
-    float4 v[4];
-    fetch(0, ml, v);
-    float m = fmaxf(fmaxf(ml[0].x, ml[1].x), fmaxf(ml[2].x, ml[3].x));
-#pragma unroll 1
-    for (int s0 = 4; s0 < nsplit; s0 += 4) {
-        float mv[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) mv[j] = s0 + j < nsplit ? ml_base[(size_t)(s0 + j) * ml_stride] : -CUDART_INF_F;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) m = fmaxf(m, mv[j]);
-    }
-    const float m_use = m == -CUDART_INF_F ? 0.f : m;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    float l = 0.f;
-#pragma unroll 1
-    for (int s0 = 0; s0 < nsplit; s0 += 4) {
-        if (s0 > 0) fetch(s0, ml, v);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float wgt = exp2f(ml[j].x - m_use);     // 0 for an absent or empty split
-            l += wgt * ml[j].y;
-            acc[0] += wgt * v[j].x; acc[1] += wgt * v[j].y; acc[2] += wgt * v[j].z; acc[3] += wgt * v[j].w;
-        }
-    }
-    const float inv = l > 0.f ? 1.f / l : 0.f;
-    __nv_bfloat16* dst = p.out + (((size_t)b * p.N + row / p.G) * p.Hq + c * p.G + row % p.G) * p.D + lane * per_lane;
-    if (per_lane == 4) {
-        uint2 v;
-        v.x = pack_bf16(acc[0] * inv, acc[1] * inv);
-        v.y = pack_bf16(acc[2] * inv, acc[3] * inv);
-        *reinterpret_cast<uint2*>(dst) = v;
-    } else {
-        *reinterpret_cast<uint32_t*>(dst) = pack_bf16(acc[0] * inv, acc[1] * inv);
     }
 }
 
@@ -484,50 +373,6 @@ int launch_attn_mma(const AttnArgs& a) {
     if (a.D == 128) return launch_mma_t<128>(a);
     if (a.D == 64) return launch_mma_t<64>(a);
     return GSD_ERR_BAD_SHAPE;
-}
-
-int launch_attn_merge(const AttnArgs& a) {
-    MergeParams p;
-    p.part_o = (const float*)a.workspace;
-    p.part_ml = (const float*)((const char*)a.workspace + plan_part_o_bytes(a.plan, a.D));
-    p.out = (__nv_bfloat16*)a.out;
-    p.plan = a.plan.dev;
-    p.N = a.N; p.Hq = a.Hq; p.Hkv = a.Hkv; p.G = a.G; p.R = a.N * a.G; p.D = a.D;
-    p.rows_per_item = a.plan.rows_per_item; p.items = a.plan.items;
-    int split_items = (a.plan.dev.splits_a > 1 ? a.plan.dev.items_a : 0) +
-                      (a.plan.dev.splits_b > 1 ? a.plan.items - a.plan.dev.items_a : 0);
-    p.bal_hdr = nullptr;
-    p.bal_merge = nullptr;
-    p.bal_groups = 0;
-    p.seq.hdr = nullptr; p.seq.nsplit = nullptr; p.seq.unit_off = nullptr; p.seq.slot_off = nullptr;
-    if (a.plan.dev.balanced == 2) {
-        p.seq = plan_seq_table(a.plan, a.D, a.B, a.workspace);
-        split_items = a.plan.items;
-    } else if (a.plan.dev.balanced) {
-        const BalTable t = plan_bal_table(a.plan, a.D, a.workspace);
-        p.bal_hdr = t.hdr;
-        p.bal_merge = t.merge;
-        const int tpu = a.plan.dev.tiles_per_unit, groups = a.plan.ctas / tpu, pairs = a.plan.items / tpu;
-        p.bal_groups = groups;
-        split_items = (pairs < groups - 1 ? pairs : groups - 1) * tpu;   // one pair per cut at most
-    }
-    p.rows_used = p.R < a.plan.rows_per_item ? p.R : a.plan.rows_per_item;
-    p.warps_total = (long)split_items * p.rows_used;
-    if (p.warps_total == 0) return GSD_OK;
-    const int warps = 8;
-    const long blocks = (p.warps_total + warps - 1) / warps;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3(warps * 32);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = a.stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_merge_kernel, p));
-    return GSD_OK;
 }
 
 }  // namespace gsd

@@ -186,6 +186,9 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t sr
         "cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
         ::"l"(map), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
@@ -392,15 +395,16 @@ struct UnitInfo {
 };
 
 // `w` is the work index of a fixed plan, or the index of the group's unit in the table of a balanced one.
-__device__ __forceinline__ UnitInfo unit_info(const TcParams& p, int w, int lane) {
+// unit_base: all but the mask - which draft tiles are live - so t_begin and ntiles count every draft tile.
+__device__ __forceinline__ UnitInfo unit_base(const TcParams& p, int w) {
     UnitInfo u;
-    int item, t0n = 0, t1n = 0;
+    int item;
     const bool bal = p.bal_units != nullptr;
     if (bal) {
         // the unit of this CTA's group, for the row-tile item this CTA has in every pair
         const int tpu = p.plan.tiles_per_unit, rt = (int)blockIdx.x % tpu;
         const int4 rec = p.bal_units[w];
-        item = rec.x * tpu + rt; t0n = rec.y; t1n = rec.z;
+        item = rec.x * tpu + rt; u.t_begin = rec.y; u.ntiles = rec.z - rec.y;
         u.slot = rec.w >= 0 ? rt * 2 * ((int)gridDim.x / tpu) + rec.w : -1;
         u.split = 0;
         u.nsplit = rec.w >= 0 ? 2 : 1;     // only "one piece or several" matters below
@@ -433,47 +437,67 @@ __device__ __forceinline__ UnitInfo unit_info(const TcParams& p, int w, int lane
     int L = p.seq_lens[u.b];
     L = L < 0 ? 0 : (L > p.Lmax ? p.Lmax : L);
     u.L = L;
-    // OR the mask rows of the unit's nodes, one node per lane
+    u.nPT = (L + BN - 1) / BN;
+    u.live = 0;
+    if (!bal) {
+        const int T = u.nPT + (p.N + BN - 1) / BN;
+        const int per = (T + u.nsplit - 1) / u.nsplit;
+        u.t_begin = min(u.split * per, T);
+        u.ntiles = min(u.t_begin + per, T) - u.t_begin;
+    }
+    return u;
+}
+
+// The draft tiles that hold a visible key for any row of the unit: the OR of the mask rows of its
+// nodes, which are consecutive in memory; eight loads of a lane are on their way at a time.
+__device__ __forceinline__ unsigned unit_live(const TcParams& p, const UnitInfo& u, int lane) {
     const int n_lo = u.row0 / p.G;
     const int n_hi = (min(u.row0 + 2 * p.RT, p.R) - 1) / p.G + 1;
+    const uint32_t* words = p.mask + ((size_t)u.b * p.N + n_lo) * p.W;
+    const uint32_t tail = (p.N & 31) ? (1u << (p.N & 31)) - 1u : 0xFFFFFFFFu;   // valid bits of a row's last word
     unsigned live = 0;
-    const uint32_t tail = (p.N & 31) ? (1u << (p.N & 31)) - 1u : 0xFFFFFFFFu;   // valid bits of the last word
     if ((p.W & 3) == 0 && (reinterpret_cast<uintptr_t>(p.mask) & 15u) == 0) {
-        // four words = one draft tile per 16-byte load; all loads of a row are issued before any is used
-        for (int n = n_lo + lane; n < n_hi; n += 32) {
-            const uint4* mrow = reinterpret_cast<const uint4*>(p.mask + ((size_t)u.b * p.N + n) * p.W);
-            uint4 q[GSD_MAX_NODES / 128];
+        // four words = one draft tile of a row per 16-byte load
+        const int nt = p.W >> 2, total = (n_hi - n_lo) * nt;
+        const uint4* quads = reinterpret_cast<const uint4*>(words);
+#pragma unroll 1
+        for (int base = lane; base < total; base += 8 * 32) {
+            uint4 q[8];
 #pragma unroll
-            for (int t = 0; t < GSD_MAX_NODES / 128; ++t) q[t] = t < (p.W >> 2) ? mrow[t] : make_uint4(0, 0, 0, 0);
+            for (int k = 0; k < 8; ++k) q[k] = base + 32 * k < total ? quads[base + 32 * k] : make_uint4(0, 0, 0, 0);
 #pragma unroll
-            for (int t = 0; t < GSD_MAX_NODES / 128; ++t) {
-                if (t == (p.W >> 2) - 1) q[t].w &= tail;
-                if (q[t].x | q[t].y | q[t].z | q[t].w) live |= 1u << t;
+            for (int k = 0; k < 8; ++k) {
+                const int t = (base + 32 * k) % nt;
+                if (t == nt - 1) q[k].w &= tail;
+                if (q[k].x | q[k].y | q[k].z | q[k].w) live |= 1u << t;
             }
         }
     } else {
-        for (int n = n_lo + lane; n < n_hi; n += 32) {
-            const uint32_t* mrow = p.mask + ((size_t)u.b * p.N + n) * p.W;
-            for (int wi = 0; wi < p.W; ++wi) {
-                uint32_t word = mrow[wi];
-                if (wi == p.W - 1) word &= tail;
-                if (word) live |= 1u << (wi >> 2);
+        const int total = (n_hi - n_lo) * p.W;
+#pragma unroll 1
+        for (int base = lane; base < total; base += 8 * 32) {
+            uint32_t q[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) q[k] = base + 32 * k < total ? words[base + 32 * k] : 0u;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int wi = (base + 32 * k) % p.W;
+                if (wi == p.W - 1) q[k] &= tail;
+                if (q[k]) live |= 1u << (wi >> 2);
             }
         }
     }
-    u.live = __reduce_or_sync(0xFFFFFFFFu, live);
-    u.nPT = (L + BN - 1) / BN;
-    if (bal) {
-        // the table counts every draft tile; here only those with a visible key are numbered
-        auto live_index = [&](int t) { return t <= u.nPT ? t : u.nPT + __popc(u.live & ((1u << (t - u.nPT)) - 1u)); };
-        u.t_begin = live_index(t0n);
-        u.ntiles = live_index(t1n) - u.t_begin;
-        return u;
-    }
-    const int T = u.nPT + __popc(u.live);
-    const int per = (T + u.nsplit - 1) / u.nsplit;
-    u.t_begin = min(u.split * per, T);
-    u.ntiles = min(u.t_begin + per, T) - u.t_begin;
+    return __reduce_or_sync(0xFFFFFFFFu, live);
+}
+
+// The whole unit: live draft tiles only are numbered.
+__device__ __forceinline__ UnitInfo unit_info(const TcParams& p, int w, int lane) {
+    UnitInfo u = unit_base(p, w);
+    u.live = unit_live(p, u, lane);
+    auto live_index = [&](int t) { return t <= u.nPT ? t : u.nPT + __popc(u.live & ((1u << (t - u.nPT)) - 1u)); };
+    const int t0 = live_index(u.t_begin), t1 = live_index(u.t_begin + u.ntiles);
+    u.t_begin = t0;
+    u.ntiles = t1 - t0;
     return u;
 }
 
@@ -509,9 +533,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
     volatile int* abort_flag = &s_wait.abort;
 
-    if (tid == 0) {
+    if (warp == 8 && lane == 0) {
         // the merge pass (a programmatic dependent launch) may be made resident as CTAs retire
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        // the first copy through a tensor map would otherwise fetch it from memory first
+        prefetch_map(&tm_q); prefetch_map(&tm_k); prefetch_map(&tm_v); prefetch_map(&tm_dk); prefetch_map(&tm_dv); prefetch_map(&tm_out);
         s_wait.abort = 0;
         s_wait.limit_ns = p.wait_limit_ns;
         mbar_init(bar(BAR_Q_FULL), 1);
@@ -532,6 +558,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             mbar_init(bar(BAR_DRAIN + i), 1);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 10) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&s_tmem_base)) : "memory");
@@ -547,15 +574,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    // This kernel is launched as a programmatic dependent of whatever precedes it on the stream:
+    // everything above may run beside the end of that, nothing below may.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // The CTA's units: work indices blockIdx.x, blockIdx.x + gridDim.x, ... of a fixed plan, or
-    // a run of the table that the planning kernel (this kernel is its programmatic dependent)
-    // has written.
+    // a run of the table that the planning kernel has written.
     int n_my;
     if (p.bal_cta) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
         n_my = p.bal_cta[blockIdx.x / p.plan.tiles_per_unit].y;
     } else if (p.seq.hdr) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
         const int units = p.seq.hdr[0];
         n_my = units > (int)blockIdx.x ? (units - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     } else {
@@ -565,13 +592,46 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     auto unit_index = [&](int it) -> int {
         return p.bal_cta ? p.bal_cta[blockIdx.x / p.plan.tiles_per_unit].x + it : (int)blockIdx.x + it * (int)gridDim.x;
     };
-    // Decoding a unit costs two dependent trips to global memory (sequence length, mask rows).
-    // Each warp decodes one of the CTA's first units here, all at once, so that no role pays
-    // that latency between units.
-    for (int k = warp; k < kUnitTable; k += kThreads / 32) {
-        if (k < n_my) {
-            const UnitInfo u = unit_info(p, unit_index(k), lane);
-            if (lane == 0) s_units[k] = u;
+    // The copies of one key tile (into ring slot n % ST, the n-th of the CTA).
+    auto load_k = [&](const UnitInfo& u, int idx, int n) {
+        const TileInfo ti = tile_info(u.t_begin + idx, u.nPT, u.L, u.live);
+        mbar_expect_tx(bar(BAR_K_FULL + n % ST), TILE_BYTES);
+        if (p.withhold_first_k && n == 0) return;        // (test hook: the bytes announced above never arrive)
+        for (int h = 0; h < T::BLOCKS; ++h)
+            tma_load_4d(sK + (n % ST) * TILE_BYTES + h * HALF_BYTES, ti.kind == 2 ? &tm_dk : &tm_k, bar(BAR_K_FULL + n % ST), h * 64, u.c, ti.key0, u.b);
+    };
+    auto load_v = [&](const UnitInfo& u, int idx, int n) {
+        const TileInfo ti = tile_info(u.t_begin + idx, u.nPT, u.L, u.live);
+        mbar_expect_tx(bar(BAR_V_FULL + n % ST), TILE_BYTES);
+        for (int h = 0; h < T::BLOCKS; ++h)
+            tma_load_4d(sV + (n % ST) * TILE_BYTES + h * HALF_BYTES, ti.kind == 2 ? &tm_dv : &tm_v, bar(BAR_V_FULL + n % ST), h * 64, u.c, ti.key0, u.b);
+    };
+    auto load_q = [&](const UnitInfo& u) {
+        const int ntile_rows = u.two ? 2 : 1;
+        mbar_expect_tx(bar(BAR_Q_FULL), (uint32_t)(ntile_rows * T::BLOCKS * RT) * 128u);
+        for (int i = 0; i < ntile_rows; ++i)
+            for (int h = 0; h < T::BLOCKS; ++h)
+                tma_load_4d(sQ + i * TILE_BYTES + h * HALF_BYTES, &tm_q, bar(BAR_Q_FULL), h * 64, u.c * G, (u.row0 + i * RT) / G, u.b);
+    };
+    // Decoding a unit costs a trip to global memory or two (sequence length, mask rows).  The warps
+    // decode the CTA's first units here, all at once, so that no role pays that latency between
+    // units.  The producer warp does not wait for the mask: it issues the copies of Q and of the
+    // first prefix tiles - as many as the empty rings hold - as soon as it knows the length.
+    int pre = 0;             // producer: key tiles of unit 0 already on their way
+    if (warp == 8) {
+        if (n_my > 0 && lane == 0) {
+            const UnitInfo u = unit_base(p, unit_index(0));
+            pre = max(0, min(ST, min(u.nPT - u.t_begin, u.ntiles)));
+            if (pre > 0) load_q(u);
+            for (int n = 0; n < pre; ++n) { load_k(u, n, n); load_v(u, n, n); }
+        }
+        pre = __shfl_sync(0xFFFFFFFFu, pre, 0);
+    } else {
+        for (int k = warp < 8 ? warp : warp - 1; k < kUnitTable; k += kThreads / 32 - 1) {
+            if (k < n_my) {
+                const UnitInfo u = unit_info(p, unit_index(k), lane);
+                if (lane == 0) s_units[k] = u;
+            }
         }
     }
     tc_fence_before();
@@ -586,58 +646,51 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     asm volatile("setmaxnreg.dec.sync.aligned.u32 96;");
     if (warp == 8) {
         // ------------------------------------------------------------ TMA producer
-        int kvc = 0;          // key tiles loaded so far (ring position)
-        int au = 0;           // non-empty units so far
-        bool ok = true, q_pending = false;
+        // K copies run one tile ahead of the V copies: K t + 1 only waits for the QK^T of tile
+        // t - 1, and its time to land passes while V t waits for the PV of tile t - 2 (4 x 40
+        // heads, N 128, L 1024-4096: 58.4 us in step with the V copies, 55.4 one ahead).
+        int kc = pre, vc = pre;         // K and V tiles loaded so far (ring positions)
+        int au = 0;                     // non-empty units so far
+        bool ok = true, q_pending = pre > 0;
         for (int it = 0; it < n_my && ok; ++it) {
             const UnitInfo u = unit_of(it);
             if (u.ntiles == 0) continue;
             if (lane == 0) {
-                // Q of the previous unit is free once its last QK^T has completed
-                ok = mbar_wait(bar(BAR_Q_EMPTY), (au & 1) ^ 1, abort_flag, p.status);
-                if (ok) {
-                    const int ntile_rows = u.two ? 2 : 1;
-                    mbar_expect_tx(bar(BAR_Q_FULL), (uint32_t)(ntile_rows * T::BLOCKS * RT) * 128u);
-                    for (int i = 0; i < ntile_rows; ++i)
-                        for (int h = 0; h < T::BLOCKS; ++h)
-                            tma_load_4d(sQ + i * TILE_BYTES + h * HALF_BYTES, &tm_q, bar(BAR_Q_FULL), h * 64, u.c * G,
-                                        (u.row0 + i * RT) / G, u.b);
-                    q_pending = true;
-                }
-                for (int idx = 0; idx < u.ntiles && ok; ++idx) {
-                    const TileInfo ti = tile_info(u.t_begin + idx, u.nPT, u.L, u.live);
-                    const CUtensorMap* mk = ti.kind == 2 ? &tm_dk : &tm_k;
-                    const CUtensorMap* mv = ti.kind == 2 ? &tm_dv : &tm_v;
-                    const int s = kvc % ST;
-                    const uint32_t par = (uint32_t)((kvc / ST) & 1) ^ 1u;
-                    ok = mbar_wait(bar(BAR_K_EMPTY + s), par, abort_flag, p.status);
-                    if (!ok) break;
-                    mbar_expect_tx(bar(BAR_K_FULL + s), TILE_BYTES);
-                    if (!(p.withhold_first_k && kvc == 0))   // (test hook: the bytes announced above never arrive)
-                        for (int h = 0; h < T::BLOCKS; ++h)
-                            tma_load_4d(sK + s * TILE_BYTES + h * HALF_BYTES, mk, bar(BAR_K_FULL + s), h * 64, u.c, ti.key0, u.b);
-                    ok = mbar_wait(bar(BAR_V_EMPTY + s), par, abort_flag, p.status);
-                    if (!ok) {
-                        // the K copy just issued is still in flight: let it land
-                        mbar_wait_slow(bar(BAR_K_FULL + s), (kvc / ST) & 1, abort_flag, nullptr, true);
-                        break;
+                const bool begun = it == 0 && pre > 0;
+                if (!begun) {
+                    // Q of the previous unit is free once its last QK^T has completed
+                    ok = mbar_wait(bar(BAR_Q_EMPTY), (au & 1) ^ 1, abort_flag, p.status);
+                    if (ok) {
+                        load_q(u);
+                        q_pending = true;
                     }
-                    mbar_expect_tx(bar(BAR_V_FULL + s), TILE_BYTES);
-                    for (int h = 0; h < T::BLOCKS; ++h)
-                        tma_load_4d(sV + s * TILE_BYTES + h * HALF_BYTES, mv, bar(BAR_V_FULL + s), h * 64, u.c, ti.key0, u.b);
-                    ++kvc;
+                }
+                int kn = begun ? pre : 0, vn = kn;      // next tile of the unit
+                while (ok && vn < u.ntiles) {
+                    if (kn < u.ntiles && kn <= vn + 1) {
+                        if (!(ok = mbar_wait(bar(BAR_K_EMPTY + kc % ST), (uint32_t)((kc / ST) & 1) ^ 1u, abort_flag, p.status))) break;
+                        load_k(u, kn, kc);
+                        ++kn;
+                        ++kc;
+                    } else {
+                        if (!(ok = mbar_wait(bar(BAR_V_EMPTY + vc % ST), (uint32_t)((vc / ST) & 1) ^ 1u, abort_flag, p.status))) break;
+                        load_v(u, vn, vc);
+                        ++vn;
+                        ++vc;
+                    }
                 }
                 if (!ok) {
                     // gave up: let the copies already in flight land before the CTA retires
                     if (q_pending) mbar_wait_slow(bar(BAR_Q_FULL), au & 1, abort_flag, nullptr, true);
-                    for (int t = max(0, kvc - ST); t < kvc; ++t) {
+                    for (int t = max(0, kc - ST); t < kc; ++t)
                         mbar_wait_slow(bar(BAR_K_FULL + t % ST), (t / ST) & 1, abort_flag, nullptr, true);
+                    for (int t = max(0, vc - ST); t < vc; ++t)
                         mbar_wait_slow(bar(BAR_V_FULL + t % ST), (t / ST) & 1, abort_flag, nullptr, true);
-                    }
                 }
             }
             ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
-            kvc = __shfl_sync(0xFFFFFFFFu, kvc, 0);
+            kc = __shfl_sync(0xFFFFFFFFu, kc, 0);
+            vc = __shfl_sync(0xFFFFFFFFu, vc, 0);
             ++au;
         }
     } else if (warp == 9) {
@@ -991,16 +1044,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     wg_barrier(1 + i);
                 }
             } else if (rvalid) {
-                {
-                    const size_t prow = (size_t)u.slot * (2 * RT) + (alt ? 0 : i * RT) + rloc;
-                    if (GSD_IN_BOUNDS(u.slot >= 0 && u.slot < p.slots, p.status)) {
-                    float* dst = p.part_o + prow * HD;
+                // a partial result: float4 columns of the row tile, so that the 32 rows of a warp
+                // are consecutive in memory (stored row by row, 32 rows per store instruction, the
+                // store took about 1 us longer)
+                const size_t tile = (size_t)u.slot * 2 + (alt ? 0 : i);
+                if (GSD_IN_BOUNDS(u.slot >= 0 && u.slot < p.slots, p.status)) {
+                    float4* dst = reinterpret_cast<float4*>(p.part_o) + tile * (HD / 4) * BM + rloc;
 #pragma unroll
-                    for (int k = 0; k < HD / 4; ++k)
-                        *reinterpret_cast<float4*>(dst + k * 4) =
-                            make_float4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
-                    *reinterpret_cast<float2*>(p.part_ml + prow * 2) = make_float2(m_ref, l_run);
-                    }
+                    for (int k = 0; k < HD / 4; ++k) dst[k * BM] = make_float4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
+                    *reinterpret_cast<float2*>(p.part_ml + (tile * BM + rloc) * 2) = make_float2(m_ref, l_run);
                 }
             }
             kvc += ntiles;
@@ -1099,32 +1151,24 @@ static int launch_tc(const AttnArgs& a) {
     p.bal_cta = nullptr;
     p.bal_units = nullptr;
     p.seq.hdr = nullptr; p.seq.nsplit = nullptr; p.seq.unit_off = nullptr; p.seq.slot_off = nullptr;
-    if (a.plan.dev.balanced) {
-        // one CTA per share of the table; the table is being written by the planning kernel,
-        // beside which this kernel may start
-        if (a.plan.dev.balanced == 2) {
-            p.seq = plan_seq_table(a.plan, a.D, a.B, a.workspace);
-        } else {
-            const BalTable t = plan_bal_table(a.plan, a.D, a.workspace);
-            p.bal_cta = t.cta;
-            p.bal_units = t.units;
-        }
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)a.plan.ctas);
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = Geo<HD>::SMEM_BYTES;
-        cfg.stream = a.stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD>, tq, tk, tv, tdk, tdv, tout, p));
-        return GSD_OK;
+    if (a.plan.dev.balanced == 2) {
+        p.seq = plan_seq_table(a.plan, a.D, a.B, a.workspace);
+    } else if (a.plan.dev.balanced) {
+        const BalTable t = plan_bal_table(a.plan, a.D, a.workspace);
+        p.bal_cta = t.cta;
+        p.bal_units = t.units;
     }
-    dim3 grid(a.plan.ctas < di.sm_count ? a.plan.ctas : di.sm_count);
-    attn_tc_kernel<HD><<<grid, kThreads, Geo<HD>::SMEM_BYTES, a.stream>>>(tq, tk, tv, tdk, tdv, tout, p);
-    GSD_CUDA_TRY(cudaGetLastError());
+    // persistent CTAs; the kernel sets itself up beside the end of its predecessor on the stream
+    cudaLaunchAttribute attr[1];
+    dependent_launch_attr(attr);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(a.plan.dev.balanced || a.plan.ctas < di.sm_count ? a.plan.ctas : di.sm_count));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Geo<HD>::SMEM_BYTES;
+    cfg.stream = a.stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD>, tq, tk, tv, tdk, tdv, tout, p));
     return GSD_OK;
 }
 

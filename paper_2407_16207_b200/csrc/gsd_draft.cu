@@ -103,6 +103,7 @@ __device__ void grow_sequence(const DraftArgs& a, int b) {
     int fl = a.frontier_len[b];
     if (n0 < 1 || n0 > Ncap || fl < 0 || fl > a.F) {
         // nothing sensible can be appended: leave the graph as it is
+        asm volatile("griddepcontrol.wait;" ::: "memory");     // (this grid never ends before the first launch)
         if (tid == 0) {
             a.new_frontier_len[b] = 0;
             if (a.status) atomicOr((unsigned*)a.status, GSD_DEV_BAD_FRONTIER);

@@ -73,7 +73,8 @@ struct PlanDev {
 };
 struct AttnPlan {
     int kernel;         // GSD_ATTN_MMA or GSD_ATTN_TCGEN05
-    int rows_per_item;  // 64 (mma.sync back end) or two row tiles of attn_tcgen05_rows(G) (tcgen05 back end)
+    int rows_per_item;  // stacked rows of an item: 64 (mma.sync back end) or two row tiles of attn_tcgen05_rows(G) (tcgen05 back end)
+    int part_rows;      // rows of a partial-result slot: 64 or 2 x 128
     int items;
     int ctas;
     int slots;          // partial-result slots; 0 when nothing is split
@@ -122,9 +123,12 @@ struct AttnArgs {
 };
 
 int attn_pick_kernel(const gsd_attn_params* p);                 // GSD_ATTN_MMA or GSD_ATTN_TCGEN05
-// partial results: fp32 accumulators [slot][rows_per_item][D], then (max, sum) [slot][rows_per_item][2]
-inline size_t plan_part_o_bytes(const AttnPlan& pl, int D) { return align_up((size_t)pl.slots * pl.rows_per_item * D * sizeof(float), 256); }
-inline size_t plan_part_ml_bytes(const AttnPlan& pl) { return align_up((size_t)pl.slots * pl.rows_per_item * 2 * sizeof(float), 256); }
+// Partial results: fp32 accumulators, then (max, sum) pairs.  A slot holds the row tiles of an item
+// (one of 64 rows, or two of 128); a tile is [D / 4 column groups][rows] of float4 - the rows of a
+// column group are consecutive, for the store of an accumulator (a lane per row) and for the merge
+// alike - and [rows] of float2.
+inline size_t plan_part_o_bytes(const AttnPlan& pl, int D) { return align_up((size_t)pl.slots * pl.part_rows * D * sizeof(float), 256); }
+inline size_t plan_part_ml_bytes(const AttnPlan& pl) { return align_up((size_t)pl.slots * pl.part_rows * 2 * sizeof(float), 256); }
 
 // The table of a per-sequence plan, in the workspace behind the partial results.
 struct SeqTable {
