@@ -56,7 +56,7 @@ int attn_pick_kernel(const gsd_attn_params* p) {
     return GSD_ATTN_MMA;
 }
 
-AttnPlan attn_make_plan(const gsd_attn_params* p, int sm_count) {
+AttnPlan attn_make_plan(const gsd_attn_params* p, int sm_count, bool by_length) {
     AttnPlan pl;
     pl.kernel = attn_pick_kernel(p);
     const bool tc = pl.kernel == GSD_ATTN_TCGEN05;
@@ -76,6 +76,7 @@ AttnPlan attn_make_plan(const gsd_attn_params* p, int sm_count) {
     pl.dev.splits_a = 1;
     pl.dev.splits_b = 1;
     pl.dev.balanced = 0;
+    pl.dev.longest_first = 0;
     // Shares of key tiles dealt out on the device from the true sequence lengths: on request
     // only.  Every cut costs a partial result (an fp32 accumulator tile written and read back,
     // as much traffic as a key tile), so it pays when the lengths of a batch differ by far
@@ -106,6 +107,14 @@ AttnPlan attn_make_plan(const gsd_attn_params* p, int sm_count) {
         pl.ws_bytes = plan_part_o_bytes(pl, p->D) + plan_part_ml_bytes(pl) + plan_bal_bytes(pl, p->B);
         return pl;
     }
+    if (tc && by_length && p->num_splits == 0 && pl.items <= resident && max_split > 1 && p->B > 1 && p->B <= 32) {
+        pl.dev.balanced = 3;
+        pl.ctas = resident;
+        pl.slots = resident;                        // unit w owns slot w
+        pl.ws_bytes = plan_part_o_bytes(pl, p->D) + plan_part_ml_bytes(pl) + plan_bal_bytes(pl, p->B);
+        return pl;
+    }
+    pl.dev.longest_first = tc && by_length && p->num_splits == 0 && pl.items > resident && p->B > 1 && p->B <= kPlanSeqs;
     if (p->num_splits > 0) {
         pl.dev.splits_a = p->num_splits;
     } else if (pl.items < resident) {
@@ -128,7 +137,7 @@ AttnPlan attn_make_plan(const gsd_attn_params* p, int sm_count) {
     pl.ctas = pl.dev.items_a * pl.dev.splits_a + items_b * pl.dev.splits_b;
     pl.slots = (pl.dev.splits_a > 1 ? pl.dev.items_a * pl.dev.splits_a : 0) +
                (pl.dev.splits_b > 1 ? items_b * pl.dev.splits_b : 0);
-    pl.ws_bytes = pl.slots ? plan_part_o_bytes(pl, p->D) + plan_part_ml_bytes(pl) : 0;
+    pl.ws_bytes = pl.slots ? plan_part_o_bytes(pl, p->D) + plan_part_ml_bytes(pl) + plan_bal_bytes(pl, p->B) : 0;
     return pl;
 }
 
@@ -161,7 +170,8 @@ extern "C" int gsd_verify_attn_num_splits(const gsd_attn_params* p) {
     if (attn_params_ok(p) != GSD_OK) return 0;
     DeviceInfo di;
     if (device_info(&di) != 0) return 0;
-    const AttnPlan pl = attn_make_plan(p, di.sm_count);
+    // (for a plan made from the lengths on the device: the count for sequences that fill the cache)
+    const AttnPlan pl = attn_make_plan(p, di.sm_count, false);
     if (pl.dev.balanced) return pl.dev.balanced == 2 ? GSD_ATTN_SPLIT_PER_SEQUENCE : GSD_ATTN_SPLIT_BALANCED;
     return pl.dev.splits_a > pl.dev.splits_b ? pl.dev.splits_a : pl.dev.splits_b;
 }
@@ -188,7 +198,9 @@ extern "C" int gsd_verify_attn(const void* q, const void* k_cache, const void* v
     if (((uintptr_t)ancestor_mask & 3u) != 0 || ((uintptr_t)seq_lens & 3u) != 0) return GSD_ERR_MISALIGNED;
     DeviceInfo di;
     if (device_info(&di) != 0) return GSD_ERR_CUDA;
-    const AttnPlan plan = attn_make_plan(p, di.sm_count);
+    AttnPlan plan = attn_make_plan(p, di.sm_count);
+    // scratch sized for the plan without the lengths is enough: that plan is then taken
+    if (plan.ws_bytes > 0 && (!workspace || workspace_bytes < plan.ws_bytes)) plan = attn_make_plan(p, di.sm_count, false);
     const size_t need = plan.ws_bytes;
     if (need > 0) {
         if (!workspace || workspace_bytes < need) return GSD_ERR_WORKSPACE;
@@ -208,7 +220,7 @@ extern "C" int gsd_verify_attn(const void* q, const void* k_cache, const void* v
     a.plan = plan; a.workspace = workspace; a.status = status;
     a.stream = (cudaStream_t)stream;
     int rc = GSD_OK;
-    if (plan.dev.balanced && (rc = launch_attn_plan(a)) != GSD_OK) return rc;
+    if ((plan.dev.balanced == 1 || plan.dev.balanced == 2) && (rc = launch_attn_plan(a)) != GSD_OK) return rc;
     rc = plan.kernel == GSD_ATTN_TCGEN05 ? launch_attn_tcgen05(a) : launch_attn_mma(a);
     if (rc != GSD_OK) return rc;
     if (plan.slots > 0) rc = launch_attn_merge(a);

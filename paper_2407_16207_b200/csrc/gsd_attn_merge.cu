@@ -32,6 +32,8 @@ struct MergeParams {
     const int4* bal_merge;   // balanced plan: (pair, first slot, slots) per pair to merge, else nullptr
     int bal_groups;          // balanced plan: groups of CTAs
     SeqTable seq;            // per-sequence plan (hdr == nullptr otherwise); the grid then covers every item
+    const int* left;         // one-wave plan: split counts, then (left_off on) first units per sequence; longest
+    int left_off;            // first: the sequences in order; else nullptr
 };
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
@@ -50,7 +52,7 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
     // after this wait.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // the k-th item that owns slots: group a comes first when it is split at all
-    int item, nsplit, slot0;
+    int item, nsplit, slot0, slot_step = 1;
     const int split_a = p.plan.splits_a > 1 ? p.plan.items_a : 0;
     if (p.bal_merge) {
         // the list of cut items was made on the device; the grid covers the most there can be
@@ -66,6 +68,14 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
         if (nsplit == 1) return;                       // the item was stored by its only unit
         item = k;
         slot0 = p.seq.slot_off[b] + (k - b * per_seq) * nsplit;
+    } else if (p.plan.balanced == 3) {
+        const int per_seq = p.Hkv * p.plan.tiles_per_unit;
+        const int b = k / per_seq;
+        nsplit = p.left[b];
+        if (nsplit == 1) return;
+        item = k;
+        slot0 = p.left[p.left_off + b] + (k - b * per_seq);
+        slot_step = per_seq;
     } else if (k < split_a) {
         item = k; nsplit = p.plan.splits_a; slot0 = k * p.plan.splits_a;
     } else {
@@ -77,12 +87,12 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
     const int unit = item / p.plan.tiles_per_unit;
     const int row = (item % p.plan.tiles_per_unit) * p.tiles * p.RT + tile * p.RT + r;
     if (r >= p.RT || row >= p.R) return;
-    const int b = unit / p.Hkv, c = unit % p.Hkv;
+    const int b = p.plan.longest_first ? p.left[unit / p.Hkv] : unit / p.Hkv, c = unit % p.Hkv;
 
     const size_t first = (size_t)slot0 * p.tiles + tile;
     const float2* ml_base = p.part_ml + first * p.tile_rows + r;
     const float4* o_base = p.part_o + (first * quads + col0) * p.tile_rows + r;
-    const size_t ml_stride = (size_t)p.tiles * p.tile_rows, o_stride = ml_stride * quads;
+    const size_t ml_stride = (size_t)slot_step * p.tiles * p.tile_rows, o_stride = ml_stride * quads;
     float2 ml[kBatch];
     float4 v[kBatch][2];
     auto fetch = [&](int s0) {
@@ -144,7 +154,11 @@ int launch_attn_merge(const AttnArgs& a) {
     p.bal_merge = nullptr;
     p.bal_groups = 0;
     p.seq.hdr = nullptr; p.seq.nsplit = nullptr; p.seq.unit_off = nullptr; p.seq.slot_off = nullptr;
-    if (a.plan.dev.balanced == 2) {
+    p.left = a.plan.dev.balanced == 3 || a.plan.dev.longest_first ? plan_left_table(a.plan, a.D, a.workspace) : nullptr;
+    p.left_off = (int)(align_up((size_t)a.B * sizeof(int), 256) / sizeof(int));
+    if (a.plan.dev.balanced == 3) {
+        split_items = a.plan.items;
+    } else if (a.plan.dev.balanced == 2) {
         p.seq = plan_seq_table(a.plan, a.D, a.B, a.workspace);
         split_items = a.plan.items;
     } else if (a.plan.dev.balanced) {

@@ -52,19 +52,31 @@ constexpr int kThreads = 384;
 // accumulators are half as wide and each stream has its own, so a stream's QK^T only waits for
 // that stream's own softmax (at HD = 64 the exponentials cost twice the tensor time: the softmax
 // warps must never wait).
+// Where a CTA's units come from is a template argument: the first microseconds of a call are bound by
+// the fetch of the kernel's own instructions, and with all the plans in one kernel a call of a few
+// tiles started 1.5 us later.
+enum PlanKind {
+    PLAN_FIXED,     // host plan
+    PLAN_ORDERED,   // host plan, longest sequences first
+    PLAN_WAVE,      // one-wave plan
+    PLAN_TABLE      // tables built by a planning kernel
+};
+
 template <int HD>
 struct Geo {
     static constexpr int BLOCKS = HD / 64;
     static constexpr uint32_t TILE_BYTES = BLOCKS * HALF_BYTES;   // a 128 x HD bf16 tile
     static constexpr int ST = HD == 128 ? 2 : 4;                  // stages of the K ring and of the V ring
-    static constexpr uint32_t SMEM_BYTES = (2 + 2 * ST) * TILE_BYTES + 2 * HALF_BYTES + 1024;  // tiles, output staging, alignment slack
+    static constexpr uint32_t SMEM_BYTES = (2 + 2 * ST) * TILE_BYTES + 1024;  // tiles, alignment slack
     static constexpr bool TWO_S = HD == 64;
     static constexpr uint32_t COL_S0 = 0, COL_P0 = 128, COL_P1 = 192, COL_O0 = 256, COL_O1 = 256 + HD;
     static constexpr uint32_t COL_S1 = TWO_S ? 384 : COL_S0;
     static_assert(COL_O1 + HD <= (TWO_S ? 384 : 512), "512 TMEM columns");
 };
 constexpr float kRescaleThreshold = 8.0f;         // log2 units
-constexpr int kUnitTable = 12;                    // units of work per CTA decoded in the prologue (one per warp)
+// Units of work per CTA decoded in the prologue.  A fixed plan with more is launched in several parts;
+// only the plans from tables decode further units where they are needed.
+constexpr int kUnitTable = 128;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // default limit of every in-kernel wait
 
 // Test hook (see gsd_debug_attn_wait): a shorter limit and, optionally, a CTA's first K tile
@@ -106,14 +118,18 @@ struct TcParams {
     float* part_o;
     float* part_ml;
     int32_t* status;
+    int out_by_32;    // `out` starts on a 32-byte boundary (16 is all that is promised)
     int B, N, Hq, Hkv, Lmax, G, W, R;
     int RT;           // stacked rows a row tile holds: the whole nodes that fit 128 rows, 128 / G * G
     float scale_log2;
     PlanDev plan;
-    int total_work;   // CTAs of the plan = units of work
+    int work0;        // first unit of this launch
+    int total_work;   // units of work of this launch
     int slots;        // partial-result slots of the plan
     const int2* bal_cta;     // balanced plan: (first unit, units) of every group of CTAs, else nullptr
     const int4* bal_units;   // balanced plan: (pair, first tile, end tile, slot or -1)
+    int* left;               // what the merge pass needs of a plan made here (plan_left_table)
+    int left_off;
     SeqTable seq;            // per-sequence plan: split counts and unit / slot offsets (hdr == nullptr otherwise)
     unsigned long long wait_limit_ns;
     int withhold_first_k;   // test hook: every CTA leaves out the K copy of its first key tile
@@ -180,27 +196,8 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
 
-// shared -> global tile store; completion is tracked by bulk async-groups of the issuing thread
-__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2, int c3) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
-        ::"l"(map), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
-}
 __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
-__device__ __forceinline__ void wg_barrier(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
-// the same hardware barrier of a warpgroup with an AND over a flag: every thread gets the answer
-__device__ __forceinline__ bool wg_all(int id, bool flag) {
-    uint32_t r;
-    asm volatile(
-        "{\n .reg .pred p, q;\n setp.ne.u32 q, %2, 0;\n bar.red.and.pred p, %1, 128, q;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(r) : "r"(id), "r"((uint32_t)flag) : "memory");
-    return r != 0;
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -250,6 +247,11 @@ __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16])
         : "memory");
 }
 
+// 32 bytes to a 32-byte aligned address
+__device__ __forceinline__ void st_global8(void* dst, const uint32_t (&v)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
 // pointer form: v[0..31] must be register-resident (constant indices after unrolling)
 __device__ __forceinline__ void tc_ld32p(uint32_t taddr, float* v) {
     uint32_t* r = reinterpret_cast<uint32_t*>(v);
@@ -384,6 +386,58 @@ __device__ __forceinline__ TileInfo tile_info(int t, int nPT, int L, unsigned li
     return ti;
 }
 
+__device__ __forceinline__ int visible_len(const TcParams& p, int b) {
+    const int L = p.seq_lens[b];
+    return L < 0 ? 0 : (L > p.Lmax ? p.Lmax : L);
+}
+
+// The order of the sequences made by the CTA itself (longest first), in shared memory.
+struct Order {
+    const int* len;      // [B] visible lengths
+    const int* seq;      // [B] sequences in order
+};
+
+// One-wave plan: what it says about unit w.  Made by one warp, a lane per sequence, without a barrier:
+// all of it lies between the launch and the first copy.
+struct WaveUnit {
+    int units;                     // of the whole call
+    int b, L, nsplit, r;           // unit w: sequence, its length and key ranges per item, unit inside the sequence
+};
+__device__ __forceinline__ WaveUnit wave_unit(const TcParams& p, int w, int lane, bool leave) {
+    const unsigned all = 0xFFFFFFFFu;
+    const bool in = lane < p.B;
+    const int nd = (p.N + BN - 1) / BN, per_seq = p.Hkv * p.plan.tiles_per_unit, resident = (int)gridDim.x;
+    const int L = in ? visible_len(p, lane) : 0;
+    const int t = in ? (L + BN - 1) / BN + nd : 0;
+    const int total = __reduce_add_sync(all, t), longest = __reduce_max_sync(all, t);
+    // lane k tries the k-th candidate for the tiles of a unit, from the lower bound on (at least four
+    // tiles, at most 32 parts an item); the longest sequence whole always fits, as there are no more
+    // items than CTAs
+    const int bound = max(max((total * per_seq + resident - 1) / resident, (longest + 31) / 32), 4);
+    const int T = bound + lane * max(1, bound / 16);
+    int units = 0;
+    for (int j = 0; j < p.B; ++j) units += (__shfl_sync(all, t, j) + T - 1) / T;
+    const int best = min(longest, (int)__reduce_min_sync(all, units * per_seq <= resident ? T : 0x7FFFFFFF));
+    const int n = in ? (t + best - 1) / best : 0;
+    int end = n;                                            // units up to and with this sequence, per item
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int before = __shfl_up_sync(all, end, o);
+        if (lane >= o) end += before;
+    }
+    WaveUnit u;
+    u.units = __shfl_sync(all, end, 31) * per_seq;
+    if (leave && in) {                                      // for the merge pass
+        p.left[lane] = n;
+        p.left[p.left_off + lane] = (end - n) * per_seq;
+    }
+    u.b = min(__popc(__ballot_sync(all, in && end * per_seq <= w)), p.B - 1);
+    u.L = __shfl_sync(all, L, u.b);
+    u.nsplit = __shfl_sync(all, n, u.b);
+    u.r = w - __shfl_sync(all, end - n, u.b) * per_seq;
+    return u;
+}
+
 // What a role needs to know about one unit of work (a row pair of one (sequence, kv head) and
 // a key range).  Every warp derives it on its own from the work index, so the roles never
 // have to meet at a CTA-wide barrier between units.
@@ -395,11 +449,13 @@ struct UnitInfo {
 };
 
 // `w` is the work index of a fixed plan, or the index of the group's unit in the table of a balanced one.
+// `wu` is set for a one-wave plan only.
 // unit_base: all but the mask - which draft tiles are live - so t_begin and ntiles count every draft tile.
-__device__ __forceinline__ UnitInfo unit_base(const TcParams& p, int w) {
+template <int PLAN>
+__device__ __forceinline__ UnitInfo unit_base(const TcParams& p, const Order& order, int w, const WaveUnit& wu) {
     UnitInfo u;
     int item;
-    const bool bal = p.bal_units != nullptr;
+    const bool bal = PLAN == PLAN_TABLE && p.bal_units != nullptr;
     if (bal) {
         // the unit of this CTA's group, for the row-tile item this CTA has in every pair
         const int tpu = p.plan.tiles_per_unit, rt = (int)blockIdx.x % tpu;
@@ -408,7 +464,13 @@ __device__ __forceinline__ UnitInfo unit_base(const TcParams& p, int w) {
         u.slot = rec.w >= 0 ? rt * 2 * ((int)gridDim.x / tpu) + rec.w : -1;
         u.split = 0;
         u.nsplit = rec.w >= 0 ? 2 : 1;     // only "one piece or several" matters below
-    } else if (p.seq.hdr) {
+    } else if (PLAN == PLAN_WAVE) {
+        const int per_seq = p.Hkv * p.plan.tiles_per_unit;
+        u.nsplit = wu.nsplit;
+        u.split = wu.r / per_seq;
+        item = wu.b * per_seq + wu.r - u.split * per_seq;
+        u.slot = w;
+    } else if (PLAN == PLAN_TABLE) {
         // unit w of the per-sequence plan: the last sequence whose first unit is <= w, then
         // (key range, item) inside it
         int lo = 0, hi = p.B - 1;
@@ -428,14 +490,13 @@ __device__ __forceinline__ UnitInfo unit_base(const TcParams& p, int w) {
     }
     const int unit = item / p.plan.tiles_per_unit;
     u.row0 = (item % p.plan.tiles_per_unit) * (2 * p.RT);
-    u.b = unit / p.Hkv;
+    u.b = PLAN == PLAN_ORDERED ? order.seq[unit / p.Hkv] : unit / p.Hkv;
     u.c = unit % p.Hkv;
     u.two = u.row0 + p.RT < p.R;
     if (!GSD_IN_BOUNDS(u.b >= 0 && u.b < p.B && u.c < p.Hkv && u.row0 < p.R, p.status)) {
         u.b = 0; u.c = 0; u.row0 = 0; u.two = false;      // checking build only: a unit outside the problem
     }
-    int L = p.seq_lens[u.b];
-    L = L < 0 ? 0 : (L > p.Lmax ? p.Lmax : L);
+    const int L = PLAN == PLAN_WAVE ? wu.L : PLAN == PLAN_ORDERED ? order.len[u.b] : visible_len(p, u.b);
     u.L = L;
     u.nPT = (L + BN - 1) / BN;
     u.live = 0;
@@ -449,7 +510,7 @@ __device__ __forceinline__ UnitInfo unit_base(const TcParams& p, int w) {
 }
 
 // The draft tiles that hold a visible key for any row of the unit: the OR of the mask rows of its
-// nodes, which are consecutive in memory; eight loads of a lane are on their way at a time.
+// nodes, which are consecutive in memory; four or eight loads of a lane are on their way at a time.
 __device__ __forceinline__ unsigned unit_live(const TcParams& p, const UnitInfo& u, int lane) {
     const int n_lo = u.row0 / p.G;
     const int n_hi = (min(u.row0 + 2 * p.RT, p.R) - 1) / p.G + 1;
@@ -475,12 +536,12 @@ __device__ __forceinline__ unsigned unit_live(const TcParams& p, const UnitInfo&
     } else {
         const int total = (n_hi - n_lo) * p.W;
 #pragma unroll 1
-        for (int base = lane; base < total; base += 8 * 32) {
-            uint32_t q[8];
+        for (int base = lane; base < total; base += 4 * 32) {
+            uint32_t q[4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) q[k] = base + 32 * k < total ? words[base + 32 * k] : 0u;
+            for (int k = 0; k < 4; ++k) q[k] = base + 32 * k < total ? words[base + 32 * k] : 0u;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
+            for (int k = 0; k < 4; ++k) {
                 const int wi = (base + 32 * k) % p.W;
                 if (wi == p.W - 1) q[k] &= tail;
                 if (q[k]) live |= 1u << (wi >> 2);
@@ -491,8 +552,9 @@ __device__ __forceinline__ unsigned unit_live(const TcParams& p, const UnitInfo&
 }
 
 // The whole unit: live draft tiles only are numbered.
-__device__ __forceinline__ UnitInfo unit_info(const TcParams& p, int w, int lane) {
-    UnitInfo u = unit_base(p, w);
+template <int PLAN>
+__device__ __forceinline__ UnitInfo unit_info(const TcParams& p, const Order& order, int w, int lane, const WaveUnit& wu = WaveUnit{}) {
+    UnitInfo u = unit_base<PLAN>(p, order, w, wu);
     u.live = unit_live(p, u, lane);
     auto live_index = [&](int t) { return t <= u.nPT ? t : u.nPT + __popc(u.live & ((1u << (t - u.nPT)) - 1u)); };
     const int t0 = live_index(u.t_begin), t1 = live_index(u.t_begin + u.ntiles);
@@ -501,16 +563,29 @@ __device__ __forceinline__ UnitInfo unit_info(const TcParams& p, int w, int lane
     return u;
 }
 
+// The sequences in descending order of length (called by the whole CTA); false: they are all alike.
+__device__ __forceinline__ bool order_by_length(const TcParams& p, int* s_len, int* s_seq) {
+    const int tid = threadIdx.x, B = p.B;
+    const int mine = tid < B ? visible_len(p, tid) : 0;
+    if (tid < B) s_len[tid] = mine;
+    __syncthreads();
+    int rank = 0;
+    if (tid < B) {
+        for (int j = 0; j < B; ++j) rank += s_len[j] > mine || (s_len[j] == mine && j < tid);
+        s_seq[rank] = tid;
+    }
+    return __syncthreads_or(tid < B && mine != s_len[0]) != 0;
+}
+
 // Persistent kernel: CTA k walks the work indices k, k + gridDim.x, ...  Barrier phases are
 // counted across units, so the producer and the QK^T issuer run ahead into the next unit
 // (Q, the first K/V tiles and the first QK^T) while the softmax warps still read out the
 // accumulators of the previous one.
-template <int HD>
+template <int HD, int PLAN>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_dk,
-               const __grid_constant__ CUtensorMap tm_dv, const __grid_constant__ CUtensorMap tm_out,
-               const TcParams p) {
+               const __grid_constant__ CUtensorMap tm_dv, const TcParams p) {
     using T = Geo<HD>;
     constexpr uint32_t TILE_BYTES = T::TILE_BYTES;
     constexpr int ST = T::ST;
@@ -519,6 +594,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     __shared__ uint32_t s_tmem_base;
     __shared__ __align__(8) WaitCtl s_wait;
     __shared__ float2 s_ml1[BM];      // (max, sum) of the odd-tile stream, one per row
+    __shared__ int s_len[kPlanSeqs], s_seq[kPlanSeqs];     // longest first: lengths, order of the sequences
+    __shared__ int s_wave_units;                           // one-wave plan: units of the call
     __shared__ UnitInfo s_units[kUnitTable];   // the CTA's first units of work, decoded once up front
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -528,16 +605,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const uint32_t sQ = smem_base;                                   // 2 tiles
     const uint32_t sK = smem_base + 2 * TILE_BYTES;                  // ST tiles
     const uint32_t sV = sK + ST * TILE_BYTES;                        // ST tiles
-    const uint32_t sStage = sV + ST * TILE_BYTES;                   // one [128][64] bf16 block per softmax warpgroup
     const uint32_t bar0 = smem_u32(s_bars);
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
     volatile int* abort_flag = &s_wait.abort;
 
     if (warp == 8 && lane == 0) {
-        // the merge pass (a programmatic dependent launch) may be made resident as CTAs retire
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        // the merge pass (a programmatic dependent launch), if there is one, may be made resident as CTAs retire
+        if (p.slots > 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         // the first copy through a tensor map would otherwise fetch it from memory first
-        prefetch_map(&tm_q); prefetch_map(&tm_k); prefetch_map(&tm_v); prefetch_map(&tm_dk); prefetch_map(&tm_dv); prefetch_map(&tm_out);
+        prefetch_map(&tm_q); prefetch_map(&tm_k); prefetch_map(&tm_v); prefetch_map(&tm_dk); prefetch_map(&tm_dv);
         s_wait.abort = 0;
         s_wait.limit_ns = p.wait_limit_ns;
         mbar_init(bar(BAR_Q_FULL), 1);
@@ -577,20 +653,34 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     // This kernel is launched as a programmatic dependent of whatever precedes it on the stream:
     // everything above may run beside the end of that, nothing below may.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    // The CTA's units: work indices blockIdx.x, blockIdx.x + gridDim.x, ... of a fixed plan, or
-    // a run of the table that the planning kernel has written.
+    const Order order{s_len, s_seq};
+    bool forth_and_back = false;
+    if (PLAN == PLAN_ORDERED) {
+        forth_and_back = order_by_length(p, s_len, s_seq);
+        if (blockIdx.x == 0 && p.left && tid < p.B) p.left[tid] = s_seq[tid];
+    }
+    // The CTA's units: work indices blockIdx.x, blockIdx.x + gridDim.x, ... of a fixed plan (every
+    // other round backwards when the lengths differ and the longest come first), or a run of the table that the planning
+    // kernel has written.
     int n_my;
-    if (p.bal_cta) {
+    if (PLAN == PLAN_TABLE && p.bal_cta) {
         n_my = p.bal_cta[blockIdx.x / p.plan.tiles_per_unit].y;
-    } else if (p.seq.hdr) {
+    } else if (PLAN == PLAN_TABLE) {
         const int units = p.seq.hdr[0];
         n_my = units > (int)blockIdx.x ? (units - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    } else if (PLAN == PLAN_WAVE) {
+        n_my = 0;                          // (set below: one unit or none)
+    } else if (forth_and_back) {
+        const int rounds = p.total_work / (int)gridDim.x, rest = p.total_work - rounds * (int)gridDim.x;
+        n_my = rounds + (((rounds & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x) < rest ? 1 : 0);
     } else {
         n_my = p.total_work > (int)blockIdx.x ? (p.total_work - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     }
     // (recomputed where it is needed rather than kept in a register through the key loops)
     auto unit_index = [&](int it) -> int {
-        return p.bal_cta ? p.bal_cta[blockIdx.x / p.plan.tiles_per_unit].x + it : (int)blockIdx.x + it * (int)gridDim.x;
+        if (PLAN == PLAN_TABLE && p.bal_cta) return p.bal_cta[blockIdx.x / p.plan.tiles_per_unit].x + it;
+        const bool back = forth_and_back && (it & 1);
+        return p.work0 + it * (int)gridDim.x + (back ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
     };
     // The copies of one key tile (into ring slot n % ST, the n-th of the CTA).
     auto load_k = [&](const UnitInfo& u, int idx, int n) {
@@ -619,17 +709,31 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     // first prefix tiles - as many as the empty rings hold - as soon as it knows the length.
     int pre = 0;             // producer: key tiles of unit 0 already on their way
     if (warp == 8) {
+        WaveUnit wu{};
+        if (PLAN == PLAN_WAVE) {
+            wu = wave_unit(p, blockIdx.x, lane, false);
+            n_my = (int)blockIdx.x < wu.units ? 1 : 0;
+        }
         if (n_my > 0 && lane == 0) {
-            const UnitInfo u = unit_base(p, unit_index(0));
+            const UnitInfo u = unit_base<PLAN>(p, order, unit_index(0), wu);
             pre = max(0, min(ST, min(u.nPT - u.t_begin, u.ntiles)));
             if (pre > 0) load_q(u);
             for (int n = 0; n < pre; ++n) { load_k(u, n, n); load_v(u, n, n); }
         }
         pre = __shfl_sync(0xFFFFFFFFu, pre, 0);
+    } else if (PLAN == PLAN_WAVE) {
+        if (warp == 0) {
+            const WaveUnit wu = wave_unit(p, blockIdx.x, lane, blockIdx.x == 0);
+            if (lane == 0) s_wave_units = wu.units;
+            if ((int)blockIdx.x < wu.units) {
+                const UnitInfo u = unit_info<PLAN>(p, order, blockIdx.x, lane, wu);
+                if (lane == 0) s_units[0] = u;
+            }
+        }
     } else {
         for (int k = warp < 8 ? warp : warp - 1; k < kUnitTable; k += kThreads / 32 - 1) {
             if (k < n_my) {
-                const UnitInfo u = unit_info(p, unit_index(k), lane);
+                const UnitInfo u = unit_info<PLAN>(p, order, unit_index(k), lane);
                 if (lane == 0) s_units[k] = u;
             }
         }
@@ -638,17 +742,23 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem_base;
+    if (PLAN == PLAN_WAVE) {
+        n_my = (int)blockIdx.x < s_wave_units ? 1 : 0;
+        asm volatile("" : "+r"(n_my));      // (knowing that the unit loops run once at most, the compiler spills in the key loop)
+    }
     auto unit_of = [&](int it) -> UnitInfo {
-        return it < kUnitTable ? s_units[it] : unit_info(p, unit_index(it), lane);
+        return PLAN != PLAN_TABLE || it < kUnitTable ? s_units[it] : unit_info<PLAN>(p, order, unit_index(it), lane);
     };
 
     if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 96;");
     if (warp == 8) {
         // ------------------------------------------------------------ TMA producer
-        // K copies run one tile ahead of the V copies: K t + 1 only waits for the QK^T of tile
-        // t - 1, and its time to land passes while V t waits for the PV of tile t - 2 (4 x 40
-        // heads, N 128, L 1024-4096: 58.4 us in step with the V copies, 55.4 one ahead).
+        // Units with one row tile, where loads are the bound: K copies run one tile ahead of the V
+        // copies.  K t + 1 only waits for the QK^T of tile t - 1, and its time to land passes while V t
+        // waits for the PV of tile t - 2 (4 x 40 heads, N 128, L 1024-4096: 58.4 us in step with the
+        // V copies, 55.4 one ahead).  Units with two keep the copies in step: the tensor pipe is the
+        // bound there and running ahead costs 1% (32 x 64/8 heads, L 8192, N 512).
         int kc = pre, vc = pre;         // K and V tiles loaded so far (ring positions)
         int au = 0;                     // non-empty units so far
         bool ok = true, q_pending = pre > 0;
@@ -667,7 +777,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 }
                 int kn = begun ? pre : 0, vn = kn;      // next tile of the unit
                 while (ok && vn < u.ntiles) {
-                    if (kn < u.ntiles && kn <= vn + 1) {
+                    if (kn < u.ntiles && kn <= vn + (u.two ? 0 : 1)) {
                         if (!(ok = mbar_wait(bar(BAR_K_EMPTY + kc % ST), (uint32_t)((kc / ST) & 1) ^ 1u, abort_flag, p.status))) break;
                         load_k(u, kn, kc);
                         ++kn;
@@ -943,12 +1053,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 tc_fence_before();
                 if (lane == 0) mbar_arrive(bar(BAR_P_READY2 + i));
             }
-            if (!ok) {
-                // gave up inside the key loop: the warpgroup's decision barrier of this unit (below)
-                // still has to see this warp, or the neighbours would wait there for ever
-                if (u.nsplit == 1 && !(alt && i == 1)) wg_all(1 + i, false);
-                break;
-            }
+            if (!ok) break;
             if (alt && i == 1) {
                 // odd-tile stream: publish (max, sum); warpgroup 0 reads the accumulator itself
                 if (my_n > 0) {
@@ -971,13 +1076,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     if (ok) ok = mbar_wait(bar(BAR_ML_READY), (uint32_t)(mlc & 1), abort_flag, p.status);
                 }
                 ok = __all_sync(0xFFFFFFFFu, ok);
-            }
-            if (u.nsplit == 1) {
-                // ... then the four warps decide together whether to go on: the store section below
-                // meets at hardware barriers, which have no time limit, so no warp may enter it while
-                // a neighbour has given up.  Every warp of the warpgroup takes part in this barrier
-                // once per unit, here or where it gave up.
-                ok = wg_all(1 + i, ok);
             }
             if (!ok) break;
             float acc[HD];
@@ -1014,34 +1112,24 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 for (int e = 0; e < HD; ++e) acc[e] = 0.f;
             }
             if (u.nsplit == 1) {
-                // Normalise, round to bf16 and stage the rows in shared memory in the swizzled tile
-                // layout; one thread then writes each 64-column half with a TMA tile store (full
-                // 128-byte lines instead of 32 scattered 16-byte pieces per store instruction;
-                // rows of nodes >= N are clipped by the tensor map).
-                const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-                const uint32_t stage = sStage + (uint32_t)i * HALF_BYTES;
-                unsigned char* srow = smem_raw + (stage - smem_u32(smem_raw)) + rloc * 128;
-                const bool issuer = (warp & 3) == 0 && lane == 0;
+                // Normalise, round to bf16 and store the row; every store of a lane fills a 32-byte
+                // sector.  (Staged in shared memory and stored by TMA it took two barriers and a wait
+                // per 64 columns: 4 x 40 heads 55.0 us instead of 54.4, D 64 37.1 instead of 36.6.)
+                if (rvalid && GSD_IN_BOUNDS(b < p.B && c < p.Hkv && row < R, p.status)) {
+                    const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+                    __nv_bfloat16* dst = p.out + (((size_t)b * N + row / G) * p.Hq + c * G + row % G) * HD;
 #pragma unroll
-                for (int h = 0; h < T::BLOCKS; ++h) {
+                    for (int k = 0; k < HD / 16; ++k) {
+                        uint32_t v[8];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const int e = h * 64 + k * 8;
-                        uint4 v;
-                        v.x = pack_bf16(acc[e + 0] * inv, acc[e + 1] * inv);
-                        v.y = pack_bf16(acc[e + 2] * inv, acc[e + 3] * inv);
-                        v.z = pack_bf16(acc[e + 4] * inv, acc[e + 5] * inv);
-                        v.w = pack_bf16(acc[e + 6] * inv, acc[e + 7] * inv);
-                        *reinterpret_cast<uint4*>(srow + ((k ^ (rloc & 7)) << 4)) = v;
+                        for (int e = 0; e < 8; ++e) v[e] = pack_bf16(acc[k * 16 + 2 * e] * inv, acc[k * 16 + 2 * e + 1] * inv);
+                        if (p.out_by_32) {
+                            st_global8(dst + k * 16, v);
+                        } else {
+                            reinterpret_cast<uint4*>(dst)[2 * k] = make_uint4(v[0], v[1], v[2], v[3]);
+                            reinterpret_cast<uint4*>(dst)[2 * k + 1] = make_uint4(v[4], v[5], v[6], v[7]);
+                        }
                     }
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    wg_barrier(1 + i);
-                    if (issuer) {
-                        tma_store_4d(&tm_out, stage, h * 64, c * G, (u.row0 + (alt ? 0 : i * RT)) / G, b);
-                        bulk_commit();
-                        bulk_wait_read();          // the staging block may be overwritten again
-                    }
-                    wg_barrier(1 + i);
                 }
             } else if (rvalid) {
                 // a partial result: float4 columns of the row tile, so that the 32 rows of a warp
@@ -1060,7 +1148,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (ntiles > 0) ++auc;
             if (n1 > 0) ++auc1;
         }
-        if ((warp & 3) == 0 && lane == 0) bulk_wait_all();   // the output stores have landed
     }
 
     // ---------------------------------------------------------------- teardown
@@ -1115,19 +1202,19 @@ int make_map(CUtensorMap* m, const void* base, uint64_t HD, uint64_t d1, uint64_
 
 }  // namespace
 
-template <int HD>
+template <int HD, int PLAN>
 static int launch_tc(const AttnArgs& a) {
     const int nodes = BM / a.G;           // whole nodes of a row tile
-    CUtensorMap tq, tk, tv, tdk, tdv, tout;
+    CUtensorMap tq, tk, tv, tdk, tdv;
     int rc;
     if ((rc = make_map(&tq, a.q, HD, a.Hq, a.N, a.B, a.G, nodes)) != GSD_OK) return rc;
     if ((rc = make_map(&tk, a.k_cache, HD, a.Hkv, a.Lmax, a.B, 1, BN)) != GSD_OK) return rc;
     if ((rc = make_map(&tv, a.v_cache, HD, a.Hkv, a.Lmax, a.B, 1, BN)) != GSD_OK) return rc;
     if ((rc = make_map(&tdk, a.draft_k, HD, a.Hkv, a.N, a.B, 1, BN)) != GSD_OK) return rc;
     if ((rc = make_map(&tdv, a.draft_v, HD, a.Hkv, a.N, a.B, 1, BN)) != GSD_OK) return rc;
-    if ((rc = make_map(&tout, a.out, HD, a.Hq, a.N, a.B, a.G, nodes)) != GSD_OK) return rc;
     TcParams p;
     p.mask = a.mask; p.seq_lens = a.seq_lens; p.out = (__nv_bfloat16*)a.out; p.status = a.status;
+    p.out_by_32 = ((uintptr_t)a.out & 31u) == 0;
     p.B = a.B; p.N = a.N; p.Hq = a.Hq; p.Hkv = a.Hkv; p.Lmax = a.Lmax; p.G = a.G; p.W = a.W;
     p.R = a.N * a.G; p.RT = nodes * a.G; p.scale_log2 = a.scale_log2; p.plan = a.plan.dev;
     p.part_o = (float*)a.workspace;
@@ -1138,10 +1225,11 @@ static int launch_tc(const AttnArgs& a) {
         int dev = 0;
         GSD_CUDA_TRY(cudaGetDevice(&dev));
         if (dev < 0 || dev >= 64 || !done[dev]) {
-            GSD_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<HD>::SMEM_BYTES));
+            GSD_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<HD, PLAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<HD>::SMEM_BYTES));
             if (dev >= 0 && dev < 64) done[dev] = true;
         }
     }
+    p.work0 = 0;
     p.total_work = a.plan.ctas;
     p.slots = a.plan.slots;
     p.wait_limit_ns = g_wait_limit_ns;
@@ -1150,15 +1238,22 @@ static int launch_tc(const AttnArgs& a) {
     if (device_info(&di) != 0) return GSD_ERR_CUDA;
     p.bal_cta = nullptr;
     p.bal_units = nullptr;
+    p.left = a.plan.slots && (a.plan.dev.balanced == 3 || a.plan.dev.longest_first) ? plan_left_table(a.plan, a.D, a.workspace) : nullptr;
+    p.left_off = (int)(align_up((size_t)a.B * sizeof(int), 256) / sizeof(int));
     p.seq.hdr = nullptr; p.seq.nsplit = nullptr; p.seq.unit_off = nullptr; p.seq.slot_off = nullptr;
     if (a.plan.dev.balanced == 2) {
         p.seq = plan_seq_table(a.plan, a.D, a.B, a.workspace);
-    } else if (a.plan.dev.balanced) {
+    } else if (a.plan.dev.balanced == 1) {
         const BalTable t = plan_bal_table(a.plan, a.D, a.workspace);
         p.bal_cta = t.cta;
         p.bal_units = t.units;
     }
-    // persistent CTAs; the kernel sets itself up beside the end of its predecessor on the stream
+    // Persistent CTAs.  A short call sets itself up beside the end of its predecessor on the stream, which
+    // saves 1 to 2 us; a long one is launched the ordinary way, as CTAs that are placed where and when
+    // SMs fall free ran 1% slower (4155 us instead of 4103 for the 1882 key tiles a CTA of 32 x 64/8
+    // heads, L 8192, N 512, power-limited).  256 tiles are about 400 us.
+    const long long tiles = (long long)a.plan.items * ((a.Lmax + BN - 1) / BN + (a.N + BN - 1) / BN);
+    const bool beside = a.plan.dev.balanced || tiles < 256ll * di.sm_count;
     cudaLaunchAttribute attr[1];
     dependent_launch_attr(attr);
     cudaLaunchConfig_t cfg = {};
@@ -1167,8 +1262,12 @@ static int launch_tc(const AttnArgs& a) {
     cfg.dynamicSmemBytes = Geo<HD>::SMEM_BYTES;
     cfg.stream = a.stream;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD>, tq, tk, tv, tdk, tdv, tout, p));
+    cfg.numAttrs = beside ? 1 : 0;
+    const int part = PLAN == PLAN_FIXED || PLAN == PLAN_ORDERED ? (int)cfg.gridDim.x * kUnitTable : a.plan.ctas;
+    for (p.work0 = 0; p.work0 < a.plan.ctas; p.work0 += part) {
+        p.total_work = a.plan.ctas - p.work0 < part ? a.plan.ctas - p.work0 : part;
+        GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD, PLAN>, tq, tk, tv, tdk, tdv, p));
+    }
     return GSD_OK;
 }
 
@@ -1181,7 +1280,12 @@ int launch_attn_tcgen05(const AttnArgs& a) {
         set_error_text("tcgen05 back end needs a head dimension of 64 or 128 and a group size of at most 128");
         return GSD_ERR_UNSUPPORTED;
     }
-    return a.D == 128 ? launch_tc<128>(a) : launch_tc<64>(a);
+    switch (a.plan.dev.balanced == 3 ? PLAN_WAVE : a.plan.dev.balanced ? PLAN_TABLE : a.plan.dev.longest_first ? PLAN_ORDERED : PLAN_FIXED) {
+        case PLAN_WAVE: return a.D == 128 ? launch_tc<128, PLAN_WAVE>(a) : launch_tc<64, PLAN_WAVE>(a);
+        case PLAN_ORDERED: return a.D == 128 ? launch_tc<128, PLAN_ORDERED>(a) : launch_tc<64, PLAN_ORDERED>(a);
+        case PLAN_TABLE: return launch_tc<128, PLAN_TABLE>(a);     // (D = 128 only)
+        default: return a.D == 128 ? launch_tc<128, PLAN_FIXED>(a) : launch_tc<64, PLAN_FIXED>(a);
+    }
 }
 
 void debug_attn_wait(unsigned long long limit_ns, int withhold_first_k) {

@@ -1,0 +1,73 @@
+"""The two plans the attention kernel makes from the sequence lengths - one wave of units when the
+items do not fill the device, longest sequences first when they do - against the fp64 oracle and
+the plan without the lengths.  Tolerance as in tests/test_gpu_attn.py; against the other plan one
+bf16 step of the largest output (both round fp32 results that differ by reassociation)."""
+import numpy as np
+import pytest
+import torch
+
+import gsd_inputs as gi
+import oracle
+from gpu_util import attn_tensors, out_to_f64
+from test_gpu_attn import assert_close_scaled, cpu_attn, sampled_rows_check
+
+pytestmark = pytest.mark.gpu
+
+NAMES = ("q", "k_cache", "v_cache", "draft_k", "draft_v", "ancestor_mask", "seq_lens")
+
+
+def inputs(B, Hq, Hkv, D, N, lens, seed=1):
+    cfg = gi.VerifyConfig("l", 7, B, Hq, Hkv, D, int(max(lens)) or 1, N, min(N - 1, 9), 4, 3, 8, 8, 0.5)
+    inp = gi.make_inputs(cfg, seed, accept=False)
+    inp["seq_lens"][:] = lens
+    for b, n in enumerate(lens):
+        inp["k_cache"][b, int(n):] = 0x7FC0
+        inp["v_cache"][b, int(n):] = 0x7FC0
+    return inp
+
+
+def call(inp, **kw):
+    import paper_2407_16207_b200 as gsd
+    t = attn_tensors(inp)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = gsd.gsd_verify_attn(*(t[n] for n in NAMES), status=status, **kw)
+    assert int(status.item()) == 0
+    return out
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,N", [(8, 2, 128, 40), (4, 4, 128, 100), (32, 2, 128, 40), (8, 2, 64, 70), (6, 2, 128, 90)])
+@pytest.mark.parametrize("lens", [(0, 3000), (0, 0, 0), (1, 1, 1, 1), (2600, 0, 130, 127, 1281), (900, 901, 899, 900, 1025, 1024, 1023), tuple(range(40, 1640, 50))])
+def test_one_wave(Hq, Hkv, D, N, lens):
+    inp = inputs(len(lens), Hq, Hkv, D, N, lens)
+    got = call(inp)
+    assert torch.equal(got, call(inp))
+    assert_close_scaled(out_to_f64(got), cpu_attn(inp))
+
+
+def test_scratch_sized_without_the_lengths_is_enough():
+    # the size that three forced key ranges need lies between that of the two automatic plans
+    import paper_2407_16207_b200 as gsd
+    inp = inputs(3, 8, 2, 128, 40, (2000, 300, 1100))
+    size = (3, 40, 8, 2, 128, inp["Lmax"])
+    need, nominal = gsd.gsd_verify_attn_workspace_bytes(*size), gsd.gsd_verify_attn_num_splits(*size)
+    without = gsd.gsd_verify_attn_workspace_bytes(*size, num_splits=nominal)
+    assert 0 < without < need
+    want = cpu_attn(inp)
+    for n in (need, without):
+        assert_close_scaled(out_to_f64(call(inp, workspace=torch.empty(n, dtype=torch.uint8, device="cuda"))), want)
+    with pytest.raises(gsd.GsdError) as e:
+        call(inp, workspace=torch.empty(without - 256, dtype=torch.uint8, device="cuda"))
+    assert e.value.code == -4
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,N,Lmax", [(24, 64, 8, 57, 1500), (5, 40, 40, 128, 1700), (75, 16, 2, 33, 700), (384, 4, 1, 20, 300), (400, 4, 1, 20, 300)])
+def test_longest_first(B, Hq, Hkv, N, Lmax):
+    rng = np.random.default_rng(B)
+    lens = rng.integers(0, Lmax + 1, B)
+    lens[rng.integers(0, B, max(2, B // 4))] = Lmax          # ties
+    lens[0], lens[B - 1] = 0, Lmax
+    inp = inputs(B, Hq, Hkv, 128, N, lens)
+    got = call(inp)
+    assert torch.equal(got, call(inp))
+    assert (got.float() - call(inp, num_splits=1).float()).abs().max().item() <= 2.0 ** -8 * max(1.0, got.float().abs().max().item())
+    sampled_rows_check(inp, got, rng, n_random=600, units=[(1, 0), (B // 2, Hkv - 1)])
