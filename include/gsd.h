@@ -87,7 +87,8 @@ typedef struct gsd_attn_params {
     int32_t D;            /* head dimension: 64 or 128 */
     int32_t Lmax;         /* padded cache length (rows per sequence in k_cache/v_cache), >= 1 */
     float softmax_scale;  /* <= 0 selects 1/sqrt(D) */
-    int32_t num_splits;   /* key-range splits per (sequence, kv head, row tile); 0 = choose;
+    int32_t num_splits;   /* key-range splits per (sequence, kv head, row tile); 0 = choose (on the
+                             device from seq_lens where the tcgen05 kernel's items are few or the batch large);
                              GSD_ATTN_SPLIT_BALANCED = equal shares of key tiles per CTA, dealt out on the
                              device from seq_lens; GSD_ATTN_SPLIT_PER_SEQUENCE = a split count per sequence,
                              chosen on the device from seq_lens so that all units are about equally long
@@ -164,7 +165,7 @@ void gsd_debug_attn_wait(uint64_t limit_ns, int32_t withhold_first_k);
 size_t gsd_verify_attn_workspace_bytes(const gsd_attn_params* p);
 
 /* The number of key-range splits gsd_verify_attn would use for *p on the current device
- * (p->num_splits if positive, else the automatic choice); GSD_ATTN_SPLIT_BALANCED or
+ * (p->num_splits if positive, else the automatic choice for sequences that fill the cache); GSD_ATTN_SPLIT_BALANCED or
  * GSD_ATTN_SPLIT_PER_SEQUENCE when the work is shared out on the device; 0 on invalid parameters. */
 int gsd_verify_attn_num_splits(const gsd_attn_params* p);
 
