@@ -52,7 +52,13 @@ int attn_pick_kernel(const gsd_attn_params* p) {
     // D 128, N 77, L 300-1999: 45.4 us there, 28.5 us here; 4 x 8 groups of 4, D 64, N 128,
     // L 1000-4000: 81 us there, 42 us here (device time of the whole call).
     const int G = p->Hq / p->Hkv;
-    if (attn_tcgen05_supports(p->D, G) && p->N * G >= 64) return GSD_ATTN_TCGEN05;
+    // Fewer rows leave most of a tile empty, and then the loads decide: at D = 128 and 512 or more cache
+    // rows the TMA rings are ahead of the mma.sync kernel's cp.async pipeline (mma.sync -> tcgen05, us:
+    // 1 x 32 heads, N 8, L 1000 13.6 -> 12.4, L 4000 32.8 -> 17.7; 32 x 32, N 8, L 2000 288 -> 176;
+    // 8 x 28/4, N 8, L 1000 15.0 -> 14.8; 8 x 32, N 1, L 2000 77.5 -> 50.6).  Short contexts and D = 64
+    // stay: the start of a unit costs more there (8 x 32, N 8, L 200 15.6 -> 17.8; 32 x 32/8, N 4, L 64
+    // 9.4 -> 15.3; D 64, 32 x 12, N 20, L 700 30.0 -> 32.9).
+    if (attn_tcgen05_supports(p->D, G) && (p->N * G >= 64 || (p->D == 128 && p->Lmax >= 512))) return GSD_ATTN_TCGEN05;
     return GSD_ATTN_MMA;
 }
 

@@ -71,3 +71,13 @@ def test_longest_first(B, Hq, Hkv, N, Lmax):
     assert torch.equal(got, call(inp))
     assert (got.float() - call(inp, num_splits=1).float()).abs().max().item() <= 2.0 ** -8 * max(1.0, got.float().abs().max().item())
     sampled_rows_check(inp, got, rng, n_random=600, units=[(1, 0), (B // 2, Hkv - 1)])
+
+
+@pytest.mark.parametrize("Hq,Hkv,N", [(4, 4, 1), (8, 2, 3), (3, 3, 31), (6, 2, 21)])
+@pytest.mark.parametrize("lens", [(511,), (512,), (0, 1, 600), (1300, 128, 129, 700)])
+def test_few_rows(Hq, Hkv, N, lens):
+    # fewer than 64 stacked rows, on either side of the cache length from which the automatic choice changes
+    inp = inputs(len(lens), Hq, Hkv, 128, N, lens)
+    want = cpu_attn(inp)
+    for splits in (0, 2):
+        assert_close_scaled(out_to_f64(call(inp, num_splits=splits)), want)
