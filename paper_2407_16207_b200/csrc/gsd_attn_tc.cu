@@ -593,7 +593,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     __shared__ __align__(8) unsigned long long s_bars[BAR_COUNT];
     __shared__ uint32_t s_tmem_base;
     __shared__ __align__(8) WaitCtl s_wait;
-    __shared__ float2 s_ml1[BM];      // (max, sum) of the odd-tile stream, one per row
+    __shared__ float2 s_ml1[BM];      // (max, sum) of the odd-tile stream, one per row; who may write when: see there
     __shared__ int s_len[kPlanSeqs], s_seq[kPlanSeqs];     // longest first: lengths, order of the sequences
     __shared__ int s_wave_units;                           // one-wave plan: units of the call
     __shared__ UnitInfo s_units[kUnitTable];   // the CTA's first units of work, decoded once up front
@@ -1057,6 +1057,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (alt && i == 1) {
                 // odd-tile stream: publish (max, sum); warpgroup 0 reads the accumulator itself
                 if (my_n > 0) {
+                    // The pair of the stream's previous unit has to have been read (warpgroup 0 says so
+                    // with O_FREE) before this one takes its place.  With one S for both streams that is
+                    // so already: this unit's scores of stream 1 were only formed after warpgroup 0 had
+                    // given S back in this unit.  With an S per stream nothing else holds this warpgroup
+                    // back when a unit has a single odd tile.  Both sides count the units in which stream
+                    // 1 had tiles, and O_FREE cannot go on by a further phase before the pair is published.
+                    if (T::TWO_S && auc > 0) {
+                        ok = mbar_wait(bar(BAR_O_FREE + 1), (uint32_t)(auc - 1) & 1u, abort_flag, p.status);
+                        ok = __all_sync(0xFFFFFFFFu, ok);
+                        if (!ok) break;
+                    }
                     s_ml1[rloc] = make_float2(m_ref, l_run);
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(BAR_ML_READY));
@@ -1102,6 +1113,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     l_run = w0 * l_run + w1 * ml1.y;
                     m_ref = m;
                     tc_fence_before();
+                    __syncwarp();                       // (every lane has read its pair)
                     if (lane == 0) mbar_arrive(bar(BAR_O_FREE + 1));
                     ++mlc;
                 }

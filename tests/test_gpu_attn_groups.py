@@ -4,9 +4,10 @@ the automatic choice takes it, against the fp64 oracle.  Same tolerance as tests
 each) and of key tiles, with NaN behind every sequence end."""
 import numpy as np
 import pytest
+import torch
 
 import gsd_inputs as gi
-from gpu_util import out_to_f64
+from gpu_util import attn_tensors, out_to_f64
 from test_gpu_attn import assert_close_scaled, cpu_attn, gpu_attn
 
 pytestmark = pytest.mark.gpu
@@ -40,7 +41,7 @@ def test_row_tile_edges(D, G, N):
 @pytest.mark.parametrize("D,G,Hkv,L,N", [(64, 4, 8, (1000, 4000), 128), (64, 1, 12, 1537, 77), (128, 3, 8, (300, 1999), 77),
                                          (128, 7, 4, 4097, 200)])
 def test_many_tiles_per_unit(D, G, Hkv, L, N):
-    # rings and barrier phases wrap many times, several units per CTA, split items and their merge
+    # rings and barrier phases wrap many times inside a unit; cut items and their merge
     cfg = gi.VerifyConfig("t", 7, 4, G * Hkv, Hkv, D, L, N, 10, 4, 3, 8, 8, 0.5)
     inp = gi.make_inputs(cfg, 11, accept=False, pad_fill="nan")
     assert_close_scaled(out_to_f64(gpu_attn(inp)), cpu_attn(inp))
@@ -59,3 +60,39 @@ def test_score_jumps_at_head_dimension_64():
     dk = gi.bf16_bits_to_f32(inp["draft_k"]); dk[0, :, 0, 5] = 0.0
     inp["draft_k"] = gi.f32_to_bf16_bits(dk)
     assert_close_scaled(out_to_f64(gpu_attn(inp)), cpu_attn(inp))
+
+
+def many_units(B, G, Hkv, D, N, lens, seed):
+    depth = int(np.ceil(np.log(2 * N + 1) / np.log(3))) + 1
+    cfg = gi.VerifyConfig("t", 7, B, G * Hkv, Hkv, D, int(max(lens)), N, depth, 3, 2, 8, 8, 0.5)
+    inp = gi.make_inputs(cfg, seed, accept=False)
+    inp["seq_lens"][:] = lens
+    for b, n in enumerate(lens):
+        inp["k_cache"][b, int(n):] = 0x7FC0
+        inp["v_cache"][b, int(n):] = 0x7FC0
+    items = B * Hkv * -(-N * G // (2 * (128 // G * G)))
+    assert items > torch.cuda.get_device_properties(0).multi_processor_count
+    return inp, items
+
+
+# Several units per CTA: the hand-overs from one unit to the next (accumulators, rings, the pair that
+# the odd key tiles of a single row tile leave for the even ones).  One row tile with two and three key
+# tiles, which is one odd tile, and with empty prefixes between them; two row tiles; a pair and a
+# single one side by side; groups whose row tiles are not full.
+@pytest.mark.parametrize("B,G,Hkv,D,N,lens", [(32, 1, 12, 64, 77, (0, 256)), (32, 1, 12, 64, 100, (200, 200)), (30, 1, 12, 64, 128, (129, 256)),
+                                              (40, 4, 8, 64, 17, (100, 700)), (20, 4, 8, 64, 70, (0, 300)), (16, 8, 16, 64, 31, (1, 520)),
+                                              (13, 3, 12, 64, 50, (0, 900)), (24, 3, 8, 128, 60, (0, 300)), (26, 3, 8, 128, 30, (100, 600)),
+                                              (12, 7, 16, 128, 21, (1, 1100)), (36, 12, 6, 128, 23, (0, 400))])
+def test_many_units_per_cta(B, G, Hkv, D, N, lens):
+    import paper_2407_16207_b200 as gsd
+    rng = np.random.default_rng(B + N)
+    inp, _ = many_units(B, G, Hkv, D, N, rng.integers(lens[0], lens[1] + 1, B), 5)
+    t = attn_tensors(inp)
+    args = [t[n] for n in ("q", "k_cache", "v_cache", "draft_k", "draft_v", "ancestor_mask", "seq_lens")]
+    want = cpu_attn(inp)
+    for splits in (0, 1, 2):
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        got = [gsd.gsd_verify_attn(*args, num_splits=splits, status=status) for _ in range(4)]
+        assert int(status.item()) == 0
+        assert all(torch.equal(got[0], g) for g in got[1:])
+        assert_close_scaled(out_to_f64(got[0]), want)
