@@ -328,3 +328,22 @@ def test_row_pointers_that_go_backwards_are_flagged_and_made_safe():
     assert int(status.item()) & 0x1
     for g, w_ in zip(got, want):
         assert np.array_equal(g, w_)
+
+
+@pytest.mark.parametrize("B,N,V", [(2, 9, 1003), (1, 40, 65536), (2, 100, 8192), (1, 300, 4099)])
+def test_scratch_on_any_8_byte_boundary(B, N, V):
+    # four, two and one thread per node read the pairs; rows in one slice and in many
+    import paper_2407_16207_b200 as gsd
+    cfg = gi.VerifyConfig("a", 7, B, 1, 1, 64, 8, N, 7, 3, 2, V, 64, 0.7)
+    inp = gi.make_inputs(cfg, 80 + N, attn=False)
+    dl = draft_logits_for(inp["logits"], 5)
+    q, u, us, want = decisive_inputs(inp, 9 + V, q_lo=2.0, q_hi=20.0, dl=dl)
+    t = accept_tensors(inp)
+    need = gsd.gsd_accept_sampled_workspace_bytes(B, N)
+    for by in (0, 8):
+        ws = torch.empty(need + 8, dtype=torch.uint8, device="cuda")[by:by + need]
+        assert ws.data_ptr() % 16 == by
+        got = gsd.gsd_accept_sampled(t["logits"], t["draft_tokens"], t["parent_ptr"], t["parent_idx"],
+                                     *(torch.from_numpy(a).cuda() for a in (q, u, us)), draft_logits=torch.from_numpy(dl).cuda(), workspace=ws)
+        for g, w in zip(got, want[:3]):
+            assert np.array_equal(g.cpu().numpy(), w)
