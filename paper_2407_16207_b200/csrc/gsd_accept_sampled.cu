@@ -32,7 +32,8 @@ constexpr int kWarps = kThreads / 32;   // each warp of a CTA sums a contiguous 
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kResidualFloor = 1e-6f;   // a residual mass at or below this is rounding noise
 
-// (maximum, sum of 2^((x - maximum) * log2 e)) of a set of logits; the empty set is (-inf, 0)
+// (maximum, sum of 2^((x - maximum) * log2 e)) of a set of logits; the empty set is (-inf, 0).  A NaN
+// among them is a NaN sum from then on, also while the maximum is still -inf.
 struct Ms {
     float m, s;
 };
@@ -45,7 +46,7 @@ __device__ __forceinline__ float ex2(float x) {
 
 __device__ __forceinline__ Ms combine(Ms a, Ms b) {
     const float m = fmaxf(a.m, b.m);
-    if (m == -CUDART_INF_F) return Ms{m, 0.f};
+    if (m == -CUDART_INF_F) return Ms{m, a.s + b.s};
     return Ms{m, a.s * ex2((a.m - m) * kLog2e) + b.s * ex2((b.m - m) * kLog2e)};
 }
 
@@ -54,7 +55,12 @@ __device__ __forceinline__ void take16(Ms& r, const float4& a, const float4& b, 
     const float m4 = fmaxf(fmaxf(fmaxf(a.x, a.y), fmaxf(a.z, a.w)), fmaxf(fmaxf(b.x, b.y), fmaxf(b.z, b.w)));
     const float m8 = fmaxf(fmaxf(fmaxf(c.x, c.y), fmaxf(c.z, c.w)), fmaxf(fmaxf(d.x, d.y), fmaxf(d.z, d.w)));
     const float m = fmaxf(r.m, fmaxf(m4, m8));
-    if (m == -CUDART_INF_F) return;
+    if (m == -CUDART_INF_F) {
+        // nothing above -inf yet: the values add up to -inf, or to NaN if there is one
+        const float t = (((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w))) + (((c.x + c.y) + (c.z + c.w)) + ((d.x + d.y) + (d.z + d.w)));
+        if (t != t) r.s = t;
+        return;
+    }
     // (the rounding of m * log2 e is a factor on every term; the sum is brought back by it)
     const float k = -m * kLog2e, off = fmaf(-m, kLog2e, -k);
     float s = ex2(fmaf(a.x, kLog2e, k)) + ex2(fmaf(a.y, kLog2e, k)) + ex2(fmaf(a.z, kLog2e, k)) + ex2(fmaf(a.w, kLog2e, k));
@@ -66,7 +72,8 @@ __device__ __forceinline__ void take16(Ms& r, const float4& a, const float4& b, 
 }
 
 __device__ __forceinline__ void take1(Ms& r, float x) {
-    r = combine(r, Ms{x, x == -CUDART_INF_F ? 0.f : 1.f});
+    const bool nan = x != x;
+    r = combine(r, Ms{nan ? -CUDART_INF_F : x, nan ? x : x == -CUDART_INF_F ? 0.f : 1.f});
 }
 
 // The row is cut into slices (one CTA each) and every slice into kWarps contiguous ranges (one
@@ -186,7 +193,11 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
                 float m = r.m;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) m = fmaxf(m, fmaxf(p[i].x, p[i].z));
-                if (m == -CUDART_INF_F) continue;
+                if (m == -CUDART_INF_F) {                              // (sums of 0 or NaN)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) r.s += p[i].y + p[i].w;
+                    continue;
+                }
                 float s = r.s * ex2((r.m - m) * kLog2e);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) s += p[i].y * ex2((p[i].x - m) * kLog2e) + p[i].w * ex2((p[i].z - m) * kLog2e);

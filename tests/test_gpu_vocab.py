@@ -99,3 +99,35 @@ def test_draft_rows_in_slices(B, F, V, k, by):
         gsd.gsd_draft_expand(shifted(torch.from_numpy(x), by), torch.from_numpy(fr[b:b + 1]).cuda(), torch.from_numpy(fl[b:b + 1]).cuda(), *t,
                              k=k, tau=2, theta_prob=tp, theta_sib=ts, status=status)
         assert int(status.item()) & 0x40
+
+
+@pytest.mark.parametrize("by", [0, 1, 2, 3])
+@pytest.mark.parametrize("V", [1, 3, 6, 1003, 16389])
+def test_nan_anywhere_in_a_row_is_flagged(V, by):
+    # target rows and the end node's draft row; the first and last entries of a row are not part of
+    # its 16-byte groups, and an entry may be the first its thread meets or follow entries of -inf
+    import paper_2407_16207_b200 as gsd
+    rng = np.random.default_rng(V)
+    B, N = 1, 4
+    lg, dl = (rng.normal(size=(B, N, V)).astype(np.float32) for _ in range(2))
+    g = [torch.tensor(x, dtype=torch.int32, device="cuda") for x in ([[0, 0, 0, 0]], [[0, 0, 1, 2, 3]], [[0, 1, 2]])]
+    q, u, us = torch.ones(B, N, device="cuda"), torch.ones(B, N, device="cuda"), torch.full((B,), 0.5, device="cuda")   # nothing is accepted
+
+    def flags(lg, dl):
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        gsd.gsd_accept_sampled(shifted(torch.from_numpy(lg), by), *g, q, u, us, draft_logits=shifted(torch.from_numpy(dl), by), status=status)
+        return int(status.item())
+    assert flags(lg, dl) == 0
+    at = sorted({0, 1, 2, 3, 4, V // 2, V - 4, V - 3, V - 2, V - 1} & set(range(V)))
+    for e in at:
+        for rest in (1.0, -np.inf):
+            bad = lg.copy()
+            bad[0, 2] += 0.0 if rest == 1.0 else rest
+            bad[0, 2, (e + 1) % V] = 1.0
+            bad[0, 2, e] = np.nan
+            assert flags(bad, dl) == 0x40, (e, rest)
+            bad = dl.copy()
+            bad[0, 0] += 0.0 if rest == 1.0 else rest
+            bad[0, 0, (e + 1) % V] = 1.0
+            bad[0, 0, e] = np.nan
+            assert flags(lg, bad) == 0x40, (e, rest)
