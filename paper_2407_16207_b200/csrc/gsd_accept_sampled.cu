@@ -51,7 +51,7 @@ __device__ __forceinline__ Ms combine(Ms a, Ms b) {
 }
 
 // sixteen values at once: one rescale of the running sum per group
-__device__ __forceinline__ void take16(Ms& r, const float4& a, const float4& b, const float4& c, const float4& d) {
+__device__ __forceinline__ void take16(Ms& r, float4 a, float4 b, float4 c, float4 d) {
     const float m4 = fmaxf(fmaxf(fmaxf(a.x, a.y), fmaxf(a.z, a.w)), fmaxf(fmaxf(b.x, b.y), fmaxf(b.z, b.w)));
     const float m8 = fmaxf(fmaxf(fmaxf(c.x, c.y), fmaxf(c.z, c.w)), fmaxf(fmaxf(d.x, d.y), fmaxf(d.z, d.w)));
     const float m = fmaxf(r.m, fmaxf(m4, m8));
@@ -61,8 +61,14 @@ __device__ __forceinline__ void take16(Ms& r, const float4& a, const float4& b, 
         if (t != t) r.s = t;
         return;
     }
-    // (the rounding of m * log2 e is a factor on every term; the sum is brought back by it)
-    const float k = -m * kLog2e, off = fmaf(-m, kLog2e, -k);
+    float ref = m;
+    if (fabsf(m) > kLargeLogit) {
+        // (entries masked with a large negative number, sixteen of them together)
+        a = minus(a, m); b = minus(b, m); c = minus(c, m); d = minus(d, m);
+        ref = 0.f;
+    }
+    // (the rounding of ref * log2 e is a factor on every term; the sum is brought back by it)
+    const float k = -ref * kLog2e, off = fmaf(-ref, kLog2e, -k);
     float s = ex2(fmaf(a.x, kLog2e, k)) + ex2(fmaf(a.y, kLog2e, k)) + ex2(fmaf(a.z, kLog2e, k)) + ex2(fmaf(a.w, kLog2e, k));
     s += ex2(fmaf(b.x, kLog2e, k)) + ex2(fmaf(b.y, kLog2e, k)) + ex2(fmaf(b.z, kLog2e, k)) + ex2(fmaf(b.w, kLog2e, k));
     s += ex2(fmaf(c.x, kLog2e, k)) + ex2(fmaf(c.y, kLog2e, k)) + ex2(fmaf(c.z, kLog2e, k)) + ex2(fmaf(c.w, kLog2e, k));

@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(kThreads, 4) draft_expand_kernel(DraftArgs a) 
 #pragma unroll
             for (int k = 0; k < kBatch; ++k) r[k] = i + k * kThreads < v1 ? __ldcs(x4 + i + k * kThreads) : none;
         };
-        auto work = [&](const float4 (&r)[kBatch], int i) {
+        auto work = [&](float4 (&r)[kBatch], int i) {
             float g = m;
 #pragma unroll
             for (int k = 0; k < kBatch; ++k) {
@@ -446,10 +446,16 @@ __global__ void __launch_bounds__(kThreads, 4) draft_expand_kernel(DraftArgs a) 
                 }
                 return;
             }
-            // One rescale per batch.  The rounding of g * log2 e (2^-21 at a logit of 12) would be a
+            float ref = g;
+            if (fabsf(g) > kLargeLogit) {
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k) r[k] = minus(r[k], g);
+                ref = 0.f;
+            }
+            // One rescale per batch.  The rounding of ref * log2 e (2^-21 at a logit of 12) would be a
             // factor on every term, while the probabilities at the end use v - maximum: the
             // batch's sum is brought back by what was rounded off.
-            const float kk = -g * kLog2e, off = fmaf(-g, kLog2e, -kk);
+            const float kk = -ref * kLog2e, off = fmaf(-ref, kLog2e, -kk);
             float acc = 0.f;
 #pragma unroll
             for (int k = 0; k < kBatch; ++k)

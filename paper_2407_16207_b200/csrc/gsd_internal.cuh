@@ -215,6 +215,14 @@ __device__ __forceinline__ RowSpan row_span(const float* x, int V) {
     return r;
 }
 
+// Sums of exponentials form (x - maximum) * log2 e as x * log2 e - maximum * log2 e in one fused
+// multiply-add.  The rounding of the second product is 2^-24 of it: harmless for logits, but at a
+// maximum of -1e10 or -3.4e38 (sixteen entries masked with such a number, next to one another in a
+// thread's share) the factor it makes overflows.  Beyond this magnitude the difference is formed
+// first.  (2^20: there the factor is still within 2^+-0.1.)
+constexpr float kLargeLogit = 1048576.f;
+__device__ __forceinline__ float4 minus(const float4& x, float m) { return make_float4(x.x - m, x.y - m, x.z - m, x.w - m); }
+
 // ---- scratch words that must start at zero ----
 // Enqueues a small kernel that zeroes `n` 32-bit words and lets the next launch on the stream
 // start beside it.  That next kernel has to be launched with the attribute set up by

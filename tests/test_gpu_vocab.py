@@ -131,3 +131,42 @@ def test_nan_anywhere_in_a_row_is_flagged(V, by):
             bad[0, 0, (e + 1) % V] = 1.0
             bad[0, 0, e] = np.nan
             assert flags(lg, bad) == 0x40, (e, rest)
+
+
+MASKS = [-1e9, -1e10, -3e30, float(np.finfo(np.float32).min)]
+
+
+@pytest.mark.parametrize("mask", MASKS)
+@pytest.mark.parametrize("V", [1003, 4099, 32000])
+def test_entries_masked_with_a_large_negative_number(V, mask):
+    # a filtered distribution whose entries are finite: whole runs of a row, of a thread's share
+    # and of its first loads hold nothing else
+    import paper_2407_16207_b200 as gsd
+    rng = np.random.default_rng(V)
+    inp = graph_inputs(2, 9, V, 70)
+    keep = np.zeros(inp["logits"].shape, bool)
+    keep[:, :, rng.integers(0, V, 40)] = True
+    keep[:, :, inp["draft_tokens"].ravel()] = True
+    inp["logits"] = np.where(keep, inp["logits"], np.float32(mask))
+    dl = np.where(keep, sampled_cases.draft_logits_for(inp["logits"], 5), np.float32(mask))
+    t = accept_tensors(inp)
+    for residual in (False, True):
+        q, u, us, want = sampled_cases.decisive_inputs(inp, 9 + V, q_lo=2.0, q_hi=20.0, dl=dl if residual else None)
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        got = gsd.gsd_accept_sampled(t["logits"], t["draft_tokens"], t["parent_ptr"], t["parent_idx"],
+                                     *(torch.from_numpy(a).cuda() for a in (q, u, us)), status=status,
+                                     draft_logits=torch.from_numpy(dl).cuda() if residual else None)
+        assert int(status.item()) == 0
+        for g, w in zip(got, want[:3]):
+            assert np.array_equal(g.cpu().numpy(), w)
+    B, F, k = 2, 9, 4
+    fr, fl = np.zeros((B, F), np.int32), np.full((B,), F, np.int32)
+    state = draft_cases.fresh(B, 64)
+    tp, ts = draft_cases.decisive_thresholds(inp["logits"], fl, k, rng, (0.001, 0.9), (0.001, 0.9))
+    out = oracle.draft_expand(inp["logits"], fr, fl, *state, k=k, tau=2, theta_prob=tp, theta_sib=ts)
+    g = [torch.from_numpy(a.copy()).cuda() for a in state]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    nf, nfl = gsd.gsd_draft_expand(t["logits"], torch.from_numpy(fr).cuda(), torch.from_numpy(fl).cuda(), *g, k=k, tau=2,
+                                   theta_prob=tp, theta_sib=ts, status=status)
+    assert int(status.item()) == 0
+    draft_cases.compare([a.cpu().numpy() for a in g], list(out[:6]), nf.cpu().numpy(), nfl.cpu().numpy(), out[6], out[7])
