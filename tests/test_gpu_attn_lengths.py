@@ -44,6 +44,19 @@ def test_one_wave(Hq, Hkv, D, N, lens):
     assert_close_scaled(out_to_f64(got), cpu_attn(inp))
 
 
+@pytest.mark.parametrize("Hq,Hkv,D,N", [(32, 8, 128, 40), (32, 8, 64, 100), (24, 8, 128, 50)])
+@pytest.mark.parametrize("long,short,n_long,B", [(1700, 100, 1, 10), (1700, 100, 2, 12), (1100, 1100, 0, 11), (1500, 0, 1, 17), (1700, 100, 1, 18)])
+def test_one_wave_that_can_cut_few(Hq, Hkv, D, N, long, short, n_long, B):
+    # more items than half the device: only some sequences can be cut (with 18 none), the others are
+    # stored by the attention kernel itself; the long one first, last and in between
+    for at in {0, B // 2, B - n_long}:
+        lens = [long if at <= b < at + n_long else short for b in range(B)]
+        inp = inputs(B, Hq, Hkv, D, N, lens)
+        got = call(inp)
+        assert torch.equal(got, call(inp))
+        assert_close_scaled(out_to_f64(got), cpu_attn(inp))
+
+
 def test_scratch_sized_without_the_lengths_is_enough():
     # the size that three forced key ranges need lies between that of the two automatic plans
     import paper_2407_16207_b200 as gsd
