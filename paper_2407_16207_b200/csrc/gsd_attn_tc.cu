@@ -67,7 +67,8 @@ struct Geo {
     static constexpr int BLOCKS = HD / 64;
     static constexpr uint32_t TILE_BYTES = BLOCKS * HALF_BYTES;   // a 128 x HD bf16 tile
     static constexpr int ST = HD == 128 ? 2 : 4;                  // stages of the K ring and of the V ring
-    static constexpr uint32_t SMEM_BYTES = (2 + 2 * ST) * TILE_BYTES + 1024;  // tiles, alignment slack
+    static constexpr uint32_t STAGE_BYTES = 32 * 64;              // output rows of a softmax warp, 32 columns at a time
+    static constexpr uint32_t SMEM_BYTES = (2 + 2 * ST) * TILE_BYTES + 8 * STAGE_BYTES + 1024;  // tiles, staging, alignment slack
     static constexpr bool TWO_S = HD == 64;
     static constexpr uint32_t COL_S0 = 0, COL_P0 = 128, COL_P1 = 192, COL_O0 = 256, COL_O1 = 256 + HD;
     static constexpr uint32_t COL_S1 = TWO_S ? 384 : COL_S0;
@@ -605,6 +606,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const uint32_t sQ = smem_base;                                   // 2 tiles
     const uint32_t sK = smem_base + 2 * TILE_BYTES;                  // ST tiles
     const uint32_t sV = sK + ST * TILE_BYTES;                        // ST tiles
+    const uint32_t sStage = sV + ST * TILE_BYTES;                    // a block per softmax warp
     const uint32_t bar0 = smem_u32(s_bars);
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
     volatile int* abort_flag = &s_wait.abort;
@@ -1123,10 +1125,46 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll
                 for (int e = 0; e < HD; ++e) acc[e] = 0.f;
             }
-            if (u.nsplit == 1) {
-                // Normalise, round to bf16 and store the row; every store of a lane fills a 32-byte
-                // sector.  (Staged in shared memory and stored by TMA it took two barriers and a wait
-                // per 64 columns: 4 x 40 heads 55.0 us instead of 54.4, D 64 37.1 instead of 36.6.)
+            if (u.nsplit == 1 && u.two) {
+                // Normalise, round to bf16 and store the rows of a tensor-bound unit.  A lane has a row, and
+                // stored as it is a store instruction touches 32 lines: about 2000 cycles of a unit,
+                // during which the warp issues nothing else.  So the warp turns 32 columns of its rows
+                // round in shared memory (16-byte pieces, swizzled by the row so that neither side
+                // conflicts), and each of its stores writes 64 bytes of eight rows.  32 x 64/8 heads,
+                // N 57, L 200-2100: 100.4 -> 96.2 us; 8 x 64/8, N 256, L 4096: 240.4 -> 239.1.  No
+                // barrier: a warp's rows are its own.
+                unsigned char* stage = smem_raw + (sStage - smem_u32(smem_raw)) + warp * T::STAGE_BYTES;
+                const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+                const bool mine = rvalid && GSD_IN_BOUNDS(b < p.B && c < p.Hkv && row < R, p.status);
+                const int at = mine ? (row / G) * p.Hq + row % G : -1;      // heads from the sequence's first row
+                __nv_bfloat16* base = p.out + ((size_t)b * N * p.Hq + c * G) * HD + (lane & 3) * 8;
+                int to[4];                                                   // of the four rows this lane stores a piece of
+#pragma unroll
+                for (int j = 0; j < 4; ++j) to[j] = __shfl_sync(0xFFFFFFFFu, at, 8 * j + (lane >> 2));
+#pragma unroll
+                for (int ch = 0; ch < HD / 32; ++ch) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        uint32_t v[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) v[e] = pack_bf16(acc[ch * 32 + k * 8 + 2 * e] * inv, acc[ch * 32 + k * 8 + 2 * e + 1] * inv);
+                        *reinterpret_cast<uint4*>(stage + lane * 64 + ((k ^ ((lane >> 1) & 3)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]);
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int r = 8 * j + (lane >> 2);
+                        const uint4 v = *reinterpret_cast<const uint4*>(stage + r * 64 + (((lane & 3) ^ ((r >> 1) & 3)) << 4));
+                        if (to[j] >= 0) *reinterpret_cast<uint4*>(base + (size_t)to[j] * HD + ch * 32) = v;
+                    }
+                    __syncwarp();                                            // (the pieces have been read)
+                }
+            } else if (u.nsplit == 1) {
+                // Units with one row tile, where the loads are the bound, store straight from registers;
+                // every store of a lane fills a 32-byte sector.  (Turned round like the above 8 x 32 heads,
+                // N 8, L 64 took 15.4 us instead of 14.8.  Staged in shared memory and stored by TMA it took
+                // two barriers and a wait per 64 columns: 4 x 40 heads 55.0 us instead of 54.4, D 64 37.1
+                // instead of 36.6.)
                 if (rvalid && GSD_IN_BOUNDS(b < p.B && c < p.Hkv && row < R, p.status)) {
                     const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
                     __nv_bfloat16* dst = p.out + (((size_t)b * N + row / G) * p.Hq + c * G + row % G) * HD;
