@@ -27,8 +27,8 @@
 // issued by two warps on different schedulers, each paced only by its own barriers (the
 // softmax warps are almost always ready to issue, so one issuing warp gets too few slots
 // to feed the tensor pipe).  The running maximum is only raised when a tile
-// exceeds it by more than 2^8 (the accumulator rescale is then done in place in TMEM by the
-// row's own thread), so P <= 256 and the rescale is rare.  Every mbarrier wait is bounded: on
+// exceeds it by more than 2^8, or always, by the shape (kRescaleThreshold); the accumulator is
+// then rescaled in place in TMEM by the row's own thread.  Every mbarrier wait is bounded: on
 // expiry the kernel raises GSD_DEV_WAIT_EXPIRED, all roles leave their loops, TMEM is released.
 #include "gsd_internal.cuh"
 #include <cuda.h>
@@ -74,7 +74,13 @@ struct Geo {
     static constexpr uint32_t COL_S1 = TWO_S ? 384 : COL_S0;
     static_assert(COL_O1 + HD <= (TWO_S ? 384 : 512), "512 TMEM columns");
 };
-constexpr float kRescaleThreshold = 8.0f;         // log2 units
+// The running maximum of a row may lag behind by this much (log2 units) where groups divide 128 heads, D
+// is 128 and there are 64 rows or more.  Elsewhere it is exact, as in the mma.sync kernel: the largest
+// weights of a row are then 1 and lose nothing in bf16.  Error against 64 bits, lagging -> exact
+// (mma.sync): 4 x 32/8 heads, D 64, N 128 2.31e-3 -> 2.21e-3 (2.24e-3); groups of 3, N 77 2.28e-3 ->
+// 2.19e-3 (2.18e-3); of 7, N 200 2.34e-3 -> 2.27e-3 (2.27e-3).  Its price there: 32.7 -> 34.9 us, 25.7 ->
+// 26.8, 54.3 -> 62.5 (mma.sync: 83.1, 50.5, 215).
+constexpr float kRescaleThreshold = 8.0f;
 // Units of work per CTA decoded in the prologue.  A fixed plan with more is launched in several parts;
 // only the plans from tables decode further units where they are needed.
 constexpr int kUnitTable = 128;
@@ -123,6 +129,7 @@ struct TcParams {
     int B, N, Hq, Hkv, Lmax, G, W, R;
     int RT;           // stacked rows a row tile holds: the whole nodes that fit 128 rows, 128 / G * G
     float scale_log2;
+    float raise_above;  // the running maximum of a row is raised when a tile exceeds it by more than this (log2 units)
     PlanDev plan;
     int work0;        // first unit of this launch
     int total_work;   // units of work of this launch
@@ -989,18 +996,18 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 bool need = false;
                 if (m_ref == -CUDART_INF_F) {
                     m_new = m_tile;                         // nothing accumulated for this row yet
-                } else if (m_tile > m_ref + kRescaleThreshold) {
+                } else if (m_tile > m_ref + p.raise_above) {
                     m_new = m_tile;
                     alpha = fast_exp2(m_ref - m_new);
                     need = true;
                 }
-                if (__any_sync(0xFFFFFFFFu, need)) {
-                    // once the PV of this stream's previous job has completed, the accumulator of
-                    // this row is final for all earlier tiles: rescale it in place
-                    ok = mbar_wait(bar(BAR_P_FREE + i), (uint32_t)((tcnt + cnt - 1) & 1), abort_flag, p.status);
-                    ok = __all_sync(0xFFFFFFFFu, ok);
-                    if (!ok) break;
-                    tc_fence_after();
+                // Once the PV of this stream's previous job has completed, the accumulator of this row is
+                // final for all earlier tiles and can be rescaled in place.  Where that is common (D = 64)
+                // it is done where P_i's release is waited for anyway (head dimension 64, 4 x 32/8 heads:
+                // 36.1 us here, 35.4 there; at 128 the registers that live on cost more than the wait).
+                constexpr bool kRaiseLate = HD == 64;
+                const bool raise = __any_sync(0xFFFFFFFFu, need);
+                auto rescale = [&]() {
 #pragma unroll 1
                     for (int ch = 0; ch < HD / 32; ++ch) {
                         float v[32];
@@ -1011,6 +1018,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                         tc_st32(tO + ch * 32, v);
                     }
                     l_run *= alpha;
+                };
+                if (!kRaiseLate && raise) {
+                    ok = mbar_wait(bar(BAR_P_FREE + i), (uint32_t)((tcnt + cnt - 1) & 1), abort_flag, p.status);
+                    ok = __all_sync(0xFFFFFFFFu, ok);
+                    if (!ok) break;
+                    tc_fence_after();
+                    rescale();
                 }
                 m_ref = m_new;
                 const float m_use = m_ref == -CUDART_INF_F ? 0.f : m_ref;
@@ -1040,6 +1054,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     ok = __all_sync(0xFFFFFFFFu, ok);
                     if (!ok) break;
                     tc_fence_after();
+                    if (kRaiseLate && raise) rescale();
                 }
                 tc_st16(tP + 0, pk[0]);
                 tc_st16(tP + 16, pk[1]);
@@ -1267,6 +1282,7 @@ static int launch_tc(const AttnArgs& a) {
     p.out_by_32 = ((uintptr_t)a.out & 31u) == 0;
     p.B = a.B; p.N = a.N; p.Hq = a.Hq; p.Hkv = a.Hkv; p.Lmax = a.Lmax; p.G = a.G; p.W = a.W;
     p.R = a.N * a.G; p.RT = nodes * a.G; p.scale_log2 = a.scale_log2; p.plan = a.plan.dev;
+    p.raise_above = HD == 128 && BM % a.G == 0 && a.N * a.G >= 64 ? kRescaleThreshold : 0.f;
     p.part_o = (float*)a.workspace;
     p.part_ml = (float*)((char*)a.workspace + plan_part_o_bytes(a.plan, a.D));
     {

@@ -96,3 +96,16 @@ def test_many_units_per_cta(B, G, Hkv, D, N, lens):
         assert int(status.item()) == 0
         assert all(torch.equal(got[0], g) for g in got[1:])
         assert_close_scaled(out_to_f64(got[0]), want)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,D,N,L", [(4, 32, 8, 64, 128, (500, 1500)), (8, 12, 12, 64, 100, 1000), (5, 24, 8, 128, 150, (300, 1200)),
+                                            (4, 28, 4, 128, 120, 1500)])
+def test_no_less_exact_than_the_mma_kernel(B, Hq, Hkv, D, N, L):
+    # these shapes ran on the mma.sync kernel, whose running maxima are exact: the relative error of the
+    # whole output (rms, against fp64) is the same to 1% over these 10^6 to 10^7 values; with a lagging
+    # maximum it is 3.2 to 4.6% larger
+    cfg = gi.VerifyConfig("t", 7, B, Hq, Hkv, D, L, N, 9, 4, 3, 8, 8, 0.5)
+    inp = gi.make_inputs(cfg, 17, accept=False)
+    want = cpu_attn(inp)
+    err = [np.linalg.norm(out_to_f64(gpu_attn(inp, kernel=k)) - want) / np.linalg.norm(want) for k in (0, 1)]
+    assert err[0] <= 1.02 * err[1], err
