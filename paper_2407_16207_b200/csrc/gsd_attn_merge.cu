@@ -2,9 +2,12 @@
 // partial results of every row.
 //   m = max_s m_s;  out = sum_s 2^(m_s - m) O_s / sum_s 2^(m_s - m) l_s
 //
-// A block takes 32 rows of a row tile and 16 of its column groups: a lane is a row, a thread has two
+// A warp takes 32 rows of a row tile and two of its column groups: a lane is a row, a thread has two
 // column groups (8 values, 16 bytes of output).  The rows of a column group are consecutive in the
-// partial results, so every load of a warp is 512 contiguous bytes.  Few registers and short code
+// partial results, so every load of a warp is 512 contiguous bytes.  For items of fewer than 64 rows of
+// the mma.sync kernel a warp takes 8 rows and four column groups, one a thread, which leaves fewer lanes
+// without a row (D 64, whole call: 2 x 12 heads, N 40, L 1500 15.2 us, 15.5 with 32 rows a warp; 32/8
+// heads, N 8, L 4000 14.6 and 14.9; the tcgen05 kernel's few rows are up to 2% slower that way).  Few registers and short code
 // on purpose: the launch lasts a few microseconds, and a form with four column groups a thread and
 // the next four parts on their way while four are added up took 1 us longer.
 #include "gsd_internal.cuh"
@@ -16,7 +19,6 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kBatch = 4;        // parts of a row on their way at a time
-constexpr int kCols = kThreads / 32 * 2;     // column groups of a block
 constexpr int kWalkers = 296;    // blocks that walk over the items of a one-wave plan (two per SM)
 
 struct MergeParams {
@@ -28,7 +30,8 @@ struct MergeParams {
     int tile_rows;           // rows of a tile in the partial results (128 or 64)
     int RT;                  // of them in use
     int tiles;               // row tiles of an item
-    int groups;              // blocks of 32 rows of an item that can hold a row
+    int groups;              // runs of kRows rows of an item that can hold a row
+    int work;                // warps' worth of work
     int B;
     const int* bal_hdr;      // balanced plan: [0] = items to merge (known on the device only)
     const int4* bal_merge;   // balanced plan: (pair, first slot, slots) per pair to merge, else nullptr
@@ -48,24 +51,29 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // 64/8 heads, N 32, L 2048: 42.4 us with blocks for every item, 39.8 walking (37.1 with a plan that
 // cannot cut, which takes 115 instead of 28.5 when one of the sequences has 8192 and the others 500).
 // Where every item may be cut, one block for each part of it is up to 0.5 us faster.
-template <bool kWalk>
+template <bool kWalk, int kRows>
 __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
     const int lane = threadIdx.x & 31;
-    const int quads = p.D / 4, parts_of_row = quads / kCols;
+    constexpr int kGroups = kRows == 32 ? 2 : 1;                   // column groups of a thread
+    constexpr int kSpan = 32 / kRows * kGroups;                    // of a warp
+    const int quads = p.D / 4, parts_of_row = quads / kSpan;
+    const int warp = (int)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
     // Launched as a programmatic dependent of the attention kernel: the blocks may become
     // resident while that kernel drains; what it (or the planning kernel) wrote is only visible
-    // after this wait.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // after this wait, which comes as late as the plan allows: working out a warp's place takes a
+    // dozen divisions.
+    auto ready = []() { asm volatile("griddepcontrol.wait;" ::: "memory"); };
     unsigned cut = 0;                                              // kWalk: the sequences that were cut
-    int blocks = (int)gridDim.x;
+    int work = p.work;
     if (kWalk) {
+        ready();
         cut = __ballot_sync(0xFFFFFFFFu, lane < p.B && p.left[lane] > 1);
-        blocks = __popc(cut) * p.Hkv * p.plan.tiles_per_unit * p.groups * parts_of_row;
+        work = __popc(cut) * p.Hkv * p.plan.tiles_per_unit * p.groups * parts_of_row;
     }
-    for (int blk = blockIdx.x; blk < blocks; blk += gridDim.x) {   // (once, unless kWalk)
-    const int col0 = (blk % parts_of_row) * kCols + (threadIdx.x >> 5) * 2;      // first column group of the thread
-    const int g = blk / parts_of_row % p.groups;
-    const int k = blk / parts_of_row / p.groups;
+    for (int w = warp; w < work; w += (int)gridDim.x * (kThreads / 32)) {      // (once, unless kWalk)
+    const int col0 = w % parts_of_row * kSpan + lane / kRows * kGroups;       // first column group of the thread
+    const int g = w / parts_of_row % p.groups;
+    const int k = w / parts_of_row / p.groups;
     // the k-th item that owns slots: group a comes first when it is split at all
     int item, nsplit, slot0, slot_step = 1;
     const int split_a = p.plan.splits_a > 1 ? p.plan.items_a : 0;
@@ -80,6 +88,7 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
     } else if (p.bal_merge) {
         // the list of cut items was made on the device; the grid covers the most there can be
         const int tpu = p.plan.tiles_per_unit, rt = k % tpu;
+        ready();
         const int listed = p.bal_hdr[0];
         const int4 rec = p.bal_merge[k / tpu];       // a (sequence, kv head) pair that was cut (read beside the count)
         if (k / tpu >= listed) return;
@@ -87,6 +96,7 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
     } else if (p.seq.hdr) {
         const int per_seq = p.Hkv * p.plan.tiles_per_unit;
         const int b = k / per_seq;
+        ready();
         nsplit = p.seq.nsplit[b];
         if (nsplit == 1) return;                       // the item was stored by its only unit
         item = k;
@@ -94,6 +104,7 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
     } else if (p.plan.balanced == 3) {
         const int per_seq = p.Hkv * p.plan.tiles_per_unit;
         const int b = k / per_seq;
+        ready();
         nsplit = p.left[b];
         if (nsplit == 1) return;
         item = k;
@@ -105,29 +116,31 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
         item = p.plan.items_a + (k - split_a); nsplit = p.plan.splits_b;
         slot0 = split_a * p.plan.splits_a + (k - split_a) * p.plan.splits_b;
     }
-    const int per_tile = p.tile_rows / 32;
-    const int tile = g / per_tile, r = (g - tile * per_tile) * 32 + lane;
+    const int per_tile = p.tile_rows / kRows;
+    const int tile = g / per_tile, r = (g - tile * per_tile) * kRows + lane % kRows;
     const int unit = item / p.plan.tiles_per_unit;
     const int row = (item % p.plan.tiles_per_unit) * p.tiles * p.RT + tile * p.RT + r;
     if (r >= p.RT || row >= p.R) {
         if (kWalk) continue;
         return;
     }
-    const int b = p.plan.longest_first ? p.left[unit / p.Hkv] : unit / p.Hkv, c = unit % p.Hkv;
+    const int place = unit / p.Hkv, c = unit % p.Hkv, node = row / p.G, head = c * p.G + row % p.G;
+    if (!kWalk) ready();
+    const int b = p.plan.longest_first ? p.left[place] : place;
 
     const size_t first = (size_t)slot0 * p.tiles + tile;
     const float2* ml_base = p.part_ml + first * p.tile_rows + r;
     const float4* o_base = p.part_o + (first * quads + col0) * p.tile_rows + r;
     const size_t ml_stride = (size_t)slot_step * p.tiles * p.tile_rows, o_stride = ml_stride * quads;
     float2 ml[kBatch];
-    float4 v[kBatch][2];
+    float4 v[kBatch][kGroups];
     auto fetch = [&](int s0) {
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
             const bool in = s0 + j < nsplit;
             ml[j] = in ? ml_base[(size_t)(s0 + j) * ml_stride] : make_float2(-CUDART_INF_F, 0.f);
 #pragma unroll
-            for (int q = 0; q < 2; ++q)
+            for (int q = 0; q < kGroups; ++q)
                 v[j][q] = in ? o_base[(size_t)(s0 + j) * o_stride + q * p.tile_rows] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
@@ -136,7 +149,7 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
 #pragma unroll 4
     for (int s = kBatch; s < nsplit; ++s) m = fmaxf(m, ml_base[(size_t)s * ml_stride].x);
     const float m_use = m == -CUDART_INF_F ? 0.f : m;
-    float acc[2][4] = {};
+    float acc[kGroups][4] = {};
     float l = 0.f;
 #pragma unroll 1
     for (int s0 = 0; s0 < nsplit; s0 += kBatch) {
@@ -146,20 +159,22 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
             const float wgt = exp2f(ml[j].x - m_use);     // 0 for an absent or empty split
             l += wgt * ml[j].y;
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
+            for (int q = 0; q < kGroups; ++q) {
                 acc[q][0] += wgt * v[j][q].x; acc[q][1] += wgt * v[j][q].y;
                 acc[q][2] += wgt * v[j][q].z; acc[q][3] += wgt * v[j][q].w;
             }
         }
     }
     const float inv = l > 0.f ? 1.f / l : 0.f;
-    __nv_bfloat16* dst = p.out + (((size_t)b * p.N + row / p.G) * p.Hq + c * p.G + row % p.G) * p.D + col0 * 4;
-    uint4 o;
-    o.x = pack_bf16(acc[0][0] * inv, acc[0][1] * inv);
-    o.y = pack_bf16(acc[0][2] * inv, acc[0][3] * inv);
-    o.z = pack_bf16(acc[1][0] * inv, acc[1][1] * inv);
-    o.w = pack_bf16(acc[1][2] * inv, acc[1][3] * inv);
-    *reinterpret_cast<uint4*>(dst) = o;
+    __nv_bfloat16* dst = p.out + (((size_t)b * p.N + node) * p.Hq + head) * p.D + col0 * 4;
+    uint32_t o[2 * kGroups];
+#pragma unroll
+    for (int q = 0; q < kGroups; ++q) {
+        o[2 * q] = pack_bf16(acc[q][0] * inv, acc[q][1] * inv);
+        o[2 * q + 1] = pack_bf16(acc[q][2] * inv, acc[q][3] * inv);
+    }
+    if constexpr (kGroups == 2) *reinterpret_cast<uint4*>(dst) = make_uint4(o[0], o[1], o[2], o[3]);
+    else *reinterpret_cast<uint2*>(dst) = make_uint2(o[0], o[1]);
     if (!kWalk) return;
     }
 }
@@ -203,13 +218,16 @@ int launch_attn_merge(const AttnArgs& a) {
         p.bal_groups = groups;
         split_items = (pairs < groups - 1 ? pairs : groups - 1) * tpu;   // one pair per cut at most
     }
-    // blocks of 32 rows that can hold a row: all of them, or those up to the last row of a lone item
-    const int per_tile = p.tile_rows / 32;
+    // runs of rows that can hold a row: all of them, or those up to the last row of a lone item
+    const int rows = p.tile_rows == 64 && p.R < 64 ? 8 : 32, span = rows == 8 ? 4 : 2;
+    const int per_tile = p.tile_rows / rows;
     p.groups = p.R >= a.plan.rows_per_item ? p.tiles * per_tile
-               : p.R <= p.RT               ? (p.R + 31) / 32
-                                           : per_tile + (p.R - p.RT + 31) / 32;
-    long blocks = (long)split_items * p.groups * (p.D / 4 / kCols);
-    if (blocks == 0) return GSD_OK;
+               : p.R <= p.RT               ? (p.R + rows - 1) / rows
+                                           : per_tile + (p.R - p.RT + rows - 1) / rows;
+    const long work = (long)split_items * p.groups * (p.D / 4 / span);
+    if (work == 0) return GSD_OK;
+    p.work = (int)work;
+    long blocks = (work + kThreads / 32 - 1) / (kThreads / 32);
     if (walk && blocks > kWalkers) blocks = kWalkers;
     cudaLaunchAttribute attr[1];
     dependent_launch_attr(attr);
@@ -219,7 +237,9 @@ int launch_attn_merge(const AttnArgs& a) {
     cfg.stream = a.stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, walk ? attn_merge_kernel<true> : attn_merge_kernel<false>, p));
+    void (*kernel)(MergeParams) = rows == 8 ? (walk ? attn_merge_kernel<true, 8> : attn_merge_kernel<false, 8>)
+                                            : (walk ? attn_merge_kernel<true, 32> : attn_merge_kernel<false, 32>);
+    GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, p));
     return GSD_OK;
 }
 
