@@ -68,9 +68,10 @@ typedef enum gsd_status {
 
 /* kernel selection for gsd_verify_attn */
 /* GSD_ATTN_AUTO takes the tcgen05 kernel when it supports the shape and the stacked rows of one
- * (sequence, kv head), N * Hq/Hkv, number at least 64 or, with head dimension 128, the cache has 512
- * rows or more (head dimension 64 or 128, groups of up to 128 heads); everything else runs on the mma.sync kernel, which reaches roughly a sixth of the
- * tensor throughput.  Asking for GSD_ATTN_TCGEN05 by name is answered for D == 128 and group
+ * (sequence, kv head), N * Hq/Hkv, number at least 64 (head dimension 64 or 128, groups of up to 128
+ * heads); with fewer rows, if the head dimension is 128, the cache has 512 rows or more and there are no
+ * more (sequence, kv head) pairs than SMs.  Everything else runs on the mma.sync kernel, which reaches
+ * roughly a sixth of the tensor throughput.  Asking for GSD_ATTN_TCGEN05 by name is answered for D == 128 and group
  * sizes that divide 128 only; other shapes return GSD_ERR_UNSUPPORTED. */
 #define GSD_ATTN_SPLIT_BALANCED (-1)      /* values of gsd_attn_params.num_splits */
 #define GSD_ATTN_SPLIT_PER_SEQUENCE (-2)

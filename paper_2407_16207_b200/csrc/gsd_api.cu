@@ -45,26 +45,30 @@ static int attn_params_ok(const gsd_attn_params* p) {
     return GSD_OK;
 }
 
-int attn_pick_kernel(const gsd_attn_params* p) {
+int attn_pick_kernel(const gsd_attn_params* p, int sm_count) {
     if (p->kernel != GSD_ATTN_AUTO) return p->kernel;
     // The TMEM kernel pays off once the stacked rows fill its 128-row tiles.  D = 64 and groups
     // that do not divide 128 ran on the mma.sync kernel before, measured at 5 x 8 groups of 3,
     // D 128, N 77, L 300-1999: 45.4 us there, 28.5 us here; 4 x 8 groups of 4, D 64, N 128,
     // L 1000-4000: 81 us there, 42 us here (device time of the whole call).
     const int G = p->Hq / p->Hkv;
-    // Fewer rows leave most of a tile empty, and then the loads decide: at D = 128 and 512 or more cache
-    // rows the TMA rings are ahead of the mma.sync kernel's cp.async pipeline (mma.sync -> tcgen05, us:
-    // 1 x 32 heads, N 8, L 1000 13.6 -> 12.4, L 4000 32.8 -> 17.7; 32 x 32, N 8, L 2000 288 -> 176;
-    // 8 x 28/4, N 8, L 1000 15.0 -> 14.8; 8 x 32, N 1, L 2000 77.5 -> 50.6).  Short contexts and D = 64
-    // stay: the start of a unit costs more there (8 x 32, N 8, L 200 15.6 -> 17.8; 32 x 32/8, N 4, L 64
-    // 9.4 -> 15.3; D 64, 32 x 12, N 20, L 700 30.0 -> 32.9).
-    if (attn_tcgen05_supports(p->D, G) && (p->N * G >= 64 || (p->D == 128 && p->Lmax >= 512))) return GSD_ATTN_TCGEN05;
+    // Fewer rows leave most of a tile empty, and then it depends on the context, which is not known
+    // here: Lmax is the room in the cache.  At D = 128 and 512 or more cache rows, with no more items than
+    // SMs, the tcgen05 kernel is the faster one for any context (mma.sync -> tcgen05, us: 1 x 32 heads, N 8,
+    // L 64 12.4 -> 8.8, L 1000 17.5 -> 12.0; 1 x 64/8, N 4, L 200 10.5 -> 9.9; 4 x 32, N 48, L 64 14.7 -> 9.3,
+    // L 4000 102 -> 46.6).  With more items its second round of units costs short contexts more than long
+    // ones gain - and the cache of a server is mostly empty early on: 8 x 32 heads, N 8: L 64 7.3 there,
+    // 14.8 here, L 200 12.2 and 17.4, L 1000 32.1 and 31.3; N 32: 9.3 and 15.1, 15.2 and 17.4, 41.4 and 32.0
+    // (L 4000 136 and 90).  Short caches and D = 64 stay there too: the start of a unit costs more here
+    // (D 64, 32 x 12, N 20, L 700 26.6 and 32.9).
+    if (!attn_tcgen05_supports(p->D, G)) return GSD_ATTN_MMA;
+    if (p->N * G >= 64 || (p->D == 128 && p->Lmax >= 512 && p->B * p->Hkv <= sm_count)) return GSD_ATTN_TCGEN05;
     return GSD_ATTN_MMA;
 }
 
 AttnPlan attn_make_plan(const gsd_attn_params* p, int sm_count, bool by_length) {
     AttnPlan pl;
-    pl.kernel = attn_pick_kernel(p);
+    pl.kernel = attn_pick_kernel(p, sm_count);
     const bool tc = pl.kernel == GSD_ATTN_TCGEN05;
     const int G = p->Hq / p->Hkv;
     const int R = p->N * G;

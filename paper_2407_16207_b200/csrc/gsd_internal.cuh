@@ -140,7 +140,7 @@ struct AttnArgs {
     cudaStream_t stream;
 };
 
-int attn_pick_kernel(const gsd_attn_params* p);                 // GSD_ATTN_MMA or GSD_ATTN_TCGEN05
+int attn_pick_kernel(const gsd_attn_params* p, int sm_count);   // GSD_ATTN_MMA or GSD_ATTN_TCGEN05
 // Partial results: fp32 accumulators, then (max, sum) pairs.  A slot holds the row tiles of an item
 // (one of 64 rows, or two of 128); a tile is [D / 4 column groups][rows] of float4 - the rows of a
 // column group are consecutive, for the store of an accumulator (a lane per row) and for the merge

@@ -94,3 +94,22 @@ def test_few_rows(Hq, Hkv, N, lens):
     want = cpu_attn(inp)
     for splits in (0, 2):
         assert_close_scaled(out_to_f64(call(inp, num_splits=splits)), want)
+
+
+@pytest.mark.parametrize("D,G,N", [(128, 1, 1), (128, 1, 15), (128, 4, 4), (128, 1, 17), (128, 2, 16), (128, 3, 11), (128, 1, 48), (128, 7, 9),
+                                   (64, 1, 16), (64, 3, 6), (64, 1, 49)])
+def test_few_rows_of_many_items(D, G, N):
+    # more (sequence, kv head) pairs than SMs: the mma.sync kernel whatever the cache length, whose warps
+    # without a row (16 rows each) only help to load; cut items are merged by eight rows
+    import paper_2407_16207_b200 as gsd
+    B, Hkv = 40, 4
+    assert B * Hkv > torch.cuda.get_device_properties(0).multi_processor_count
+    lens = np.random.default_rng(N).integers(0, 600, B)
+    lens[:3] = 0, 600, 64
+    inp = inputs(B, G * Hkv, Hkv, D, N, lens)
+    want = cpu_attn(inp)
+    got = call(inp)
+    assert torch.equal(got, call(inp, kernel=gsd.GSD_ATTN_MMA))
+    assert_close_scaled(out_to_f64(got), want)
+    for splits in (1, 3):
+        assert_close_scaled(out_to_f64(call(inp, num_splits=splits, kernel=gsd.GSD_ATTN_MMA)), want)
