@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 from typing import Optional, Tuple
 
 import torch
@@ -135,11 +136,40 @@ def native():
         except ImportError as e:
             raise GsdError(-100, f"the extension _native.so is missing or does not load ({e}): run "
                                  "`python -m paper_2407_16207_b200.build`") from e
+        if module.torch_version != torch.__version__:
+            raise GsdError(-100, f"the extension _native.so was built against torch {module.torch_version}, this is "
+                                 f"{torch.__version__}: run `python -m paper_2407_16207_b200.build`")
         _native = module
     if _native_lib is not L:
         _native.bind(*(ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in _NATIVE_CALLS))
         _native_lib = L
     return _native
+
+
+class _Declines:
+    """In the extension's place where it cannot be loaded: takes no call."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
+_declines: Optional[_Declines] = None
+
+
+def _marshal():
+    """What the calls try first: the extension, or nothing but the ctypes path if it does not load (the
+    library and its kernels are the same, a call takes 20 us longer)."""
+    global _declines
+    if _native is not None and _lib is not None and _lib is _native_lib:
+        return _native
+    if _declines is None:
+        lib()                                   # (a missing library is an error)
+        try:
+            return native()
+        except GsdError as e:
+            _declines = _Declines()
+            warnings.warn(f"{e}; the calls go through ctypes", RuntimeWarning, stacklevel=3)
+    return _declines
 
 
 def _check(rc: int) -> None:
@@ -219,7 +249,7 @@ def gsd_verify_attn(q, k_cache, v_cache, draft_k, draft_v, ancestor_mask, seq_le
                     status: Optional[torch.Tensor] = None) -> torch.Tensor:
     """DAG-masked attention of the draft nodes; see gsd_verify_attn in include/gsd.h.
     Enqueued on the current stream; returns `out` [B,N,Hq,D] bf16."""
-    fast = _native if _lib is not None and _lib is _native_lib else native()
+    fast = _native if _lib is not None and _lib is _native_lib else _marshal()
     r = fast.verify_attn(q, k_cache, v_cache, draft_k, draft_v, ancestor_mask, seq_lens, out, softmax_scale, num_splits, kernel,
                          workspace, status)
     if r is not None:
@@ -257,7 +287,7 @@ def gsd_accept(logits, draft_tokens, parent_ptr, parent_idx, *, Tcap: int = 0,
     """Greedy verification + longest accepted path; see gsd_accept in include/gsd.h.
     Returns (accepted_tokens [B,Tcap], accepted_len [B], accepted_nodes [B,Tcap] or None)."""
     if out is None:
-        fast = _native if _lib is not None and _lib is _native_lib else native()
+        fast = _native if _lib is not None and _lib is _native_lib else _marshal()
         r = fast.accept(logits, draft_tokens, parent_ptr, parent_idx, Tcap, want_nodes, workspace, status)
         if r is not None:
             if r.__class__ is int:
@@ -310,7 +340,7 @@ def gsd_accept_sampled(logits, draft_tokens, parent_ptr, parent_idx, draft_q, u_
     residual max(0, P - Q).  Returns (accepted_tokens [B,Tcap], accepted_len [B], accepted_nodes
     or None)."""
     if out is None:
-        fast = _native if _lib is not None and _lib is _native_lib else native()
+        fast = _native if _lib is not None and _lib is _native_lib else _marshal()
         r = fast.accept_sampled(logits, draft_tokens, parent_ptr, parent_idx, draft_q, u_accept, u_sample, draft_logits, Tcap,
                                 want_nodes, workspace, status)
         if r is not None:
@@ -365,7 +395,7 @@ def gsd_draft_expand(logits, frontier, frontier_len, tokens, tree_parent, merge_
     """One growth step of the draft token graph, in place; see gsd_draft_expand in include/gsd.h.
     Returns (new_frontier [B,F*k], new_frontier_len [B])."""
     if out is None:
-        fast = _native if _lib is not None and _lib is _native_lib else native()
+        fast = _native if _lib is not None and _lib is _native_lib else _marshal()
         r = fast.draft_expand(logits, frontier, frontier_len, tokens, tree_parent, merge_to, leaf, prob, num_nodes, k, tau,
                               theta_prob, theta_sib, workspace, status)
         if r is not None:
@@ -408,7 +438,7 @@ def gsd_build_mask(parent_ptr, parent_idx, out: Optional[torch.Tensor] = None, *
                    status: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Ancestor bitmask [B,N,ceil(N/32)] (int32 words) from the parent CSR; see gsd_build_mask in
     include/gsd.h.  Enqueued on the current stream."""
-    fast = _native if _lib is not None and _lib is _native_lib else native()
+    fast = _native if _lib is not None and _lib is _native_lib else _marshal()
     r = fast.build_mask(parent_ptr, parent_idx, out, status)
     if r is not None:
         if r.__class__ is int:
@@ -461,7 +491,7 @@ def gsd_commit_kv(k_cache, v_cache, draft_k, draft_v, accepted_nodes, accepted_l
                   status: Optional[torch.Tensor] = None) -> None:
     """Append the draft K/V rows of the accepted path to the cache in place and advance
     seq_lens; see gsd_commit_kv in include/gsd.h.  Enqueued on the current stream."""
-    fast = _native if _lib is not None and _lib is _native_lib else native()
+    fast = _native if _lib is not None and _lib is _native_lib else _marshal()
     r = fast.commit_kv(k_cache, v_cache, draft_k, draft_v, accepted_nodes, accepted_len, seq_lens, status)
     if r is not None:
         return _check(r)

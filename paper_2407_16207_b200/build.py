@@ -38,13 +38,16 @@ def build_native(force: bool = False) -> str:
     """Compile csrc/gsd_native.cpp (host code only) against the installed torch and CPython."""
     import torch
     src = os.path.join(CSRC, "gsd_native.cpp")
-    if not force and not _stale(NATIVE, [src, os.path.join(ROOT, "include", "gsd.h"), torch.__file__]):
+    built_for = os.path.join(OBJ_DIR, "native_torch_version")
+    same = os.path.exists(built_for) and open(built_for).read() == torch.__version__
+    if not force and same and not _stale(NATIVE, [src, os.path.join(ROOT, "include", "gsd.h")]):
         return NATIVE
+    os.makedirs(OBJ_DIR, exist_ok=True)
     base = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.sep in _nvcc() else "/usr/local/cuda"
     tmp = NATIVE + f".tmp{os.getpid()}"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f'-DGSD_TORCH_VERSION="{torch.__version__}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            "-I", os.path.join(ROOT, "include"), "-isystem", os.path.join(base, "include"),
            "-isystem", os.path.join(base, "include", "torch", "csrc", "api", "include"),
            "-isystem", os.path.join(cuda, "include"), "-isystem", sysconfig.get_paths()["include"],
@@ -55,6 +58,8 @@ def build_native(force: bool = False) -> str:
         sys.stderr.write(r.stdout + r.stderr)
         raise RuntimeError("c++ failed: " + " ".join(cmd))
     os.replace(tmp, NATIVE)
+    with open(built_for, "w") as f:
+        f.write(torch.__version__)
     return NATIVE
 
 

@@ -385,4 +385,9 @@ PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__native(void) { return PyModule_Create(&module_def); }
+// (the classes of torch's headers are compiled in: binding.py refuses another version's)
+PyMODINIT_FUNC PyInit__native(void) {
+    PyObject* m = PyModule_Create(&module_def);
+    if (m && PyModule_AddStringConstant(m, "torch_version", GSD_TORCH_VERSION) != 0) Py_CLEAR(m);
+    return m;
+}

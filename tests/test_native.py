@@ -35,6 +35,30 @@ def test_the_table_names_the_calls_in_order():
     assert tuple(re.findall(r"decltype\(&(gsd_\w+)\)", table)) == gsd.binding._NATIVE_CALLS
 
 
+@pytest.mark.parametrize("why", ["missing", "another torch"])
+def test_without_the_extension_the_calls_go_through_ctypes(why, monkeypatch):
+    import sys
+    import types
+    import warnings
+    import paper_2407_16207_b200 as gsd
+    b = gsd.binding
+    for name in ("_native", "_native_lib", "_declines"):
+        monkeypatch.setattr(b, name, None)
+    other = None if why == "missing" else types.SimpleNamespace(torch_version="0.0")
+    monkeypatch.setitem(sys.modules, b.__package__ + "._native", other)
+    monkeypatch.delattr(sys.modules[b.__package__], "_native", raising=False)
+    if other is not None:
+        monkeypatch.setattr(sys.modules[b.__package__], "_native", other, raising=False)
+    with pytest.raises(gsd.GsdError, match="_native.so"):
+        b.native()
+    i32 = lambda *s: torch.zeros(s, dtype=torch.int32)
+    with pytest.warns(RuntimeWarning, match="ctypes"), pytest.raises(ValueError, match="parent_ptr: expected a CUDA tensor"):
+        gsd.gsd_build_mask(i32(1, 5), i32(1, 4))
+    with warnings.catch_warnings(), pytest.raises(ValueError, match="logits: expected contiguous torch.float32"):
+        warnings.simplefilter("error")              # said once
+        gsd.gsd_accept(torch.zeros(1, 4, 8).double(), i32(1, 4), i32(1, 5), i32(1, 4))
+
+
 def inputs(seed, Hkv=2, D=128, N=70):
     cfg = gi.VerifyConfig("n", 7, 3, 4 * Hkv, Hkv, D, (50, 700), N, 9, 3, 2, 1003, 64, 0.6)
     inp = gi.make_inputs(cfg, seed)
