@@ -113,3 +113,16 @@ def test_few_rows_of_many_items(D, G, N):
     assert_close_scaled(out_to_f64(got), want)
     for splits in (1, 3):
         assert_close_scaled(out_to_f64(call(inp, num_splits=splits, kernel=gsd.GSD_ATTN_MMA)), want)
+
+
+@pytest.mark.parametrize("B,Hkv,splits", [(384, 52, 0), (400, 48, 0), (25, 12, 64)])
+def test_more_units_than_one_launch_takes(B, Hkv, splits):
+    # more than 128 units a CTA go out in several launches: longest first (up to 384 sequences), in
+    # order, and cut (most of the 64 parts are empty), where each launch is a dependent of the one before
+    N, D = 64, 64
+    rng = np.random.default_rng(B)
+    inp = inputs(B, Hkv, Hkv, D, N, rng.integers(0, 40 if splits == 0 else 900, B))
+    assert B * Hkv * max(splits, 1) > 128 * torch.cuda.get_device_properties(0).multi_processor_count
+    got = call(inp, num_splits=splits)
+    assert torch.equal(got, call(inp, num_splits=splits))
+    sampled_rows_check(inp, got, rng, n_random=2000, units=[(0, 0), (B // 2, Hkv - 1), (B - 1, Hkv - 1)])
