@@ -221,8 +221,9 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
         "{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n"
         " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar) : "memory");
 }
-// 32 lanes x 32 consecutive fp32 columns: thread t of the warp gets lane (base + t)
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
+// 32 lanes x 32 consecutive fp32 columns: thread t of the warp gets lane (base + t).  v[0..31] must be
+// register-resident (constant indices after unrolling).
+__device__ __forceinline__ void tc_ld32(uint32_t taddr, float* v) {
     uint32_t* r = reinterpret_cast<uint32_t*>(v);
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -259,19 +260,6 @@ __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16])
 __device__ __forceinline__ void st_global8(void* dst, const uint32_t (&v)[8]) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                  ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
-}
-// pointer form: v[0..31] must be register-resident (constant indices after unrolling)
-__device__ __forceinline__ void tc_ld32p(uint32_t taddr, float* v) {
-    uint32_t* r = reinterpret_cast<uint32_t*>(v);
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ float max3(float a, float b, float c) {
     float d;
@@ -976,7 +964,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 // the whole score row of this thread: 128 fp32 registers
                 float sc[BN];
 #pragma unroll
-                for (int ch = 0; ch < 4; ++ch) tc_ld32p(tS + ch * 32, sc + ch * 32);
+                for (int ch = 0; ch < 4; ++ch) tc_ld32(tS + ch * 32, sc + ch * 32);
                 tc_wait_ld();
                 tc_fence_before();
                 if (lane == 0) mbar_arrive(bar(BAR_S_FREE + i));   // the next job's QK^T may overwrite S
@@ -1110,7 +1098,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (ntiles > 0) {
                 tc_fence_after();
 #pragma unroll
-                for (int ch = 0; ch < HD / 32; ++ch) tc_ld32p(tO + ch * 32, acc + ch * 32);
+                for (int ch = 0; ch < HD / 32; ++ch) tc_ld32(tO + ch * 32, acc + ch * 32);
                 tc_wait_ld();
                 if (alt && n1 > 0) {
                     // merge the odd-tile stream: O = w0 O0 + w1 O1, l = w0 l0 + w1 l1 at the common maximum
