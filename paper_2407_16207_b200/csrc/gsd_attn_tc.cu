@@ -1303,13 +1303,11 @@ static int launch_tc(const AttnArgs& a) {
         p.bal_units = t.units;
     }
     // Persistent CTAs.  A short call sets itself up beside the end of its predecessor on the stream, which
-    // saves about 0.7 us (beside / after it: 16 x 64/8 heads, N 32, L 256 14.0 / 14.7 us, L 1024 27.2 /
-    // 27.6).  From 16 key tiles a CTA on, about 40 us, that is no longer seen (L 4096 70.8 / 70.7; 8 x 64/8,
-    // N 256, L 4096 236.6 / 236.2; 32 x 64/8, N 512, L 8192 4091 / 4085), and CTAs placed where and when SMs
-    // fall free were up to 5% slower (20 x 40 heads, N 64, L 500 59.2 / 56.2; 30 x 64/8, N 64, L 700 77.5 /
-    // 74.9): such calls are launched the ordinary way.
+    // saves 1 to 2 us; a long one is launched the ordinary way, as CTAs that are placed where and when
+    // SMs fall free ran 1% slower (4155 us instead of 4103 for the 1882 key tiles a CTA of 32 x 64/8
+    // heads, L 8192, N 512, power-limited).  256 tiles are about 400 us.
     const long long tiles = (long long)a.plan.items * ((a.Lmax + BN - 1) / BN + (a.N + BN - 1) / BN);
-    const bool beside = a.plan.dev.balanced || tiles < 16ll * di.sm_count;
+    const bool beside = a.plan.dev.balanced || tiles < 256ll * di.sm_count;
     cudaLaunchAttribute attr[1];
     dependent_launch_attr(attr);
     cudaLaunchConfig_t cfg = {};
