@@ -197,7 +197,7 @@ int gsd_verify_attn_num_splits(const gsd_attn_params* p);
  *   status          device int32 word or NULL
  *   stream          cudaStream_t
  *
- * logits must be 4-byte aligned; 16-byte alignment with V % 4 == 0 enables vector loads.
+ * logits must be 4-byte aligned.  Rows are read 16 bytes at a time whatever the vocabulary and the alignment.
  */
 int gsd_accept(const float* logits, const int32_t* draft_tokens, const int32_t* parent_ptr,
                const int32_t* parent_idx, int32_t* accepted_tokens, int32_t* accepted_len,

@@ -521,8 +521,10 @@ int pick_slices(long rows, int V, int sm_count) {
 }
 
 // CTAs of the second launch per sequence: only the two passes over the end node's rows are shared,
-// so a CTA should have at least 2048 entries of them (one round of loads), and all clusters should
-// be resident at once (two CTAs per SM).  Without draft logits there is no residual and no pass.
+// so a CTA should have at least 2048 entries of them (half a round of loads), and all of them together take
+// one CTA per SM at most: they are resident while the first launch still streams, and the SMs they take
+// are missing there (32 x 64 rows of 32000: 62.9 us with one CTA per sequence, 64.7 with eight, 56.9 with
+// the four that this allows).  Without draft logits there is no residual and no pass.
 int pick_cluster(int B, int V, bool residual, int sm_count) {
     int c = 1;
     while (residual && c * 2 <= kMaxCluster && V / (c * 2) >= 2048 && (long)B * c * 2 <= sm_count) c *= 2;

@@ -1303,9 +1303,11 @@ static int launch_tc(const AttnArgs& a) {
         p.bal_units = t.units;
     }
     // Persistent CTAs.  A short call sets itself up beside the end of its predecessor on the stream, which
-    // saves 1 to 2 us; a long one is launched the ordinary way, as CTAs that are placed where and when
-    // SMs fall free ran 1% slower (4155 us instead of 4103 for the 1882 key tiles a CTA of 32 x 64/8
-    // heads, L 8192, N 512, power-limited).  256 tiles are about 400 us.
+    // saves 1 to 2 us where that is other work (beside / behind: 4 x 40 heads, N 128, L 1024-4096, 36 key
+    // tiles a CTA, 51.0 / 52.5 us; the step of 8 x 64/8 heads, N 256, L 4096, 118 tiles, 340 / 342).  A
+    // long one, which has nothing to gain, is launched the ordinary way: CTAs placed where and when SMs
+    // fall free ran up to 1% slower (32 x 64/8 heads, L 8192, N 512, 1882 tiles, power-limited: 4155 / 4103
+    // once, 4091 / 4085 another time).  256 tiles are about 400 us.
     const long long tiles = (long long)a.plan.items * ((a.Lmax + BN - 1) / BN + (a.N + BN - 1) / BN);
     const bool beside = a.plan.dev.balanced || tiles < 256ll * di.sm_count;
     cudaLaunchAttribute attr[1];
