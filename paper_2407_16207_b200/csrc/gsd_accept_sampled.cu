@@ -55,15 +55,15 @@ __device__ __forceinline__ void take16(Ms& r, float4 a, float4 b, float4 c, floa
     const float m4 = fmaxf(fmaxf(fmaxf(a.x, a.y), fmaxf(a.z, a.w)), fmaxf(fmaxf(b.x, b.y), fmaxf(b.z, b.w)));
     const float m8 = fmaxf(fmaxf(fmaxf(c.x, c.y), fmaxf(c.z, c.w)), fmaxf(fmaxf(d.x, d.y), fmaxf(d.z, d.w)));
     const float m = fmaxf(r.m, fmaxf(m4, m8));
-    if (m == -CUDART_INF_F) {
-        // nothing above -inf yet: the values add up to -inf, or to NaN if there is one
-        const float t = (((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w))) + (((c.x + c.y) + (c.z + c.w)) + ((d.x + d.y) + (d.z + d.w)));
-        if (t != t) r.s = t;
-        return;
-    }
     float ref = m;
-    if (fabsf(m) > kLargeLogit) {
-        // (entries masked with a large negative number, sixteen of them together)
+    if (!(fabsf(m) <= kLargeLogit)) {
+        if (m == -CUDART_INF_F) {
+            // nothing above -inf yet: the values add up to -inf, or to NaN if there is one
+            const float t = (((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w))) + (((c.x + c.y) + (c.z + c.w)) + ((d.x + d.y) + (d.z + d.w)));
+            if (t != t) r.s = t;
+            return;
+        }
+        // entries masked with a large negative number, sixteen of them together
         a = minus(a, m); b = minus(b, m); c = minus(c, m); d = minus(d, m);
         ref = 0.f;
     }

@@ -435,19 +435,17 @@ __global__ void __launch_bounds__(kThreads, 4) draft_expand_kernel(DraftArgs a) 
                 g = fmaxf(g, g4);
                 offer_group(best, g4, i + k * kThreads);
             }
-            if (g == -CUDART_INF_F) {
-                // nothing finite yet: a NaN would otherwise go unnoticed (below it poisons the sum)
-#pragma unroll
-                for (int k = 0; k < kBatch; ++k) {
-                    const float q[4] = {r[k].x, r[k].y, r[k].z, r[k].w};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (q[j] != q[j]) s = q[j];
-                }
-                return;
-            }
             float ref = g;
-            if (fabsf(g) > kLargeLogit) {
+            if (!(fabsf(g) <= kLargeLogit)) {
+                if (g == -CUDART_INF_F) {
+                    // nothing finite yet: a NaN would otherwise go unnoticed (below it poisons the sum)
+#pragma unroll
+                    for (int k = 0; k < kBatch; ++k) {
+                        const float t = (r[k].x + r[k].y) + (r[k].z + r[k].w);
+                        if (t != t) s = t;
+                    }
+                    return;
+                }
 #pragma unroll
                 for (int k = 0; k < kBatch; ++k) r[k] = minus(r[k], g);
                 ref = 0.f;
