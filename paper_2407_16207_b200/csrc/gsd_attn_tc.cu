@@ -754,8 +754,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         // Units with one row tile, where loads are the bound: K copies run one tile ahead of the V
         // copies.  K t + 1 only waits for the QK^T of tile t - 1, and its time to land passes while V t
         // waits for the PV of tile t - 2 (4 x 40 heads, N 128, L 1024-4096: 58.4 us in step with the
-        // V copies, 55.4 one ahead).  Units with two keep the copies in step: the tensor pipe is the
-        // bound there and running ahead costs 1% (32 x 64/8 heads, L 8192, N 512).
+        // V copies, 55.4 one ahead).  Units with two keep the copies in step, in a loop of
+        // their own: the tensor pipe is the bound there, and the choice between the two kinds of copy at
+        // every step cost 2% of the cycles of the key loop (32 x 64/8 heads, N 128, L 8192: 1566 -> 1539
+        // thousand; 8 x 64/8, N 512, L 2048: 494 -> 485).
         int kc = pre, vc = pre;         // K and V tiles loaded so far (ring positions)
         int au = 0;                     // non-empty units so far
         bool ok = true, q_pending = pre > 0;
@@ -773,17 +775,28 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     }
                 }
                 int kn = begun ? pre : 0, vn = kn;      // next tile of the unit
-                while (ok && vn < u.ntiles) {
-                    if (kn < u.ntiles && kn <= vn + (u.two ? 0 : 1)) {
+                if (u.two) {
+                    for (; vn < u.ntiles && ok; ++vn) {
                         if (!(ok = mbar_wait(bar(BAR_K_EMPTY + kc % ST), (uint32_t)((kc / ST) & 1) ^ 1u, abort_flag, p.status))) break;
-                        load_k(u, kn, kc);
-                        ++kn;
+                        load_k(u, vn, kc);
                         ++kc;
-                    } else {
                         if (!(ok = mbar_wait(bar(BAR_V_EMPTY + vc % ST), (uint32_t)((vc / ST) & 1) ^ 1u, abort_flag, p.status))) break;
                         load_v(u, vn, vc);
-                        ++vn;
                         ++vc;
+                    }
+                } else {
+                    while (ok && vn < u.ntiles) {
+                        if (kn < u.ntiles && kn <= vn + 1) {
+                            if (!(ok = mbar_wait(bar(BAR_K_EMPTY + kc % ST), (uint32_t)((kc / ST) & 1) ^ 1u, abort_flag, p.status))) break;
+                            load_k(u, kn, kc);
+                            ++kn;
+                            ++kc;
+                        } else {
+                            if (!(ok = mbar_wait(bar(BAR_V_EMPTY + vc % ST), (uint32_t)((vc / ST) & 1) ^ 1u, abort_flag, p.status))) break;
+                            load_v(u, vn, vc);
+                            ++vn;
+                            ++vc;
+                        }
                     }
                 }
                 if (!ok) {
