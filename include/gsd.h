@@ -193,7 +193,9 @@ int gsd_verify_attn_num_splits(const gsd_attn_params* p);
  *   accepted_len    [B] int32 device out
  *   accepted_nodes  [B, Tcap] int32 device out or NULL: v0..vm then -1 padding
  *   p               host
- *   workspace       device scratch >= gsd_accept_workspace_bytes(p), 8-byte aligned
+ *   workspace       device scratch of gsd_accept_workspace_bytes(p) bytes, 8-byte aligned, arbitrary
+ *                   contents.  8 bytes per node and 4 per sequence, rounded up to 256, are accepted too;
+ *                   few rows are then cut into fewer slices, which takes longer
  *   status          device int32 word or NULL
  *   stream          cudaStream_t
  *
@@ -313,8 +315,7 @@ int gsd_draft_expand(const float* logits, const int32_t* frontier, const int32_t
  * whose host application has already claimed the GPU's memory for its own pool, a caller
  * that is handed tensors by another runtime and has no allocator of its own, or code on a
  * latency-critical path where cudaMalloc (which may synchronise the whole device) is off
- * limits.  For them the scratch that gsd_accept needs (8 bytes per draft node + 4 bytes per
- * sequence) lives in a fixed array inside the library image, GSD_STATIC_SCRATCH_BYTES long;
+ * limits.  For them the scratch that gsd_accept needs lives in a fixed array inside the library image, GSD_STATIC_SCRATCH_BYTES long;
  * every GPU on which the library is used holds that array until the process exits.
  *
  * Same arguments, results, status bits and error codes as gsd_accept, minus workspace and
@@ -324,8 +325,7 @@ int gsd_draft_expand(const float* logits, const int32_t* frontier, const int32_t
  *
  * The first call on each device looks up the array's device address (the device must be
  * current, as for every call here); make that first call outside any stream capture.
- * All calls on a device share the one array: it keeps whatever the last call left in it, the
- * part a call uses is cleared on `stream` before its kernel touches it, and two calls that can
+ * All calls on a device share the one array: it keeps whatever the last call left in it, and two calls that can
  * overlap on the GPU (different streams, no dependency) race on it - serialise them.
  */
 #define GSD_STATIC_MAX_ROWS 16384

@@ -2,20 +2,22 @@
 // accepted root path through the draft DAG (Sec. 3 deterministic verification and the
 // rejection cascade; Sec. 4.1 longest-path selection).
 //
-// One launch.  Grid (splits, B*N): each CTA streams one slice of one logits row with
-// 16-byte loads and reduces (value, index) pairs; slices of a row meet in a packed 64-bit
-// atomicMax.  The CTA that finishes last for a sequence runs the path pass for it
-// (gsd_path.cuh: level-synchronous relaxation of best[v] = 1 + max over accepted parents,
-// selection of the end node, backtracking, emission).
+// Two launches.  Grid (splits, B*N): each CTA streams one slice of one logits row with 16-byte
+// loads, reduces (value, index) pairs and leaves the best as a packed 64-bit key in scratch.  The
+// second launch (one CTA per sequence, a programmatic dependent of the first) fetches the graph
+// beside the stream, takes the best key of every node and runs the path pass (gsd_path.cuh).
 #include "gsd_internal.cuh"
 #include "gsd_path.cuh"
 #include <math_constants.h>
+#include <algorithm>
 
 namespace gsd {
 namespace {
 
 constexpr int kThreads = kPathThreads;
 constexpr int kNone = 0x7FFFFFFF;
+constexpr int kMaxSplits = 32;          // slices of a row
+constexpr int kWantCtas = 148 * 32;     // four waves of eight CTAs per SM
 
 struct Best {
     float v;
@@ -84,46 +86,15 @@ struct AcceptArgs {
     int32_t* out_tok;
     int32_t* out_len;
     int32_t* out_nodes;
-    unsigned long long* keys;  // [B*N], zeroed before the launch
-    unsigned* done;            // [B], zeroed before the launch
+    unsigned long long* keys;  // [splits][B*N]
     int32_t* status;
     int B, N, V, Ecap, Tcap, splits;
 };
 
-__device__ void path_pass(const AcceptArgs& a, int b) {
-    __shared__ int s_amax[GSD_MAX_NODES];
-    const int N = a.N, tid = threadIdx.x;
-    // the keys were written by other CTAs: read them past L1.  (No barrier of its own: the path
-    // routine fetches the graph first and meets at a barrier before any step is tested, so the
-    // two trips to memory overlap.)
-    for (int v = tid; v < N; v += kThreads) s_amax[v] = key_index(__ldcg(a.keys + (size_t)b * N + v));
-    const int32_t* tok = a.tok + (size_t)b * N;
-    PathIo io;
-    io.tok = tok;
-    io.pptr = a.pptr + (size_t)b * (N + 1);
-    io.pidx = a.pidx + (size_t)b * a.Ecap;
-    io.out_tok = a.out_tok + (size_t)b * a.Tcap;
-    io.out_nodes = a.out_nodes ? a.out_nodes + (size_t)b * a.Tcap : nullptr;
-    io.out_len = a.out_len + b;
-    io.status = a.status;
-    io.N = N; io.V = a.V; io.Ecap = a.Ecap; io.Tcap = a.Tcap;
-    // a step parent -> v is accepted iff v's token is what the target model would emit after the parent
-    const PathResult res = longest_accepted_path<false>(io, 0u, [&](int p, int v) { return tok[v] == s_amax[p]; });
-    // the target model's own next token
-    if (tid == 0 && res.edges < a.Tcap && GSD_IN_BOUNDS(res.end >= 0 && res.end < N && res.edges >= 0, a.status))
-        io.out_tok[res.edges] = s_amax[res.end];
-}
-
-// Zeroes scratch words.  The kernel that uses them is launched as a programmatic dependent: it
-// may start streaming its input at once and only waits for these zeros before its first atomic.
-__global__ void clear_words_kernel(unsigned* words, int n) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) words[i] = 0u;
-}
-
 __global__ void __launch_bounds__(kThreads) accept_kernel(AcceptArgs a) {
     __shared__ Best sh[kThreads / 32];
-    __shared__ int s_last;
+    // the second launch may become resident as CTAs retire
+    if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int row = blockIdx.y;  // b * N + n
     const int split = blockIdx.x;
     const float* x = a.logits + (size_t)row * a.V;
@@ -169,37 +140,66 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(AcceptArgs a) {
         best.i = f.i;
         best.v = -CUDART_INF_F;
     }
-    if (threadIdx.x == 0) {
-        // the scratch is zeroed by the launch before this one; everything above ran beside it
+    if (threadIdx.x == 0 && GSD_IN_BOUNDS(row < a.B * a.N && (best.i == kNone || (best.i >= 0 && best.i < a.V)), a.status))
+        a.keys[(size_t)split * a.B * a.N + row] = best.i == kNone ? 0ull : pack_key(best.v, best.i);
+}
+
+// Second launch: the best key of every node, then the path.
+__global__ void __launch_bounds__(kThreads) accept_tail_kernel(AcceptArgs a) {
+    __shared__ int s_amax[GSD_MAX_NODES];
+    const int N = a.N, b = blockIdx.x, tid = threadIdx.x;
+    PathIo io;
+    io.tok = a.tok + (size_t)b * N;
+    io.pptr = a.pptr + (size_t)b * (N + 1);
+    io.pidx = a.pidx + (size_t)b * a.Ecap;
+    io.out_tok = a.out_tok + (size_t)b * a.Tcap;
+    io.out_nodes = a.out_nodes ? a.out_nodes + (size_t)b * a.Tcap : nullptr;
+    io.out_len = a.out_len + b;
+    io.status = a.status;
+    io.N = N; io.V = a.V; io.Ecap = a.Ecap; io.Tcap = a.Tcap;
+    // the keys of a thread's nodes: neighbouring threads read neighbouring keys
+    auto best_keys = [&]() -> unsigned {
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        if (best.i != kNone && GSD_IN_BOUNDS(row < a.B * a.N && best.i >= 0 && best.i < a.V, a.status))
-            atomicMax(a.keys + row, pack_key(best.v, best.i));
-        __threadfence();
-        const int b = row / a.N;
-        const unsigned prev = atomicAdd(a.done + b, 1u);
-        s_last = (prev == (unsigned)(a.N * a.splits) - 1u);
-    }
-    __syncthreads();
-    if (s_last) {
-        __threadfence();
-        path_pass(a, row / a.N);
-    }
+        constexpr int kTrip = 8;                          // slices whose keys are on their way at a time
+        const size_t rows = (size_t)a.B * N;
+        const unsigned long long* keys = a.keys + (size_t)b * N + tid;
+        unsigned long long best[kPathNodeSlots] = {};
+        for (int s0 = 0; s0 < a.splits; s0 += kTrip) {
+            unsigned long long k[kPathNodeSlots][kTrip];
+#pragma unroll
+            for (int j = 0; j < kTrip; ++j)
+#pragma unroll
+                for (int i = 0; i < kPathNodeSlots; ++i)
+                    k[i][j] = s0 + j < a.splits && tid + i * kThreads < N ? __ldcg(keys + (s0 + j) * rows + i * kThreads) : 0ull;
+#pragma unroll
+            for (int j = 0; j < kTrip; ++j)
+#pragma unroll
+                for (int i = 0; i < kPathNodeSlots; ++i) best[i] = max(best[i], k[i][j]);
+        }
+#pragma unroll
+        for (int i = 0; i < kPathNodeSlots; ++i)
+            if (tid + i * kThreads < N) s_amax[tid + i * kThreads] = key_index(best[i]);
+        return 0u;
+    };
+    // a step parent -> v is accepted iff v's token is what the target model would emit after the parent
+    const PathResult res = longest_accepted_path_ex<false>(
+        io, 0u, [&](float, int p, int, int t) { return t == s_amax[p]; }, [](int, int) { return 0.f; }, best_keys);
+    // the target model's own next token
+    if (tid == 0 && res.edges < a.Tcap && GSD_IN_BOUNDS(res.end >= 0 && res.end < N && res.edges >= 0, a.status))
+        io.out_tok[res.edges] = s_amax[res.end];
 }
 
 }  // namespace
-
-int launch_clear_words(unsigned* words, int n, cudaStream_t stream) {
-    const int blocks = (n + 1023) / 1024;
-    clear_words_kernel<<<blocks < 64 ? blocks : 64, 256, 0, stream>>>(words, n);
-    GSD_CUDA_TRY(cudaGetLastError());
-    return GSD_OK;
-}
 
 }  // namespace gsd
 
 extern "C" size_t gsd_accept_workspace_bytes(const gsd_accept_params* p) {
     if (!p || p->B < 1 || p->N < 1 || p->N > GSD_MAX_NODES) return 0;
-    return gsd::align_up((size_t)p->B * p->N * 8 + (size_t)p->B * 4, 256);
+    // a key per slice: as many as the rule in gsd_accept can make of this many rows (the vocabulary may be
+    // given as anything here)
+    const size_t rows = (size_t)p->B * p->N;
+    const size_t keys = std::max(rows, std::min(rows * gsd::kMaxSplits, (size_t)2 * gsd::kWantCtas));
+    return std::max(gsd::accept_least_workspace(p->B, p->N), gsd::align_up(keys * 8, 256));
 }
 
 extern "C" int gsd_accept(const float* logits, const int32_t* draft_tokens,
@@ -215,34 +215,29 @@ extern "C" int gsd_accept(const float* logits, const int32_t* draft_tokens,
         return GSD_ERR_BAD_SHAPE;
     if ((long long)p->B * p->N > (1ll << 30)) return GSD_ERR_BAD_SHAPE;
     if (((uintptr_t)logits & 3u) != 0) return GSD_ERR_MISALIGNED;
-    const size_t need = gsd_accept_workspace_bytes(p);
+    // (a key per row is enough: the rows then go whole)
+    const size_t need = accept_least_workspace(p->B, p->N);
     if (!workspace || workspace_bytes < need) return GSD_ERR_WORKSPACE;
     if (((uintptr_t)workspace & 7u) != 0) return GSD_ERR_MISALIGNED;
-    DeviceInfo di;
-    if (device_info(&di) != 0) return GSD_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
 
     AcceptArgs a;
     a.logits = logits; a.tok = draft_tokens; a.pptr = parent_ptr; a.pidx = parent_idx;
     a.out_tok = accepted_tokens; a.out_len = accepted_len; a.out_nodes = accepted_nodes;
     a.keys = (unsigned long long*)workspace;
-    a.done = (unsigned*)((char*)workspace + (size_t)p->B * p->N * 8);
     a.status = status;
     a.B = p->B; a.N = p->N; a.V = p->V; a.Ecap = p->Ecap; a.Tcap = p->Tcap;
     // Slices of at least 4096 floats and CTAs for four waves (eight CTAs are resident per SM), so
     // that the last, partly filled wave is short: 2048 rows of 32000 take 50.7 us in one slice each
     // (1.7 waves), 48.0 in two, 46.6 in four.
-    const long rows = (long)p->B * p->N;
+    const size_t rows = (size_t)p->B * p->N;
     int splits = 1;
-    const long want = (long)di.sm_count * 32;
-    while (rows * splits < want && (p->V / (splits * 2)) >= 4096) splits *= 2;
+    while (rows * splits < kWantCtas && splits < kMaxSplits && p->V / (splits * 2) >= 4096 && rows * splits * 2 * 8 <= workspace_bytes) splits *= 2;
     a.splits = splits;
 
-    if (launch_clear_words((unsigned*)workspace, p->B * p->N * 2 + p->B, st) != GSD_OK) return GSD_ERR_CUDA;
     cudaLaunchAttribute attr[1];
     dependent_launch_attr(attr);
     // grid.y holds at most 65535 rows: larger problems go out in blocks of whole sequences
-    // so that the per-sequence completion counter still works
     const int seq_per = 65535 / p->N;
     for (int b0 = 0; b0 < p->B; b0 += seq_per) {
         const int nb = (p->B - b0 < seq_per) ? p->B - b0 : seq_per;
@@ -251,14 +246,16 @@ extern "C" int gsd_accept(const float* logits, const int32_t* draft_tokens,
         s.pptr += (size_t)b0 * (p->N + 1); s.pidx += (size_t)b0 * p->Ecap;
         s.out_tok += (size_t)b0 * p->Tcap; s.out_len += b0;
         if (s.out_nodes) s.out_nodes += (size_t)b0 * p->Tcap;
-        s.keys += (size_t)b0 * p->N; s.done += b0; s.B = nb;
+        s.keys += (size_t)b0 * p->N * splits; s.B = nb;
+        accept_kernel<<<dim3(splits, (unsigned)(nb * p->N)), kThreads, 0, st>>>(s);
+        GSD_CUDA_TRY(cudaGetLastError());
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(splits, (unsigned)(nb * p->N));
+        cfg.gridDim = dim3((unsigned)nb);
         cfg.blockDim = dim3(kThreads);
         cfg.stream = st;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_kernel, s));
+        GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_tail_kernel, s));
     }
     GSD_CUDA_TRY(cudaGetLastError());
     return GSD_OK;
@@ -303,7 +300,6 @@ extern "C" int gsd_accept_static(const float* logits, const int32_t* draft_token
         if (!ptr) return GSD_ERR_CUDA;
         if (dev >= 0 && dev < 64) addr[dev] = ptr;
     }
-    // gsd_accept clears the part of the scratch it uses before every launch
     return gsd_accept(logits, draft_tokens, parent_ptr, parent_idx, accepted_tokens, accepted_len,
                       accepted_nodes, p, ptr, (size_t)GSD_STATIC_SCRATCH_BYTES, status, stream);
 }

@@ -163,7 +163,6 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
     static_assert(kMaxCluster <= kMaxSlices, "one range sum per warp of the cluster");
     cluster_arrive();                    // (every CTA has started before any writes to another)
     const int N = a.N, V = a.V, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t* tok = a.tok + (size_t)b * N;
     const float* lg = a.logits + (size_t)b * N * V;
     const float* q = a.q + (size_t)b * N;
     const float* u = a.u + (size_t)b * N;
@@ -226,7 +225,7 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
     int32_t* out_tok = a.out_tok + (size_t)b * a.Tcap;
     if (rank == 0) {
         PathIo io;
-        io.tok = tok;
+        io.tok = a.tok + (size_t)b * N;
         io.pptr = a.pptr + (size_t)b * (N + 1);
         io.pidx = a.pidx + (size_t)b * a.Ecap;
         io.out_tok = out_tok;
@@ -238,10 +237,10 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
         // logit gathered from global memory) against u q
         const PathResult res = longest_accepted_path_ex<true>(
             io, 0u,
-            [&](float logit, int p, int v) { return s_uq[v] < ex2((logit - s_mx[p]) * kLog2e) / s_sum[p]; },
-            [&](int p, int v) -> float {
-                if (!GSD_IN_BOUNDS(p >= 0 && p < N && tok[v] >= 0 && tok[v] < V, a.status)) return -CUDART_INF_F;
-                return lg[(size_t)p * V + tok[v]];
+            [&](float logit, int p, int v, int) { return s_uq[v] < ex2((logit - s_mx[p]) * kLog2e) / s_sum[p]; },
+            [&](int p, int t) -> float {
+                if (!GSD_IN_BOUNDS(p >= 0 && p < N && t >= 0 && t < V, a.status)) return -CUDART_INF_F;
+                return lg[(size_t)p * V + t];
             },
             combine_pairs);
         if (tid == 0) s_outcome = Outcome{res.edges, res.end, res.end_has_child ? 1 : 0, s_mx[res.end], s_sum[res.end]};

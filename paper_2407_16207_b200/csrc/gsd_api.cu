@@ -270,7 +270,7 @@ bool arena_layout(const gsd_attn_params* ap, const gsd_accept_params* cp, ArenaL
     L->pidx = take(L->b_pidx); L->atok = take(L->b_acc); L->alen = take(L->b_len);
     L->anodes = take(L->b_acc); L->status = take(4);
     L->ws_attn = take(gsd_verify_attn_workspace_bytes(ap));
-    L->ws_acc = take(gsd_accept_workspace_bytes(cp));
+    L->ws_acc = take(accept_least_workspace(cp->B, cp->N));    // (the copies bound the step: a key per row is enough)
     L->total = off;
     return true;
 }
@@ -379,7 +379,7 @@ extern "C" int gsd_verify_step_host(const void* q, const void* k_cache, const vo
                     (const int32_t*)(base + L.pptr), (const int32_t*)(base + L.pidx),
                     (int32_t*)(base + L.atok), (int32_t*)(base + L.alen),
                     (int32_t*)(base + L.anodes), cp, base + L.ws_acc,
-                    gsd_accept_workspace_bytes(cp), (int32_t*)(base + L.status), stream);
+                    arena_bytes - L.ws_acc, (int32_t*)(base + L.status), stream);
     if (rc != GSD_OK) return rc;
     GSD_CUDA_TRY(cudaMemcpyAsync(accepted_tokens, base + L.atok, L.b_acc, cudaMemcpyDeviceToHost, st));
     GSD_CUDA_TRY(cudaMemcpyAsync(accepted_len, base + L.alen, L.b_len, cudaMemcpyDeviceToHost, st));

@@ -223,11 +223,12 @@ __device__ __forceinline__ RowSpan row_span(const float* x, int V) {
 constexpr float kLargeLogit = 1048576.f;
 __device__ __forceinline__ float4 minus(const float4& x, float m) { return make_float4(x.x - m, x.y - m, x.z - m, x.w - m); }
 
-// ---- scratch words that must start at zero ----
-// Enqueues a small kernel that zeroes `n` 32-bit words and lets the next launch on the stream
-// start beside it.  That next kernel has to be launched with the attribute set up by
-// dependent_launch_attr() and to execute griddepcontrol.wait before it first touches the words.
-int launch_clear_words(unsigned* words, int n, cudaStream_t stream);
+// The least scratch gsd_accept takes: a key per row (and four bytes per sequence, which it needed once).
+inline size_t accept_least_workspace(int B, int N) { return align_up((size_t)B * N * 8 + (size_t)B * 4, 256); }
+
+// ---- programmatic dependent launches ----
+// A kernel launched with this attribute may start while its predecessor on the stream still runs; it
+// executes griddepcontrol.wait before it first touches what that one (or anything before it) writes.
 inline void dependent_launch_attr(cudaLaunchAttribute* attr) {
     attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr->val.programmaticStreamSerializationAllowed = 1;

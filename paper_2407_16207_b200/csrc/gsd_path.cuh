@@ -1,23 +1,26 @@
 // Longest accepted root path through the draft DAG (Sec. 4.1 longest-path selection; Sec. 3
 // rejection cascade), shared by the deterministic and the non-deterministic verification.
 // One CTA of kPathThreads threads per sequence.  The caller supplies the test of one step
-// parent -> v; this file does the rest: parent lists on chip, level-synchronous relaxation of
-// best[v] = 1 + max over accepted steps into v, choice of the end node (longest, then lowest
-// index), walk back (lowest predecessor that carries length - 1), emission of the path's node
+// parent -> v; this file does the rest: parent lists on chip, the accepted steps, level-synchronous
+// relaxation of best[v] = 1 + max over accepted steps into v, choice of the end node (longest, then
+// lowest index), walk back (lowest predecessor that carries length - 1), emission of the path's node
 // ids and drafted tokens.  The token the target model contributes at the end is the caller's.
 //
-// The pass runs on one SM while the rest of the device may already be idle, so it is laid out
-// for few dependent trips to memory: tokens, row pointers and the parent indices are fetched in
-// one go; the relaxation costs one barrier per round (two copies of best[]); every node picks
-// its predecessor in parallel, after which the walk back is a pointer chase in shared memory
-// and the outputs are written by the whole block.
+// The pass runs on one SM while the rest of the device may already be idle, so it is laid out for
+// short chains: tokens, row pointers and the parent indices are fetched in one trip; a node belongs
+// to one thread, which tests the steps into it once and keeps the accepted ones, the first in a register
+// - most nodes have one or none - so that a round of the relaxation is a read of shared memory and
+// a barrier; every node picks its predecessor in parallel, after which the walk back is a pointer
+// chase in shared memory.  (Steps tested again in every round, with the parent lists walked in shared
+// memory: 3 sequences of N 507, the relaxation alone 4.3 us, now 1.3.  One warp doing the relaxation with votes
+// instead of barriers, the accepted steps in its registers: 1 to 2 us slower than eight warps, an
+// instruction of a lone warp takes as long as a barrier.)
 #pragma once
 #include "gsd_internal.cuh"
 
 namespace gsd {
 
 constexpr int kPathThreads = 256;
-constexpr int kPathNone = 0x7FFFFFFF;
 constexpr int kPathNodeSlots = (GSD_MAX_NODES + kPathThreads - 1) / kPathThreads;
 constexpr int kPathEdgeCache = 3 * GSD_MAX_NODES;   // parent edges of one sequence kept in shared memory
 static_assert(kPathEdgeCache % kPathThreads == 0, "the edge prefetch is dealt out in whole rounds");
@@ -36,32 +39,30 @@ struct PathIo {
 struct PathResult {
     int edges;           // m: the accepted path has m + 1 nodes
     int end;             // its last node
-    bool end_has_child;  // some node lists `end` as a parent (only filled in with kCacheOutcome)
+    bool end_has_child;  // some node lists `end` as a parent
 };
 
-// The test of a step p -> v comes in two halves: `edge_pre(p, v)` fetches what the test needs
-// from global memory (a float), `step_ok(pre, p, v)` decides.  With kCacheOutcome both are
-// called once per step when the parent lists fit the on-chip cache (one thread per step, all at
-// once - for tests that touch global memory); otherwise they are called again on every use (for
-// tests that cost a comparison).  Between the two halves the function calls `mid()` (all
-// threads; it returns status bits) and meets at a barrier: a caller whose decision needs results
-// of an earlier kernel waits for them there, AFTER the graph and the values of `edge_pre` have
-// been fetched.  `flags` carries status bits the caller has already found; the function adds its
-// own and publishes them.  All threads of the CTA must call it; all return the same result.
-// out_tok[edges] is left for the caller, entries past it are set to -1.
-template <bool kCacheOutcome, class StepOk, class EdgePre, class Mid>
+// The test of a step p -> v comes in two halves: `edge_pre(p, t)` fetches what the test needs from
+// global memory (a float; t is v's token), `step_ok(pre, p, v, t)` decides.  With kFetch the first is
+// called for all steps of a node at once and what it returned is kept on chip.  Between the two
+// halves the function calls `mid()` (all threads; it returns status bits) and meets at a barrier: a
+// caller whose decision needs results of an earlier kernel waits for them there, AFTER the graph
+// and the values of `edge_pre` have been fetched.  `flags` carries status bits the caller has already
+// found; the function adds its own and publishes them.  All threads of the CTA must call it; all
+// return the same result.  out_tok[edges] is left for the caller, entries past it are set to -1.
+//
+template <bool kFetch, class StepOk, class EdgePre, class Mid>
 __device__ PathResult longest_accepted_path_ex(const PathIo& io, unsigned flags, StepOk step_ok, EdgePre edge_pre, Mid mid) {
-    __shared__ int s_best[2][GSD_MAX_NODES];      // two copies: a round reads one and writes the other
+    __shared__ int s_best[GSD_MAX_NODES];         // edges of the longest accepted root path, -1: none
     __shared__ int s_tok[GSD_MAX_NODES];
     __shared__ int s_ptr[GSD_MAX_NODES + 1];
     __shared__ int s_edge[kPathEdgeCache];
-    __shared__ unsigned char s_eok[kPathEdgeCache];
-    __shared__ float s_eval[kCacheOutcome ? kPathEdgeCache : 1];   // what edge_pre fetched for each step
-    __shared__ short s_enode[kPathEdgeCache];   // the node a step leads into
-    __shared__ short s_path[GSD_MAX_NODES];     // the chosen path, root first
+    __shared__ float s_pre[kFetch ? kPathEdgeCache : 1];   // what edge_pre fetched for each step
+    __shared__ short s_pred[GSD_MAX_NODES];       // a node's predecessor on its best path
+    __shared__ short s_path[GSD_MAX_NODES];       // the chosen path, root first
+    __shared__ unsigned char s_child[GSD_MAX_NODES];   // the node is some node's parent
     __shared__ int s_red[kPathThreads / 32];
     __shared__ unsigned s_flags;
-    __shared__ int s_m, s_end;
     const int N = io.N, tid = threadIdx.x;
     if (tid == 0) s_flags = 0;
     // tokens, row pointers and (speculatively: the row holds Ecap entries whatever the pointers
@@ -83,7 +84,8 @@ __device__ PathResult longest_accepted_path_ex(const PathIo& io, unsigned flags,
         if (v < N) {
             s_tok[v] = r_tok[k];
             if (r_tok[k] < 0 || r_tok[k] >= io.V) flags |= GSD_DEV_BAD_TOKEN;
-            s_best[0][v] = v == 0 ? 0 : -1;
+            s_best[v] = v == 0 ? 0 : -1;
+            s_child[v] = 0;
         }
     }
 #pragma unroll
@@ -122,110 +124,128 @@ __device__ PathResult longest_accepted_path_ex(const PathIo& io, unsigned flags,
             __syncthreads();
         }
     }
-    // the relaxation rounds walk the parent lists again and again: keep them, and the outcome
-    // of every step, on chip
-    const int n_edges = s_ptr[N];
-    const bool cached = n_edges <= kPathEdgeCache;
-    if (cached && kCacheOutcome) {
-        for (int v = tid; v < N; v += kPathThreads)
-            for (int e = s_ptr[v]; e < s_ptr[v + 1]; ++e) s_enode[e] = (short)v;
-        __syncthreads();
-        for (int e = tid; e < n_edges; e += kPathThreads) {
-            const int p = s_edge[e], v = s_enode[e];
-            s_eval[e] = (p >= 0 && p < v && s_tok[v] >= 0 && s_tok[v] < io.V) ? edge_pre(p, v) : 0.f;
+    // Lists that do not fit on chip stay where they are: their steps are tested again on every use.
+    const bool cached = s_ptr[N] <= kPathEdgeCache;
+    auto parent_at = [&](int e) -> int { return cached ? s_edge[e] : io.pidx[e]; };
+    auto token_ok = [&](int t) -> bool { return t >= 0 && t < io.V; };
+    if (kFetch && cached) {
+        // (four steps of a node at a time)
+        for (int v = tid; v < N; v += kPathThreads) {
+            const int e1 = s_ptr[v + 1], t = s_tok[v];
+            for (int e = s_ptr[v]; e < e1; e += 4) {
+                float got[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int p = e + k < e1 ? s_edge[e + k] : -1;
+                    got[k] = p >= 0 && p < v && token_ok(t) ? edge_pre(p, t) : 0.f;
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (e + k < e1) s_pre[e + k] = got[k];
+            }
         }
     }
     flags |= mid();
     __syncthreads();
-    if (cached && kCacheOutcome) {
-        for (int e = tid; e < n_edges; e += kPathThreads) {
-            const int p = s_edge[e], v = s_enode[e];
-            s_eok[e] = (p >= 0 && p < v && s_tok[v] >= 0 && s_tok[v] < io.V) ? (unsigned char)step_ok(s_eval[e], p, v) : 0;
+    // The accepted steps.  A node's thread writes its accepted parents over the front of its parent list.
+    auto accepted = [&](int e, int p, int v, int t) -> bool {
+        return token_ok(t) && step_ok(!kFetch ? 0.f : cached ? s_pre[e] : edge_pre(p, t), p, v, t);
+    };
+    int n_acc[kPathNodeSlots], first[kPathNodeSlots];      // of the thread's nodes: accepted parents, the first of them
+#pragma unroll
+    for (int k = 0; k < kPathNodeSlots; ++k) {
+        const int v = tid + k * kPathThreads;
+        n_acc[k] = 0;
+        first[k] = 0;
+        if (v < 1 || v >= N) continue;
+        const int e0 = s_ptr[v], e1 = s_ptr[v + 1], t = s_tok[v];
+        for (int e = e0; e < e1; ++e) {
+            const int p = parent_at(e);
+            if (p < 0 || p >= v) {
+                flags |= GSD_DEV_BAD_CSR;
+                continue;
+            }
+            s_child[p] = 1;
+            if (!accepted(e, p, v, t)) continue;
+            if (n_acc[k] == 0) first[k] = p;
+            if (cached) s_edge[e0 + n_acc[k]] = p;
+            ++n_acc[k];
         }
-        __syncthreads();
     }
-    auto parent_at = [&](int e) -> int { return cached ? s_edge[e] : io.pidx[e]; };
-    auto ok_at = [&](int e, int p, int v) -> bool {
-        if (cached && kCacheOutcome) return s_eok[e] != 0;
-        return s_tok[v] >= 0 && s_tok[v] < io.V && step_ok(edge_pre(p, v), p, v);
+    // calls f(p) for every accepted parent of the thread's k-th node
+    auto each_accepted = [&](int k, auto f) {
+        if (n_acc[k] > 0) f(first[k]);
+        if (n_acc[k] > 1) {
+            const int v = tid + k * kPathThreads, e0 = s_ptr[v];
+            if (cached) {
+                for (int e = e0 + 1; e < e0 + n_acc[k]; ++e) f(s_edge[e]);
+            } else {
+                for (int e = e0; e < s_ptr[v + 1]; ++e) {
+                    const int p = io.pidx[e];
+                    if (p >= 0 && p < v && accepted(e, p, v, s_tok[v])) f(p);
+                }
+            }
+        }
     };
 
-    // level-synchronous relaxation: after round r every node whose longest accepted root
-    // path has <= r edges is final; values only grow, so it stops when nothing changed
-    int cur_buf = 0;
+    // Level-synchronous relaxation: after round r every node whose longest accepted root path has at
+    // most r edges is final.  Values only grow, so a node may be met before or after its parent's update of
+    // the round, and it stops when nothing changed.
+    volatile int* best = s_best;
+    int mine[kPathNodeSlots];
+#pragma unroll
+    for (int k = 0; k < kPathNodeSlots; ++k) mine[k] = tid + k * kPathThreads == 0 ? 0 : -1;
     for (int round = 0; round < N; ++round) {
-        const int* rd = s_best[cur_buf];
-        int* wr = s_best[cur_buf ^ 1];
         int changed = 0;
 #pragma unroll
         for (int k = 0; k < kPathNodeSlots; ++k) {
-            const int v = tid + k * kPathThreads;
-            if (v < N) {
-                int cur = rd[v];
-                if (v > 0) {
-                    for (int e = s_ptr[v]; e < s_ptr[v + 1]; ++e) {
-                        const int p = parent_at(e);
-                        if (p < 0 || p >= v) {
-                            flags |= GSD_DEV_BAD_CSR;
-                            continue;
-                        }
-                        const int bp = rd[p];
-                        if (bp >= 0 && bp + 1 > cur && ok_at(e, p, v)) cur = bp + 1;
-                    }
-                }
-                wr[v] = cur;
-                changed |= (cur != rd[v]);
+            int to = mine[k];
+            each_accepted(k, [&](int p) {
+                const int bp = best[p];
+                if (bp >= 0) to = max(to, bp + 1);
+            });
+            if (to != mine[k]) {
+                mine[k] = to;
+                best[tid + k * kPathThreads] = to;
+                changed = 1;
             }
         }
-        cur_buf ^= 1;
         if (!__syncthreads_or(changed)) break;
     }
-    const int* best = s_best[cur_buf];
-    int* pred = s_best[cur_buf ^ 1];   // the other copy now takes every node's predecessor on its best path
-    __syncthreads();                   // (every thread has left the last round's reads of it)
 
-    // every node: the lowest predecessor with an accepted step that carries length - 1
+    // every node's predecessor: the lowest one with an accepted step that carries length - 1; and the end
+    // node: longest, then lowest index
     int key = -1;
-    for (int v = tid; v < N; v += kPathThreads) {
-        const int bv = best[v];
-        int pr = kPathNone;
-        if (v > 0 && bv > 0) {
-            for (int e = s_ptr[v]; e < s_ptr[v + 1]; ++e) {
-                const int p = parent_at(e);
-                if (p < 0 || p >= v) continue;
-                if (best[p] == bv - 1 && p < pr && ok_at(e, p, v)) pr = p;
-            }
-        }
-        pred[v] = pr;
-        // end node: longest, then lowest index
-        if (bv >= 0) key = max(key, (bv << 10) | (1023 - v));
-    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xFFFFFFFFu, key, o));
+    for (int k = 0; k < kPathNodeSlots; ++k) {
+        const int v = tid + k * kPathThreads;
+        if (mine[k] < 0) continue;
+        int pred = N;
+        each_accepted(k, [&](int p) {
+            if (p < pred && best[p] == mine[k] - 1) pred = p;
+        });
+        s_pred[v] = (short)(pred == N ? 0 : pred);
+        key = max(key, (mine[k] << 10) | (1023 - v));
+    }
+    key = __reduce_max_sync(0xFFFFFFFFu, key);
     if ((tid & 31) == 0) s_red[tid >> 5] = key;
     if (flags) atomicOr(&s_flags, flags);
     __syncthreads();
-
+#pragma unroll
+    for (int w = 0; w < kPathThreads / 32; ++w) key = max(key, s_red[w]);
+    const int m = key >> 10, end = 1023 - (key & 1023);
     if (tid == 0) {
-        for (int w = 1; w < kPathThreads / 32; ++w) key = max(key, s_red[w]);
-        const int m = key >> 10;
-        int v = 1023 - (key & 1023);
-        s_end = v;
         unsigned fl = s_flags;
         if (m + 1 > io.Tcap) fl |= GSD_DEV_TCAP;
-        // walk back along the predecessors (cannot break off for a consistent best[])
-        for (int len = m; len >= 0; --len) {
-            s_path[len] = (short)v;
-            if (len == 0) break;
-            const int pr = pred[v];
-            v = pr == kPathNone ? 0 : pr;
+        int v = end;
+        for (int l = m; l >= 0; --l) {
+            s_path[l] = (short)v;
+            v = s_pred[v];
         }
         *io.out_len = m + 1;
-        s_m = m;
         if (fl && io.status) atomicOr((unsigned*)io.status, fl);
     }
     __syncthreads();
-    const int m = s_m;
     for (int i = tid; i <= io.Tcap; i += kPathThreads) {
         if (i <= m) {
             const int node = s_path[i];
@@ -237,22 +257,14 @@ __device__ PathResult longest_accepted_path_ex(const PathIo& io, unsigned flags,
             if (io.out_nodes) io.out_nodes[i] = -1;
         }
     }
-    bool end_has_child = false;
-    if (kCacheOutcome) {
-        int has = 0;
-        const int end = s_end;
-        for (int v = end + 1 + tid; v < N; v += kPathThreads)
-            for (int e = s_ptr[v]; e < s_ptr[v + 1]; ++e) has |= (parent_at(e) == end);
-        end_has_child = __syncthreads_or(has) != 0;
-    }
-    return PathResult{s_m, s_end, end_has_child};
+    return PathResult{m, end, s_child[end] != 0};
 }
 
-// The plain form: a test `step_ok(p, v)` that needs nothing fetched and nothing waited for.
-template <bool kCacheOutcome, class StepOk>
+// The plain form: a test `step_ok(p, v, t)` that needs nothing fetched and nothing waited for.
+template <class StepOk>
 __device__ PathResult longest_accepted_path(const PathIo& io, unsigned flags, StepOk step_ok) {
-    return longest_accepted_path_ex<kCacheOutcome>(
-        io, flags, [&](float, int p, int v) { return step_ok(p, v); }, [](int, int) { return 0.f; }, []() { return 0u; });
+    return longest_accepted_path_ex<false>(
+        io, flags, [&](float, int p, int v, int t) { return step_ok(p, v, t); }, [](int, int) { return 0.f; }, []() { return 0u; });
 }
 
 }  // namespace gsd
