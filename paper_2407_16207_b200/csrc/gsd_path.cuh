@@ -151,34 +151,42 @@ __device__ PathResult longest_accepted_path_ex(const PathIo& io, unsigned flags,
     auto accepted = [&](int e, int p, int v, int t) -> bool {
         return token_ok(t) && step_ok(!kFetch ? 0.f : cached ? s_pre[e] : edge_pre(p, t), p, v, t);
     };
-    int n_acc[kPathNodeSlots], first[kPathNodeSlots];      // of the thread's nodes: accepted parents, the first of them
+    // Up to three of them sit in a register, ten bits each (fewer: some of them twice), -1 when there is none;
+    // with more the list is walked.
+    constexpr int kHeld = 3;
+    int held[kPathNodeSlots], n_acc[kPathNodeSlots];       // of the thread's nodes
+    bool many = false;
 #pragma unroll
     for (int k = 0; k < kPathNodeSlots; ++k) {
         const int v = tid + k * kPathThreads;
-        n_acc[k] = 0;
-        first[k] = 0;
-        if (v < 1 || v >= N) continue;
-        const int e0 = s_ptr[v], e1 = s_ptr[v + 1], t = s_tok[v];
-        for (int e = e0; e < e1; ++e) {
-            const int p = parent_at(e);
-            if (p < 0 || p >= v) {
-                flags |= GSD_DEV_BAD_CSR;
-                continue;
+        int n = 0, h = -1;
+        if (v > 0 && v < N) {
+            const int e0 = s_ptr[v], e1 = s_ptr[v + 1], t = s_tok[v];
+            for (int e = e0; e < e1; ++e) {
+                const int p = parent_at(e);
+                if ((unsigned)p >= (unsigned)v) {
+                    flags |= GSD_DEV_BAD_CSR;
+                    continue;
+                }
+                s_child[p] = 1;
+                if (!accepted(e, p, v, t)) continue;
+                if (n < kHeld) h = n == 0 ? p * 0x100401 : n == 1 ? (h & 1023) | p * 0x100400 : (h & 0xFFFFF) | p << 20;
+                if (cached) s_edge[e0 + n] = p;
+                ++n;
             }
-            s_child[p] = 1;
-            if (!accepted(e, p, v, t)) continue;
-            if (n_acc[k] == 0) first[k] = p;
-            if (cached) s_edge[e0 + n_acc[k]] = p;
-            ++n_acc[k];
         }
+        held[k] = h;
+        n_acc[k] = n;
+        many |= n > kHeld;
     }
-    // calls f(p) for every accepted parent of the thread's k-th node
+    // calls f(p) for every accepted parent of the thread's k-th node, of which there is one at least
     auto each_accepted = [&](int k, auto f) {
-        if (n_acc[k] > 0) f(first[k]);
-        if (n_acc[k] > 1) {
+#pragma unroll
+        for (int j = 0; j < kHeld; ++j) f(held[k] >> (10 * j) & 1023);
+        if (many && n_acc[k] > kHeld) {
             const int v = tid + k * kPathThreads, e0 = s_ptr[v];
             if (cached) {
-                for (int e = e0 + 1; e < e0 + n_acc[k]; ++e) f(s_edge[e]);
+                for (int e = e0 + kHeld; e < e0 + n_acc[k]; ++e) f(s_edge[e]);
             } else {
                 for (int e = e0; e < s_ptr[v + 1]; ++e) {
                     const int p = io.pidx[e];
@@ -199,14 +207,12 @@ __device__ PathResult longest_accepted_path_ex(const PathIo& io, unsigned flags,
         int changed = 0;
 #pragma unroll
         for (int k = 0; k < kPathNodeSlots; ++k) {
-            int to = mine[k];
-            each_accepted(k, [&](int p) {
-                const int bp = best[p];
-                if (bp >= 0) to = max(to, bp + 1);
-            });
-            if (to != mine[k]) {
-                mine[k] = to;
-                best[tid + k * kPathThreads] = to;
+            if (held[k] < 0) continue;
+            int from = -1;
+            each_accepted(k, [&](int p) { from = max(from, best[p]); });
+            if (from >= 0 && from + 1 > mine[k]) {
+                mine[k] = from + 1;
+                best[tid + k * kPathThreads] = mine[k];
                 changed = 1;
             }
         }
@@ -215,11 +221,11 @@ __device__ PathResult longest_accepted_path_ex(const PathIo& io, unsigned flags,
 
     // every node's predecessor: the lowest one with an accepted step that carries length - 1; and the end
     // node: longest, then lowest index
-    int key = -1;
+    int key = tid == 0 ? 1023 : -1;                        // (the root: length 0)
 #pragma unroll
     for (int k = 0; k < kPathNodeSlots; ++k) {
         const int v = tid + k * kPathThreads;
-        if (mine[k] < 0) continue;
+        if (mine[k] < 1) continue;
         int pred = N;
         each_accepted(k, [&](int p) {
             if (p < pred && best[p] == mine[k] - 1) pred = p;
@@ -238,10 +244,11 @@ __device__ PathResult longest_accepted_path_ex(const PathIo& io, unsigned flags,
         unsigned fl = s_flags;
         if (m + 1 > io.Tcap) fl |= GSD_DEV_TCAP;
         int v = end;
-        for (int l = m; l >= 0; --l) {
+        for (int l = m; l > 0; --l) {
             s_path[l] = (short)v;
             v = s_pred[v];
         }
+        s_path[0] = (short)v;
         *io.out_len = m + 1;
         if (fl && io.status) atomicOr((unsigned*)io.status, fl);
     }
