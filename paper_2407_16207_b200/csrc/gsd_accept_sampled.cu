@@ -16,8 +16,8 @@
 // the stream ends): the leading CTA combines the pairs per node, tests the steps, runs the
 // level-synchronous longest-path relaxation and walks back; then the regenerated token: range sums
 // (for P those in scratch; for the residual one per warp of the cluster, formed on the spot from
-// the two rows of the end node and exchanged through distributed shared memory) give the range of
-// the crossing, a block-wide scan over that range gives the index.
+// the two rows of the end node, which stay in registers, and exchanged through distributed shared memory) give the range of
+// the crossing, a scan over that range by its warp (or, when it was not kept, by a CTA) gives the index.
 #include "gsd_internal.cuh"
 #include "gsd_path.cuh"
 #include <math_constants.h>
@@ -48,6 +48,17 @@ __device__ __forceinline__ Ms combine(Ms a, Ms b) {
     const float m = fmaxf(a.m, b.m);
     if (m == -CUDART_INF_F) return Ms{m, a.s + b.s};
     return Ms{m, a.s * ex2((a.m - m) * kLog2e) + b.s * ex2((b.m - m) * kLog2e)};
+}
+
+// the pairs of a warp's lanes, all of them with the same result
+__device__ __forceinline__ Ms warp_combine(Ms r) {
+    float m = r.m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+    float s = m == -CUDART_INF_F ? r.s : r.s * ex2((r.m - m) * kLog2e);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+    return Ms{m, s};
 }
 
 // sixteen values at once: one rescale of the running sum per group
@@ -154,71 +165,87 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
     __shared__ float s_uq[GSD_MAX_NODES];
     __shared__ int s_red[kThreads / 32];
     __shared__ float s_scan[kThreads / 32];
-    __shared__ float s_rm[kThreads / 32];
-    __shared__ float s_cm[kMaxCluster], s_cs[kMaxCluster];
+    __shared__ float s_cm[kMaxCluster * kWarps], s_cs[kMaxCluster * kWarps];
     __shared__ float s_rsum[kMaxSlices * kWarps];
     __shared__ Outcome s_outcome;
     __shared__ int s_pick;
     const int C = a.cluster, rank = C > 1 ? cluster_rank() : 0;
+    static_assert(kPathNodeSlots == 2, "two nodes a thread at most");
     static_assert(kMaxCluster <= kMaxSlices, "one range sum per warp of the cluster");
     cluster_arrive();                    // (every CTA has started before any writes to another)
     const int N = a.N, V = a.V, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float* lg = a.logits + (size_t)b * N * V;
     const float* q = a.q + (size_t)b * N;
     const float* u = a.u + (size_t)b * N;
-    // Softmax statistics of every node from the pairs of the first launch, and the left sides
-    // of the step tests.  This is the first thing that needs the first launch's results: the path
+    const float u_draw = a.us[b];
+    float uq[kPathNodeSlots];            // the left sides of the step tests
+#pragma unroll
+    for (int k = 0; k < kPathNodeSlots; ++k) uq[k] = tid + k * kThreads < N ? u[tid + k * kThreads] * q[tid + k * kThreads] : 0.f;
+    // Softmax statistics of every node from the pairs of the first launch.  This is the first thing that needs the first launch's results: the path
     // routine calls it after the graph and one logit per step have been fetched, so those two
     // trips to memory are over when the first launch ends.
     auto combine_pairs = [&]() -> unsigned {
         unsigned flags = 0;
+#pragma unroll
+        for (int k = 0; k < kPathNodeSlots; ++k)
+            if (tid + k * kThreads < N) s_uq[tid + k * kThreads] = uq[k];
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        // a node's pairs are shared by up to four neighbouring threads when there are fewer nodes than
-        // threads: with few rows the rows are cut into many slices, and one thread per node had 128
-        // pairs to go through (2 sequences of N 40, V 128256: 3.7 us of the call)
-        const int tpn = 4 * N <= kThreads ? 4 : 2 * N <= kThreads ? 2 : 1;
+        // A node's pairs are shared by neighbouring threads when there are fewer nodes than threads (with few rows
+        // the rows are cut into many slices: 1 x 11 rows of 128256, 128 pairs a node, by at most four
+        // threads: 2.5 us); with more nodes than threads a thread goes through two of them at once.
+        int tpn = 1;
+        while (tpn < 2 * a.slices && 2 * tpn * N <= kThreads && tpn < 32) tpn *= 2;
         const int quads = a.slices * (kWarps / 2) / tpn;               // float4s (two pairs each) of one thread
         // (a workspace has to be on an 8-byte boundary only; 8-byte loads throughout took up to 1.3 us more:
         // 4 x 100 rows of 50257, 34.8 -> 36.1)
         const bool by16 = (reinterpret_cast<uintptr_t>(a.part) & 15u) == 0;
-        auto two_pairs = [&](const float4* at) -> float4 {
+        auto two_pairs = [&](const float4* at) -> float4 {             // (written by other CTAs: read past L1)
             if (by16) return __ldcg(at);
             const float2 lo = __ldcg(reinterpret_cast<const float2*>(at)), hi = __ldcg(reinterpret_cast<const float2*>(at) + 1);
             return make_float4(lo.x, lo.y, hi.x, hi.y);
         };
-        for (int t = tid; t < (N * tpn + 31) / 32 * 32; t += kThreads) {
-            const int v = min(t / tpn, N - 1);
-            // the pairs were written by other CTAs: read them past L1
-            Ms r{-CUDART_INF_F, 0.f};
-            const float4* pp = reinterpret_cast<const float4*>(a.part + ((size_t)b * N + v) * a.slices * kWarps) + (t % tpn) * quads;
-            for (int k = 0; k < quads; k += 4) {                       // eight pairs (64 bytes) per round, loaded at once
-                float4 p[4];
+        const float4* pairs = reinterpret_cast<const float4*>(a.part + (size_t)b * N * a.slices * kWarps) + tid * quads;
+        const bool two = N > kThreads + tid;                           // (a second node: tpn is 1 then)
+        Ms r[2] = {{-CUDART_INF_F, 0.f}, {-CUDART_INF_F, 0.f}};
+        if (tid < N * tpn) {
+            for (int k = 0; k < quads; k += 4) {                       // eight pairs (64 bytes) a round and node
+                float4 p[2][4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) p[i] = k + i < quads ? two_pairs(pp + k + i) : make_float4(-CUDART_INF_F, 0.f, -CUDART_INF_F, 0.f);
-                float m = r.m;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) m = fmaxf(m, fmaxf(p[i].x, p[i].z));
-                if (m == -CUDART_INF_F) {                              // (sums of 0 or NaN)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) r.s += p[i].y + p[i].w;
-                    continue;
+                for (int i = 0; i < 4; ++i) {
+                    const float4 none = make_float4(-CUDART_INF_F, 0.f, -CUDART_INF_F, 0.f);
+                    p[0][i] = k + i < quads ? two_pairs(pairs + k + i) : none;
+                    p[1][i] = two && k + i < quads ? two_pairs(pairs + kThreads * quads + k + i) : none;
                 }
-                float s = r.s * ex2((r.m - m) * kLog2e);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) s += p[i].y * ex2((p[i].x - m) * kLog2e) + p[i].w * ex2((p[i].z - m) * kLog2e);
-                r = Ms{m, s};
+                for (int h = 0; h < 2; ++h) {
+                    float m = r[h].m;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) m = fmaxf(m, fmaxf(p[h][i].x, p[h][i].z));
+                    if (m == -CUDART_INF_F) {                          // (sums of 0 or NaN)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) r[h].s += p[h][i].y + p[h][i].w;
+                        continue;
+                    }
+                    float s = r[h].s * ex2((r[h].m - m) * kLog2e);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) s += p[h][i].y * ex2((p[h][i].x - m) * kLog2e) + p[h][i].w * ex2((p[h][i].z - m) * kLog2e);
+                    r[h] = Ms{m, s};
+                }
             }
-            for (int o = 1; o < tpn; o *= 2) {
-                Ms other;
-                other.m = __shfl_xor_sync(0xFFFFFFFFu, r.m, o);
-                other.s = __shfl_xor_sync(0xFFFFFFFFu, r.s, o);
-                r = combine(r, other);
-            }
-            if (t >= N * tpn || t % tpn != 0) continue;
-            s_mx[v] = r.m;
-            s_sum[v] = r.s;
-            s_uq[v] = u[v] * q[v];       // the left side of the step test, fetched beside the pairs
-            if (!(r.s > 0.f) || r.m == CUDART_INF_F) flags |= GSD_DEV_BAD_LOGITS;   // no finite entry, +inf or NaN
+        }
+        for (int o = 1; o < tpn; o *= 2) {
+            Ms other;
+            other.m = __shfl_xor_sync(0xFFFFFFFFu, r[0].m, o);
+            other.s = __shfl_xor_sync(0xFFFFFFFFu, r[0].s, o);
+            r[0] = combine(r[0], other);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int v = h == 0 ? tid / tpn : tid + kThreads;
+            if (v >= N || (h == 0 && tid % tpn != 0)) continue;
+            s_mx[v] = r[h].m;
+            s_sum[v] = r[h].s;
+            if (!(r[h].s > 0.f) || r[h].m == CUDART_INF_F) flags |= GSD_DEV_BAD_LOGITS;   // no finite entry, +inf or NaN
         }
         return flags;
     };
@@ -273,8 +300,16 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
     // with one CTA per sequence the two passes took 9 us at V 32000 and four times that at
     // 128256; eight CTAs make each pass one trip.  8 x 256 rows of 32000, whole call: 64.8 us with
     // one CTA per sequence, 61.9 with two, 59.2 with four, 59.7 with eight.
+    // A warp's part of the rows that fits its registers (up to 32768 entries a row on eight CTAs) is read once:
+    // the weights take the target row's place there, and the warp with the crossing finds the token
+    // itself.  8 x 256 rows of 32000, whole call: 56.5 us with both rows read again for the weights and for
+    // the token, 52.9 this way.
+    constexpr int kBatch = 4;            // groups a thread has in flight (eight made short rows 0.5 to 1 us slower: more code to fetch)
+    float4 xv[kBatch], yv[kBatch];
+    float w_head = 0.f, w_tail = 0.f;
+    bool kept = false;
     bool residual = false;
-    float q_m = 0.f, inv_sp = 0.f, inv_sq = 0.f, res_total = 0.f;
+    float q_m = 0.f, inv_sp = 0.f, inv_sq = 0.f;
     const float* y = nullptr;
     bool same = false;                   // both rows have their 16-byte groups at the same entries
     if (a.dlogits && s_outcome.end_has_child) {
@@ -284,77 +319,191 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
         // entries of the range outside its groups: before (first range) and behind (last range)
         const int e_head = g.lo + lane, e_tail = xs.head + g.a1 * 4 + lane;
         const bool in_head = e_head < xs.head, in_tail = e_tail < g.hi;
-        constexpr int kBatch = 4;        // groups a thread has in flight (eight made short rows 0.5 to 1 us slower: more code to fetch)
         const float4 none = make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
         auto group = [&](const float* row, bool vec, int i) { return i < g.a1 ? load4(row + xs.head + 4 * i, vec) : none; };
-        // softmax statistics of the draft row; the target's row is brought into L2 beside it
+        // Softmax statistics of the draft row.  The first batch of both rows stays in registers; of what is
+        // behind it the target's row is brought into L2.
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+            yv[k] = group(y, same, g.a0 + lane + k * 32);
+            xv[k] = group(x, true, g.a0 + lane + k * 32);
+        }
+        float hx = 0.f, hy = 0.f, tx = 0.f, ty = 0.f;
+        if (in_head) { hy = __ldg(y + e_head); hx = __ldg(x + e_head); }
+        if (in_tail) { ty = __ldg(y + e_tail); tx = __ldg(x + e_tail); }
         Ms r{-CUDART_INF_F, 0.f};
-        if (in_head) take1(r, __ldg(y + e_head));
-        if (in_tail) take1(r, __ldg(y + e_tail));
-        for (int i = g.a0 + lane; i < g.a1; i += kBatch * 32) {
+        if (in_head) take1(r, hy);
+        if (in_tail) take1(r, ty);
+        take16(r, yv[0], yv[1], yv[2], yv[3]);
+        for (int i = g.a0 + lane + kBatch * 32; i < g.a1; i += kBatch * 32) {
             float4 t[kBatch];
 #pragma unroll
             for (int k = 0; k < kBatch; ++k) t[k] = group(y, same, i + k * 32);
 #pragma unroll
             for (int k = 0; k < kBatch; ++k)
                 if (i + k * 32 < g.a1) asm volatile("prefetch.global.L2 [%0];" ::"l"(x + xs.head + 4 * (i + k * 32)));
-#pragma unroll
-            for (int k = 0; k < kBatch; k += 4) take16(r, t[k], t[k + 1], t[k + 2], t[k + 3]);
+            take16(r, t[0], t[1], t[2], t[3]);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            Ms t;
-            t.m = __shfl_xor_sync(0xFFFFFFFFu, r.m, o);
-            t.s = __shfl_xor_sync(0xFFFFFFFFu, r.s, o);
-            r = combine(r, t);
-        }
-        if (lane == 0) { s_rm[warp] = r.m; s_scan[warp] = r.s; }
-        __syncthreads();
-        if (tid < C) {
-            r = Ms{-CUDART_INF_F, 0.f};
-            for (int w = 0; w < kWarps; ++w) r = combine(r, Ms{s_rm[w], s_scan[w]});
-            put_remote(s_cm + rank, tid, __float_as_uint(r.m));
-            put_remote(s_cs + rank, tid, __float_as_uint(r.s));
+        r = warp_combine(r);
+        // every warp hands its pair to every CTA of the cluster, and every warp combines them all
+        if (lane < C) {
+            put_remote(s_cm + rank * kWarps + warp, lane, __float_as_uint(r.m));
+            put_remote(s_cs + rank * kWarps + warp, lane, __float_as_uint(r.s));
         }
         cluster_arrive();
+        // (the target's probabilities, while the pairs travel)
+        inv_sp = 1.f / p_sum;
+        auto p_of = [&](float v) { return ex2((v - mx) * kLog2e) * inv_sp; };
+        auto p_of4 = [&](const float4& v) { return make_float4(p_of(v.x), p_of(v.y), p_of(v.z), p_of(v.w)); };
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) xv[k] = p_of4(xv[k]);
+        if (in_head) hx = p_of(hx);
+        if (in_tail) tx = p_of(tx);
         cluster_wait();
         r = Ms{-CUDART_INF_F, 0.f};
-        for (int c = 0; c < C; ++c) r = combine(r, Ms{s_cm[c], s_cs[c]});
+        for (int w = lane; w < C * kWarps; w += 32) r = combine(r, Ms{s_cm[w], s_cs[w]});
+        r = warp_combine(r);
         if (!(r.s > 0.f) || r.m == CUDART_INF_F) {
             if (rank == 0 && tid == 0 && a.status) atomicOr((unsigned*)a.status, GSD_DEV_BAD_LOGITS);
         } else {
             q_m = r.m;
-            inv_sp = 1.f / p_sum;
             inv_sq = 1.f / r.s;
-            auto res1 = [&](float xv, float yv) -> float {
-                return fmaxf(ex2((xv - mx) * kLog2e) * inv_sp - ex2((yv - q_m) * kLog2e) * inv_sq, 0.f);
+            auto rest = [&](float p, float yv) { return fmaxf(p - ex2((yv - q_m) * kLog2e) * inv_sq, 0.f); };
+            if (in_head) w_head = rest(hx, hy);
+            if (in_tail) w_tail = rest(tx, ty);
+            float part = w_head;
+            auto weigh = [&](const float4& pv, const float4& yv) -> float4 {
+                const float4 w = make_float4(rest(pv.x, yv.x), rest(pv.y, yv.y), rest(pv.z, yv.z), rest(pv.w, yv.w));
+                part += (w.x + w.y) + (w.z + w.w);
+                return w;
             };
-            float part = 0.f;
-            if (in_head) part += res1(__ldg(x + e_head), __ldg(y + e_head));
-            for (int i = g.a0 + lane; i < g.a1; i += kBatch * 32) {
-                float4 xv[kBatch], yv[kBatch];
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k) xv[k] = weigh(xv[k], yv[k]);
+            for (int i = g.a0 + lane + kBatch * 32; i < g.a1; i += kBatch * 32) {
+                float4 xa[kBatch], ya[kBatch];
 #pragma unroll
                 for (int k = 0; k < kBatch; ++k) {
-                    xv[k] = group(x, true, i + k * 32);
-                    yv[k] = group(y, same, i + k * 32);
+                    xa[k] = group(x, true, i + k * 32);
+                    ya[k] = group(y, same, i + k * 32);
                 }
 #pragma unroll
-                for (int k = 0; k < kBatch; ++k)
-                    part += (res1(xv[k].x, yv[k].x) + res1(xv[k].y, yv[k].y)) + (res1(xv[k].z, yv[k].z) + res1(xv[k].w, yv[k].w));
+                for (int k = 0; k < kBatch; ++k) weigh(p_of4(xa[k]), ya[k]);
             }
-            if (in_tail) part += res1(__ldg(x + e_tail), __ldg(y + e_tail));
+            part += w_tail;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
             if (lane < C) put_remote(s_rsum + rank * kWarps + warp, lane, __float_as_uint(part));
             cluster_arrive();
             cluster_wait();
-            for (int w = 0; w < C * kWarps; ++w) res_total += s_rsum[w];
-            // a residual without mass (the two distributions agree to rounding) leaves P
-            residual = res_total > kResidualFloor;
-            __syncthreads();             // (P's range sums may take the place of the residual's)
+            kept = ((xs.nvec + C - 1) / C + kWarps - 1) / kWarps <= kBatch * 32;      // (the longest range of the cluster)
+            residual = true;             // (if it has any mass, see below)
         }
     }
-    if (!residual && rank != 0) return;  // (no CTA of the cluster touches another one's memory any more)
+    // The range of the crossing, found by every warp of the cluster with the same result: the first range whose
+    // inclusive prefix exceeds the target, or the last one with any mass if rounding leaves none.  Four
+    // range sums a lane (walked one by one by every thread it took 1.5 us).
+    static_assert(kMaxSlices * kWarps <= 128, "four range sums a lane");
+    int rsel = 0;
+    float before_range = 0.f, target = 0.f;
+    bool crossing = false;
+    auto find_range = [&](int nr, auto target_of) -> bool {
+        float w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = 4 * lane + j < nr ? s_rsum[4 * lane + j] : 0.f;
+        float inc = (w[0] + w[1]) + (w[2] + w[3]);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+            if (lane >= o) inc += t;
+        }
+        const float total = __shfl_sync(0xFFFFFFFFu, inc, 31);
+        if (!target_of(total)) return false;
+        float c[5];                      // the cumulative axis at the ends of the lane's ranges
+        c[0] = __shfl_up_sync(0xFFFFFFFFu, inc, 1);
+        if (lane == 0) c[0] = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) c[j + 1] = c[j] + w[j];
+        const float end_before = __shfl_up_sync(0xFFFFFFFFu, c[4], 1);
+        if (lane > 0) c[0] = end_before;     // (a lane's first range begins where the one before it ends)
+        int at = kNone, last = kNone;
+        float c_at = 0.f, c_last = 0.f;
+#pragma unroll
+        for (int j = 3; j >= 0; --j) {
+            // (rounding can put the end of a range without mass past a target that nothing before it has reached)
+            if (w[j] > 0.f && c[j + 1] > target) { at = 4 * lane + j; c_at = c[j]; }
+            if (w[j] > 0.f && last == kNone) { last = 4 * lane + j; c_last = c[j]; }
+        }
+        const unsigned hit = __ballot_sync(0xFFFFFFFFu, at != kNone), mass = __ballot_sync(0xFFFFFFFFu, last != kNone);
+        crossing = hit != 0u;
+        if (hit | mass) {
+            const int from = crossing ? __ffs(hit) - 1 : 31 - __clz(mass);
+            rsel = __shfl_sync(0xFFFFFFFFu, crossing ? at : last, from);
+            before_range = __shfl_sync(0xFFFFFFFFu, crossing ? c_at : c_last, from);
+        }
+        return true;
+    };
+    if (residual)                        // a residual without mass (the two distributions agree to rounding) leaves P
+        residual = find_range(C * kWarps, [&](float total) { target = u_draw * total; return total > kResidualFloor; });
+    if (!residual) {
+        if (rank != 0) return;           // (no CTA of the cluster touches another one's memory any more)
+        const int nr = a.slices * kWarps;
+        __syncthreads();                 // (P's range sums take the place of the residual's)
+        if (tid < nr) {                  // one range sum per thread, brought to the row's maximum
+            const float2 t = __ldcg(a.part + ((size_t)b * N + s_end) * a.slices * kWarps + tid);
+            s_rsum[tid] = t.x == -CUDART_INF_F ? 0.f : t.y * ex2((t.x - mx) * kLog2e);
+        }
+        __syncthreads();
+        find_range(nr, [&](float) { target = u_draw * p_sum; return true; });
+    }
+    // the CTA that formed a residual range goes on with it (its part of the rows is close by)
+    if (residual && rank != rsel / kWarps) return;
+    if (residual && kept) {
+        // The weights of the range are in this warp's registers, in runs of 128 entries, four a lane.
+        if (warp != rsel % kWarps) return;
+        const Range g = range_of(xs, V, C, rsel);
+        float cum = before_range;
+        int pick = -1, last = -1;
+        bool open = crossing;            // the crossing is still ahead
+        auto run = [&](const float4& w4, int e) {                  // the lane's entries e .. e + 3 of a run
+            const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+            const float own = (w[0] + w[1]) + (w[2] + w[3]);
+            float in = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const float t = __shfl_up_sync(0xFFFFFFFFu, in, o);
+                if (lane >= o) in += t;
+            }
+            in += cum;
+            // (a lane's entries begin where those of the lane before end)
+            float c = __shfl_up_sync(0xFFFFFFFFu, in, 1);
+            if (lane == 0) c = cum;
+            cum = __shfl_sync(0xFFFFFFFFu, in, 31);
+            const unsigned hit = __ballot_sync(0xFFFFFFFFu, open && own > 0.f && in > target);
+            const int first = hit ? __ffs(hit) - 1 : 31;
+            if (open || !crossing) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    c += w[j];
+                    if (hit && lane == first && w[j] > 0.f && c > target) pick = pick < 0 ? e + j : pick;
+                    if (w[j] > 0.f && lane <= first) last = e + j;
+                }
+            }
+            open = open && !hit;
+        };
+        if (rsel == 0 && xs.head > 0) run(make_float4(w_head, 0.f, 0.f, 0.f), lane);
+#pragma unroll 1
+        for (int k = 0; k < kBatch; ++k) {
+            run(xv[0], xs.head + 4 * (g.a0 + lane + k * 32));
+#pragma unroll
+            for (int j = 0; j + 1 < kBatch; ++j) xv[j] = xv[j + 1];
+        }
+        if (rsel == C * kWarps - 1) run(make_float4(w_tail, 0.f, 0.f, 0.f), xs.head + g.a1 * 4 + lane);
+        pick = __reduce_max_sync(0xFFFFFFFFu, pick);
+        // rounding left no entry above the target: the last one with any mass up to there
+        if (pick < 0) pick = __reduce_max_sync(0xFFFFFFFFu, last);
+        if (lane == 0 && s_m < a.Tcap && GSD_IN_BOUNDS(s_m >= 0 && pick < V, a.status)) out_tok[s_m] = pick;
+        return;
+    }
     // weight of one entry from its two logits (-inf stands for "past the end": weight 0)
     auto weight = [&](float xv, float yv) -> float {
         const float e = ex2((xv - mx) * kLog2e);
@@ -374,30 +523,6 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
             for (int k = 0; k < 16; ++k) v[k] = j + k < jend ? row[j + k] : -CUDART_INF_F;
         }
     };
-    const float target = a.us[b] * (residual ? res_total : p_sum);
-    // every thread walks the range sums: the first range whose inclusive prefix exceeds the
-    // target, or the last one with any mass if rounding leaves none
-    int rsel = -1, last_r = 0;
-    float before_range = 0.f, before_last = 0.f;
-    {
-        const int nr = residual ? C * kWarps : a.slices * kWarps;
-        if (!residual && tid < nr) {          // one range sum per thread, brought to the row's maximum
-            const float2 t = __ldcg(a.part + ((size_t)b * N + s_end) * a.slices * kWarps + tid);
-            s_rsum[tid] = t.x == -CUDART_INF_F ? 0.f : t.y * ex2((t.x - mx) * kLog2e);
-        }
-        __syncthreads();
-        float run = 0.f;
-        for (int r = 0; r < nr; ++r) {
-            const float sr = s_rsum[r];
-            if (rsel < 0 && run + sr > target) { rsel = r; before_range = run; }
-            if (sr > 0.f) { last_r = r; before_last = run; }
-            run += sr;
-        }
-    }
-    const bool crossing = rsel >= 0;
-    if (!crossing) { rsel = last_r; before_range = before_last; }
-    // the CTA that formed a residual range goes on with it (its part of the rows is close by)
-    if (residual && rank != rsel / kWarps) return;
     if (tid == 0) s_pick = kNone;
     const Range rg = range_of(xs, V, residual ? C : a.slices, rsel);
     const int r0 = rg.lo, r1 = rg.hi;
@@ -435,7 +560,7 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
     // the target holds the crossing.
     float before = __shfl_up_sync(0xFFFFFFFFu, inc, 1);
     if (lane == 0) before = base;
-    if (crossing && inc > target) atomicMin(&s_pick, tid);
+    if (crossing && piece > 0.f && inc > target) atomicMin(&s_pick, tid);
     __syncthreads();
     const int first = s_pick;           // kNone: rounding left no crossing in this range
     __syncthreads();
@@ -448,8 +573,9 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
             if (residual) load16(y, c0, j1, yv);
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
-                cum += weight(xv[k], residual ? yv[k] : 0.f);
-                if (pick < 0 && cum > target) pick = c0 + k;
+                const float e = weight(xv[k], residual ? yv[k] : 0.f);
+                cum += e;
+                if (pick < 0 && e > 0.f && cum > target) pick = c0 + k;
             }
         }
         s_pick = pick;                  // -1: the serial sum stayed at or below the target
@@ -495,13 +621,7 @@ __global__ void __launch_bounds__(kThreads, 8) accept_sampled_kernel(SampledArgs
         }
         if (sp.head + g.a1 * 4 + lane < g.hi) take1(r, __ldcs(x + sp.head + g.a1 * 4 + lane));   // (last range only)
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        Ms t;
-        t.m = __shfl_xor_sync(0xFFFFFFFFu, r.m, o);
-        t.s = __shfl_xor_sync(0xFFFFFFFFu, r.s, o);
-        r = combine(r, t);
-    }
+    r = warp_combine(r);
     if (lane == 0) a.part[((size_t)row * a.slices + slice) * kWarps + warp] = make_float2(r.m, r.s);
 }
 
