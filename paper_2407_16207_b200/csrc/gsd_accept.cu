@@ -93,8 +93,9 @@ struct AcceptArgs {
 
 __global__ void __launch_bounds__(kThreads) accept_kernel(AcceptArgs a) {
     __shared__ Best sh[kThreads / 32];
-    // the second launch may become resident as CTAs retire
-    if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    wait_for_predecessor();
+    // the second launch may become resident as CTAs retire; it reads the graph before it waits
+    if (threadIdx.x == 0) let_successor_start();
     const int row = blockIdx.y;  // b * N + n
     const int split = blockIdx.x;
     const float* x = a.logits + (size_t)row * a.V;
@@ -147,6 +148,7 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(AcceptArgs a) {
 // Second launch: the best key of every node, then the path.
 __global__ void __launch_bounds__(kThreads) accept_tail_kernel(AcceptArgs a) {
     __shared__ int s_amax[GSD_MAX_NODES];
+    let_successor_start();
     const int N = a.N, b = blockIdx.x, tid = threadIdx.x;
     PathIo io;
     io.tok = a.tok + (size_t)b * N;
@@ -159,7 +161,7 @@ __global__ void __launch_bounds__(kThreads) accept_tail_kernel(AcceptArgs a) {
     io.N = N; io.V = a.V; io.Ecap = a.Ecap; io.Tcap = a.Tcap;
     // the keys of a thread's nodes: neighbouring threads read neighbouring keys
     auto best_keys = [&]() -> unsigned {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        wait_for_predecessor();
         constexpr int kTrip = 8;                          // slices whose keys are on their way at a time
         const size_t rows = (size_t)a.B * N;
         const unsigned long long* keys = a.keys + (size_t)b * N + tid;
@@ -235,8 +237,6 @@ extern "C" int gsd_accept(const float* logits, const int32_t* draft_tokens,
     while (rows * splits < kWantCtas && splits < kMaxSplits && p->V / (splits * 2) >= 4096 && rows * splits * 2 * 8 <= workspace_bytes) splits *= 2;
     a.splits = splits;
 
-    cudaLaunchAttribute attr[1];
-    dependent_launch_attr(attr);
     // grid.y holds at most 65535 rows: larger problems go out in blocks of whole sequences
     const int seq_per = 65535 / p->N;
     for (int b0 = 0; b0 < p->B; b0 += seq_per) {
@@ -247,17 +247,9 @@ extern "C" int gsd_accept(const float* logits, const int32_t* draft_tokens,
         s.out_tok += (size_t)b0 * p->Tcap; s.out_len += b0;
         if (s.out_nodes) s.out_nodes += (size_t)b0 * p->Tcap;
         s.keys += (size_t)b0 * p->N * splits; s.B = nb;
-        accept_kernel<<<dim3(splits, (unsigned)(nb * p->N)), kThreads, 0, st>>>(s);
-        GSD_CUDA_TRY(cudaGetLastError());
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)nb);
-        cfg.blockDim = dim3(kThreads);
-        cfg.stream = st;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_tail_kernel, s));
+        GSD_CUDA_TRY(launch_dependent(accept_kernel, dim3(splits, (unsigned)(nb * p->N)), dim3(kThreads), 0, st, s));
+        GSD_CUDA_TRY(launch_dependent(accept_tail_kernel, dim3((unsigned)nb), dim3(kThreads), 0, st, s));
     }
-    GSD_CUDA_TRY(cudaGetLastError());
     return GSD_OK;
 }
 

@@ -189,7 +189,7 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
 #pragma unroll
         for (int k = 0; k < kPathNodeSlots; ++k)
             if (tid + k * kThreads < N) s_uq[tid + k * kThreads] = uq[k];
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        wait_for_predecessor();
         // A node's pairs are shared by neighbouring threads when there are fewer nodes than threads (with few rows
         // the rows are cut into many slices: 1 x 11 rows of 128256, 128 pairs a node, by at most four
         // threads: 2.5 us); with more nodes than threads a thread goes through two of them at once.
@@ -598,8 +598,9 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
 // First launch: one CTA per (slice, row) streams its part of the row and leaves the warps'
 // (maximum, sum) pairs in scratch.
 __global__ void __launch_bounds__(kThreads, 8) accept_sampled_kernel(SampledArgs a) {
-    // the per-sequence pass (a programmatic dependent launch) may become resident as CTAs retire
-    if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    wait_for_predecessor();
+    // the per-sequence pass may become resident as CTAs retire; it reads the graph before it waits
+    if (threadIdx.x == 0) let_successor_start();
     const int row = blockIdx.y;  // b * N + n
     const int slice = blockIdx.x;
     const float* x = a.logits + (size_t)row * a.V;
@@ -628,6 +629,7 @@ __global__ void __launch_bounds__(kThreads, 8) accept_sampled_kernel(SampledArgs
 // Second launch: one cluster per sequence does the rest (statistics per node, step tests, longest
 // path, regenerated token) once every pair of the first launch is visible.
 __global__ void __launch_bounds__(kThreads, 1) accept_sampled_tail_kernel(SampledArgs a) {
+    let_successor_start();
     finish_sequence(a, (int)blockIdx.x / a.cluster);      // (waits for the first launch inside, as late as it can)
 }
 
@@ -704,8 +706,7 @@ extern "C" int gsd_accept_sampled(const float* logits, const int32_t* draft_toke
         if (s.out_nodes) s.out_nodes += (size_t)b0 * p->Tcap;
         s.part += (size_t)b0 * p->N * a.slices * kWarps; s.B = nb;
         const dim3 grid(a.slices, (unsigned)(nb * p->N));
-        accept_sampled_kernel<<<grid, kThreads, 0, st>>>(s);
-        GSD_CUDA_TRY(cudaGetLastError());
+        GSD_CUDA_TRY(launch_dependent(accept_sampled_kernel, grid, dim3(kThreads), 0, st, s));
         s.cluster = pick_cluster(nb, p->V, draft_logits != nullptr, di.sm_count);
         cudaLaunchAttribute attr[2];
         dependent_launch_attr(attr);

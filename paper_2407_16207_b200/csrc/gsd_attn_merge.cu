@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
     // resident while that kernel drains; what it (or the planning kernel) wrote is only visible
     // after this wait, which comes as late as the plan allows: working out a warp's place takes a
     // dozen divisions.
-    auto ready = []() { asm volatile("griddepcontrol.wait;" ::: "memory"); };
+    auto ready = []() { wait_for_predecessor(); };
     unsigned cut = 0;                                              // kWalk: the sequences that were cut
     int work = p.work;
     if (kWalk) {
@@ -122,6 +122,7 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
     const int row = (item % p.plan.tiles_per_unit) * p.tiles * p.RT + tile * p.RT + r;
     if (r >= p.RT || row >= p.R) {
         if (kWalk) continue;
+        ready();                           // (the grid must not end before its predecessor)
         return;
     }
     const int place = unit / p.Hkv, c = unit % p.Hkv, node = row / p.G, head = c * p.G + row % p.G;
@@ -229,17 +230,9 @@ int launch_attn_merge(const AttnArgs& a) {
     p.work = (int)work;
     long blocks = (work + kThreads / 32 - 1) / (kThreads / 32);
     if (walk && blocks > kWalkers) blocks = kWalkers;
-    cudaLaunchAttribute attr[1];
-    dependent_launch_attr(attr);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3(kThreads);
-    cfg.stream = a.stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
     void (*kernel)(MergeParams) = rows == 8 ? (walk ? attn_merge_kernel<true, 8> : attn_merge_kernel<false, 8>)
                                             : (walk ? attn_merge_kernel<true, 32> : attn_merge_kernel<false, 32>);
-    GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, p));
+    GSD_CUDA_TRY(launch_dependent(kernel, dim3((unsigned)blocks), dim3(kThreads), 0, a.stream, p));
     return GSD_OK;
 }
 

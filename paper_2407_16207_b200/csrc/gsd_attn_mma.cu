@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
     unsigned char* sV[2] = {smem + TILE, smem + 3 * TILE};
     __shared__ unsigned s_live;
 
+    let_successor_start();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int item, split, nsplit, slot;
     plan_decode(p.plan, blockIdx.x, item, split, nsplit, slot);
@@ -97,6 +98,7 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
     const int b = unit / p.Hkv, c = unit % p.Hkv;
     const int N = p.N, G = p.G, R = p.R;
 
+    wait_for_predecessor();
     int L = p.seq_lens[b];
     if (L < 0 || L > p.Lmax) {
         if (tid == 0 && p.status) atomicOr((unsigned*)p.status, GSD_DEV_BAD_SEQ_LEN);
@@ -367,9 +369,7 @@ int launch_mma_t(const AttnArgs& a) {
             if (dev >= 0 && dev < 64) done[dev] = true;
         }
     }
-    dim3 grid(a.plan.ctas);
-    attn_mma_kernel<D><<<grid, kThreads, smem, a.stream>>>(p);
-    GSD_CUDA_TRY(cudaGetLastError());
+    GSD_CUDA_TRY(launch_dependent(attn_mma_kernel<D>, dim3(a.plan.ctas), dim3(kThreads), smem, a.stream, p));
     return GSD_OK;
 }
 

@@ -607,8 +607,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     volatile int* abort_flag = &s_wait.abort;
 
     if (warp == 8 && lane == 0) {
-        // the merge pass (a programmatic dependent launch), if there is one, may be made resident as CTAs retire
-        if (p.slots > 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        // The merge pass, if there is one, may be made resident as CTAs retire.  Other successors may not, here
+        // and in the merge pass: the CTAs of a next call that settle where SMs fall free cost it more than
+        // its start gains (32 x 64/8 heads, N 57, L 200-2100: 109 us a call, 117 so; the step of 3 x 40 heads, N
+        // 363, L 228: 142 and 162 - one of 1 x 8/1, N 27, L 97: 10.3 and 9.8).
+        if (p.slots > 0) let_successor_start();
         // the first copy through a tensor map would otherwise fetch it from memory first
         prefetch_map(&tm_q); prefetch_map(&tm_k); prefetch_map(&tm_v); prefetch_map(&tm_dk); prefetch_map(&tm_dv);
         s_wait.abort = 0;

@@ -27,9 +27,11 @@ struct CommitArgs {
 };
 
 __global__ void __launch_bounds__(kThreads) commit_kernel(CommitArgs a) {
+    let_successor_start();
     const int b = blockIdx.x;
     __shared__ int s_src[GSD_MAX_NODES];   // source node of each destination position
     __shared__ int s_count;
+    wait_for_predecessor();
     int L = a.seq_lens[b];
     unsigned flags = 0;
     if (L < 0 || L > a.Lmax) {
@@ -110,7 +112,6 @@ extern "C" int gsd_commit_kv(void* k_cache, void* v_cache, const void* draft_k, 
     a.nodes = accepted_nodes; a.len = accepted_len; a.seq_lens = seq_lens; a.status = status;
     a.N = p->N; a.Lmax = p->Lmax; a.Tcap = p->Tcap;
     a.row16 = p->Hkv * p->D * 2 / 16;
-    commit_kernel<<<p->B, kThreads, 0, (cudaStream_t)stream>>>(a);
-    GSD_CUDA_TRY(cudaGetLastError());
+    GSD_CUDA_TRY(launch_dependent(commit_kernel, dim3(p->B), dim3(kThreads), 0, (cudaStream_t)stream, a));
     return GSD_OK;
 }

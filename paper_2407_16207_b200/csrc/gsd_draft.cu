@@ -103,7 +103,7 @@ __device__ void grow_sequence(const DraftArgs& a, int b) {
     int fl = a.frontier_len[b];
     if (n0 < 1 || n0 > Ncap || fl < 0 || fl > a.F) {
         // nothing sensible can be appended: leave the graph as it is
-        asm volatile("griddepcontrol.wait;" ::: "memory");     // (this grid never ends before the first launch)
+        wait_for_predecessor();                                // (this grid never ends before the first launch)
         if (tid == 0) {
             a.new_frontier_len[b] = 0;
             if (a.status) atomicOr((unsigned*)a.status, GSD_DEV_BAD_FRONTIER);
@@ -180,7 +180,7 @@ __device__ void grow_sequence(const DraftArgs& a, int b) {
     for (int v = tid; v < n0; v += kThreads) enter(v);
 
     // the children: k per frontier node, in frontier order, best first
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_predecessor();
 #pragma unroll
     for (int s = 0; s < kChildSlots; ++s) {
         const int j = tid + s * kThreads;
@@ -390,8 +390,9 @@ __global__ void __launch_bounds__(kThreads, 4) draft_expand_kernel(DraftArgs a) 
     __shared__ int s_bi[K];
     __shared__ float s_pv[kMaxCluster * K], s_pm[kMaxCluster], s_ps[kMaxCluster];   // what the cluster's CTAs hand in
     __shared__ int s_pi[kMaxCluster * K];
-    // the per-sequence pass (a programmatic dependent launch) may become resident as CTAs retire
-    if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    wait_for_predecessor();
+    // the per-sequence pass may become resident as CTAs retire; it reads the graph before it waits
+    if (threadIdx.x == 0) let_successor_start();
     const int C = a.cluster, slice = C > 1 ? cluster_rank() : 0;
     const int fi = (int)blockIdx.x / C, b = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -620,6 +621,7 @@ __global__ void __launch_bounds__(kThreads, 4) draft_expand_kernel(DraftArgs a) 
 // Second launch: one CTA per sequence appends the children and updates the graph once every
 // row's result of the first launch is visible.
 __global__ void __launch_bounds__(kThreads) draft_grow_kernel(DraftArgs a) {
+    let_successor_start();
     grow_sequence(a, blockIdx.x);        // (waits for the first launch inside, as late as it can)
 }
 
@@ -674,24 +676,18 @@ extern "C" int gsd_draft_expand(const float* logits, const int32_t* frontier, co
     // every scratch entry is written before it is read: nothing has to start at zero
     a.cluster = pick_cluster((long)p->B * p->F, p->V, di.sm_count);
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)a.cluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute attr[2];
+    dependent_launch_attr(attr);
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)a.cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.gridDim = dim3((unsigned)p->F * (unsigned)a.cluster, (unsigned)p->B);
     cfg.blockDim = dim3(kThreads);
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = a.cluster > 1 ? 1 : 0;
+    cfg.numAttrs = a.cluster > 1 ? 2 : 1;
     GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, draft_expand_kernel, a));
-    dependent_launch_attr(attr);
-    cfg.gridDim = dim3((unsigned)p->B);
-    cfg.blockDim = dim3(kThreads);
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, draft_grow_kernel, a));
-    GSD_CUDA_TRY(cudaGetLastError());
+    GSD_CUDA_TRY(launch_dependent(draft_grow_kernel, dim3((unsigned)p->B), dim3(kThreads), 0, st, a));
     return GSD_OK;
 }

@@ -233,5 +233,28 @@ inline void dependent_launch_attr(cudaLaunchAttribute* attr) {
     attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr->val.programmaticStreamSerializationAllowed = 1;
 }
+// All small kernels of an iteration are launched this way, wait first and let their own successor start at
+// once, so that the launches of a chain of them overlap.  Among other passes, one by one launched -> so:
+// the step of 6 x 32/8 heads, D 64, N 9, L 200, V 128256 37.3 -> 29.2 us; gsd_accept, 3 x 61 rows of 50257, 14.0 ->
+// 11.6; gsd_accept_sampled, 8 x 256 of 32000, 53.5 -> 50.8.  A kernel whose second half reads inputs before
+// it waits (the acceptance and draft calls: the graph, while the logits are streamed) lets it start only
+// after its own wait: by then everything that precedes the call is over.
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchAttribute attr[1];
+    dependent_launch_attr(attr);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
 
 }  // namespace gsd

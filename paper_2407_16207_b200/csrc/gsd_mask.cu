@@ -29,6 +29,7 @@ build_mask_kernel(const int32_t* __restrict__ parent_ptr, const int32_t* __restr
     __shared__ uint32_t s_rows[GSD_MAX_NODES];
     __shared__ int s_edge[kEdgeCache];
     volatile uint32_t* rows = s_rows;
+    let_successor_start();
     const int w = blockIdx.x, b = b0 + blockIdx.y, v = threadIdx.x;
     const int32_t* pp = parent_ptr + (size_t)b * (N + 1);
     const int32_t* pi = parent_idx + (size_t)b * Ecap;
@@ -36,6 +37,7 @@ build_mask_kernel(const int32_t* __restrict__ parent_ptr, const int32_t* __restr
     // (the row of parent indices holds Ecap entries whatever the pointers say)
     const int cached = min(Ecap, kEdgeCache);
     int e0 = 0, e1 = 0;
+    wait_for_predecessor();
     if (mine) {
         e0 = pp[v];
         e1 = pp[v + 1];
@@ -97,9 +99,8 @@ extern "C" int gsd_build_mask(const int32_t* parent_ptr, const int32_t* parent_i
     const int threads = (N + 31) / 32 * 32;                 // one per node
     for (int b0 = 0; b0 < B; b0 += 65535) {                 // (grid.y holds 65535 sequences)
         const int nb = B - b0 < 65535 ? B - b0 : 65535;
-        build_mask_kernel<<<dim3(W, nb), threads, 0, (cudaStream_t)stream>>>(parent_ptr, parent_idx, ancestor_mask, b0, N, W,
-                                                                             Ecap, status);
+        GSD_CUDA_TRY(launch_dependent(build_mask_kernel, dim3(W, nb), dim3(threads), 0, (cudaStream_t)stream, parent_ptr, parent_idx,
+                                      ancestor_mask, b0, N, W, Ecap, status));
     }
-    GSD_CUDA_TRY(cudaGetLastError());
     return GSD_OK;
 }
