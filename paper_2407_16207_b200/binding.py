@@ -120,7 +120,7 @@ def lib() -> ctypes.CDLL:
 
 # The library's functions the extension calls, in the order of its table.
 _NATIVE_CALLS = ("gsd_verify_attn", "gsd_verify_attn_workspace_bytes", "gsd_accept", "gsd_accept_workspace_bytes",
-                 "gsd_accept_sampled", "gsd_accept_sampled_workspace_bytes", "gsd_draft_expand",
+                 "gsd_accept_sampled", "gsd_accept_sampled_workspace_bytes", "gsd_binding_draft_expand",
                  "gsd_draft_expand_workspace_bytes", "gsd_build_mask", "gsd_commit_kv")
 _native = None
 _native_lib: Optional[ctypes.CDLL] = None      # the library the extension is bound to

@@ -40,7 +40,7 @@ def build_native(force: bool = False) -> str:
     src = os.path.join(CSRC, "gsd_native.cpp")
     built_for = os.path.join(OBJ_DIR, "native_torch_version")
     same = os.path.exists(built_for) and open(built_for).read() == torch.__version__
-    if not force and same and not _stale(NATIVE, [src, os.path.join(ROOT, "include", "gsd.h")]):
+    if not force and same and not _stale(NATIVE, [src, os.path.join(CSRC, "gsd_binding.h"), os.path.join(ROOT, "include", "gsd.h")]):
         return NATIVE
     os.makedirs(OBJ_DIR, exist_ok=True)
     base = os.path.dirname(torch.__file__)
@@ -48,7 +48,7 @@ def build_native(force: bool = False) -> str:
     tmp = NATIVE + f".tmp{os.getpid()}"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
            f'-DGSD_TORCH_VERSION="{torch.__version__}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-           "-I", os.path.join(ROOT, "include"), "-isystem", os.path.join(base, "include"),
+           "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-isystem", os.path.join(base, "include"),
            "-isystem", os.path.join(base, "include", "torch", "csrc", "api", "include"),
            "-isystem", os.path.join(cuda, "include"), "-isystem", sysconfig.get_paths()["include"],
            src, "-o", tmp, "-L", os.path.join(base, "lib"), "-Wl,-rpath," + os.path.join(base, "lib"),

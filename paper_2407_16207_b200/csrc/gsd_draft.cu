@@ -10,6 +10,7 @@
 // an earlier node with the same tau-gram for every new node (first occurrence = lowest id),
 // and compacts the new frontier.
 #include "gsd_internal.cuh"
+#include "gsd_binding.h"
 #include <math_constants.h>
 
 namespace gsd {
@@ -79,6 +80,7 @@ struct DraftArgs {
     int32_t* status;
     int B, F, V, Ncap, k, tau;
     int cluster;         // CTAs per row of logits
+    int pad;             // fill the rest of new_frontier with -1
     float theta_prob, theta_sib;
 };
 
@@ -104,6 +106,8 @@ __device__ void grow_sequence(const DraftArgs& a, int b) {
     if (n0 < 1 || n0 > Ncap || fl < 0 || fl > a.F) {
         // nothing sensible can be appended: leave the graph as it is
         wait_for_predecessor();                                // (this grid never ends before the first launch)
+        if (a.pad)
+            for (int i = tid; i < a.F * k; i += kThreads) a.new_frontier[(size_t)b * a.F * k + i] = -1;
         if (tid == 0) {
             a.new_frontier_len[b] = 0;
             if (a.status) atomicOr((unsigned*)a.status, GSD_DEV_BAD_FRONTIER);
@@ -252,6 +256,8 @@ __device__ void grow_sequence(const DraftArgs& a, int b) {
         for (int w = 0; w < kWarps; ++w) base += s_cnt[w];
         __syncthreads();
     }
+    if (a.pad)
+        for (int i = base + tid; i < a.F * k; i += kThreads) nf[i] = -1;
     if (tid == 0) {
         a.new_frontier_len[b] = base;
         a.num_nodes[b] = n1;
@@ -644,11 +650,11 @@ extern "C" size_t gsd_draft_expand_workspace_bytes(const gsd_draft_params* p) {
     return gsd::align_up((size_t)p->B * p->F * GSD_DRAFT_MAX_K * 8, 256);
 }
 
-extern "C" int gsd_draft_expand(const float* logits, const int32_t* frontier, const int32_t* frontier_len,
-                                int32_t* tokens, int32_t* tree_parent, int32_t* merge_to, uint8_t* leaf,
-                                float* prob, int32_t* num_nodes, int32_t* new_frontier,
-                                int32_t* new_frontier_len, const gsd_draft_params* p, void* workspace,
-                                size_t workspace_bytes, int32_t* status, void* stream) {
+static int draft_expand(const float* logits, const int32_t* frontier, const int32_t* frontier_len,
+                        int32_t* tokens, int32_t* tree_parent, int32_t* merge_to, uint8_t* leaf,
+                        float* prob, int32_t* num_nodes, int32_t* new_frontier,
+                        int32_t* new_frontier_len, const gsd_draft_params* p, void* workspace,
+                        size_t workspace_bytes, int32_t* status, void* stream, bool pad) {
     using namespace gsd;
     if (!p || !logits || !frontier || !frontier_len || !tokens || !tree_parent || !merge_to || !leaf ||
         !prob || !num_nodes || !new_frontier || !new_frontier_len)
@@ -673,6 +679,7 @@ extern "C" int gsd_draft_expand(const float* logits, const int32_t* frontier, co
     a.status = status;
     a.B = p->B; a.F = p->F; a.V = p->V; a.Ncap = p->Ncap; a.k = p->k; a.tau = p->tau;
     a.theta_prob = p->theta_prob; a.theta_sib = p->theta_sib;
+    a.pad = pad;
     // every scratch entry is written before it is read: nothing has to start at zero
     a.cluster = pick_cluster((long)p->B * p->F, p->V, di.sm_count);
     cudaLaunchConfig_t cfg = {};
@@ -690,4 +697,22 @@ extern "C" int gsd_draft_expand(const float* logits, const int32_t* frontier, co
     GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, draft_expand_kernel, a));
     GSD_CUDA_TRY(launch_dependent(draft_grow_kernel, dim3((unsigned)p->B), dim3(kThreads), 0, st, a));
     return GSD_OK;
+}
+
+extern "C" int gsd_draft_expand(const float* logits, const int32_t* frontier, const int32_t* frontier_len,
+                                int32_t* tokens, int32_t* tree_parent, int32_t* merge_to, uint8_t* leaf,
+                                float* prob, int32_t* num_nodes, int32_t* new_frontier,
+                                int32_t* new_frontier_len, const gsd_draft_params* p, void* workspace,
+                                size_t workspace_bytes, int32_t* status, void* stream) {
+    return draft_expand(logits, frontier, frontier_len, tokens, tree_parent, merge_to, leaf, prob, num_nodes, new_frontier,
+                        new_frontier_len, p, workspace, workspace_bytes, status, stream, false);
+}
+
+extern "C" int gsd_binding_draft_expand(const float* logits, const int32_t* frontier, const int32_t* frontier_len,
+                                        int32_t* tokens, int32_t* tree_parent, int32_t* merge_to, uint8_t* leaf,
+                                        float* prob, int32_t* num_nodes, int32_t* new_frontier,
+                                        int32_t* new_frontier_len, const gsd_draft_params* p, void* workspace,
+                                        size_t workspace_bytes, int32_t* status, void* stream) {
+    return draft_expand(logits, frontier, frontier_len, tokens, tree_parent, merge_to, leaf, prob, num_nodes, new_frontier,
+                        new_frontier_len, p, workspace, workspace_bytes, status, stream, true);
 }

@@ -18,7 +18,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <initializer_list>
-#include "gsd.h"
+#include "gsd_binding.h"
 
 namespace {
 
@@ -29,7 +29,7 @@ struct Table {
     decltype(&gsd_accept_workspace_bytes) accept_workspace_bytes;
     decltype(&gsd_accept_sampled) accept_sampled;
     decltype(&gsd_accept_sampled_workspace_bytes) accept_sampled_workspace_bytes;
-    decltype(&gsd_draft_expand) draft_expand;
+    decltype(&gsd_binding_draft_expand) draft_expand;
     decltype(&gsd_draft_expand_workspace_bytes) draft_expand_workspace_bytes;
     decltype(&gsd_build_mask) build_mask;
     decltype(&gsd_commit_kv) commit_kv;
@@ -319,8 +319,7 @@ PyObject* py_draft_expand(PyObject*, PyObject* const* argv, Py_ssize_t nargs) {
     GSD_PY_PLAIN;
     if (p.k < 1 || p.k > GSD_DRAFT_MAX_K) Py_RETURN_NONE;
     Call c(a.device);
-    // (the library writes the first new_frontier_len entries only, and every length)
-    at::Tensor nf = at::full({p.B, (int64_t)p.F * p.k}, -1, at::TensorOptions().dtype(at::kInt).device(logits->device()));
+    at::Tensor nf = empty({p.B, (int64_t)p.F * p.k}, at::kInt, a.device);
     at::Tensor nfl = empty({p.B}, at::kInt, a.device);
     c.scratch(ws, ws ? 0 : std::max<size_t>(lib.draft_expand_workspace_bytes(&p), 8), a.device);
     const int rc = unlocked([&] {
