@@ -2,14 +2,18 @@
 // partial results of every row.
 //   m = max_s m_s;  out = sum_s 2^(m_s - m) O_s / sum_s 2^(m_s - m) l_s
 //
-// A warp takes 32 rows of a row tile and two of its column groups: a lane is a row, a thread has two
-// column groups (8 values, 16 bytes of output).  The rows of a column group are consecutive in the
+// A block of four warps has 32 rows of a row tile and eight of their column groups: a lane is a row, a thread
+// has two column groups (8 values, 16 bytes of output).  The rows of a column group are consecutive in the
 // partial results, so every load of a warp is 512 contiguous bytes.  For items of fewer than 64 rows of
 // the mma.sync kernel a warp takes 8 rows and four column groups, one a thread, which leaves fewer lanes
 // without a row (D 64, whole call: 2 x 12 heads, N 40, L 1500 15.2 us, 15.5 with 32 rows a warp; 32/8
-// heads, N 8, L 4000 14.6 and 14.9; the tcgen05 kernel's few rows are up to 2% slower that way).  Few registers and short code
-// on purpose: the launch lasts a few microseconds, and a form with four column groups a thread and
-// the next four parts on their way while four are added up took 1 us longer.
+// heads, N 8, L 4000 14.6 and 14.9; the tcgen05 kernel's few rows are up to 2% slower that way).
+//
+// The launch lasts a few microseconds: a few dependent trips to memory, in as few waves of blocks as possible.
+// One pass: the sum is brought to a batch's maximum when that is larger (a pass over the maxima before it was two more
+// trips for 18 parts).  Small blocks spread evenly, and what a block works on is the same for all its threads (two
+// waves of blocks of 256 threads, every warp with a place of its own: D 64, 1 x 32/8 heads, N 8, L 4000, whole
+// call 12.2 us, now 10.6; 1 x 32/8, N 37, L 3103 15.7, now 14.9).
 #include "gsd_internal.cuh"
 #include <cuda_bf16.h>
 #include <math_constants.h>
@@ -17,9 +21,14 @@
 namespace gsd {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kBatch = 4;        // parts of a row on their way at a time
-constexpr int kWalkers = 296;    // blocks that walk over the items of a one-wave plan (two per SM)
+constexpr int kThreads = 128;
+// Parts of a row on their way at a time, and blocks per SM that have to be resident: many parts are worth
+// more than occupancy as long as all blocks are resident at once (1 x 8 items of 18 parts, 256 rows: 49.5 us
+// the whole call with four, 46.4 with eight), else it is the other way round (40 items of 3 to 5 parts: 24.2
+// with four, 26.0 with eight; limited to 64 registers, eight blocks an SM, calls took up to 2 us more).
+constexpr int kBatchFew = 8, kBlocksFew = 3;
+constexpr int kBatchMany = 4, kBlocksMany = 4;
+constexpr int kWalkers = 592;    // blocks that walk over the items of a one-wave plan (four per SM)
 
 struct MergeParams {
     const float4* part_o;
@@ -51,13 +60,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // 64/8 heads, N 32, L 2048: 42.4 us with blocks for every item, 39.8 walking (37.1 with a plan that
 // cannot cut, which takes 115 instead of 28.5 when one of the sequences has 8192 and the others 500).
 // Where every item may be cut, one block for each part of it is up to 0.5 us faster.
-template <bool kWalk, int kRows>
-__global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
+template <bool kWalk, int kRows, bool kFew>
+__global__ void __launch_bounds__(kThreads, kFew ? kBlocksFew : kBlocksMany) attn_merge_kernel(MergeParams p) {
     const int lane = threadIdx.x & 31;
+    constexpr int kBatch = kFew ? kBatchFew : kBatchMany;
     constexpr int kGroups = kRows == 32 ? 2 : 1;                   // column groups of a thread
     constexpr int kSpan = 32 / kRows * kGroups;                    // of a warp
-    const int quads = p.D / 4, parts_of_row = quads / kSpan;
-    const int warp = (int)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+    const int quads = p.D / 4, parts_of_row = quads / kSpan / (kThreads / 32);     // blocks that share a row
     // Launched as a programmatic dependent of the attention kernel: the blocks may become
     // resident while that kernel drains; what it (or the planning kernel) wrote is only visible
     // after this wait, which comes as late as the plan allows: working out a warp's place takes a
@@ -70,8 +79,9 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
         cut = __ballot_sync(0xFFFFFFFFu, lane < p.B && p.left[lane] > 1);
         work = __popc(cut) * p.Hkv * p.plan.tiles_per_unit * p.groups * parts_of_row;
     }
-    for (int w = warp; w < work; w += (int)gridDim.x * (kThreads / 32)) {      // (once, unless kWalk)
-    const int col0 = w % parts_of_row * kSpan + lane / kRows * kGroups;       // first column group of the thread
+    for (int w = (int)blockIdx.x; w < work; w += (int)gridDim.x) {                 // (once, unless kWalk)
+    // first column group of the thread
+    const int col0 = (w % parts_of_row * (kThreads / 32) + (int)(threadIdx.x >> 5)) * kSpan + lane / kRows * kGroups;
     const int g = w / parts_of_row % p.groups;
     const int k = w / parts_of_row / p.groups;
     // the k-th item that owns slots: group a comes first when it is split at all
@@ -130,34 +140,39 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(MergeParams p) {
     const int b = p.plan.longest_first ? p.left[place] : place;
 
     const size_t first = (size_t)slot0 * p.tiles + tile;
-    const float2* ml_base = p.part_ml + first * p.tile_rows + r;
-    const float4* o_base = p.part_o + (first * quads + col0) * p.tile_rows + r;
-    const size_t ml_stride = (size_t)slot_step * p.tiles * p.tile_rows, o_stride = ml_stride * quads;
-    float2 ml[kBatch];
-    float4 v[kBatch][kGroups];
-    auto fetch = [&](int s0) {
+    const float2* ml_at = p.part_ml + first * p.tile_rows + r;
+    const float4* o_at = p.part_o + (first * quads + col0) * p.tile_rows + r;
+    const unsigned ml_stride = (unsigned)(slot_step * p.tiles * p.tile_rows), o_stride = ml_stride * (unsigned)quads;
+    float m = -CUDART_INF_F, l = 0.f;
+    float acc[kGroups][4] = {};
+#pragma unroll 1
+    for (int s0 = 0; s0 < nsplit; s0 += kBatch) {
+        float2 ml[kBatch];
+        float4 v[kBatch][kGroups];
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
             const bool in = s0 + j < nsplit;
-            ml[j] = in ? ml_base[(size_t)(s0 + j) * ml_stride] : make_float2(-CUDART_INF_F, 0.f);
+            ml[j] = in ? *ml_at : make_float2(-CUDART_INF_F, 0.f);
 #pragma unroll
-            for (int q = 0; q < kGroups; ++q)
-                v[j][q] = in ? o_base[(size_t)(s0 + j) * o_stride + q * p.tile_rows] : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int q = 0; q < kGroups; ++q) v[j][q] = in ? o_at[q * p.tile_rows] : make_float4(0.f, 0.f, 0.f, 0.f);
+            ml_at += ml_stride;
+            o_at += o_stride;
         }
-    };
-    fetch(0);
-    float m = fmaxf(fmaxf(ml[0].x, ml[1].x), fmaxf(ml[2].x, ml[3].x));
-#pragma unroll 4
-    for (int s = kBatch; s < nsplit; ++s) m = fmaxf(m, ml_base[(size_t)s * ml_stride].x);
-    const float m_use = m == -CUDART_INF_F ? 0.f : m;
-    float acc[kGroups][4] = {};
-    float l = 0.f;
-#pragma unroll 1
-    for (int s0 = 0; s0 < nsplit; s0 += kBatch) {
-        if (s0 > 0) fetch(s0);
+        // what has been added up so far is brought to the batch's maximum, if that is larger
+        float top = m;
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) top = fmaxf(top, ml[j].x);
+        const float top_use = top == -CUDART_INF_F ? 0.f : top;
+        const float back = exp2f(m - top_use);
+        m = top;
+        l *= back;
+#pragma unroll
+        for (int q = 0; q < kGroups; ++q)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[q][e] *= back;
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
-            const float wgt = exp2f(ml[j].x - m_use);     // 0 for an absent or empty split
+            const float wgt = exp2f(ml[j].x - top_use);   // 0 for an absent or empty split
             l += wgt * ml[j].y;
 #pragma unroll
             for (int q = 0; q < kGroups; ++q) {
@@ -225,13 +240,18 @@ int launch_attn_merge(const AttnArgs& a) {
     p.groups = p.R >= a.plan.rows_per_item ? p.tiles * per_tile
                : p.R <= p.RT               ? (p.R + rows - 1) / rows
                                            : per_tile + (p.R - p.RT + rows - 1) / rows;
-    const long work = (long)split_items * p.groups * (p.D / 4 / span);
+    const long work = (long)split_items * p.groups * (p.D / 4 / span / (kThreads / 32));
     if (work == 0) return GSD_OK;
     p.work = (int)work;
-    long blocks = (work + kThreads / 32 - 1) / (kThreads / 32);
+    long blocks = work;
     if (walk && blocks > kWalkers) blocks = kWalkers;
-    void (*kernel)(MergeParams) = rows == 8 ? (walk ? attn_merge_kernel<true, 8> : attn_merge_kernel<false, 8>)
-                                            : (walk ? attn_merge_kernel<true, 32> : attn_merge_kernel<false, 32>);
+    DeviceInfo di;
+    if (device_info(&di) != 0) return GSD_ERR_CUDA;
+    const bool few = blocks <= (long)kBlocksFew * di.sm_count;
+    void (*kernel)(MergeParams) = nullptr;
+    if (rows == 8) kernel = few ? attn_merge_kernel<false, 8, true> : attn_merge_kernel<false, 8, false>;    // (the mma.sync kernel has no one-wave plan)
+    else if (walk) kernel = few ? attn_merge_kernel<true, 32, true> : attn_merge_kernel<true, 32, false>;
+    else kernel = few ? attn_merge_kernel<false, 32, true> : attn_merge_kernel<false, 32, false>;
     GSD_CUDA_TRY(launch_dependent(kernel, dim3((unsigned)blocks), dim3(kThreads), 0, a.stream, p));
     return GSD_OK;
 }
