@@ -547,15 +547,60 @@ __device__ __forceinline__ unsigned unit_live(const TcParams& p, const UnitInfo&
     return __reduce_or_sync(0xFFFFFFFFu, live);
 }
 
-// The whole unit: live draft tiles only are numbered.
-template <int PLAN>
-__device__ __forceinline__ UnitInfo unit_info(const TcParams& p, const Order& order, int w, int lane, const WaveUnit& wu = WaveUnit{}) {
-    UnitInfo u = unit_base<PLAN>(p, order, w, wu);
-    u.live = unit_live(p, u, lane);
-    auto live_index = [&](int t) { return t <= u.nPT ? t : u.nPT + __popc(u.live & ((1u << (t - u.nPT)) - 1u)); };
+// The same for many mask words, a slice of them: part `part` of `parts`, eight 16-byte loads of a lane on their way
+// whatever the width of a row.
+__device__ __forceinline__ unsigned unit_live_slice(const TcParams& p, const UnitInfo& u, int part, int parts, int lane) {
+    const int n_lo = u.row0 / p.G;
+    const int n_hi = (min(u.row0 + 2 * p.RT, p.R) - 1) / p.G + 1;
+    const int total = (n_hi - n_lo) * p.W, lo = total * part / parts, hi = total * (part + 1) / parts;
+    const uint32_t* words = p.mask + ((size_t)u.b * p.N + n_lo) * p.W;
+    const uint32_t tail = (p.N & 31) ? (1u << (p.N & 31)) - 1u : 0xFFFFFFFFu;   // valid bits of a row's last word
+    unsigned live = 0;
+    auto note = [&](uint32_t v, int col) {
+        if (col == p.W - 1) v &= tail;
+        if (v) live |= 1u << (col >> 2);
+    };
+    // (words before the first 16-byte boundary and behind the last one go one by one)
+    const int to_boundary = (int)((0u - (unsigned)(reinterpret_cast<uintptr_t>(words + lo) >> 2)) & 3u);
+    const int q0 = min(lo + to_boundary, hi), nq = (hi - q0) >> 2, rest = q0 + 4 * nq;
+    const uint32_t v_head = lo + lane < q0 ? words[lo + lane] : 0u, v_tail = rest + lane < hi ? words[rest + lane] : 0u;
+    const uint4* quads = reinterpret_cast<const uint4*>(words + q0);
+#pragma unroll 1
+    for (int base = lane; base < nq; base += 8 * 32) {
+        uint4 q[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) q[k] = base + 32 * k < nq ? quads[base + 32 * k] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (!(q[k].x | q[k].y | q[k].z | q[k].w)) continue;
+            const uint32_t v[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
+            int col = (q0 + 4 * (base + 32 * k)) % p.W;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                note(v[j], col);
+                col = col + 1 == p.W ? 0 : col + 1;
+            }
+        }
+    }
+    note(v_head, (lo + lane) % p.W);
+    note(v_tail, (rest + lane) % p.W);
+    return __reduce_or_sync(0xFFFFFFFFu, live);
+}
+
+// Of the draft tiles only the live ones are numbered.
+__device__ __forceinline__ void unit_use_live(UnitInfo& u, unsigned live) {
+    u.live = live;
+    auto live_index = [&](int t) { return t <= u.nPT ? t : u.nPT + __popc(live & ((1u << (t - u.nPT)) - 1u)); };
     const int t0 = live_index(u.t_begin), t1 = live_index(u.t_begin + u.ntiles);
     u.t_begin = t0;
     u.ntiles = t1 - t0;
+}
+
+// The whole unit.
+template <int PLAN>
+__device__ __forceinline__ UnitInfo unit_info(const TcParams& p, const Order& order, int w, int lane, const WaveUnit& wu = WaveUnit{}) {
+    UnitInfo u = unit_base<PLAN>(p, order, w, wu);
+    unit_use_live(u, unit_live(p, u, lane));
     return u;
 }
 
@@ -577,7 +622,7 @@ __device__ __forceinline__ bool order_by_length(const TcParams& p, int* s_len, i
 // counted across units, so the producer and the QK^T issuer run ahead into the next unit
 // (Q, the first K/V tiles and the first QK^T) while the softmax warps still read out the
 // accumulators of the previous one.
-template <int HD, int PLAN>
+template <int HD, int PLAN, bool LONG_MASK>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_dk,
@@ -593,6 +638,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     __shared__ int s_len[kPlanSeqs], s_seq[kPlanSeqs];     // longest first: lengths, order of the sequences
     __shared__ int s_wave_units;                           // one-wave plan: units of the call
     __shared__ UnitInfo s_units[kUnitTable];   // the CTA's first units of work, decoded once up front
+    __shared__ unsigned s_live[kThreads / 32]; // live draft tiles in the slices of their mask rows
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int N = p.N, G = p.G, R = p.R, RT = p.RT;
@@ -721,6 +767,38 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             for (int n = 0; n < pre; ++n) { load_k(u, n, n); load_v(u, n, n); }
         }
         pre = __shfl_sync(0xFFFFFFFFu, pre, 0);
+    } else if (LONG_MASK) {
+        // Mask rows of many words (256 nodes, one head a group: up to 16 KB a unit): few units are shared by the
+        // warps, a slice each, and put together behind a barrier (one warp a unit with four words of a lane on
+        // their way took 13 us at N 338: 2 x 32 heads, N 407, L 4081 88.6 -> 83 us; D 64, 2 x 12 heads, N 346, L
+        // 3900 38.2 -> 35.2).
+        constexpr int kDecoders = kThreads / 32 - 1;
+        WaveUnit wu{};
+        int n = n_my;
+        if (PLAN == PLAN_WAVE) {
+            wu = wave_unit(p, blockIdx.x, lane, blockIdx.x == 0 && warp == 0);
+            if (warp == 0 && lane == 0) s_wave_units = wu.units;
+            n = (int)blockIdx.x < wu.units ? 1 : 0;
+        }
+        const int slices = max(1, kDecoders / max(n, 1)), me = warp < 8 ? warp : warp - 1;
+        for (int t = me; t < min(n, kUnitTable) * slices; t += kDecoders) {
+            const int k = t / slices, part = t - k * slices;
+            UnitInfo u = unit_base<PLAN>(p, order, PLAN == PLAN_WAVE ? (int)blockIdx.x : unit_index(k), wu);
+            const unsigned live = unit_live_slice(p, u, part, slices, lane);
+            if (lane == 0) {
+                if (slices > 1) s_live[t] = live;
+                else unit_use_live(u, live);
+                if (part == 0) s_units[k] = u;
+            }
+        }
+        if (slices > 1) {
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kDecoders) : "memory");
+            if (lane == 0 && me < n) {
+                unsigned live = 0;
+                for (int k = 0; k < slices; ++k) live |= s_live[me * slices + k];
+                unit_use_live(s_units[me], live);
+            }
+        }
     } else if (PLAN == PLAN_WAVE) {
         if (warp == 0) {
             const WaveUnit wu = wave_unit(p, blockIdx.x, lane, blockIdx.x == 0);
@@ -1271,7 +1349,7 @@ int make_map(CUtensorMap* m, const void* base, uint64_t HD, uint64_t d1, uint64_
 
 }  // namespace
 
-template <int HD, int PLAN>
+template <int HD, int PLAN, bool LONG_MASK>
 static int launch_tc(const AttnArgs& a) {
     const int nodes = BM / a.G;           // whole nodes of a row tile
     CUtensorMap tq, tk, tv, tdk, tdv;
@@ -1295,7 +1373,7 @@ static int launch_tc(const AttnArgs& a) {
         int dev = 0;
         GSD_CUDA_TRY(cudaGetDevice(&dev));
         if (dev < 0 || dev >= 64 || !done[dev]) {
-            GSD_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<HD, PLAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<HD>::SMEM_BYTES));
+            GSD_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<HD, PLAN, LONG_MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<HD>::SMEM_BYTES));
             if (dev >= 0 && dev < 64) done[dev] = true;
         }
     }
@@ -1338,7 +1416,7 @@ static int launch_tc(const AttnArgs& a) {
     const int part = PLAN == PLAN_FIXED || PLAN == PLAN_ORDERED ? (int)cfg.gridDim.x * kUnitTable : a.plan.ctas;
     for (p.work0 = 0; p.work0 < a.plan.ctas; p.work0 += part) {
         p.total_work = a.plan.ctas - p.work0 < part ? a.plan.ctas - p.work0 : part;
-        GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD, PLAN>, tq, tk, tv, tdk, tdv, p));
+        GSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD, PLAN, LONG_MASK>, tq, tk, tv, tdk, tdv, p));
     }
     return GSD_OK;
 }
@@ -1347,17 +1425,30 @@ int attn_tcgen05_rows(int G) { return G <= BM ? BM / G * G : BM; }
 
 bool attn_tcgen05_supports(int D, int G) { return (D == 128 || D == 64) && G >= 1 && G <= BM; }
 
+template <bool LONG_MASK>
+static int launch_plan(const AttnArgs& a) {
+    switch (a.plan.dev.balanced == 3 ? PLAN_WAVE : a.plan.dev.balanced ? PLAN_TABLE : a.plan.dev.longest_first ? PLAN_ORDERED : PLAN_FIXED) {
+        case PLAN_WAVE: return a.D == 128 ? launch_tc<128, PLAN_WAVE, LONG_MASK>(a) : launch_tc<64, PLAN_WAVE, LONG_MASK>(a);
+        case PLAN_ORDERED: return a.D == 128 ? launch_tc<128, PLAN_ORDERED, LONG_MASK>(a) : launch_tc<64, PLAN_ORDERED, LONG_MASK>(a);
+        case PLAN_TABLE: return launch_tc<128, PLAN_TABLE, LONG_MASK>(a);     // (D = 128 only)
+        default: return a.D == 128 ? launch_tc<128, PLAN_FIXED, LONG_MASK>(a) : launch_tc<64, PLAN_FIXED, LONG_MASK>(a);
+    }
+}
+
+// The mask words of a unit are more than a warp fetches in one round of 16-byte loads (N above 128 with one head a
+// group).  A kernel of its own: the code for slices in the others' prologue cost calls of a few tiles up to
+// 4%; with up to 1024 words it is a wash (D 64, 4 x 32/8 heads, N 428, L 20322, 896 words: 586 us, 592 so).
+static bool long_mask(const AttnArgs& a) {
+    const int nodes = 2 * (BM / a.G);
+    return (nodes < a.N ? nodes : a.N) * a.W > 8 * 32 * 4;
+}
+
 int launch_attn_tcgen05(const AttnArgs& a) {
     if (!attn_tcgen05_supports(a.D, a.G)) {
         set_error_text("tcgen05 back end needs a head dimension of 64 or 128 and a group size of at most 128");
         return GSD_ERR_UNSUPPORTED;
     }
-    switch (a.plan.dev.balanced == 3 ? PLAN_WAVE : a.plan.dev.balanced ? PLAN_TABLE : a.plan.dev.longest_first ? PLAN_ORDERED : PLAN_FIXED) {
-        case PLAN_WAVE: return a.D == 128 ? launch_tc<128, PLAN_WAVE>(a) : launch_tc<64, PLAN_WAVE>(a);
-        case PLAN_ORDERED: return a.D == 128 ? launch_tc<128, PLAN_ORDERED>(a) : launch_tc<64, PLAN_ORDERED>(a);
-        case PLAN_TABLE: return launch_tc<128, PLAN_TABLE>(a);     // (D = 128 only)
-        default: return a.D == 128 ? launch_tc<128, PLAN_FIXED>(a) : launch_tc<64, PLAN_FIXED>(a);
-    }
+    return long_mask(a) ? launch_plan<true>(a) : launch_plan<false>(a);
 }
 
 void debug_attn_wait(unsigned long long limit_ns, int withhold_first_k) {
