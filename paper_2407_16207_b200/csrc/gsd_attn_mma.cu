@@ -7,7 +7,8 @@
 // once per row tile.
 //
 // Grid: one CTA per (work item, key-range split) of the call's plan.  A CTA of 4 warps owns
-// 64 stacked rows and walks its share of the key tiles (64 keys each; prefix tiles first, then draft tiles) with a
+// 64 stacked rows - 16 a warp, or, when an item has at most 32 or 16 rows, with two or four warps for the same rows and a
+// share of each tile's keys each - and walks its share of the key tiles (64 keys each; prefix tiles first, then draft tiles) with a
 // two-stage cp.async pipeline.  Rows of the cache at positions >= seq_lens[b] and draft
 // rows >= N are zero-filled by the copy itself, so junk (even NaN patterns) never reaches
 // the arithmetic.  Draft tiles whose mask words are all zero for the CTA's rows are
@@ -77,20 +78,26 @@ struct MmaParams {
     float scale_log2;
 };
 
-template <int D>
+template <int D, int KEY_WARPS>
 __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
     constexpr int CH = D / 8;              // 16-byte chunks per row
     constexpr int TILE = BN * D * 2;       // bytes of one K or V tile
     constexpr int KS = D / 16;             // k-steps of the QK^T product
-    constexpr int NT = BN / 8;             // score n-tiles per warp
+    constexpr int ROW_WARPS = 4 / KEY_WARPS;
+    constexpr int KEYS = BN / KEY_WARPS;   // keys of a tile a warp works on
+    constexpr int NT = KEYS / 8;           // score n-tiles per warp
     constexpr int DT = D / 8;              // output n-tiles per warp
     extern __shared__ __align__(128) unsigned char smem[];
-    unsigned char* sK[2] = {smem, smem + 2 * TILE};
-    unsigned char* sV[2] = {smem + TILE, smem + 3 * TILE};
+    auto sK = [&](int stage) { return smem + stage * (2 * TILE); };
+    auto sV = [&](int stage) { return smem + stage * (2 * TILE) + TILE; };
     __shared__ unsigned s_live;
 
-    let_successor_start();
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // (the merge pass only: CTAs of a next call that settle beside this one's leave it unevenly filled SMs - 8 x 32
+    // heads, N 32, L 4000 126 us a call, 96 without)
+    if (p.slots > 0) let_successor_start();
+    const int tid = threadIdx.x, lane = tid & 31;
+    // the 16 rows and the keys of a tile that this warp works on
+    const int warp = (tid >> 5) % ROW_WARPS, kg = (tid >> 5) / ROW_WARPS, k_lo = kg * KEYS;
     int item, split, nsplit, slot;
     plan_decode(p.plan, blockIdx.x, item, split, nsplit, slot);
     const int unit = item / p.plan.tiles_per_unit;   // b * Hkv + c
@@ -129,7 +136,7 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
 
     // ---- Q tile -> smem (borrowing the second V stage) -> A fragments
     {
-        unsigned char* sQ = sV[1];
+        unsigned char* sQ = sV(1);
         for (int i = tid; i < BM * CH; i += kThreads) {
             const int r = i / CH, ch = i % CH;
             const int row = row0 + r;
@@ -145,7 +152,7 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
     const unsigned live_tiles = s_live;
     uint32_t qf[KS][4];
     {
-        unsigned char* sQ = sV[1];
+        unsigned char* sQ = sV(1);
         const int r = warp * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks)
@@ -170,8 +177,8 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
             const int key = key0 + r;
             const bool ok = key < limit;
             const size_t off = (size_t)(ok ? key : 0) * rstride + ch * 8;
-            cp_async16(smem_u32(sK[stage] + tile_off<D>(r, ch)), kb + off, ok ? 16 : 0);
-            cp_async16(smem_u32(sV[stage] + tile_off<D>(r, ch)), vb + off, ok ? 16 : 0);
+            cp_async16(smem_u32(sK(stage) + tile_off<D>(r, ch)), kb + off, ok ? 16 : 0);
+            cp_async16(smem_u32(sV(stage) + tile_off<D>(r, ch)), vb + off, ok ? 16 : 0);
         }
     };
     auto next_live = [&](int t) -> int {
@@ -214,7 +221,7 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
 #pragma unroll
             for (int kp = 0; kp < KS / 2; ++kp) {
                 uint32_t kf[4];
-                ldmatrix_x4(kf, smem_u32(sK[stage] + tile_off<D>(nt * 8 + (lane & 7), kp * 4 + (lane >> 3))));
+                ldmatrix_x4(kf, smem_u32(sK(stage) + tile_off<D>(k_lo + nt * 8 + (lane & 7), kp * 4 + (lane >> 3))));
                 mma_bf16(s[nt], qf[kp * 2], kf[0], kf[1]);
                 mma_bf16(s[nt], qf[kp * 2 + 1], kf[2], kf[3]);
             }
@@ -241,7 +248,7 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
             for (int nt = 0; nt < NT; ++nt) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const int col = nt * 8 + (lane & 3) * 2 + (e & 1);
+                    const int col = k_lo + nt * 8 + (lane & 3) * 2 + (e & 1);
                     const int h = e >> 1;
                     const uint32_t w = (col >> 5) ? mw[h][1] : mw[h][0];
                     const bool vis = ((w >> (col & 31)) & 1u) && (key0 + col < N) && rvalid[h];
@@ -253,7 +260,7 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
             for (int nt = 0; nt < NT; ++nt) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const int col = nt * 8 + (lane & 3) * 2 + (e & 1);
+                    const int col = k_lo + nt * 8 + (lane & 3) * 2 + (e & 1);
                     const bool vis = (key0 + col < L) && rvalid[e >> 1];
                     s[nt][e] = vis ? s[nt][e] * p.scale_log2 : -CUDART_INF_F;
                 }
@@ -290,7 +297,7 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
 
         // ---- O += P V
 #pragma unroll
-        for (int ks = 0; ks < BN / 16; ++ks) {
+        for (int ks = 0; ks < KEYS / 16; ++ks) {
             uint32_t pf[4];
             pf[0] = pack_bf16(s[2 * ks][0], s[2 * ks][1]);
             pf[1] = pack_bf16(s[2 * ks][2], s[2 * ks][3]);
@@ -299,8 +306,8 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
 #pragma unroll
             for (int dp = 0; dp < DT / 2; ++dp) {
                 uint32_t vf[4];
-                const int key = ks * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-                ldmatrix_x4_trans(vf, smem_u32(sV[stage] + tile_off<D>(key, dp * 2 + (lane >> 4))));
+                const int key = k_lo + ks * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
+                ldmatrix_x4_trans(vf, smem_u32(sV(stage) + tile_off<D>(key, dp * 2 + (lane >> 4))));
                 mma_bf16(o[dp * 2], pf, vf[0], vf[1]);
                 mma_bf16(o[dp * 2 + 1], pf, vf[2], vf[3]);
             }
@@ -318,37 +325,94 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
         l_run[h] += __shfl_xor_sync(0xFFFFFFFFu, l_run[h], 1);
         l_run[h] += __shfl_xor_sync(0xFFFFFFFFu, l_run[h], 2);
     }
-    if (nsplit == 1) {
+    // stores the thread's values of `tiles` output n-tiles from dt0 on
+    auto store = [&](auto& r, int dt0) {
+        constexpr int tiles = sizeof(r) / sizeof(r[0]);
+        if (nsplit == 1) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (!rvalid[h]) continue;
-            const int row = row0 + rloc[h];
-            if (!GSD_IN_BOUNDS(b < p.B && c < p.Hkv && row < p.R, p.status)) continue;
-            const float inv = l_run[h] > 0.f ? 1.f / l_run[h] : 0.f;
-            __nv_bfloat16* dst = p.out + (((size_t)b * N + row / G) * p.Hq + c * G + row % G) * D;
+            for (int h = 0; h < 2; ++h) {
+                if (!rvalid[h]) continue;
+                const int row = row0 + rloc[h];
+                if (!GSD_IN_BOUNDS(b < p.B && c < p.Hkv && row < p.R, p.status)) continue;
+                const float inv = l_run[h] > 0.f ? 1.f / l_run[h] : 0.f;
+                __nv_bfloat16* dst = p.out + (((size_t)b * N + row / G) * p.Hq + c * G + row % G) * D + dt0 * 8;
 #pragma unroll
-            for (int dt = 0; dt < DT; ++dt) {
-                const int col = dt * 8 + (lane & 3) * 2;
-                *reinterpret_cast<uint32_t*>(dst + col) = pack_bf16(o[dt][h * 2] * inv, o[dt][h * 2 + 1] * inv);
+                for (int dt = 0; dt < tiles; ++dt) {
+                    const int col = dt * 8 + (lane & 3) * 2;
+                    *reinterpret_cast<uint32_t*>(dst + col) = pack_bf16(r[dt][h * 2] * inv, r[dt][h * 2 + 1] * inv);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (!rvalid[h]) continue;
+                if (!GSD_IN_BOUNDS(slot >= 0 && slot < p.slots, p.status)) continue;
+#pragma unroll
+                for (int dt = 0; dt < tiles; ++dt) {
+                    const int col = (dt0 + dt) * 8 + (lane & 3) * 2;
+                    float* dst = p.part_o + (((size_t)slot * (D / 4) + col / 4) * BM + rloc[h]) * 4 + col % 4;
+                    *reinterpret_cast<float2*>(dst) = make_float2(r[dt][h * 2], r[dt][h * 2 + 1]);
+                }
+                if (dt0 == 0 && (lane & 3) == 0) *reinterpret_cast<float2*>(p.part_ml + ((size_t)slot * BM + rloc[h]) * 2) = make_float2(m_run[h], l_run[h]);
             }
         }
+    };
+    if constexpr (KEY_WARPS == 1) {
+        store(o, 0);
     } else {
+        // The warps of a row group leave their parts in the memory of the tiles (every copy has landed and every warp
+        // has left the loop), and each brings a share of the columns together.
+        constexpr int VALUES = DT * 4 + 4;                 // of a thread
+        constexpr int SHARE = DT / KEY_WARPS;
+        static_assert(4 * VALUES * 32 * 4 <= 4 * TILE, "the parts fit the tiles");
+        float* part = reinterpret_cast<float*>(smem) + lane;
+        auto part_of = [&](int k) { return part + (k * ROW_WARPS + warp) * (VALUES * 32); };
+        __syncthreads();
+        if (active) {
+            float* at = part_of(kg);
+#pragma unroll
+            for (int dt = 0; dt < DT; ++dt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) at[(dt * 4 + e) * 32] = o[dt][e];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                at[(DT * 4 + h) * 32] = m_run[h];
+                at[(DT * 4 + 2 + h) * 32] = l_run[h];
+            }
+        }
+        __syncthreads();
+        if (!active) return;
+        float w[KEY_WARPS][2], r[SHARE][4];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            if (!rvalid[h]) continue;
-            if (!GSD_IN_BOUNDS(slot >= 0 && slot < p.slots, p.status)) continue;
+            float m = -CUDART_INF_F, l = 0.f;
 #pragma unroll
-            for (int dt = 0; dt < DT; ++dt) {
-                const int col = dt * 8 + (lane & 3) * 2;
-                float* dst = p.part_o + (((size_t)slot * (D / 4) + col / 4) * BM + rloc[h]) * 4 + col % 4;
-                *reinterpret_cast<float2*>(dst) = make_float2(o[dt][h * 2], o[dt][h * 2 + 1]);
+            for (int k = 0; k < KEY_WARPS; ++k) {
+                w[k][h] = part_of(k)[(DT * 4 + h) * 32];
+                m = fmaxf(m, w[k][h]);
             }
-            if ((lane & 3) == 0) *reinterpret_cast<float2*>(p.part_ml + ((size_t)slot * BM + rloc[h]) * 2) = make_float2(m_run[h], l_run[h]);
+            const float m_use = m == -CUDART_INF_F ? 0.f : m;
+#pragma unroll
+            for (int k = 0; k < KEY_WARPS; ++k) {
+                w[k][h] = exp2f(w[k][h] - m_use);
+                l += w[k][h] * part_of(k)[(DT * 4 + 2 + h) * 32];
+            }
+            m_run[h] = m;
+            l_run[h] = l;
         }
+#pragma unroll
+        for (int dt = 0; dt < SHARE; ++dt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                r[dt][e] = 0.f;
+#pragma unroll
+                for (int k = 0; k < KEY_WARPS; ++k) r[dt][e] += w[k][e >> 1] * part_of(k)[((kg * SHARE + dt) * 4 + e) * 32];
+            }
+        store(r, kg * SHARE);
     }
 }
 
-template <int D>
+template <int D, int KEY_WARPS>
 int launch_mma_t(const AttnArgs& a) {
     MmaParams p;
     p.q = (const __nv_bfloat16*)a.q; p.k_cache = (const __nv_bfloat16*)a.k_cache;
@@ -365,19 +429,23 @@ int launch_mma_t(const AttnArgs& a) {
         int dev = 0;
         GSD_CUDA_TRY(cudaGetDevice(&dev));
         if (dev < 0 || dev >= 64 || !done[dev]) {
-            GSD_CUDA_TRY(cudaFuncSetAttribute(attn_mma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            GSD_CUDA_TRY(cudaFuncSetAttribute(attn_mma_kernel<D, KEY_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
             if (dev >= 0 && dev < 64) done[dev] = true;
         }
     }
-    GSD_CUDA_TRY(launch_dependent(attn_mma_kernel<D>, dim3(a.plan.ctas), dim3(kThreads), smem, a.stream, p));
+    GSD_CUDA_TRY(launch_dependent(attn_mma_kernel<D, KEY_WARPS>, dim3(a.plan.ctas), dim3(kThreads), smem, a.stream, p));
     return GSD_OK;
 }
 
 }  // namespace
 
 int launch_attn_mma(const AttnArgs& a) {
-    if (a.D == 128) return launch_mma_t<128>(a);
-    if (a.D == 64) return launch_mma_t<64>(a);
+    // Few rows leave warps without any: two or four of them then share the 64 keys of a tile.  Among other passes, one
+    // warp for all keys -> shared: 8 x 32 heads, N 8, L 64 / 200 / 1000 7.2 / 12.0 / 32.5 -> 6.4 / 9.5 / 25.4 us; N 32, L 64
+    // / 1000 / 4000 9.0 / 41.2 / 137.7 -> 8.1 / 30.8 / 95.5; D 64, 32 x 32/8, N 8, L 1500 47.3 -> 31.0.
+    const int rows = a.N * a.G;
+    if (a.D == 128) return rows <= 16 ? launch_mma_t<128, 4>(a) : rows <= 32 ? launch_mma_t<128, 2>(a) : launch_mma_t<128, 1>(a);
+    if (a.D == 64) return rows <= 16 ? launch_mma_t<64, 4>(a) : rows <= 32 ? launch_mma_t<64, 2>(a) : launch_mma_t<64, 1>(a);
     return GSD_ERR_BAD_SHAPE;
 }
 
