@@ -59,7 +59,8 @@ int attn_pick_kernel(const gsd_attn_params* p, int sm_count) {
     // L 4000 102 -> 46.6).  With more items its second round of units costs short contexts more than long
     // ones gain - and the cache of a server is mostly empty early on: 8 x 32 heads, N 8: L 64 7.3 there,
     // 14.8 here, L 200 12.2 and 17.4, L 1000 32.1 and 31.3; N 32: 9.3 and 15.1, 15.2 and 17.4, 41.4 and 32.0
-    // (L 4000 136 and 90).  Short caches and D = 64 stay there too: the start of a unit costs more here
+    // (L 4000 136 and 90).  (The mma.sync kernel has become faster with at most 32 rows since: N 8 6.5, 9.7 and 25.4
+    // there, N 32 8.3, 13.4, 30.8 and, at L 4000, 94.7.)  Short caches and D = 64 stay there too: the start of a unit costs more here
     // (D 64, 32 x 12, N 20, L 700 26.6 and 32.9).
     if (!attn_tcgen05_supports(p->D, G)) return GSD_ATTN_MMA;
     if (p->N * G >= 64 || (p->D == 128 && p->Lmax >= 512 && p->B * p->Hkv <= sm_count)) return GSD_ATTN_TCGEN05;

@@ -1,8 +1,8 @@
 // The marshalling of the calls that a serving loop makes every iteration, as a CPython extension:
 // dtype / shape / contiguity checks, output and scratch tensors from torch's allocator, the current
 // stream, and the C ABI call.  binding.py has the same in Python over ctypes, which takes 20 to 33 us a
-// call - longer than the kernels of a small step - against 4 to 12 us here (17 for the draft step, with
-// three launches); mask 4, acceptance 9, attention 7 to 12.
+// call - longer than the kernels of a small step - against 3 to 9 us here (commit 3, attention 4 to 5,
+// acceptance and draft step 8 to 9).
 //
 // Every function returns the call's result, a negative gsd_status as an int (binding.py raises), or
 // None when an argument is not the plain case (wrong dtype or shape, another device, a tensor
