@@ -23,9 +23,11 @@ namespace {
 constexpr int kRegParents = 4;
 constexpr int kEdgeCache = 4 * GSD_MAX_NODES;     // parent indices of one sequence kept in shared memory
 
+// (Plain pointers: the kernel is resident while its predecessor may still write the graph, so the inputs must
+// not be declared as data that nobody writes, which would let their loads go ahead of the wait.)
 __global__ void __launch_bounds__(GSD_MAX_NODES)
-build_mask_kernel(const int32_t* __restrict__ parent_ptr, const int32_t* __restrict__ parent_idx,
-                  uint32_t* __restrict__ mask, int b0, int N, int W, int Ecap, int32_t* status) {
+build_mask_kernel(const int32_t* parent_ptr, const int32_t* parent_idx, uint32_t* mask, int b0, int N, int W, int Ecap,
+                  int32_t* status) {
     __shared__ uint32_t s_rows[GSD_MAX_NODES];
     __shared__ int s_edge[kEdgeCache];
     volatile uint32_t* rows = s_rows;
