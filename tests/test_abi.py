@@ -80,3 +80,13 @@ def test_host_side_validation_needs_no_gpu(library):
                                                             ctypes.c_size_t(1 << 30), None, None]
     library.gsd_verify_step_host.restype = ctypes.c_int
     assert library.gsd_verify_step_host(*args) == -2
+
+
+def test_the_host_step_reserves_what_its_acceptance_asks_for(library):
+    # a key per slice of a row, so that few rows are cut there as they are in gsd_accept itself
+    import paper_2407_16207_b200 as gsd
+    B, N, Hq, Hkv, D, Lmax, V, Ecap = 1, 11, 8, 1, 128, 64, 128256, 40
+    parts = [B * N * Hq * D * 2] * 2 + [B * Lmax * Hkv * D * 2] * 2 + [B * N * Hkv * D * 2] * 2 + \
+            [B * N * 4, B * 4, B * N * V * 4, B * N * 4, B * (N + 1) * 4, B * Ecap * 4, B * N * 4, B * 4, B * N * 4, 4,
+             gsd.gsd_verify_attn_workspace_bytes(B, N, Hq, Hkv, D, Lmax), gsd.gsd_accept_workspace_bytes(B, N)]
+    assert gsd.gsd_verify_step_host_arena_bytes(B, N, Hq, Hkv, D, Lmax, V, Ecap, N) >= sum((n + 255) // 256 * 256 for n in parts)
