@@ -16,8 +16,8 @@ namespace {
 
 constexpr int kThreads = kPathThreads;
 constexpr int kNone = 0x7FFFFFFF;
-constexpr int kMaxSplits = 32;          // slices of a row
-constexpr int kWantCtas = 148 * 32;     // four waves of eight CTAs per SM
+constexpr int kWaveCtas = 32;           // CTAs of a call per SM: four waves of eight
+constexpr int kScratchSms = 148;        // SMs for which the scratch has room (with more of them the rows get fewer slices)
 
 struct Best {
     float v;
@@ -145,7 +145,10 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(AcceptArgs a) {
         a.keys[(size_t)split * a.B * a.N + row] = best.i == kNone ? 0ull : pack_key(best.v, best.i);
 }
 
-// Second launch: the best key of every node, then the path.
+// Second launch: the best key of every node, then the path.  kShare: the many slices of few rows are shared by
+// neighbouring threads (a form of its own: the two shifts cost the other calls 0.1 us).
+constexpr int kTrip = 8;                // slices whose keys a thread has on their way at a time
+template <bool kShare>
 __global__ void __launch_bounds__(kThreads) accept_tail_kernel(AcceptArgs a) {
     __shared__ int s_amax[GSD_MAX_NODES];
     let_successor_start();
@@ -161,26 +164,29 @@ __global__ void __launch_bounds__(kThreads) accept_tail_kernel(AcceptArgs a) {
     io.N = N; io.V = a.V; io.Ecap = a.Ecap; io.Tcap = a.Tcap;
     // the keys of a thread's nodes: neighbouring threads read neighbouring keys
     auto best_keys = [&]() -> unsigned {
+        int log_share = 0;
+        while (kShare && (kTrip << log_share) < a.splits && (2 * N << log_share) <= kThreads && log_share < 5) ++log_share;
+        const int share = 1 << log_share, node = tid >> log_share, mine = tid & (share - 1);
         wait_for_predecessor();
-        constexpr int kTrip = 8;                          // slices whose keys are on their way at a time
         const size_t rows = (size_t)a.B * N;
-        const unsigned long long* keys = a.keys + (size_t)b * N + tid;
+        const unsigned long long* keys = a.keys + (size_t)b * N + node;
         unsigned long long best[kPathNodeSlots] = {};
-        for (int s0 = 0; s0 < a.splits; s0 += kTrip) {
+        for (int s0 = mine; s0 < a.splits; s0 += kTrip * share) {
             unsigned long long k[kPathNodeSlots][kTrip];
 #pragma unroll
             for (int j = 0; j < kTrip; ++j)
 #pragma unroll
                 for (int i = 0; i < kPathNodeSlots; ++i)
-                    k[i][j] = s0 + j < a.splits && tid + i * kThreads < N ? __ldcg(keys + (s0 + j) * rows + i * kThreads) : 0ull;
+                    k[i][j] = s0 + j * share < a.splits && node + i * kThreads < N ? __ldcg(keys + (s0 + j * share) * rows + i * kThreads) : 0ull;
 #pragma unroll
             for (int j = 0; j < kTrip; ++j)
 #pragma unroll
                 for (int i = 0; i < kPathNodeSlots; ++i) best[i] = max(best[i], k[i][j]);
         }
+        for (int o = 1; o < share; o *= 2) best[0] = max(best[0], __shfl_xor_sync(0xFFFFFFFFu, best[0], o));
 #pragma unroll
         for (int i = 0; i < kPathNodeSlots; ++i)
-            if (tid + i * kThreads < N) s_amax[tid + i * kThreads] = key_index(best[i]);
+            if (mine == 0 && node + i * kThreads < N) s_amax[node + i * kThreads] = key_index(best[i]);
         return 0u;
     };
     // a step parent -> v is accepted iff v's token is what the target model would emit after the parent
@@ -198,9 +204,8 @@ __global__ void __launch_bounds__(kThreads) accept_tail_kernel(AcceptArgs a) {
 extern "C" size_t gsd_accept_workspace_bytes(const gsd_accept_params* p) {
     if (!p || p->B < 1 || p->N < 1 || p->N > GSD_MAX_NODES) return 0;
     // a key per slice: as many as the rule in gsd_accept can make of this many rows (the vocabulary may be
-    // given as anything here)
-    const size_t rows = (size_t)p->B * p->N;
-    const size_t keys = std::max(rows, std::min(rows * gsd::kMaxSplits, (size_t)2 * gsd::kWantCtas));
+    // given as anything here, and nothing asks for a device)
+    const size_t keys = std::max((size_t)p->B * p->N, (size_t)2 * gsd::kWaveCtas * gsd::kScratchSms);
     return std::max(gsd::accept_least_workspace(p->B, p->N), gsd::align_up(keys * 8, 256));
 }
 
@@ -221,6 +226,8 @@ extern "C" int gsd_accept(const float* logits, const int32_t* draft_tokens,
     const size_t need = accept_least_workspace(p->B, p->N);
     if (!workspace || workspace_bytes < need) return GSD_ERR_WORKSPACE;
     if (((uintptr_t)workspace & 7u) != 0) return GSD_ERR_MISALIGNED;
+    DeviceInfo di;
+    if (device_info(&di) != 0) return GSD_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
 
     AcceptArgs a;
@@ -231,11 +238,13 @@ extern "C" int gsd_accept(const float* logits, const int32_t* draft_tokens,
     a.B = p->B; a.N = p->N; a.V = p->V; a.Ecap = p->Ecap; a.Tcap = p->Tcap;
     // Slices of at least 4096 floats and CTAs for four waves (eight CTAs are resident per SM), so
     // that the last, partly filled wave is short: 2048 rows of 32000 take 50.7 us in one slice each
-    // (1.7 waves), 48.0 in two, 46.6 in four.
-    const size_t rows = (size_t)p->B * p->N;
+    // (1.7 waves), 48.0 in two, 46.6 in four.  (2 rows of 1048576, among other passes: 9.4 us with at most 32
+    // slices, 5.6 with the 256 that come of this.)
+    const size_t rows = (size_t)p->B * p->N, want = (size_t)kWaveCtas * di.sm_count;
     int splits = 1;
-    while (rows * splits < kWantCtas && splits < kMaxSplits && p->V / (splits * 2) >= 4096 && rows * splits * 2 * 8 <= workspace_bytes) splits *= 2;
+    while (rows * splits < want && p->V / (splits * 2) >= 4096 && rows * splits * 2 * 8 <= workspace_bytes) splits *= 2;
     a.splits = splits;
+    void (*tail)(AcceptArgs) = splits > kTrip && 2 * p->N <= kThreads ? accept_tail_kernel<true> : accept_tail_kernel<false>;
 
     // grid.y holds at most 65535 rows: larger problems go out in blocks of whole sequences
     const int seq_per = 65535 / p->N;
@@ -248,7 +257,7 @@ extern "C" int gsd_accept(const float* logits, const int32_t* draft_tokens,
         if (s.out_nodes) s.out_nodes += (size_t)b0 * p->Tcap;
         s.keys += (size_t)b0 * p->N * splits; s.B = nb;
         GSD_CUDA_TRY(launch_dependent(accept_kernel, dim3(splits, (unsigned)(nb * p->N)), dim3(kThreads), 0, st, s));
-        GSD_CUDA_TRY(launch_dependent(accept_tail_kernel, dim3((unsigned)nb), dim3(kThreads), 0, st, s));
+        GSD_CUDA_TRY(launch_dependent(tail, dim3((unsigned)nb), dim3(kThreads), 0, st, s));
     }
     return GSD_OK;
 }
@@ -258,7 +267,8 @@ extern "C" int gsd_accept(const float* logits, const int32_t* draft_tokens,
 // that lives in the library image, for callers that cannot hand over device memory.
 namespace gsd {
 namespace {
-// 8 bytes per draft node plus 4 bytes per sequence, for at most GSD_STATIC_MAX_ROWS rows.
+// A key per slice of every row, for at most GSD_STATIC_MAX_ROWS rows (the size is of an earlier layout with
+// more to keep per row).
 // Every GPU that loads the library holds these bytes until the process exits.
 static __device__ __align__(256) unsigned char g_accept_scratch[GSD_STATIC_SCRATCH_BYTES];
 }  // namespace

@@ -90,3 +90,10 @@ def test_the_host_step_reserves_what_its_acceptance_asks_for(library):
             [B * N * 4, B * 4, B * N * V * 4, B * N * 4, B * (N + 1) * 4, B * Ecap * 4, B * N * 4, B * 4, B * N * 4, 4,
              gsd.gsd_verify_attn_workspace_bytes(B, N, Hq, Hkv, D, Lmax), gsd.gsd_accept_workspace_bytes(B, N)]
     assert gsd.gsd_verify_step_host_arena_bytes(B, N, Hq, Hkv, D, Lmax, V, Ecap, N) >= sum((n + 255) // 256 * 256 for n in parts)
+
+
+def test_scratch_for_the_slices_of_few_rows(library):
+    # two rows of 2^20 entries are cut into 256 slices each, however few rows the call has
+    import paper_2407_16207_b200 as gsd
+    assert gsd.gsd_accept_workspace_bytes(1, 2) >= 2 * 256 * 8
+    assert gsd.gsd_accept_workspace_bytes(64, 256) >= 64 * 256 * 8

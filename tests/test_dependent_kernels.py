@@ -14,12 +14,10 @@ def sources():
 
 
 def dependents():
-    """Kernels launched by launch_dependent or with a launch configuration of their own, by name."""
+    """All kernels but those launched with <<<>>>, which start when everything before them is over."""
     text = "\n".join(sources().values())
-    names = set(re.findall(r"(?:launch_dependent\(|cudaLaunchKernelEx\(&cfg, )(\w+_kernel)\b", text))
-    for line in re.findall(r"kernel = .*", text):                  # (chosen among instances first)
-        names |= set(re.findall(r"\b(\w+_kernel)<", line))
-    return sorted(names)
+    names = set(re.findall(r"__global__ void[^;{]*?\b(\w+_kernel)\(", text))
+    return sorted(names - set(re.findall(r"\b(\w+_kernel)(?:<[^;<>]*>)?<<<", text)))
 
 
 def test_the_dependent_kernels_are_found():

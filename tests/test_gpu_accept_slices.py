@@ -39,7 +39,11 @@ def check(B, N, V, parents, agree=0.7):
 
 
 @pytest.mark.parametrize("B,N,V", [(1, 1, 8191), (1, 2, 8192), (1, 3, 131075), (2, 5, 16385), (3, 61, 50257), (5, 33, 12289),
-                                   (1, 512, 8200), (2, 257, 4096)])
+                                   (1, 512, 8200), (2, 257, 4096),
+                                   # more slices than a thread reads keys of at a time: shared by 2 to 32 threads a node, N
+                                   # on both sides of the half and the quarter of the threads, more than 32 slices
+                                   (1, 2, 1048576), (2, 1, 524289), (1, 20, 262147), (3, 63, 65536), (1, 64, 262144), (1, 65, 131072),
+                                   (1, 128, 131075), (1, 129, 131072)])
 def test_slices(B, N, V):
     rng = np.random.default_rng(N)
     check(B, N, V, [random_graph(rng, N, 2) for _ in range(B)], agree=0.4)
