@@ -2,8 +2,8 @@
 // partial results of every row.
 //   m = max_s m_s;  out = sum_s 2^(m_s - m) O_s / sum_s 2^(m_s - m) l_s
 //
-// A block of four warps has 32 rows of a row tile and eight of their column groups: a lane is a row, a thread
-// has two column groups (8 values, 16 bytes of output).  The rows of a column group are consecutive in the
+// A block of four warps has 32 rows of a row tile and eight of their column groups (one of eight warps sixteen): a lane
+// is a row, a thread has two column groups (8 values, 16 bytes of output).  The rows of a column group are consecutive in the
 // partial results, so every load of a warp is 512 contiguous bytes.  For items of fewer than 64 rows of
 // the mma.sync kernel a warp takes 8 rows and four column groups, one a thread, which leaves fewer lanes
 // without a row (D 64, whole call: 2 x 12 heads, N 40, L 1500 15.2 us, 15.5 with 32 rows a warp; 32/8
@@ -29,6 +29,12 @@ constexpr int kThreads = 128;
 constexpr int kBatchFew = 8, kBlocksFew = 3;
 constexpr int kBatchMany = 4, kBlocksMany = 4;
 constexpr int kWalkers = 592;    // blocks that walk over the items of a one-wave plan (four per SM)
+// Blocks of eight warps (sixteen column groups), half as many of them, where four small blocks a SM would do but not
+// three: the SMs that fall free first take five small blocks each and others are left with one or two.  512 small
+// blocks -> 256 of these, whole call: 4 x 24/8 heads, N 40, L 1500 17.2 -> 16.8 us (16.7 with the former pass), D 64, 8 x
+// 32/8, N 32, L 1500 18.9 -> 18.7, 2 x 64/8, N 32, L 4000 22.0 -> 21.6.  640 and 1280 small blocks are better small (1 x
+// 40 heads, N 100, L 8000 36.4 and 37.3; 5 x 24/8, N 77, L 300-1999 25.5 and 27.1): the eight warps end together.
+constexpr int kWideWarps = 8, kWideBlocks = 2, kWideUpTo = 4;
 
 struct MergeParams {
     const float4* part_o;
@@ -40,7 +46,7 @@ struct MergeParams {
     int RT;                  // of them in use
     int tiles;               // row tiles of an item
     int groups;              // runs of kRows rows of an item that can hold a row
-    int work;                // warps' worth of work
+    int work;                // blocks' worth of work
     int B;
     const int* bal_hdr;      // balanced plan: [0] = items to merge (known on the device only)
     const int4* bal_merge;   // balanced plan: (pair, first slot, slots) per pair to merge, else nullptr
@@ -60,13 +66,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // 64/8 heads, N 32, L 2048: 42.4 us with blocks for every item, 39.8 walking (37.1 with a plan that
 // cannot cut, which takes 115 instead of 28.5 when one of the sequences has 8192 and the others 500).
 // Where every item may be cut, one block for each part of it is up to 0.5 us faster.
-template <bool kWalk, int kRows, bool kFew>
-__global__ void __launch_bounds__(kThreads, kFew ? kBlocksFew : kBlocksMany) attn_merge_kernel(MergeParams p) {
+template <bool kWalk, int kRows, bool kFew, int kWarps = kThreads / 32>
+__global__ void __launch_bounds__(kWarps * 32, kWarps == kWideWarps ? kWideBlocks : kFew ? kBlocksFew : kBlocksMany) attn_merge_kernel(MergeParams p) {
     const int lane = threadIdx.x & 31;
     constexpr int kBatch = kFew ? kBatchFew : kBatchMany;
     constexpr int kGroups = kRows == 32 ? 2 : 1;                   // column groups of a thread
     constexpr int kSpan = 32 / kRows * kGroups;                    // of a warp
-    const int quads = p.D / 4, parts_of_row = quads / kSpan / (kThreads / 32);     // blocks that share a row
+    const int quads = p.D / 4, parts_of_row = quads / kSpan / kWarps;     // blocks that share a row
     // Launched as a programmatic dependent of the attention kernel: the blocks may become
     // resident while that kernel drains; what it (or the planning kernel) wrote is only visible
     // after this wait, which comes as late as the plan allows: working out a warp's place takes a
@@ -81,7 +87,7 @@ __global__ void __launch_bounds__(kThreads, kFew ? kBlocksFew : kBlocksMany) att
     }
     for (int w = (int)blockIdx.x; w < work; w += (int)gridDim.x) {                 // (once, unless kWalk)
     // first column group of the thread
-    const int col0 = (w % parts_of_row * (kThreads / 32) + (int)(threadIdx.x >> 5)) * kSpan + lane / kRows * kGroups;
+    const int col0 = (w % parts_of_row * kWarps + (int)(threadIdx.x >> 5)) * kSpan + lane / kRows * kGroups;
     const int g = w / parts_of_row % p.groups;
     const int k = w / parts_of_row / p.groups;
     // the k-th item that owns slots: group a comes first when it is split at all
@@ -252,7 +258,14 @@ int launch_attn_merge(const AttnArgs& a) {
     if (rows == 8) kernel = few ? attn_merge_kernel<false, 8, true> : attn_merge_kernel<false, 8, false>;    // (the mma.sync kernel has no one-wave plan)
     else if (walk) kernel = few ? attn_merge_kernel<true, 32, true> : attn_merge_kernel<true, 32, false>;
     else kernel = few ? attn_merge_kernel<false, 32, true> : attn_merge_kernel<false, 32, false>;
-    GSD_CUDA_TRY(launch_dependent(kernel, dim3((unsigned)blocks), dim3(kThreads), 0, a.stream, p));
+    int threads = kThreads;
+    if (rows == 32 && !walk && !few && blocks <= (long)kWideUpTo * di.sm_count) {
+        kernel = attn_merge_kernel<false, 32, false, kWideWarps>;
+        threads = kWideWarps * 32;
+        blocks = blocks * kThreads / threads;                      // (a row has two small blocks at least)
+        p.work = (int)blocks;
+    }
+    GSD_CUDA_TRY(launch_dependent(kernel, dim3((unsigned)blocks), dim3(threads), 0, a.stream, p));
     return GSD_OK;
 }
 

@@ -10,6 +10,9 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,D,N,kernel", [(1, 8, 2, 128, 40, "tc"), (9, 32, 8, 128, 70, "tc"),       # few blocks, many
+                                                 # 448, 512 and 592 of them: blocks of eight warps, 64 columns and 128
+                                                 (28, 4, 1, 128, 25, "tc"), (4, 32, 8, 128, 30, "tc"), (37, 4, 1, 128, 32, "tc"),
+                                                 (8, 32, 8, 64, 32, "auto"),
                                                  (1, 6, 6, 64, 21, "mma"), (3, 8, 2, 128, 30, "mma"), (40, 12, 12, 64, 33, "mma")])
 def test_number_of_parts(B, Hq, Hkv, D, N, kernel):
     import paper_2407_16207_b200 as gsd
@@ -18,7 +21,7 @@ def test_number_of_parts(B, Hq, Hkv, D, N, kernel):
     t = attn_tensors(gi.make_inputs(cfg, 3, accept=False))
     t["seq_lens"][0] = 5                               # nearly all of its parts are empty
     args = [t[n] for n in ("q", "k_cache", "v_cache", "draft_k", "draft_v", "ancestor_mask", "seq_lens")]
-    kern = gsd.GSD_ATTN_TCGEN05 if kernel == "tc" else gsd.GSD_ATTN_MMA
+    kern = {"tc": gsd.GSD_ATTN_TCGEN05, "mma": gsd.GSD_ATTN_MMA, "auto": gsd.GSD_ATTN_AUTO}[kernel]
     whole = out_to_f64(gsd.gsd_verify_attn(*args, kernel=kern, num_splits=1))
     for parts in (2, 3, 4, 5, 7, 8, 9, 12, 16, 17, 33, 64):
         got = out_to_f64(gsd.gsd_verify_attn(*args, kernel=kern, num_splits=parts))
