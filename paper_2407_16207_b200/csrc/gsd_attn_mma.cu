@@ -196,10 +196,10 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
     const int rloc[2] = {warp * 16 + (lane >> 2), warp * 16 + (lane >> 2) + 8};
     const bool rvalid[2] = {row0 + rloc[0] < R, row0 + rloc[1] < R};
 
-    // A warp whose 16 rows are all past the last one only helps to load: its share of the issue slots and
-    // of shared memory goes to the others (8 x 32 heads, N 8, L 200: 15.6 -> 12.2 us, L 1000: 43.4 -> 32.1;
-    // D 64, 4 x 12 heads, N 12, L 2000: 18.7 -> 15.4).
-    const bool active = row0 + warp * 16 < R;
+    // A warp whose 16 rows are all past the last one only helps to load: its share of the issue slots and of
+    // shared memory goes to the others (D 64, 4 x 12 heads, N 34, L 2000: 17.4 -> 17.2 us; at D 128 the test costs more
+    // than that: 8 x 32 heads, N 40, L 1500 56.7 -> 57.4).  Warps that share the keys of a tile all have rows.
+    const bool active = KEY_WARPS > 1 || row0 + warp * 16 < R;
     int t = next_live(t_begin);
     if (t < t_end) load_tile(t, 0);
     cp_async_commit();
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
         __syncthreads();
 
         if (active) {
-        // ---- S = Q K^T for 16 rows x 64 keys
+        // ---- S = Q K^T for 16 rows x KEYS keys
         float s[NT][4];
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
@@ -368,20 +368,17 @@ __global__ void __launch_bounds__(kThreads) attn_mma_kernel(MmaParams p) {
         float* part = reinterpret_cast<float*>(smem) + lane;
         auto part_of = [&](int k) { return part + (k * ROW_WARPS + warp) * (VALUES * 32); };
         __syncthreads();
-        if (active) {
-            float* at = part_of(kg);
+        float* at = part_of(kg);
 #pragma unroll
-            for (int dt = 0; dt < DT; ++dt)
+        for (int dt = 0; dt < DT; ++dt)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) at[(dt * 4 + e) * 32] = o[dt][e];
+            for (int e = 0; e < 4; ++e) at[(dt * 4 + e) * 32] = o[dt][e];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                at[(DT * 4 + h) * 32] = m_run[h];
-                at[(DT * 4 + 2 + h) * 32] = l_run[h];
-            }
+        for (int h = 0; h < 2; ++h) {
+            at[(DT * 4 + h) * 32] = m_run[h];
+            at[(DT * 4 + 2 + h) * 32] = l_run[h];
         }
         __syncthreads();
-        if (!active) return;
         float w[KEY_WARPS][2], r[SHARE][4];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
