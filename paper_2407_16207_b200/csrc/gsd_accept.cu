@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kThreads) accept_tail_kernel(AcceptArgs a) {
         return 0u;
     };
     // a step parent -> v is accepted iff v's token is what the target model would emit after the parent
-    const PathResult res = longest_accepted_path_ex<false>(
+    const PathResult res = longest_accepted_path<false>(
         io, 0u, [&](float, int p, int, int t) { return t == s_amax[p]; }, [](int, int) { return 0.f; }, best_keys);
     // the target model's own next token
     if (tid == 0 && res.edges < a.Tcap && GSD_IN_BOUNDS(res.end >= 0 && res.end < N && res.edges >= 0, a.status))

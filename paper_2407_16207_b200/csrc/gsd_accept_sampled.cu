@@ -262,7 +262,7 @@ __device__ void finish_sequence(const SampledArgs& a, int b) {
         io.N = N; io.V = V; io.Ecap = a.Ecap; io.Tcap = a.Tcap;
         // the test of one step: the target's probability of v's token under its parent p (one
         // logit gathered from global memory) against u q
-        const PathResult res = longest_accepted_path_ex<true>(
+        const PathResult res = longest_accepted_path<true>(
             io, 0u,
             [&](float logit, int p, int v, int) { return s_uq[v] < ex2((logit - s_mx[p]) * kLog2e) / s_sum[p]; },
             [&](int p, int t) -> float {

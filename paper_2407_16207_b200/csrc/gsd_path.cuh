@@ -50,9 +50,8 @@ struct PathResult {
 // and the values of `edge_pre` have been fetched.  `flags` carries status bits the caller has already
 // found; the function adds its own and publishes them.  All threads of the CTA must call it; all
 // return the same result.  out_tok[edges] is left for the caller, entries past it are set to -1.
-//
 template <bool kFetch, class StepOk, class EdgePre, class Mid>
-__device__ PathResult longest_accepted_path_ex(const PathIo& io, unsigned flags, StepOk step_ok, EdgePre edge_pre, Mid mid) {
+__device__ PathResult longest_accepted_path(const PathIo& io, unsigned flags, StepOk step_ok, EdgePre edge_pre, Mid mid) {
     __shared__ int s_best[GSD_MAX_NODES];         // edges of the longest accepted root path, -1: none
     __shared__ int s_tok[GSD_MAX_NODES];
     __shared__ int s_ptr[GSD_MAX_NODES + 1];
@@ -265,13 +264,6 @@ __device__ PathResult longest_accepted_path_ex(const PathIo& io, unsigned flags,
         }
     }
     return PathResult{m, end, s_child[end] != 0};
-}
-
-// The plain form: a test `step_ok(p, v, t)` that needs nothing fetched and nothing waited for.
-template <class StepOk>
-__device__ PathResult longest_accepted_path(const PathIo& io, unsigned flags, StepOk step_ok) {
-    return longest_accepted_path_ex<false>(
-        io, flags, [&](float, int p, int v, int t) { return step_ok(p, v, t); }, [](int, int) { return 0.f; }, []() { return 0u; });
 }
 
 }  // namespace gsd
