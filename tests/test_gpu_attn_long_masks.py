@@ -12,7 +12,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,D,N,L", [(1, 2, 2, 128, 129, 100), (2, 3, 3, 128, 161, 300), (1, 24, 8, 128, 512, 130), (2, 2, 2, 64, 346, 700),
-                                            (3, 60, 60, 128, 289, 40), (7, 64, 64, 128, 257, 20), (1, 1, 1, 128, 512, 0)])
+                                            (3, 60, 60, 128, 289, 40), (7, 64, 64, 128, 257, 20), (1, 1, 1, 128, 512, 0),
+                                            # one word fewer than the shared form needs and one more, groups of one to three
+                                            (2, 3, 3, 128, 170, 100), (2, 3, 3, 128, 171, 100), (1, 4, 2, 128, 256, 100),
+                                            (1, 4, 2, 128, 257, 100), (1, 6, 2, 64, 384, 60), (1, 6, 2, 64, 385, 60)])
 @pytest.mark.parametrize("shift", [0, 1])
 def test_live_tiles_of_long_masks(B, Hq, Hkv, D, N, L, shift):
     import paper_2407_16207_b200 as gsd
