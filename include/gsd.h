@@ -244,7 +244,7 @@ size_t gsd_accept_workspace_bytes(const gsd_accept_params* p);
  *   accepted_tokens, accepted_len, accepted_nodes   device outputs as for gsd_accept; the entry
  *                    after the drafted tokens of the path is the regenerated token
  *   workspace        device scratch of gsd_accept_sampled_workspace_bytes(p) bytes, 8-byte
- *                    aligned, arbitrary contents; the call clears what has to start at zero
+ *                    aligned, arbitrary contents
  * The softmax statistics are accumulated in fp32 (ex2.approx); a step whose two sides differ by
  * less than a few 1e-6 relative may be decided differently from an exact evaluation.
  * Errors and status bits as for gsd_accept, plus GSD_DEV_BAD_LOGITS.  Asynchronous on `stream`.

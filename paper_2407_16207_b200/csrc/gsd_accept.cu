@@ -237,9 +237,9 @@ extern "C" int gsd_accept(const float* logits, const int32_t* draft_tokens,
     a.status = status;
     a.B = p->B; a.N = p->N; a.V = p->V; a.Ecap = p->Ecap; a.Tcap = p->Tcap;
     // Slices of at least 4096 floats and CTAs for four waves (eight CTAs are resident per SM), so
-    // that the last, partly filled wave is short: 2048 rows of 32000 take 50.7 us in one slice each
-    // (1.7 waves), 48.0 in two, 46.6 in four.  (2 rows of 1048576, among other passes: 9.4 us with at most 32
-    // slices, 5.6 with the 256 that come of this.)
+    // that the last, partly filled wave is short: in captured graphs 2048 rows of 32000 take 44.5 us in one slice
+    // each (1.7 waves), 42.5 in four; 60 rows of 128256 24.8 in one, 10.6 in sixteen; 2 rows of 1048576 9.3 in 32, 5.5
+    // in the 256 that come of this.
     const size_t rows = (size_t)p->B * p->N, want = (size_t)kWaveCtas * di.sm_count;
     int splits = 1;
     while (rows * splits < want && p->V / (splits * 2) >= 4096 && rows * splits * 2 * 8 <= workspace_bytes) splits *= 2;

@@ -55,14 +55,16 @@ int attn_pick_kernel(const gsd_attn_params* p, int sm_count) {
     const int G = p->Hq / p->Hkv;
     // Fewer rows leave most of a tile empty, and then it depends on the context, which is not known
     // here: Lmax is the room in the cache.  At D = 128 and 512 or more cache rows, with no more items than
-    // SMs, the tcgen05 kernel is the faster one for any context (mma.sync -> tcgen05, us: 1 x 32 heads, N 8,
-    // L 64 12.4 -> 8.8, L 1000 17.5 -> 12.0; 1 x 64/8, N 4, L 200 10.5 -> 9.9; 4 x 32, N 48, L 64 14.7 -> 9.3,
-    // L 4000 102 -> 46.6).  With more items its second round of units costs short contexts more than long
-    // ones gain - and the cache of a server is mostly empty early on: 8 x 32 heads, N 8: L 64 7.3 there,
-    // 14.8 here, L 200 12.2 and 17.4, L 1000 32.1 and 31.3; N 32: 9.3 and 15.1, 15.2 and 17.4, 41.4 and 32.0
-    // (L 4000 136 and 90).  (The mma.sync kernel has become faster with at most 32 rows since: N 8 6.5, 9.7 and 25.4
-    // there, N 32 8.3, 13.4, 30.8 and, at L 4000, 94.7.)  Short caches and D = 64 stay there too: the start of a unit costs more here
-    // (D 64, 32 x 12, N 20, L 700 26.6 and 32.9).
+    // SMs, the tcgen05 kernel is the faster one from about 24 rows on, for any context (mma.sync and tcgen05,
+    // us, in 4096 cache rows: 4 x 32 heads, N 48, L 64 14.7 and 9.5, L 4000 96.9 and 47.3; 4 x 32, N 24, L 1000 21.7 and
+    // 18.1; 1 x 32, N 24, L 64 9.5 and 9.6, L 4000 20.6 and 19.9).  With at most 16 rows the mma.sync kernel, as it is
+    // now, is 1 to 4 us faster on up to 64 items (1 x 32, N 8, L 64 7.9 and 9.2, L 1000 11.5 and 13.1, L 16000 48.6 and
+    // 47.7; 2 x 32, N 8, L 1000 13.0 and 16.6) and even on 128 (4 x 32, N 8, L 1000 18.1 and 18.0): the line was drawn
+    // with an earlier form of it.  With more items than SMs a second round of units here costs short contexts more than
+    // long ones gain, and the cache of a server is mostly empty early on: 8 x 32 heads, L 64 / 200 / 1000 / 4000, N 8
+    // 7.0 / 11.3 / 25.5 / 79.4 there, 15.3 / 18.2 / 32.6 / 92.7 here; N 32 10.4 / 14.4 / 30.0 / 91.7 and 16.6 / 19.3 /
+    // 33.5 / 94.7; N 48 11.9 / 18.2 / 41.9 / 136 and 16.5 / 19.6 / 34.0 / 95.7.  Short caches and D = 64 stay there too:
+    // the start of a unit costs more here (D 64, 32 x 12, N 20, L 700 26.6 and 32.9 with that earlier form).
     if (!attn_tcgen05_supports(p->D, G)) return GSD_ATTN_MMA;
     if (p->N * G >= 64 || (p->D == 128 && p->Lmax >= 512 && p->B * p->Hkv <= sm_count)) return GSD_ATTN_TCGEN05;
     return GSD_ATTN_MMA;

@@ -23,9 +23,10 @@ namespace {
 
 constexpr int kThreads = 128;
 // Parts of a row on their way at a time, and blocks per SM that have to be resident: many parts are worth
-// more than occupancy as long as all blocks are resident at once (1 x 8 items of 18 parts, 256 rows: 49.5 us
-// the whole call with four, 46.4 with eight), else it is the other way round (40 items of 3 to 5 parts: 24.2
-// with four, 26.0 with eight; limited to 64 registers, eight blocks an SM, calls took up to 2 us more).
+// more than occupancy as long as all blocks are resident at once (the whole call in captured graphs: 8 items of 18
+// parts, 256 rows, 42.2 us with four, 40.9 with eight; 32 items of 4 parts, 64 rows, 15.8 and 15.5), else it is the other
+// way round (40 items of 3 to 5 parts: 24.2 with four, 26.0 with eight; limited to 64 registers, eight blocks an SM,
+// calls took up to 2 us more).
 constexpr int kBatchFew = 8, kBlocksFew = 3;
 constexpr int kBatchMany = 4, kBlocksMany = 4;
 constexpr int kWalkers = 592;    // blocks that walk over the items of a one-wave plan (four per SM)

@@ -1436,8 +1436,9 @@ static int launch_plan(const AttnArgs& a) {
 }
 
 // The mask words of a unit are more than a warp fetches in one round of 16-byte loads (one head a group: N above
-// 170, two: above 256, three: above 384, four and more: never).  A kernel of its own: the code for slices in the others' prologue cost calls of a few tiles up to
-// 4%; with up to 1024 words it is a wash (D 64, 4 x 32/8 heads, N 428, L 20322, 896 words: 586 us, 592 so).
+// 170, two: above 256, three: above 384, four and more: never).  A kernel of its own: the code for slices in the
+// others' prologue cost calls of a few tiles up to 4%; with up to 1024 words it is a wash (D 64, 4 x 32/8 heads, N 428,
+// L 20322, 896 words: 586 us, 592 so).
 static bool long_mask(const AttnArgs& a) {
     const int nodes = 2 * (BM / a.G);
     return (nodes < a.N ? nodes : a.N) * a.W > 8 * 32 * 4;
