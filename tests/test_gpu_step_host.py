@@ -66,3 +66,21 @@ def test_step_from_host_buffers_with_plans_made_on_the_device(num_splits):
         assert err.max() <= 1e-2 and err.mean() <= 1e-3
         wt, wl, wn, _ = oracle.accept(inp["logits"], inp["draft_tokens"], inp["parent_ptr"], inp["parent_idx"])
         assert np.array_equal(toks.numpy(), wt) and np.array_equal(lens.numpy(), wl) and np.array_equal(nodes.numpy(), wn)
+
+
+def test_an_arena_with_scratch_for_whole_rows_only_is_accepted():
+    # a key per row behind everything else, as the arena once was; one page less is refused
+    import paper_2407_16207_b200 as gsd
+    cfg = gi.VerifyConfig("h", 7, 1, 4, 4, 64, 100, 11, 5, 3, 2, 70000, 11, 0.6)
+    inp = gi.make_inputs(cfg, 4)
+    h = {k: v.pin_memory() for k, v in {**attn_tensors(inp, "cpu"), **accept_tensors(inp, "cpu")}.items()}
+    names = ("q", "k_cache", "v_cache", "draft_k", "draft_v", "ancestor_mask", "seq_lens", "logits", "draft_tokens", "parent_ptr", "parent_idx")
+    nbytes = gsd.gsd_verify_step_host_arena_bytes(cfg.B, cfg.N, cfg.Hq, cfg.Hkv, cfg.D, inp["Lmax"], cfg.V, h["parent_idx"].shape[1], cfg.N)
+    least = nbytes - gsd.gsd_accept_workspace_bytes(cfg.B, cfg.N) + (cfg.B * cfg.N * 8 + cfg.B * 4 + 255) // 256 * 256
+    wt, wl, wn, _ = oracle.accept(inp["logits"], inp["draft_tokens"], inp["parent_ptr"], inp["parent_idx"])
+    for size in (least, nbytes, nbytes + (1 << 20)):
+        arena = torch.empty(size, dtype=torch.uint8, device="cuda")
+        _, toks, lens, nodes, status = gsd.gsd_verify_step_host(*(h[n] for n in names), arena)
+        assert status == 0 and np.array_equal(toks.numpy(), wt) and np.array_equal(lens.numpy(), wl) and np.array_equal(nodes.numpy(), wn)
+    with pytest.raises(gsd.GsdError):
+        gsd.gsd_verify_step_host(*(h[n] for n in names), torch.empty(least - 256, dtype=torch.uint8, device="cuda"))
